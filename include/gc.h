@@ -64,9 +64,9 @@ typedef struct {
     int32_t region_hops; /* k of the k-hop region; 0 -> 3 as in Sec. 4.2; must be >= 2 */
     float slack;         /* spare capacity per adjacency row; 0 -> 0.25 */
     int32_t device;      /* CUDA device ordinal; 0 -> current device */
-    int32_t dense_cluster; /* CTAs per cluster of the heavy 4-cycle kernel: 0 auto, 8 or 16 */
-    int32_t chunk_threshold; /* wedge bound above which a 4-cycle pivot is counted in shared memory
-                                over id-range chunks; <= 0: never (the cluster kernel takes them) */
+    int32_t dense_cluster; /* 0, 8 or 16; no effect (heavy 4-cycle pivots use no clusters) */
+    int32_t chunk_threshold; /* initial gc_tuning.c4_chunk_min when > 0; no effect (every heavy
+                                4-cycle pivot is counted in shared memory over id-range chunks) */
     int32_t local_max_pairs; /* batches of at most this many pairs (as passed) to gc_apply_batch,
                                 gc_count_batch and their _device forms, and such batches within
                                 gc_apply_batches* runs (taken one at a time, in order), take the
@@ -109,8 +109,8 @@ typedef struct {
     /* device time per stage (CUDA events):
        [0] normalise  [1] region walk  [2] union graph  [3] triangles + 4-cliques
        [4] 4-cycles   [5] edge terms + closed forms     [6] commit
-       [7] the heavy-pivot 4-cycle kernels alone (k_c4_dense_t and, when a
-           tuning enables it, k_c4_chunk), timed on the stream they run on
+       [7] the heavy-pivot 4-cycle kernels alone (plan, runs and k_c4_pivot),
+           timed on the stream they run on
        Stages 3 and 4 run side by side: each is timed from the start of the
        counting pass to its own end. */
     float ms_stage[8];
@@ -123,8 +123,7 @@ typedef struct {
                                        (open wedges), [1] triangles */
     /* work of the heavy-pivot 4-cycle kernels of ms_stage[7], for their own
        roofline: the wedges they walked, and the counter updates they sent to
-       L2 (reductions that return nothing; atomics that return the old value;
-       the shared-memory counters of k_c4_chunk send none) */
+       L2 (none: they count in shared memory) */
     int64_t work_wedges_heavy;
     int64_t l2_red_heavy, l2_atom_heavy;
 } gc_stats;
@@ -366,11 +365,10 @@ typedef struct {
     int32_t c4_reg_max;     /* registers                        [32]    */
     int32_t c4_warp_max;    /* warp hash in shared memory       [512]   */
     int32_t c4_block_max;   /* block hash in shared memory      [8192]  */
-    int64_t c4_cta_max;     /* per-CTA hash table in L2         [32768] */
-    int64_t c4_chunk_min;   /* above this and up to c4_chunk_max: shared-memory counters over
-                               id-range chunks; other pivots above c4_cta_max: a CTA cluster on a
-                               dense array in L2; 0 = never */
-    int64_t c4_chunk_max;   /* 0 = no upper bound */
+    int64_t c4_cta_max;     /* block hash, large table; at most 19456 is used, pivots beyond are
+                               counted in shared memory over id-range chunks     [32768] */
+    int64_t c4_chunk_min;   /* kept as set; no effect */
+    int64_t c4_chunk_max;   /* kept as set; no effect */
     int64_t local_max_pairs; /* batches of at most this many pairs take the edge-local delta
                                 (gc_options.local_max_pairs); 0 = never */
     int64_t local_c4_heavy_min; /* gc_vertex_* and gc_edge_*: 4-cycle pivots with w~ at least this

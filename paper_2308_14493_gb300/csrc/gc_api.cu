@@ -82,13 +82,7 @@ struct gc_graph {
     Buf<unsigned long long> out_dev;     // per-batch results of a batched run
     Buf<int32_t> vids, vdeg;             // vertex deletion: ids and their degrees
     Buf<long long> voff;                 // vertex deletion: pair offsets
-    Buf<unsigned long long> dense;       // counter arrays of the heaviest 4-cycle pivots (per cluster)
-    int dense_clusters = 0;
-    int dense_cluster_size = 8;
-    Buf<unsigned long long> cta_tables;  // hash tables of the medium 4-cycle pivots (per CTA)
-    int cta_groups = 0;
-    Buf<unsigned char> chunk_table;      // per-CTA run bounds of the chunked 4-cycle kernel
-    long long chunk_cap = 0;             // run-bound entries per CTA in it
+    Buf<unsigned char> c4_buf;           // plan, run bounds and lists of the shared-memory 4-cycle pivots
     Tuning tune = default_tuning();     // bin boundaries of the counting pass
     long long loc_heavy_min = 65536;   // w~ from which local-count 4-cycle pivots take k_c4_group (0 = never)
     int32_t* bins = nullptr;             // NBINS * n work lists of the counting pass
@@ -567,15 +561,29 @@ static void trim_scratch(gc_graph* g) {
     if (g->s) cudaStreamSynchronize(g->s);
 }
 
-// Scratch of the chunked 4-cycle kernel: per CTA, the run bounds of one
-// pivot's lower neighbours (c4_chunk_cap entries for this n), allocated when
-// a tuning first enables that tier.
-static bool ensure_chunk_table(gc_graph* g) {
-    const long long cap = c4_chunk_cap(std::max(g->n, 1));
-    if (!ensure(g, g->chunk_table, (size_t)g->sms * c4_chunk_cta_bytes(cap))) return false;
-    g->chunk_cap = cap;
-    return true;
+// Buffers of the shared-memory 4-cycle pivots for the current n, carved from
+// one allocation.
+static size_t carve_c4(const gc_graph* g, C4Bufs* b) {
+    const long long n = std::max(g->n, 1);
+    const C4Geom m = c4_geom(n, g->sms);
+    size_t at = 0;
+    auto take = [&](size_t bytes) {
+        void* p = g->c4_buf.p ? g->c4_buf.p + at : nullptr;
+        at += (bytes + 255) & ~(size_t)255;
+        return p;
+    };
+    C4Bufs o;
+    o.head = (C4Head*)take(sizeof(C4Head));
+    o.chunk = (C4Chunk*)take(sizeof(C4Chunk) * (size_t)m.nchmax);
+    o.gmax = (int32_t*)take(4 * (size_t)m.ngran);
+    o.sorted = (int32_t*)take(4 * (size_t)n);
+    o.list = (uint32_t*)take(4 * (size_t)m.ctas * C4_LIST);
+    o.lcap = C4_LIST;
+    o.run = (unsigned long long*)take(8 * (size_t)m.group * (size_t)n);
+    if (b) *b = o;
+    return at;
 }
+static bool ensure_c4(gc_graph* g) { return ensure(g, g->c4_buf, carve_c4(g, nullptr)); }
 
 static int ensure_desc(gc_graph* g, long long words) {
     if (g->desc && g->desc_cap >= words) return GC_OK;
@@ -632,15 +640,8 @@ static int count_region(gc_graph* g, int fin, bool set_F, bool timed, bool twin 
     ca.db = g->db;
     ca.tpack = g->tpack.p;
     ca.bins = g->bins;
-    ca.dense = g->dense.p;
     ca.n_alloc = std::max(g->n, 1);
-    ca.dense_clusters = g->dense_clusters;
-    ca.dense_cluster_size = g->dense_cluster_size;
-    ca.cta_tables = g->cta_tables.p;
-    ca.cta_table_words = 2 * C4_T3;
-    ca.cta_groups = g->cta_groups;
-    ca.chunk_scratch = g->chunk_table.p;
-    ca.chunk_cap = g->chunk_table.p ? g->chunk_cap : 0;
+    carve_c4(g, &ca.c4);
     ca.tune = g->tune;
     ca.sms = g->sms;
     for (int i = 0; i < 3; i++) {
@@ -1386,9 +1387,7 @@ static void destroy(gc_graph* g) {
     release(g, g->vids);
     release(g, g->vdeg);
     release(g, g->voff);
-    release(g, g->dense);
-    release(g, g->cta_tables);
-    release(g, g->chunk_table);
+    release(g, g->c4_buf);
     dfree(g, g->bins);
     if (g->s) cudaStreamSynchronize(g->s);
     if (g->h_ctl) cudaFreeHost(g->h_ctl);
@@ -1532,20 +1531,11 @@ static int open_device(gc_graph* g, const int32_t* row_ptr, const int32_t* colh)
     dfree(g, d_rp); dfree(g, d_col); dfree(g, deg0); dfree(g, key_off); dfree(g, bad); dfree(g, k1); dfree(g, k2);
     if (rc) return rc;
     g->m = m2 / 2;
-    // counting pass: work lists, one dense counter array per cluster of the
-    // heaviest 4-cycle pivots and one hash table per CTA of the medium ones
-    // (all kept zero between pivots)
+    // counting pass: work lists and the buffers of the shared-memory 4-cycle pivots
     count_setup_attributes();
     local_setup_attributes();
     g->bins = (int32_t*)dalloc(g, sizeof(int32_t) * (size_t)NBINS * nn);
-    g->dense_clusters = dense_cluster_plan(g->opt.dense_cluster, g->sms, &g->dense_cluster_size);
-    if (!g->bins || !ensure(g, g->dense, (size_t)g->dense_clusters * (size_t)dense_stride((long long)nn)))
-        return nomem(g, "counting work lists");
-    CK(cudaMemsetAsync(g->dense.p, 0, 8 * g->dense.cap, s));
-    g->cta_groups = g->sms;
-    if (!ensure(g, g->cta_tables, (size_t)g->cta_groups * 2 * C4_T3)) return nomem(g, "4-cycle hash tables");
-    if (g->tune.c4_chunk_min < NEVER && !ensure_chunk_table(g)) return nomem(g, "4-cycle chunk table");
-    CK(cudaMemsetAsync(g->cta_tables.p, 0, 8 * g->cta_tables.cap, s));
+    if (!g->bins || !ensure_c4(g)) return nomem(g, "counting work lists");
     return count_static(g, true, nullptr);
 }
 
@@ -2068,16 +2058,9 @@ static int grow_vertices(gc_graph* g, long long k) {
     pdl_launch(k_init_new_vertices, dim3(grid_elems(g, k)), dim3(TPB), 0, s, g->perm, g->iperm, g->deg, g->cap,
                g->row_start, n0, n1);
     CKL();
-    release(g, g->dense);
-    if (!ensure(g, g->dense, (size_t)g->dense_clusters * (size_t)dense_stride((long long)nn)))
-        return nomem(g, "4-cycle counter arrays");
-    CK(cudaMemsetAsync(g->dense.p, 0, 8 * g->dense.cap, s));
     g->n = n1;
     g->S = std::max(1, bitlen(n1 > 0 ? n1 - 1 : 0));
-    if (g->chunk_table.p) {
-        release(g, g->chunk_table);
-        if (!ensure_chunk_table(g)) return nomem(g, "4-cycle chunk table");
-    }
+    if (!ensure_c4(g)) return nomem(g, "4-cycle buffers");
     for (int i = 0; i < 3; i++)
         if (g->qexec[i]) {
             cudaGraphExecDestroy(g->qexec[i]);
@@ -2358,7 +2341,6 @@ int gc_set_tuning(gc_graph* g, const gc_tuning* t) {
     n.c4_cta_max = t->c4_cta_max;
     n.c4_chunk_min = t->c4_chunk_min == 0 ? NEVER : t->c4_chunk_min;
     n.c4_chunk_max = t->c4_chunk_max == 0 ? NEVER : t->c4_chunk_max;
-    if (n.c4_chunk_min < NEVER && !ensure_chunk_table(g)) return nomem(g, "4-cycle chunk table");
     g->tune = n;
     g->opt.local_max_pairs = (int32_t)std::min<int64_t>(t->local_max_pairs, INT32_MAX);
     g->loc_heavy_min = t->local_c4_heavy_min;
@@ -2483,53 +2465,37 @@ int gc_autotune(gc_graph* g, int32_t reps, gc_tuning* best, float* best_ms) {
     int rc = time_static(g, reps, &cur_ms, ref);
     if (rc) return rc;
     // candidate values per boundary; coordinate descent, at most three sweeps
-    // (a bound below the tier beneath it empties the tier; the chunked
-    // kernel only takes pivots above c4_cta_max, so lowering that one after
-    // c4_chunk_min opens the chunked tier to medium pivots)
-    const long long cand[9][6] = {
-        {16, 32, -1, -1, -1, -1},                          // tri_warp_max
-        {64, 128, -1, -1, -1, -1},                         // tri_small_max
-        {256, 512, -1, -1, -1, -1},                        // tri_block_max
-        {16, 32, -1, -1, -1, -1},                          // c4_reg_max
-        {128, 512, -1, -1, -1, -1},                        // c4_warp_max
-        {512, 2048, 8192, -1, -1, -1},                     // c4_block_max
-        {2048, 8192, 16384, 32768, -1, -1},                // c4_cta_max
-        {NEVER, 2048, 8192, 32768, 262144, 1048576},       // c4_chunk_min
-        {NEVER, 131072, 524288, 2097152, -1, -1}            // c4_chunk_max
+    // (a bound below the tier beneath it empties the tier)
+    const int cand[7][3] = {
+        {16, 32, -1},       // tri_warp_max
+        {64, 128, -1},      // tri_small_max
+        {256, 512, -1},     // tri_block_max
+        {16, 32, -1},       // c4_reg_max
+        {128, 512, -1},     // c4_warp_max
+        {512, 2048, 8192},  // c4_block_max
+        {2048, 8192, 32768}, // c4_cta_max
     };
-    auto field = [](Tuning& t, int i) -> long long {
+    auto field = [](const Tuning& t, int i) -> int {
+        const int v[7] = {t.tri_warp_max, t.tri_small_max, t.tri_block_max, t.c4_reg_max,
+                          t.c4_warp_max,  t.c4_block_max,  (int)std::min<long long>(t.c4_cta_max, INT32_MAX)};
+        return v[i];
+    };
+    auto set = [](Tuning& t, int i, int v) {
         switch (i) {
-            case 0: return t.tri_warp_max;
-            case 1: return t.tri_small_max;
-            case 2: return t.tri_block_max;
-            case 3: return t.c4_reg_max;
-            case 4: return t.c4_warp_max;
-            case 5: return t.c4_block_max;
-            case 6: return t.c4_cta_max;
-            case 7: return t.c4_chunk_min;
-            default: return t.c4_chunk_max;
+            case 0: t.tri_warp_max = v; break;
+            case 1: t.tri_small_max = v; break;
+            case 2: t.tri_block_max = v; break;
+            case 3: t.c4_reg_max = v; break;
+            case 4: t.c4_warp_max = v; break;
+            case 5: t.c4_block_max = v; break;
+            default: t.c4_cta_max = v; break;
         }
     };
-    auto set = [](Tuning& t, int i, long long v) {
-        switch (i) {
-            case 0: t.tri_warp_max = (int)v; break;
-            case 1: t.tri_small_max = (int)v; break;
-            case 2: t.tri_block_max = (int)v; break;
-            case 3: t.c4_reg_max = (int)v; break;
-            case 4: t.c4_warp_max = (int)v; break;
-            case 5: t.c4_block_max = (int)v; break;
-            case 6: t.c4_cta_max = v; break;
-            case 7: t.c4_chunk_min = v; break;
-            default: t.c4_chunk_max = v; break;
-        }
-    };
-    const bool chunk_ok = ensure_chunk_table(g);
     for (int sweep = 0; sweep < 3; sweep++) {
         bool moved = false;
-        for (int i = 8; i >= 0; i--) {
-            if (i >= 7 && !chunk_ok) continue;
-            for (int k = 0; k < 6; k++) {
-                const long long v = cand[i][k];
+        for (int i = 6; i >= 0; i--) {
+            for (int k = 0; k < 3; k++) {
+                const int v = cand[i][k];
                 if (v < 0 || v == field(cur, i)) continue;
                 Tuning t = cur;
                 set(t, i, v);

@@ -37,26 +37,23 @@ enum {
     BIN_TRI_MERGE = 2,  // k > TRI_KM                      merge per out-edge
     BIN_C4_REG = 3,     // w~ <= 32                        registers (match)
     BIN_C4_WARP = 4,    // w~ <= C4_T1                     warp hash in shared memory
-    BIN_C4_BLOCK = 5,   // C4B_SMALL_MAX < w~ <= C4_T2     block hash in shared memory
-    BIN_C4_DENSE = 6,   // C4_T3 < w~ <= c4_chunk_min      cluster, shared dense counter array
-    BIN_C4_CTA = 7,     // C4_T2 < w~ <= C4_T3             CTA, own hash table in global memory
-    BIN_C4_CHUNK = 8,   // w~ > c4_chunk_min (off)         CTA, shared-memory counters over id-range chunks
-    BIN_TRI_SMALL = 9,  // 32 < k <= TRI_KS                block per root, small shared footprint
-    BIN_C4_BSMALL = 10, // w~ <= C4B_SMALL_MAX             block hash in shared memory, small table
-    NBINS = 11
+    BIN_C4_BLOCK = 5,   // C4B_SMALL_MAX < w~ <= C4_T2     block hash in shared memory, medium table
+    BIN_C4_DENSE = 6,   // w~ > C4_T3                      counters of an id chunk in shared memory
+    BIN_TRI_SMALL = 7,  // 32 < k <= TRI_KS                block per root, small shared footprint
+    BIN_C4_BSMALL = 8,  // w~ <= C4B_SMALL_MAX             block hash in shared memory, small table
+    BIN_C4_BIG = 9,     // C4_T2 < w~ <= C4_T3             block hash in shared memory, large table
+    NBINS = 10
 };
 
 // Work counters (Ctl::work) of the kernels that take their roots or pivots
 // one at a time; kernels that run side by side need different counters.
 enum {
     WORK_TRI_BLOCK = 1,   // k_tri_block, long out-lists
-    WORK_C4_BLOCK = 2,    // k_c4_block, large table
-    WORK_C4_DENSE = 3,    // k_c4_dense_t, clusters
-    WORK_C4_CTA = 4,      // k_c4_hash (and k_c4_dense_t without clusters)
-    WORK_C4_CHUNK = 5,    // k_c4_chunk
-    WORK_TRI_SMALL = 6,   // k_tri_block, short out-lists
-    WORK_C4_BSMALL = 7,   // k_c4_block, small table
-    NWORK = 8
+    WORK_C4_BLOCK = 2,    // k_c4_table, medium table
+    WORK_TRI_SMALL = 3,   // k_tri_block, short out-lists
+    WORK_C4_BSMALL = 4,   // k_c4_table, small table
+    WORK_C4_BIG = 5,      // k_c4_table, large table
+    NWORK = 6
 };
 
 constexpr int ACC_STRIPES = 32;  // copies of each accumulator (spreads the atomics of many warps)
@@ -76,8 +73,8 @@ struct Ctl {
                                      // [12] |E(G_a)|, [13] |E(G_b)|, [14] triangle work, [15] wedges
                                      // [16] sum of t_e in G_a (3 triangles), [17] in G_b,
                                      // [18] sum C(d,2) in G_a (2-paths), [19] in G_b
-                                     // heavy-pivot 4-cycle tier: [20] wedges, [21] L2
-                                     // reductions, [22] L2 atomics returning the old value
+                                     // shared-memory 4-cycle pivots: [20] wedges ([21] L2
+                                     // reductions and [22] L2 atomics of theirs: none)
     unsigned long long F[6];         // maintained counts
     long long Ca[6], Cb[6];          // induced counts of G_a, G_b of the last pass
     long long sa[6], sb[6];          // their non-induced sums (TT halved)
@@ -116,6 +113,8 @@ struct Ctl {
                                      // [3] 4-cycle tasks [4] 4-cycle probes
     long long l_need;                // entries the largest local array needed
     int l_nw3;                       // third vertices listed after V_X (maintained triangle sums)
+    // wedge bounds of the pivots counted in shared memory (BIN_C4_DENSE): sum and maximum
+    unsigned long long c4_wt, c4_wmax;
     // (device-only tail: the host mirror copies the block up to here)
     unsigned long long accs[NACC][ACC_STRIPES];  // acc, striped: kernels add here, k_finalize sums
 };
@@ -125,10 +124,7 @@ constexpr int TRI_KS = 128;
 constexpr int C4_T1 = 512;
 constexpr int C4_T2 = 8192;
 constexpr int C4B_SMALL_MAX = 2048;  // block-hash pivots up to this bound use the small table
-constexpr long long C4_T3 = 32768;
-constexpr int C4_CLUSTER = 8;       // CTAs per cluster of the dense 4-cycle kernel
-constexpr int CH_BYTES = 196608;    // shared counter bytes of the chunked 4-cycle kernel
-constexpr int CH_R = CH_BYTES / 4;  // ids per chunk (49,152)
+constexpr long long C4_T3 = 19456;   // 3/4 of the large table's slots, less a few
 
 // Bin boundaries of the counting pass (upper bounds of each tier; each at
 // most the capacity its kernel was compiled for).  Chosen per graph by the
@@ -140,13 +136,13 @@ struct Tuning {
     int c4_reg_max;          // wedge bound w~: registers up to this (<= 32)
     int c4_warp_max;         // warp hash (<= C4_T1)
     int c4_block_max;        // block hash (<= C4_T2)
-    long long c4_cta_max;    // global hash tables (<= half the table words)
-    long long c4_chunk_min;  // chunked shared-memory kernel above this ...
-    long long c4_chunk_max;  // ... and up to this (the cluster kernel takes the rest)
+    long long c4_cta_max;    // block hash, large table (<= C4_T3); chunk counters beyond
+    // bounds of a kernel that the chunk counters replaced: kept for the
+    // callers that set and read them, no kernel looks at them
+    long long c4_chunk_min, c4_chunk_max;
 };
 constexpr long long NEVER = 1ll << 62;
-inline Tuning default_tuning() { return Tuning{32, TRI_KS, TRI_KM, 32, C4_T1, C4_T2, C4_T3, NEVER, NEVER}; }
-constexpr int C4_DENSE_THREADS = 1024;
+inline Tuning default_tuning() { return Tuning{32, TRI_KS, TRI_KM, 32, C4_T1, C4_T2, 32768, NEVER, NEVER}; }
 
 // Handle-independent launch geometry.
 struct Dims {

@@ -1,6 +1,7 @@
 // gc_kernels.cuh -- declarations of the kernels, for the launchers in gc_api.cu.
 #pragma once
 
+#include "gc_c4.cuh"
 #include "gc_internal.cuh"
 
 namespace gcx {
@@ -92,15 +93,8 @@ struct CountArgs {
     const int32_t* db;             // degree in G_b
     unsigned long long* tpack;     // per-entry triangle counters, zeroed
     int32_t* bins;                 // NBINS * n_alloc
-    unsigned long long* dense;     // dense_clusters * dense_stride(n_alloc) zeroed words
     int n_alloc;                   // vertex id bound
-    int dense_clusters;            // clusters of the heavy 4-cycle kernel
-    int dense_cluster_size;        // CTAs per such cluster (8 or 16)
-    unsigned long long* cta_tables; // cta_groups * cta_table_words zeroed words
-    long long cta_table_words;      // power of two; pivots up to half of it use the hash tier
-    int cta_groups;                 // CTAs of the medium 4-cycle kernel (one table each)
-    unsigned char* chunk_scratch;   // sms * c4_chunk_cta_bytes(chunk_cap): per-CTA run bounds of the chunked kernel
-    long long chunk_cap;            // run-bound entries per CTA (0: the chunked tier is off)
+    C4Bufs c4;                     // buffers of the shared-memory 4-cycle pivots (c4_geom(n_alloc))
     Tuning tune;                    // bin boundaries (clamped to the capacities)
     int sms;
     cudaStream_t aux[3] = {nullptr, nullptr, nullptr};  // side streams of the counting pass (or none)
@@ -112,22 +106,6 @@ Tuning effective_tuning(const CountArgs& a);
 // Dynamic shared-memory limits of the counting kernels (once per device).
 void count_setup_attributes();
 void local_setup_attributes();
-size_t c4_chunk_smem_bytes();
-int c4_chunk_width(long long n);                 // id-range chunks + 1
-long long c4_chunk_cap(long long n);             // run-bound entries per CTA for ids below n
-// bytes of one CTA's scratch of the chunked kernel: run bounds int32[cap],
-// row starts int64[cap / 2], row flags uint32[cap / 2]
-__host__ __device__ inline size_t c4_chunk_cta_bytes(long long cap) {
-    return (size_t)cap * 4 + (size_t)(cap / 2) * 12;
-}
-// Cluster shape of the heavy 4-cycle kernel: CTAs per cluster (want = 0:
-// 16 if the device can co-schedule it, else 8) and the number of clusters.
-int dense_cluster_plan(int want, int sms, int* size_out);
-
-// 64-bit words of one cluster's counter region in the heavy 4-cycle kernel
-// for n vertices: an even count (16-byte aligned regions) with room for the
-// narrow layout's arrays, list counter and padding at every n.
-__host__ __device__ constexpr long long dense_stride(long long n) { return ((n + 1) & ~1ll) + 8; }
 // Device buffers of the edge-local path (gc_local.cu).  V_X = wlist[0 ..
 // lvl[0]), marked in `visited`; its union rows in U_off / U_col, degrees in
 // G_a / G_b in da / db.  The scratch arrays hold `cap` entries (the offset

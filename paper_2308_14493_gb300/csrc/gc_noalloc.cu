@@ -30,9 +30,8 @@ namespace {
 
 constexpr int NA_MAX_N = GC_NOALLOC_MAX_VERTICES;      // vertices
 constexpr long long NA_MAX_E = GC_NOALLOC_MAX_ENTRIES;  // directed adjacency entries (2m)
-constexpr int NA_DENSE_CLUSTERS = 2;                   // clusters of the heaviest 4-cycle pivots
-constexpr int NA_CTA_GROUPS = 4;                       // CTAs of the medium 4-cycle pivots
-constexpr long long NA_TABLE_WORDS = 1 << 15;          // hash table words per such CTA
+constexpr int NA_CHUNKS = 32;                           // id chunks of the shared-memory 4-cycle pivots, at most
+constexpr int NA_GROUP = 32;                            // chunks whose run bounds are held at a time, at most
 constexpr int NA_TPB = 256;
 
 // byte offsets of the pieces inside the scratch array
@@ -47,9 +46,11 @@ constexpr size_t OFF_WL = al(OFF_DB + 4 * (size_t)NA_MAX_N);
 constexpr size_t OFF_UCOL = al(OFF_WL + 4 * (size_t)NA_MAX_N);
 constexpr size_t OFF_TPACK = al(OFF_UCOL + 4 * (size_t)NA_MAX_E);
 constexpr size_t OFF_BINS = al(OFF_TPACK + 8 * (size_t)NA_MAX_E);
-constexpr size_t OFF_DENSE = al(OFF_BINS + 4 * (size_t)NA_MAX_N * NBINS);
-constexpr size_t OFF_CTA = al(OFF_DENSE + 8 * (size_t)dense_stride(NA_MAX_N) * NA_DENSE_CLUSTERS);
-constexpr size_t OFF_ERR = al(OFF_CTA + 8 * (size_t)NA_TABLE_WORDS * NA_CTA_GROUPS);
+constexpr size_t OFF_HEAD = al(OFF_BINS + 4 * (size_t)NA_MAX_N * NBINS);
+constexpr size_t OFF_CHUNK = al(OFF_HEAD + sizeof(C4Head));
+constexpr size_t OFF_SORTED = al(OFF_CHUNK + sizeof(C4Chunk) * NA_CHUNKS);
+constexpr size_t OFF_RUN = al(OFF_SORTED + 4 * (size_t)NA_MAX_N);
+constexpr size_t OFF_ERR = al(OFF_RUN + 8 * (size_t)NA_MAX_N * NA_GROUP);
 constexpr size_t SCRATCH_BYTES = al(OFF_ERR + 16);
 
 __device__ __align__(256) unsigned char g_noalloc_scratch[SCRATCH_BYTES];
@@ -179,23 +180,17 @@ extern "C" int gc_count_static_noalloc(int32_t n, const int32_t* d_row_ptr, cons
     uint32_t* U_col = (uint32_t*)(b + OFF_UCOL);
     unsigned long long* tpack = (unsigned long long*)(b + OFF_TPACK);
     int32_t* bins = (int32_t*)(b + OFF_BINS);
-    unsigned long long* dense = (unsigned long long*)(b + OFF_DENSE);
-    unsigned long long* cta_tables = (unsigned long long*)(b + OFF_CTA);
     int* bad = (int*)(b + OFF_ERR);
     cudaStream_t s = (cudaStream_t)stream;
     int nn = n > 0 ? n : 1;
     int grid = (int)((std::max<long long>(n, nnz) + NA_TPB - 1) / NA_TPB);
     if (grid < 1) grid = 1;
     if (grid > 1024) grid = 1024;
-    // what must start at zero: flags, accumulators, triangle counters and the
-    // 4-cycle counters (an interrupted earlier call may have left them dirty)
+    // what must start at zero: flags, accumulators and triangle counters (an
+    // interrupted earlier call may have left them dirty)
     const bool stale = cudaPeekAtLastError() != cudaSuccess;
     k_na_reset<<<1, 32, 0, s>>>(ctl, bad);
-    // per-cluster counter regions of dense_stride(n) words
-    if (cudaMemsetAsync(tpack, 0, 8 * (size_t)std::max<long long>(nnz, 1), s) != cudaSuccess ||
-        cudaMemsetAsync(dense, 0, 8 * (size_t)dense_stride(nn) * NA_DENSE_CLUSTERS, s) != cudaSuccess ||
-        cudaMemsetAsync(cta_tables, 0, 8 * (size_t)NA_TABLE_WORDS * NA_CTA_GROUPS, s) != cudaSuccess)
-        return GC_ECUDA;
+    if (cudaMemsetAsync(tpack, 0, 8 * (size_t)std::max<long long>(nnz, 1), s) != cudaSuccess) return GC_ECUDA;
     k_reset_count<<<1, 32, 0, s>>>(ctl);
     k_na_build<<<grid, NA_TPB, 0, s>>>(d_row_ptr, d_col, n, nnz, ctl, U_off, U_col, U_split, da, db, wlist, bad);
     k_na_fill<<<grid, NA_TPB, 0, s>>>(d_row_ptr, d_col, n, nnz, U_col, bad);
@@ -221,16 +216,17 @@ extern "C" int gc_count_static_noalloc(int32_t n, const int32_t* d_row_ptr, cons
     ca.db = db;
     ca.tpack = tpack;
     ca.bins = bins;
-    ca.dense = dense;
     ca.n_alloc = nn;
-    ca.dense_clusters = NA_DENSE_CLUSTERS;
-    ca.dense_cluster_size = 8;
-    ca.cta_tables = cta_tables;
-    ca.cta_table_words = NA_TABLE_WORDS;
-    ca.chunk_scratch = nullptr;  // no chunked 4-cycle tier in the fixed scratch
-    ca.chunk_cap = 0;
+    const C4Geom geom = c4_geom(nn, sms);
+    if (geom.nchmax > NA_CHUNKS || geom.group > NA_GROUP || !geom.narrow) return GC_EINVAL;
+    ca.c4.head = (C4Head*)(b + OFF_HEAD);
+    ca.c4.chunk = (C4Chunk*)(b + OFF_CHUNK);
+    ca.c4.gmax = nullptr;  // every degree is below 2^16
+    ca.c4.sorted = (int32_t*)(b + OFF_SORTED);
+    ca.c4.run = (unsigned long long*)(b + OFF_RUN);
+    ca.c4.list = nullptr;  // a static count has no one-graph wedges
+    ca.c4.lcap = 0;
     ca.tune = default_tuning();
-    ca.cta_groups = NA_CTA_GROUPS;
     ca.sms = sms;
     enqueue_counting(ca, s, nullptr, nullptr, nullptr, 1);
     if (!stale && cudaGetLastError() != cudaSuccess) return GC_ECUDA;
