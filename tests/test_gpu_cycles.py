@@ -94,3 +94,26 @@ def test_full_tables(gcb, extra):
     with gcb.Graph(n, rp, col) as g:
         g.set_tuning(**TABLES)
         assert g.count_static() == oracle.static_counts(rp, col)
+
+
+def test_repeated_static_counts(gcb):
+    """Static counts of a small graph replay a captured sequence from the
+    third on: between batches that move buffers, tuning changes and new
+    vertices every count is that of the graph as it is then."""
+    n = 3000
+    keys = hub_graph(n, 6000, 500, 12)
+    rp, col = gen.csr_from_keys(n, keys)
+    og = oracle.OracleGraph(rp, col)
+    with gcb.Graph(n, rp, col) as g:
+        for i, size in enumerate((0, 50, 4000, 10, 0, 0)):
+            if size:
+                grp, gcol = g.export_csr()
+                ins, dels = gen.random_batch(g.n, gen.keys_from_csr(grp, gcol), size, size // 2, 100 + i)
+                assert g.apply(ins, dels) == og.apply(ins, dels)["F"]
+            if i == 4:
+                g.set_tuning(**ALL_DENSE)
+            if i == 5:
+                g.add_vertices(20000)
+            for _ in range(5):
+                assert g.count_static() == og.F
+            assert g.counts() == og.F
