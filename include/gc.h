@@ -179,11 +179,11 @@ int gc_counts_all(const gc_graph *g, uint64_t out[22]);
    The containment identity of the global counts holds per vertex, so the
    non-induced copies through each vertex, counted by its role in them,
    invert the same way; the sum over vertices is 4 x gc_counts.  Runs a
-   static pass plus the per-vertex kernels (device scratch of about 4 bytes
-   per adjacency entry, 64 bytes per vertex, and one 4-byte counter array
-   per 4-cycle block, 2 GB at most, all freed on return); the maintained
-   counts are not changed.  gc_batch_stats().ms_device gives the device
-   time of the per-vertex kernels. */
+   static pass that also credits its 4-cycles to their vertices, then the
+   per-vertex kernels (device scratch of 4 bytes per adjacency entry, 32 bytes
+   per vertex and the device copy of the output, freed on return); the
+   maintained counts are not changed.  gc_batch_stats().ms_device gives the
+   device time of all of it. */
 int gc_vertex_counts(gc_graph *g, uint64_t *out);
 
 /* The same per vertex and orbit: out[11 x + j] = the induced connected
@@ -205,11 +205,10 @@ int gc_vertex_orbits(gc_graph *g, uint64_t *out);
    each connected 4-vertex subgraph through the edge, counted by the edge's
    role in them, invert with a triangular matrix.  Summed over the edges,
    type k gives (3, 3, 4, 4, 5, 6)[k] x gc_counts.  Runs a static pass plus
-   the per-edge kernels (device scratch of 52 bytes per adjacency entry,
-   two per edge; 8 bytes per vertex; the device copy of the output; and one
-   4-byte counter array per 4-cycle block, 2 GB at most; all freed on
-   return); the maintained counts are not changed.  gc_batch_stats().ms_device gives the device time of the
-   per-edge kernels. */
+   the per-edge kernels (device scratch of 36 bytes per adjacency entry, 16
+   per edge, 20 per vertex and the device copy of the output, freed on
+   return); the maintained counts are not changed.  gc_batch_stats().ms_device
+   gives the device time of all of it. */
 int gc_edge_counts(gc_graph *g, int32_t *edges, uint64_t *out);
 
 /* The same per edge orbit: out[10 r + j] = the induced connected 4-vertex
@@ -372,9 +371,8 @@ typedef struct {
     int64_t local_max_pairs; /* batches of at most this many pairs take the edge-local delta
                                 (gc_options.local_max_pairs); 0 = never */
     int64_t local_c4_heavy_min; /* gc_vertex_* and gc_edge_*: 4-cycle pivots with w~ at least this
-                                   are walked 8 at a time by the whole GPU, each with its own
-                                   counter array in L2; the others by one CTA each on per-CTA
-                                   arrays; 0 = never (default 65536) */
+                                   skip the hash-table tiers and are counted over id-range
+                                   chunks; 0 = the bounds above alone (default 65536) */
     int64_t pair_min_share; /* gc_apply_batches*, sequential runs: when the region pass of a run's
                                first batch holds at least this many per mille of the graph's 2m
                                adjacency entries, the later batches go in pairs: the first of a

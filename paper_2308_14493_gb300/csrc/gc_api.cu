@@ -616,7 +616,9 @@ static int ensure_desc(gc_graph* g, long long words) {
 //   set_F: a static count that initialises F; timed: record stage events
 // all: the region is every vertex (no per-entry region test in the union
 // graph); twin: the twin pass's union graph of two batches
-static int count_region(gc_graph* g, int fin, bool set_F, bool timed, bool twin = false, bool all = false) {
+// c4_mode, c4_credit: the 4-cycle credits of the local counts (static counts)
+static int count_region(gc_graph* g, int fin, bool set_F, bool timed, bool twin = false, bool all = false,
+                        int c4_mode = C4_COUNT, unsigned long long* c4_credit = nullptr) {
     cudaStream_t s = g->s;
     int gw = grid_warps(g);
     pdl_launch(k_reset_count, dim3(1), dim3(32), 0, s, g->ctl);
@@ -653,6 +655,9 @@ static int count_region(gc_graph* g, int fin, bool set_F, bool timed, bool twin 
     ca.n_alloc = std::max(g->n, 1);
     carve_c4(g, &ca.c4);
     ca.tune = g->tune;
+    ca.c4_mode = c4_mode;
+    ca.c4_credit = c4_credit;
+    ca.local_heavy_min = g->loc_heavy_min;
     ca.sms = g->sms;
     for (int i = 0; i < 3; i++) {
         ca.aux[i] = g->opt.serial_count ? nullptr : g->aux[i];
@@ -1321,7 +1326,7 @@ static int apply_batches_region(gc_graph* g, const int32_t* d_ins, const int32_t
 
 // The launch sequence of a static count: W = V, the counting pass, the
 // triangle sums of the edge-local path.
-static int enqueue_static(gc_graph* g, bool set_F) {
+static int enqueue_static(gc_graph* g, bool set_F, int c4_mode = C4_COUNT, unsigned long long* c4_credit = nullptr) {
     cudaStream_t s = g->s;
     CK(cudaMemsetAsync(g->visited, 0xFF, sizeof(uint32_t) * (size_t)((g->n + 31) / 32 + 1), s));
     pdl_launch(k_region_all, dim3(grid_elems(g, g->n)), dim3(TPB), 0, s, g->ctl, g->n, g->wlist);
@@ -1329,7 +1334,7 @@ static int enqueue_static(gc_graph* g, bool set_F) {
     g->launches += 2;
     CKL();
     CK(record_stage(g->ev[2], s));
-    int rc = count_region(g, 1, set_F, true, false, true);
+    int rc = count_region(g, 1, set_F, true, false, true, c4_mode, c4_credit);
     if (rc) return rc;
     // the static pass also gives the triangle sums of the edge-local path
     CK(cudaMemsetAsync(g->T2, 0, 8 * (size_t)std::max(g->n, 1), s));
@@ -1348,7 +1353,8 @@ static int enqueue_static(gc_graph* g, bool set_F) {
 // hide their launches.
 constexpr long long STATIC_GRAPH_ENTRIES = 1 << 22;
 
-static int count_static(gc_graph* g, bool set_F, uint64_t out[6]) {
+static int count_static(gc_graph* g, bool set_F, uint64_t out[6], int c4_mode = C4_COUNT,
+                        unsigned long long* c4_credit = nullptr) {
     cudaStream_t s = g->s;
     int rc = plan_region_buffers(g, g->m, 0);
     if (rc) return rc;
@@ -1361,7 +1367,8 @@ static int count_static(gc_graph* g, bool set_F, uint64_t out[6]) {
         g->s_tune = g->tune;
         g->s_seen = 0;
     }
-    const bool replay = !set_F && 2 * g->m <= STATIC_GRAPH_ENTRIES && ++g->s_seen > 2;
+    const bool replay =
+        !set_F && c4_mode == C4_COUNT && 2 * g->m <= STATIC_GRAPH_ENTRIES && ++g->s_seen > 2;
     if (replay) {
         if (!g->sexec) {
             rc = capture(g, &g->sexec, &g->s_launches, [&] { return enqueue_static(g, false); });
@@ -1370,7 +1377,7 @@ static int count_static(gc_graph* g, bool set_F, uint64_t out[6]) {
         CK(cudaGraphLaunch(g->sexec, s));
         g->launches = g->s_launches;
     } else {
-        rc = enqueue_static(g, set_F);
+        rc = enqueue_static(g, set_F, c4_mode, c4_credit);
         if (rc) return rc;
     }
     rc = read_ctl(g);
@@ -1785,32 +1792,6 @@ int gc_counts_all(const gc_graph* g, uint64_t out[22]) {
     return GC_OK;
 }
 
-// Scratch of the heavy 4-cycle pivots of the local counts (none when the
-// grouped walk is off); returns false when an allocation failed.
-static bool alloc_heavy(gc_graph* g, HeavyC4& h) {
-    h.heavy_min = g->loc_heavy_min;
-    h.U_wt = g->U_wt;
-    h.heavy = nullptr;
-    h.hlist = nullptr;
-    h.hcount = nullptr;
-    h.cnt_g = nullptr;
-    if (h.heavy_min <= 0) return true;
-    const size_t n = (size_t)std::max(g->n, 1);
-    h.heavy = (uint8_t*)dalloc(g, n);
-    h.hlist = (int32_t*)dalloc(g, 4 * n);
-    h.hcount = (int*)dalloc(g, 16);
-    h.cnt_g = (uint32_t*)dalloc(g, 4 * (size_t)C4G * n);
-    return h.heavy && h.hlist && h.hcount && h.cnt_g &&
-           cudaMemsetAsync(h.cnt_g, 0, 4 * (size_t)C4G * n, g->s) == cudaSuccess;
-}
-
-static void free_heavy(gc_graph* g, HeavyC4& h) {
-    if (h.heavy) dfree(g, h.heavy);
-    if (h.hlist) dfree(g, h.hlist);
-    if (h.hcount) dfree(g, h.hcount);
-    if (h.cnt_g) dfree(g, h.cnt_g);
-}
-
 static int vertex_counts(gc_graph* g, uint64_t* out, int orbits) {
     if (!g || (!out && g->n > 0)) return GC_EINVAL;
     if (!on_device(g)) {
@@ -1819,38 +1800,31 @@ static int vertex_counts(gc_graph* g, uint64_t* out, int orbits) {
     }
     g->err.clear();
     if (g->n == 0) return GC_OK;
-    // the union graph, per-entry t and T2 of the current graph
-    int rc = count_static(g, false, nullptr);
-    if (rc) return rc;
     cudaStream_t s = g->s;
     const size_t n = (size_t)g->n;
-    const long long nU = std::max<long long>(g->h_ctl->nU, 1);
-    // one dense counter array per 4-cycle block, at most 2 GB in all
-    const int blocks = (int)std::max<long long>(1, std::min<long long>(g->sms, (2LL << 30) / (4LL * (long long)n)));
-    uint32_t* tall = (uint32_t*)dalloc(g, 4 * (size_t)nU);
-    long long* sdeg = (long long*)dalloc(g, 8 * n);
     const int k = orbits ? 11 : 6;
-    long long* NV = (long long*)dalloc(g, 88 * n);
-    uint32_t* cnt = (uint32_t*)dalloc(g, 4 * n * (size_t)blocks);
+    uint32_t* tall = (uint32_t*)dalloc(g, 4 * (size_t)std::max<long long>(2 * g->m, 1));
+    long long* sdeg = (long long*)dalloc(g, 8 * n);
+    unsigned long long* credit = (unsigned long long*)dalloc(g, 24 * n);  // diamonds, 4-cliques, 4-cycles
     unsigned long long* dout = (unsigned long long*)dalloc(g, 8 * (size_t)k * n);
-    HeavyC4 hv;
-    const bool hv_ok = alloc_heavy(g, hv);
     auto cleanup = [&]() {
         dfree(g, tall);
         dfree(g, sdeg);
-        dfree(g, NV);
-        dfree(g, cnt);
+        dfree(g, credit);
         dfree(g, dout);
-        free_heavy(g, hv);
     };
-    if (!tall || !sdeg || !NV || !cnt || !dout || !hv_ok) {
+    if (!tall || !sdeg || !credit || !dout) {
         cleanup();
         return nomem(g, "per-vertex counts");
     }
-    if (cudaMemsetAsync(NV, 0, 88 * n, s) != cudaSuccess || cudaMemsetAsync(cnt, 0, 4 * n * (size_t)blocks, s) != cudaSuccess) {
+    // the union graph, per-entry t, T2 and the 4-cycle credits of the current graph
+    cudaError_t ce = cudaEventRecord(g->e0, s);
+    if (ce == cudaSuccess) ce = cudaMemsetAsync(credit, 0, 24 * n, s);
+    int rc = GC_OK;
+    if (ce == cudaSuccess) rc = count_static(g, false, nullptr, C4_VERTEX, credit + 2 * n);
+    if (rc) {
         cleanup();
-        g->err = "cudaMemsetAsync failed";
-        return GC_ECUDA;
+        return rc;
     }
     VertexArgs va;
     va.ctl = g->ctl;
@@ -1860,21 +1834,21 @@ static int vertex_counts(gc_graph* g, uint64_t* out, int orbits) {
     va.U_split = g->U_split;
     va.tpack = g->tpack.p;
     va.T2 = g->T2;
+    va.bins = g->bins;
     va.tall = tall;
     va.sdeg = sdeg;
-    va.NV = NV;
-    va.cnt = cnt;
-    va.c4_blocks = blocks;
+    va.d2 = credit;
+    va.k4 = credit + n;
+    va.c4 = credit + 2 * n;
     va.n = (int)n;
     va.iperm = g->iperm;
     va.out = dout;
     va.orbits = orbits;
     va.sms = g->sms;
-    va.hv = hv;
-    cudaError_t ce = cudaEventRecord(g->e0, s);
-    g->launches = enqueue_vertex_counts(va, s);
-    if (g->launches < 0 && ce == cudaSuccess) ce = cudaErrorUnknown;
-    if (ce == cudaSuccess) ce = cudaEventRecord(g->e1, s);
+    if (ce == cudaSuccess) {
+        g->launches += enqueue_vertex_counts(va, s);
+        ce = cudaEventRecord(g->e1, s);
+    }
     if (ce == cudaSuccess) ce = cudaMemcpyAsync(out, dout, 8 * (size_t)k * n, cudaMemcpyDeviceToHost, s);
     if (ce == cudaSuccess) ce = cudaStreamSynchronize(s);
     if (ce == cudaSuccess) ce = cudaGetLastError();
@@ -1901,51 +1875,50 @@ static int edge_counts(gc_graph* g, int32_t* edges, uint64_t* out, int orbits) {
     }
     g->err.clear();
     if (g->m == 0) return GC_OK;
-    // the union graph, per-entry t and T2 of the current graph
-    int rc = count_static(g, false, nullptr);
-    if (rc) return rc;
     cudaStream_t s = g->s;
     const size_t n = (size_t)g->n;
-    const long long nU = g->h_ctl->nU, m = nU / 2;
-    if (nU != 2 * g->m) {
-        g->err = "per-edge counts: the union graph does not hold every edge twice";
-        return GC_ECUDA;
-    }
-    const int blocks = (int)std::max<long long>(1, std::min<long long>(g->sms, (2LL << 30) / (4LL * (long long)n)));
-    const int sg = radix_grid(nU, g->sms);
+    const long long m = g->m, nU = 2 * m;
+    const int sg = radix_grid(m, g->sms);
     const int k = orbits ? 10 : 6;
     uint32_t* tall = (uint32_t*)dalloc(g, 4 * (size_t)nU);
     long long* sdeg = (long long*)dalloc(g, 8 * n);
-    long long* NE = (long long*)dalloc(g, 32 * (size_t)nU);
-    unsigned long long* keys = (unsigned long long*)dalloc(g, 8 * (size_t)nU);
-    unsigned long long* ktmp = (unsigned long long*)dalloc(g, 8 * (size_t)nU);
+    // per entry: opposite and diamond-outer credits, 4-cliques, 4-cycles
+    unsigned long long* credit = (unsigned long long*)dalloc(g, 32 * (size_t)nU);
+    int32_t* outdeg = (int32_t*)dalloc(g, 4 * n);
+    long long* out_off = (long long*)dalloc(g, 8 * (n + 1));
+    unsigned long long* keys = (unsigned long long*)dalloc(g, 8 * (size_t)m);
+    unsigned long long* ktmp = (unsigned long long*)dalloc(g, 8 * (size_t)m);
     uint32_t* hist = (uint32_t*)dalloc(g, 4 * 256 * (size_t)sg);
-    uint32_t* cnt = (uint32_t*)dalloc(g, 4 * n * (size_t)blocks);
     unsigned long long* dout = (unsigned long long*)dalloc(g, 8 * (size_t)k * (size_t)m);
     int32_t* dedges = edges ? (int32_t*)dalloc(g, 8 * (size_t)m) : nullptr;
-    HeavyC4 hv;
-    const bool hv_ok = alloc_heavy(g, hv);
     auto cleanup = [&]() {
-        free_heavy(g, hv);
         dfree(g, tall);
         dfree(g, sdeg);
-        dfree(g, NE);
+        dfree(g, credit);
+        dfree(g, outdeg);
+        dfree(g, out_off);
         dfree(g, keys);
         dfree(g, ktmp);
         dfree(g, hist);
-        dfree(g, cnt);
         dfree(g, dout);
         if (dedges) dfree(g, dedges);
     };
-    if (!tall || !sdeg || !NE || !keys || !ktmp || !hist || !cnt || !dout || (edges && !dedges) || !hv_ok) {
+    if (!tall || !sdeg || !credit || !outdeg || !out_off || !keys || !ktmp || !hist || !dout || (edges && !dedges)) {
         cleanup();
         return nomem(g, "per-edge counts");
     }
-    if (cudaMemsetAsync(NE, 0, 32 * (size_t)nU, s) != cudaSuccess ||
-        cudaMemsetAsync(cnt, 0, 4 * n * (size_t)blocks, s) != cudaSuccess) {
+    // the union graph, per-entry t, T2 and the 4-cycle credits of the current graph
+    cudaError_t ce = cudaEventRecord(g->e0, s);
+    if (ce == cudaSuccess) ce = cudaMemsetAsync(credit, 0, 32 * (size_t)nU, s);
+    int rc = GC_OK;
+    if (ce == cudaSuccess) rc = count_static(g, false, nullptr, C4_EDGE, credit + 3 * nU);
+    if (!rc && g->h_ctl->nU != nU) {
+        g->err = "per-edge counts: the union graph does not hold every edge twice";
+        rc = GC_ECUDA;
+    }
+    if (rc) {
         cleanup();
-        g->err = "cudaMemsetAsync failed";
-        return GC_ECUDA;
+        return rc;
     }
     EdgeArgs ea;
     ea.ctl = g->ctl;
@@ -1955,30 +1928,31 @@ static int edge_counts(gc_graph* g, int32_t* edges, uint64_t* out, int orbits) {
     ea.U_split = g->U_split;
     ea.tpack = g->tpack.p;
     ea.T2 = g->T2;
+    ea.bins = g->bins;
     ea.tall = tall;
     ea.sdeg = sdeg;
-    ea.NE = NE;
+    ea.to = credit;
+    ea.k4 = credit + 2 * nU;
+    ea.c4 = credit + 3 * nU;
+    ea.outdeg = outdeg;
+    ea.out_off = out_off;
+    ea.bsum = g->bsum.p;
     ea.keys = keys;
     ea.keys_tmp = ktmp;
     ea.hist = hist;
     ea.sort_grid = sg;
-    ea.d_count = &g->ctl->nU;
-    ea.nU = nU;
     ea.m = m;
     ea.nb = g->S;
-    ea.cnt = cnt;
-    ea.c4_blocks = blocks;
     ea.n = (int)n;
     ea.iperm = g->iperm;
     ea.out = dout;
     ea.edges = dedges;
     ea.orbits = orbits;
     ea.sms = g->sms;
-    ea.hv = hv;
-    cudaError_t ce = cudaEventRecord(g->e0, s);
-    g->launches = enqueue_edge_counts(ea, s);
-    if (g->launches < 0 && ce == cudaSuccess) ce = cudaErrorUnknown;
-    if (ce == cudaSuccess) ce = cudaEventRecord(g->e1, s);
+    if (ce == cudaSuccess) {
+        g->launches += enqueue_edge_counts(ea, s);
+        ce = cudaEventRecord(g->e1, s);
+    }
     if (ce == cudaSuccess) ce = cudaMemcpyAsync(out, dout, 8 * (size_t)k * (size_t)m, cudaMemcpyDeviceToHost, s);
     if (ce == cudaSuccess && edges) ce = cudaMemcpyAsync(edges, dedges, 8 * (size_t)m, cudaMemcpyDeviceToHost, s);
     if (ce == cudaSuccess) ce = cudaStreamSynchronize(s);

@@ -81,6 +81,8 @@ struct PivotArgs {
 // The hash-table tiers, then plan, run bounds and pivot kernels, on stream s
 // (bins: the work lists, NBINS * n); both return the launches made.
 int enqueue_c4_tables(const PivotArgs& a, int mode, const int32_t* bins, int sms, cudaStream_t s);
+// (the credits of the pivots below the tables: C4_VERTEX and C4_EDGE only)
+int enqueue_c4_warp_credit(const PivotArgs& a, int mode, const int32_t* bins, int sms, cudaStream_t s);
 int enqueue_c4_pivots(const PivotArgs& a, int mode, const C4Geom& g, cudaStream_t s);
 void c4_setup_attributes();
 

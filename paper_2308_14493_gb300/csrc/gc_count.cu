@@ -829,7 +829,14 @@ int enqueue_counting(const CountArgs& a, cudaStream_t s, cudaEvent_t ev_tri, cud
     auto lists = [&](int b) { return a.bins + (size_t)b * a.n_alloc; };
     long long nw = a.n_alloc > 0 ? a.n_alloc : 1;
     int gb = (int)std::min<long long>((nw + 255) / 256, 8LL * sms);
-    const Tuning t = effective_tuning(a);
+    Tuning t = effective_tuning(a);
+    if (a.c4_mode != C4_COUNT && a.local_heavy_min > 0) {
+        const long long cap = std::max<long long>(1, a.local_heavy_min - 1);
+        t.c4_reg_max = (int)std::min<long long>(t.c4_reg_max, cap);
+        t.c4_warp_max = (int)std::min<long long>(t.c4_warp_max, cap);
+        t.c4_block_max = (int)std::min<long long>(t.c4_block_max, cap);
+        t.c4_cta_max = std::min(t.c4_cta_max, cap);
+    }
     pdl_launch(k_wedge_bound, dim3(8 * sms), dim3(256), 0, s, a.ctl, a.wlist, a.U_off, a.U_col, a.U_split, a.U_wt);
     pdl_launch(k_bin, dim3(gb), dim3(256), 0, s, a.ctl, a.wlist, a.U_off, a.U_split, a.U_wt, a.bins, a.n_alloc, t);
     nl += 2;
@@ -853,9 +860,6 @@ int enqueue_counting(const CountArgs& a, cudaStream_t s, cudaEvent_t ev_tri, cud
     k_tri_merge<<<sms, 256, 0, sT>>>(a.ctl, lists(BIN_TRI_MERGE), a.U_off, a.U_col, a.U_split, a.tpack);
     nl += 4;
     if (ev_c4) record_stage(ev_c4, sT);
-    k_c4_reg<<<4 * sms, 256, 0, sC1>>>(a.ctl, lists(BIN_C4_REG), a.U_off, a.U_col, a.U_split);
-    k_c4_warp<<<7 * sms, C4W_WARPS * 32, 0, sC1>>>(a.ctl, lists(BIN_C4_WARP), a.U_off, a.U_col, a.U_split,
-                                                   a.U_wt);
     PivotArgs pa;
     pa.ctl = a.ctl;
     pa.pivots = lists(BIN_C4_DENSE);
@@ -868,12 +872,19 @@ int enqueue_counting(const CountArgs& a, cudaStream_t s, cudaEvent_t ev_tri, cud
     const C4Geom geom = c4_geom(a.n_alloc, sms);
     pa.words = geom.words;
     pa.group = geom.group;
-    pa.credit = nullptr;
-    nl += enqueue_c4_tables(pa, C4_COUNT, a.bins, sms, sC1);
+    pa.credit = a.c4_credit;
+    if (a.c4_mode == C4_COUNT) {
+        k_c4_reg<<<4 * sms, 256, 0, sC1>>>(a.ctl, lists(BIN_C4_REG), a.U_off, a.U_col, a.U_split);
+        k_c4_warp<<<7 * sms, C4W_WARPS * 32, 0, sC1>>>(a.ctl, lists(BIN_C4_WARP), a.U_off, a.U_col, a.U_split,
+                                                       a.U_wt);
+        nl += 2;
+    } else {
+        nl += enqueue_c4_warp_credit(pa, a.c4_mode, a.bins, sms, sC1);
+    }
+    nl += enqueue_c4_tables(pa, a.c4_mode, a.bins, sms, sC1);
     if (a.ev_heavy[0]) record_stage(a.ev_heavy[0], sC2);
-    nl += enqueue_c4_pivots(pa, C4_COUNT, geom, sC2);
+    nl += enqueue_c4_pivots(pa, a.c4_mode, geom, sC2);
     if (a.ev_heavy[1]) record_stage(a.ev_heavy[1], sC2);
-    nl += 2;
     if (par) {
         cudaEventRecord(a.join[1], sC1);
         cudaEventRecord(a.join[2], sC2);

@@ -535,13 +535,97 @@ __global__ void __launch_bounds__(THREADS, MINB) k_c4_pivot(PivotArgs a, int c0)
     acc_add(a.ctl, 20, wedges);
 }
 
-// Pivots whose endpoints all fit a hash table of SLOTS entries (a bound of at
-// most 3/4 SLOTS wedges), a block per pivot.  A slot is an id and a packed
-// count (G_a high, G_b low 16 bits; a count is at most the pivot's lower
-// neighbours, below 2^15).  Four wedges a lane are inserted together, so their
-// probes overlap.  Only the first 4/3 w~ slots are used, so small pivots clear
-// little.
+// A pivot's hash table in shared memory: a slot is an id and a packed count
+// (G_a high, G_b low 16 bits; a count is at most the pivot's lower neighbours,
+// below 2^15 in every table tier).
 constexpr uint32_t TAB_EMPTY = 0xFFFFFFFFu;
+struct Table {
+    uint32_t *keys, *cnts;
+    uint32_t slots;
+    __device__ __forceinline__ uint32_t home(uint32_t w) const { return __umulhi(w * 0x9E3779B1u, slots); }
+    __device__ __forceinline__ uint32_t next(uint32_t h) const { return h + 1 == slots ? 0u : h + 1; }
+    // slots for a pivot of at most wt wedges: 3/4 filled at most
+    __device__ static __forceinline__ uint32_t size_for(int wt) { return (uint32_t)(wt + wt / 3 + 32); }
+};
+
+// Insert four wedges of pivot u (q[i] null: none); their probes overlap.  Old
+// counts are added to qa, qb.
+__device__ __forceinline__ void tab_insert(const Table& T, uint32_t u, const uint32_t* const (&q)[PV_UNROLL],
+                                           const uint32_t (&e)[PV_UNROLL], const uint32_t (&f)[PV_UNROLL],
+                                           unsigned long long& wedges, unsigned long long& qa,
+                                           unsigned long long& qb) {
+    uint32_t h[PV_UNROLL], inc[PV_UNROLL];
+    unsigned todo = 0;
+#pragma unroll
+    for (int i = 0; i < PV_UNROLL; i++) {
+        const uint32_t w = vid(e[i]), both = e[i] & f[i];
+        h[i] = T.home(w);
+        inc[i] = ((both & FLAG_A) ? 0x10000u : 0u) | (both >> 31);
+        if (q[i] && w < u) {
+            wedges++;
+            if (inc[i]) todo |= 1u << i;
+        }
+    }
+    while (todo) {
+        uint32_t k[PV_UNROLL];
+#pragma unroll
+        for (int i = 0; i < PV_UNROLL; i++) k[i] = (todo >> i) & 1u ? T.keys[h[i]] : 0u;
+#pragma unroll
+        for (int i = 0; i < PV_UNROLL; i++)
+            if (((todo >> i) & 1u) && k[i] == TAB_EMPTY) {
+                const uint32_t was = atomicCAS(&T.keys[h[i]], TAB_EMPTY, vid(e[i]));
+                k[i] = was == TAB_EMPTY ? vid(e[i]) : was;
+            }
+#pragma unroll
+        for (int i = 0; i < PV_UNROLL; i++)
+            if ((todo >> i) & 1u) {
+                if (k[i] == vid(e[i])) {
+                    const uint32_t c = atomicAdd(&T.cnts[h[i]], inc[i]);
+                    if (inc[i] >> 16) qa += c >> 16;
+                    if (inc[i] & 1u) qb += c & 0xFFFFu;
+                    todo &= ~(1u << i);
+                } else {
+                    h[i] = T.next(h[i]);
+                }
+            }
+    }
+}
+
+// Credits of four wedges (every one was inserted): c_w - 1 to x[i], and to the
+// second edge's entry.
+template <int MODE>
+__device__ __forceinline__ void tab_credit(const Table& T, uint32_t u, const uint32_t* U_col,
+                                           unsigned long long* credit, const uint32_t* const (&q)[PV_UNROLL],
+                                           const uint32_t (&e)[PV_UNROLL], uint32_t (&x)[PV_UNROLL]) {
+#pragma unroll
+    for (int i = 0; i < PV_UNROLL; i++) {
+        const uint32_t w = vid(e[i]);
+        x[i] = 0;
+        if (q[i] && w < u) {
+            uint32_t h = T.home(w);
+            while (T.keys[h] != w) h = T.next(h);
+            x[i] = (T.cnts[h] >> 16) - 1;
+            if (MODE == C4_EDGE && x[i]) red_u64(&credit[q[i] - U_col], x[i]);
+        }
+    }
+}
+
+// Clear the table; per vertex, every endpoint takes its C(c_w, 2).
+template <int MODE>
+__device__ __forceinline__ void tab_clear(const Table& T, unsigned long long* credit, uint32_t first, uint32_t step) {
+    for (uint32_t i = first; i < T.slots; i += step) {
+        if (MODE == C4_VERTEX) {
+            const unsigned long long c = T.cnts[i] >> 16;
+            if (c >= 2) red_u64(&credit[T.keys[i]], c * (c - 1) / 2);
+        }
+        T.keys[i] = TAB_EMPTY;
+        T.cnts[i] = 0;
+    }
+}
+
+// Pivots whose endpoints all fit a hash table of SLOTS entries (a bound of at
+// most 3/4 SLOTS wedges), a block per pivot.  Only the first 4/3 w~ slots are
+// used, so small pivots clear little.
 // Measured alone (ncu) on a Chung-Lu graph of 800,000 vertices and 15 M edges:
 // 0.65 / 1.27 / 1.06 ms for the small / medium / large table; the kernels
 // before (one hash insertion at a time per lane, 32 rows to a warp, the large
@@ -583,66 +667,27 @@ __global__ void __launch_bounds__(THREADS, MINB) k_c4_table(PivotArgs a, const i
         if (t.id >= (unsigned)npiv) break;
         const uint32_t u = t.u;
         const uint32_t* const row = a.U_col + t.rb;
-        const uint32_t slots = (uint32_t)min(SLOTS, t.k + t.k / 3 + 32);
+        const Table T{keys, cnts, min((uint32_t)SLOTS, Table::size_for(t.k))};
         const Deal deal = deal_groups(t.nlow, (float)t.k, NW);
         auto run = [&](uint32_t v, const uint32_t** p, int* len) {
             const long long b = a.U_off[v];
             *p = a.U_col + b;
             *len = (int)(a.U_off[v + 1] - b);
         };
-        auto slot = [&](uint32_t w) { return __umulhi(w * 0x9E3779B1u, slots); };
         if (tid == 0) s_grp[1] = 0;
         if (tid == THREADS - 1) fetch(s_task[(it + 1) & 1]);
-        unsigned long long old = 0;
+        unsigned long long old = 0, oldb = 0;
         walk_lower<false>(
             row, t.nlow, deal, &s_grp[0], W, run,
             [&](const auto& q, const auto& e, const auto& f, auto&) {
-                uint32_t h[PV_UNROLL], inc[PV_UNROLL];
-                unsigned todo = 0;
-#pragma unroll
-                for (int i = 0; i < PV_UNROLL; i++) {
-                    const uint32_t w = vid(e[i]), both = e[i] & f[i];
-                    h[i] = slot(w);
-                    inc[i] = ((both & FLAG_A) ? 0x10000u : 0u) | (both >> 31);
-                    if (q[i] && w < u) {
-                        wedges++;
-                        if (inc[i]) todo |= 1u << i;
-                    }
-                }
-                while (todo) {
-                    uint32_t k[PV_UNROLL];
-#pragma unroll
-                    for (int i = 0; i < PV_UNROLL; i++) k[i] = (todo >> i) & 1u ? keys[h[i]] : 0u;
-#pragma unroll
-                    for (int i = 0; i < PV_UNROLL; i++)
-                        if (((todo >> i) & 1u) && k[i] == TAB_EMPTY) {
-                            const uint32_t was = atomicCAS(&keys[h[i]], TAB_EMPTY, vid(e[i]));
-                            k[i] = was == TAB_EMPTY ? vid(e[i]) : was;
-                        }
-#pragma unroll
-                    for (int i = 0; i < PV_UNROLL; i++)
-                        if ((todo >> i) & 1u) {
-                            if (k[i] == vid(e[i])) {
-                                const uint32_t c = atomicAdd(&cnts[h[i]], inc[i]);
-                                if (MODE == C4_COUNT) {
-                                    if (inc[i] >> 16) qa += c >> 16;
-                                    if (inc[i] & 1u) qb += c & 0xFFFFu;
-                                } else {
-                                    old += c >> 16;
-                                }
-                                todo &= ~(1u << i);
-                            } else {
-                                h[i] = h[i] + 1 == slots ? 0 : h[i] + 1;
-                            }
-                        }
-                }
+                tab_insert(T, u, q, e, f, wedges, old, oldb);
             },
             [](unsigned long long, uint32_t, int) {});
+        qa += old;
+        qb += oldb;
         __syncthreads();
         if (tid == 0) s_grp[0] = 0;
         if (MODE != C4_COUNT) {
-            qa += old;
-            qb += old;
             if (MODE == C4_VERTEX) {
                 old = warp_sum_u64(old);
                 if ((tid & 31) == 0 && old) red_u64(&a.credit[u], old);
@@ -650,35 +695,87 @@ __global__ void __launch_bounds__(THREADS, MINB) k_c4_table(PivotArgs a, const i
             walk_lower<true>(
                 row, t.nlow, deal, &s_grp[1], W, run,
                 [&](const auto& q, const auto& e, const auto&, auto& x) {
-#pragma unroll
-                    for (int i = 0; i < PV_UNROLL; i++) {
-                        const uint32_t w = vid(e[i]);
-                        x[i] = 0;
-                        if (q[i] && w < u) {
-                            uint32_t h = slot(w);
-                            while (keys[h] != w) h = h + 1 == slots ? 0 : h + 1;
-                            x[i] = (cnts[h] >> 16) - 1;
-                            if (MODE == C4_EDGE && x[i]) red_u64(&a.credit[q[i] - a.U_col], x[i]);
-                        }
-                    }
+                    tab_credit<MODE>(T, u, a.U_col, a.credit, q, e, x);
                 },
                 [&](unsigned long long sum, uint32_t fv, int j) {
                     red_u64(&a.credit[MODE == C4_EDGE ? (size_t)(t.rb + j) : (size_t)vid(fv)], sum);
                 });
             __syncthreads();
         }
-        for (uint32_t i = tid; i < slots; i += THREADS) {
-            if (MODE == C4_VERTEX) {
-                const unsigned long long c = cnts[i] >> 16;
-                if (c >= 2) red_u64(&a.credit[keys[i]], c * (c - 1) / 2);
-            }
-            keys[i] = TAB_EMPTY;
-            cnts[i] = 0;
-        }
+        tab_clear<MODE>(T, a.credit, tid, THREADS);
         __syncthreads();
     }
     acc_add(a.ctl, 5, qa);
     acc_add(a.ctl, 11, qb);
+    acc_add(a.ctl, 15, wedges);
+}
+
+// Credits of the small pivots (registers and warp tiers, w~ <= C4_T1): a warp
+// per pivot with its own table.
+constexpr int CW_WARPS = 8;
+constexpr int CW_SLOTS = C4_T1 + C4_T1 / 3 + 32;
+struct CreditWarp {
+    WarpRuns runs;
+    uint32_t keys[CW_SLOTS], cnts[CW_SLOTS];
+    int ctr[2];
+};
+template <int MODE>
+__global__ void __launch_bounds__(CW_WARPS * 32, 4) k_c4_warp_credit(PivotArgs a, const int32_t* __restrict__ bins) {
+    pdl_enter();
+    extern __shared__ __align__(16) unsigned char cw_smem[];
+    CreditWarp& S = ((CreditWarp*)cw_smem)[threadIdx.x >> 5];
+    const int lane = threadIdx.x & 31;
+    const int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, nw = (gridDim.x * blockDim.x) >> 5;
+    for (int i = lane; i < CW_SLOTS; i += 32) {
+        S.keys[i] = TAB_EMPTY;
+        S.cnts[i] = 0;
+    }
+    const int n0 = a.ctl->nbin[BIN_C4_REG], n1 = n0 + a.ctl->nbin[BIN_C4_WARP];
+    unsigned long long q = 0, wedges = 0;
+    for (int i = gw; i < n1; i += nw) {
+        const uint32_t u = (uint32_t)(i < n0 ? bins[(size_t)BIN_C4_REG * a.n + i]
+                                             : bins[(size_t)BIN_C4_WARP * a.n + i - n0]);
+        const long long rb = a.U_off[u];
+        const int nlow = a.U_split[u];
+        const Table T{S.keys, S.cnts, min((uint32_t)CW_SLOTS, Table::size_for((int)a.U_wt[u]))};
+        const uint32_t* const row = a.U_col + rb;
+        const Deal deal{5, 1};  // 32 rows at a time
+        auto run = [&](uint32_t v, const uint32_t** p, int* len) {
+            const long long b = a.U_off[v];
+            *p = a.U_col + b;
+            *len = (int)(a.U_off[v + 1] - b);
+        };
+        if (lane < 2) S.ctr[lane] = 0;
+        __syncwarp();
+        unsigned long long old = 0, oldb = 0;
+        walk_lower<false>(
+            row, nlow, deal, &S.ctr[0], S.runs, run,
+            [&](const auto& qq, const auto& e, const auto& f, auto&) {
+                tab_insert(T, u, qq, e, f, wedges, old, oldb);
+            },
+            [](unsigned long long, uint32_t, int) {});
+        __syncwarp();
+        q += old;
+        if (__any_sync(FULL, old != 0)) {  // else every c_w is 1 at most: no credits
+            if (MODE == C4_VERTEX) {
+                old = warp_sum_u64(old);
+                if (lane == 0) red_u64(&a.credit[u], old);
+            }
+            walk_lower<true>(
+                row, nlow, deal, &S.ctr[1], S.runs, run,
+                [&](const auto& qq, const auto& e, const auto&, auto& x) {
+                    tab_credit<MODE>(T, u, a.U_col, a.credit, qq, e, x);
+                },
+                [&](unsigned long long sum, uint32_t fv, int j) {
+                    red_u64(&a.credit[MODE == C4_EDGE ? (size_t)(rb + j) : (size_t)vid(fv)], sum);
+                });
+            __syncwarp();
+        }
+        tab_clear<MODE>(T, a.credit, lane, 32);
+        __syncwarp();
+    }
+    acc_add(a.ctl, 5, q);
+    acc_add(a.ctl, 11, q);
     acc_add(a.ctl, 15, wedges);
 }
 
@@ -710,6 +807,12 @@ struct C4Kernels {
         set((const void*)tab_s, table_smem<C4_TAB_S, 128>());
         set((const void*)tab_m, table_smem<C4_TAB_M, 512>());
         set((const void*)tab_l, table_smem<C4_TAB_L, 1024>());
+        if constexpr (MODE != C4_COUNT)
+            set((const void*)k_c4_warp_credit<MODE>, CW_WARPS * sizeof(CreditWarp));
+    }
+    static void warps(const PivotArgs& a, const int32_t* bins, int sms, cudaStream_t s) {
+        if constexpr (MODE != C4_COUNT)
+            k_c4_warp_credit<MODE><<<4 * sms, CW_WARPS * 32, CW_WARPS * sizeof(CreditWarp), s>>>(a, bins);
     }
     static int tables(const PivotArgs& a, const int32_t* bins, int sms, cudaStream_t s) {
         tab_s<<<8 * sms, 128, table_smem<C4_TAB_S, 128>(), s>>>(a, bins + (size_t)BIN_C4_BSMALL * a.n);
@@ -752,6 +855,12 @@ int enqueue_c4_tables(const PivotArgs& a, int mode, const int32_t* bins, int sms
     return mode == C4_VERTEX ? C4Kernels<C4_VERTEX>::tables(a, bins, sms, s)
            : mode == C4_EDGE ? C4Kernels<C4_EDGE>::tables(a, bins, sms, s)
                              : C4Kernels<C4_COUNT>::tables(a, bins, sms, s);
+}
+
+int enqueue_c4_warp_credit(const PivotArgs& a, int mode, const int32_t* bins, int sms, cudaStream_t s) {
+    if (mode == C4_VERTEX) C4Kernels<C4_VERTEX>::warps(a, bins, sms, s);
+    else C4Kernels<C4_EDGE>::warps(a, bins, sms, s);
+    return 1;
 }
 
 int enqueue_c4_pivots(const PivotArgs& a, int mode, const C4Geom& g, cudaStream_t s) {

@@ -53,7 +53,9 @@ enum {
     WORK_TRI_SMALL = 3,   // k_tri_block, short out-lists
     WORK_C4_BSMALL = 4,   // k_c4_table, small table
     WORK_C4_BIG = 5,      // k_c4_table, large table
-    NWORK = 6
+    WORK_LT_SMALL = 6,    // k_l_tri_block, short out-lists
+    WORK_LT_BLOCK = 7,    // k_l_tri_block, long out-lists
+    NWORK = 8
 };
 
 constexpr int ACC_STRIPES = 32;  // copies of each accumulator (spreads the atomics of many warps)

@@ -96,6 +96,9 @@ struct CountArgs {
     int n_alloc;                   // vertex id bound
     C4Bufs c4;                     // buffers of the shared-memory 4-cycle pivots (c4_geom(n_alloc))
     Tuning tune;                    // bin boundaries (clamped to the capacities)
+    int c4_mode = C4_COUNT;         // credits of the 4-cycles as well (static counts only) ...
+    unsigned long long* c4_credit = nullptr;  // ... added here, per vertex or per entry
+    long long local_heavy_min = 0;  // with credits: pivots of at least this bound (> 0) skip the tables
     int sms;
     cudaStream_t aux[3] = {nullptr, nullptr, nullptr};  // side streams of the counting pass (or none)
     cudaEvent_t fork = nullptr;     // fork / join events for them (timing disabled)
@@ -150,21 +153,8 @@ __global__ void k_t2_from_region(const Ctl* c, const int32_t* wlist, const long 
 int enqueue_local(const LocalArgs& a, cudaStream_t s, cudaEvent_t ev_tri, cudaEvent_t ev_sub, cudaEvent_t ev_fin,
                   int commit);
 
-// Per-vertex graphlet counts of a static pass (gc_vertex.cu).
-// Heavy 4-cycle pivots of the per-vertex and per-edge counts (gc_vertex.cu):
-// pivots with w~ >= heavy_min are walked C4G at a time by the whole grid,
-// each with its own counter array in cnt_g; heavy_min = 0 leaves every
-// pivot to the per-block walk.
-constexpr int C4G = 8;
-struct HeavyC4 {
-    long long heavy_min;
-    const long long* U_wt;         // w~ per pivot (static pass)
-    uint8_t* heavy;                // n flags
-    int32_t* hlist;                // n
-    int* hcount;                   // 1
-    uint32_t* cnt_g;               // C4G * n, zeroed
-};
-
+// Per-vertex and per-edge graphlet counts after a static pass with the credits
+// of its 4-cycles (gc_vertex.cu).
 struct VertexArgs {
     Ctl* ctl;
     const int32_t* wlist;          // all vertices (c->nW = n)
@@ -173,19 +163,18 @@ struct VertexArgs {
     const int32_t* U_split;
     const unsigned long long* tpack;
     const unsigned long long* T2;
+    const int32_t* bins;           // work lists of the pass (NBINS * n)
     uint32_t* tall;                // nU: t of every entry
     long long* sdeg;               // n
-    long long* NV;                 // 11 n role counts, zeroed
-    uint32_t* cnt;                 // c4_blocks * n, zeroed
-    int c4_blocks;
+    unsigned long long *d2, *k4;   // n each, zeroed: diamond degree-2 corners, 4-cliques
+    const unsigned long long* c4;  // n: 4-cycles through each vertex
     int n;
     const int32_t* iperm;
     unsigned long long* out;       // 6 n (graphlets) or 11 n (orbits), by external id
     int orbits;
     int sms;
-    HeavyC4 hv;
 };
-// Returns the kernels launched, or -1 on a CUDA error.
+// Returns the kernels launched.
 int enqueue_vertex_counts(const VertexArgs& a, cudaStream_t s);
 
 struct EdgeArgs {
@@ -196,27 +185,29 @@ struct EdgeArgs {
     const int32_t* U_split;
     const unsigned long long* tpack;
     const unsigned long long* T2;
+    const int32_t* bins;           // work lists of the pass (NBINS * n)
     uint32_t* tall;                // nU: t of every entry
     long long* sdeg;               // n
-    long long* NE;                 // 4 nU per-entry credits, zeroed
-    unsigned long long* keys;      // nU sort keys (the first m sorted are the edges)
-    unsigned long long* keys_tmp;  // nU
+    unsigned long long* to;        // 2 nU, zeroed: opposite and diamond-outer credits
+    unsigned long long* k4;        // nU, zeroed
+    const unsigned long long* c4;  // nU: 4-cycle credits of each entry
+    int32_t* outdeg;               // n
+    long long* out_off;            // n + 1
+    long long* bsum;               // 1024
+    unsigned long long* keys;      // m sort keys
+    unsigned long long* keys_tmp;  // m
     uint32_t* hist;                // 256 sort_grid
     int sort_grid;
-    const long long* d_count;      // device copy of nU
-    long long nU, m;
+    long long m;
     int nb;                        // bits of an external id
-    uint32_t* cnt;                 // c4_blocks * n, zeroed
-    int c4_blocks;
     int n;
     const int32_t* iperm;
     unsigned long long* out;       // 10 m (edge orbits) or 6 m (graphlets), by external (lo, hi) order
     int32_t* edges;                // 2 m: (lo, hi) per output row
     int orbits;
     int sms;
-    HeavyC4 hv;
 };
-// Returns the kernels launched, or -1 on a CUDA error.
+// Returns the kernels launched.
 int enqueue_edge_counts(const EdgeArgs& a, cudaStream_t s);
 
 // Enqueue the counting kernels (binning, triangles / 4-cliques, 4-cycles,

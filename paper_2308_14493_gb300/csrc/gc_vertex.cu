@@ -21,23 +21,20 @@
 //   diamond  degree-2 corner: for each triangle {v, a, b}, t_ab - 1;
 //            degree-3 corner sum_u C(t_vu, 2)
 //   4-clique listed once (oriented), each of its four vertices credited
-// NV[v] holds the eleven role counts in orbit order.  The input is the
-// union graph U of a static count (both flags on every entry, t of each
-// out-entry in tpack, T2 filled, w~ per pivot in U_wt).
+// The 4-cycle credits come from the counting pass itself (gc_cycles.cu in
+// its credit modes, in place of the global 4-cycle kernels), the triangle
+// and 4-clique credits from the root kernels below, everything else from one
+// row scan at the end.  The input is the union graph U of a static count (both
+// flags on every entry, t of each out-entry in tpack, T2 filled, the work bins
+// of the triangle roots).
 //
-// The second half of the file gives the same per edge (ten edge orbits,
-// k_e_*), and the 4-cycle walk of the heavy pivots shared by both
-// (k_c4_group: a few pivots at a time over the whole grid, their counters
-// resident in L2).
+// The second half of the file gives the same per edge (ten edge orbits).
+#include <algorithm>
+
 #include "gc_internal.cuh"
 #include "gc_kernels.cuh"
 
 namespace gcx {
-
-// role slots of NV, in orbit order 4..14
-enum { R_PEND, R_PMID, R_SLEAF, R_SCTR, R_C4, R_TTAIL, R_TOTH, R_TATT, R_D2, R_D3, R_K4, NROLE };
-// per-entry credit slots of the per-edge counts (the two entries of an edge are added at the end)
-enum { E_OPP, E_OUTER, E_C4, E_K4, NEROLE };
 
 // t of every entry (out-entries carry it; an in-entry reads its twin).
 __global__ void k_v_tsym(const Ctl* c, const int32_t* __restrict__ wlist, const long long* __restrict__ U_off,
@@ -80,13 +77,451 @@ __global__ void k_v_s(const Ctl* c, const int32_t* __restrict__ wlist, const lon
     }
 }
 
-// The row terms of each vertex: 3-path end and middle, 3-star leaf and
-// centre, tailed triangle tail end, other corner and attachment, diamond
-// degree-3 corner.
-__global__ void k_v_terms(const Ctl* c, const int32_t* __restrict__ wlist, const long long* __restrict__ U_off,
-                          const uint32_t* __restrict__ U_col, const uint32_t* __restrict__ tall,
-                          const long long* __restrict__ sdeg, const unsigned long long* __restrict__ T2,
-                          long long* __restrict__ NV) {
+
+// ---- triangles and 4-cliques of a root, credited ------------------------------
+//
+// As in the counting pass (gc_count.cu): root u, X = the entries of its
+// out-list, every entry y of N+(v), v in X, that is also in X closes the
+// triangle (u, v, y), listed once.  Here t of every edge is known, so X keeps
+// only entries with t > 0 (an edge in no triangle closes none): shorter lists,
+// fewer rows to walk.  Credits of a triangle:
+//   per vertex  t of the opposite edge - 1 to each corner (diamond degree 2)
+//   per edge    degree of the opposite corner - 2 (E_OPP), and the t of the
+//               two other edges - 2 (E_OUTER)
+// X's adjacency is kept as symmetric bit rows S; the 4-cliques through u and
+// X[q] are the triangles of S at q (half of sum over p in S[q] of
+// popcount(S[q] & S[p])), those through u, X[q], X[p] popcount(S[q] & S[p]).
+// Per edge, the pair credits go to the entry (X[q], X[p]), found by walking the
+// candidates a second time, only for roots with a 4-clique.
+//
+// A lane per out-edge merging two rows in global memory took 187 ms on the
+// 1.6M/30M graph (32 lanes on rows of very different lengths, three dependent
+// loads a step); the root kernels take about 12.
+
+struct TriCredits {
+    unsigned long long* d2;   // per vertex: diamond degree-2 corners
+    unsigned long long* k4v;  // per vertex: 4-cliques
+    unsigned long long* to;   // per entry, two words: E_OPP, E_OUTER
+    unsigned long long* k4e;  // per entry: 4-cliques
+};
+
+__device__ __forceinline__ void add_u64(unsigned long long* p, unsigned long long x) {
+    if (x) atomicAdd(p, x);
+}
+
+__device__ __forceinline__ int find_id(const uint32_t* s, int k, uint32_t y) {
+    int lo = 0, hi = k;
+    while (lo < hi) {
+        const int mid = (lo + hi) >> 1;
+        if (s[mid] < y) lo = mid + 1;
+        else hi = mid;
+    }
+    return (lo < k && s[lo] == y) ? lo : -1;
+}
+
+// Shared state of one root with up to KM kept entries.
+template <bool EDGE, int KM>
+struct RootState {
+    long long nb[KM];                 // start of N+(X[q])
+    unsigned long long c0[KM];        // per vertex: D2 of X[q]; per edge: E_OPP of (u, X[q])
+    unsigned long long c1[EDGE ? KM : 1];  // E_OUTER of (u, X[q])
+    uint32_t x[KM];                   // ids
+    uint32_t t[KM];                   // t of (u, X[q])
+    int pre[KM + 1];                  // candidates before row q
+    int at[KM];                       // position in u's out-list
+    int dg[EDGE ? KM : 1];            // degrees
+};
+
+// One triangle (u, X[q], X[p]) whose third edge is entry `slot`.
+template <bool EDGE, int KM>
+__device__ __forceinline__ void credit_triangle(RootState<EDGE, KM>& S, int q, int p, long long slot, uint32_t t3,
+                                                long long du, const TriCredits& cr, unsigned long long& mine) {
+    const unsigned long long tq = S.t[q], tp = S.t[p];
+    if (EDGE) {
+        atomicAdd(&S.c0[q], (unsigned long long)(S.dg[p] - 2));
+        atomicAdd(&S.c1[q], tp + t3 - 2);
+        atomicAdd(&S.c0[p], (unsigned long long)(S.dg[q] - 2));
+        atomicAdd(&S.c1[p], tq + t3 - 2);
+        add_u64(&cr.to[2 * slot], (unsigned long long)(du - 2));
+        add_u64(&cr.to[2 * slot + 1], tq + tp - 2);
+    } else {
+        mine += t3 - 1;
+        if (tp > 1) atomicAdd(&S.c0[q], tp - 1);
+        if (tq > 1) atomicAdd(&S.c0[p], tq - 1);
+    }
+}
+
+// Roots with short out-lists: a warp per root.
+constexpr int LT_WARPS = 8;
+template <bool EDGE>
+struct WarpRoot {
+    RootState<EDGE, 32> r;
+    uint32_t row[32];
+};
+template <bool EDGE>
+__global__ void __launch_bounds__(LT_WARPS * 32) k_l_tri_warp(const Ctl* c, const int32_t* __restrict__ list,
+                                                              const long long* __restrict__ U_off,
+                                                              const uint32_t* __restrict__ U_col,
+                                                              const int32_t* __restrict__ U_split,
+                                                              const uint32_t* __restrict__ tall, TriCredits cr) {
+    pdl_enter();
+    __shared__ WarpRoot<EDGE> s_w[LT_WARPS];
+    const int lane = threadIdx.x & 31;
+    WarpRoot<EDGE>& W = s_w[threadIdx.x >> 5];
+    RootState<EDGE, 32>& S = W.r;
+    const int cnt = c->nbin[BIN_TRI_WARP];
+    for (int i = blockIdx.x * LT_WARPS + (threadIdx.x >> 5); i < cnt; i += gridDim.x * LT_WARPS) {
+        const uint32_t u = (uint32_t)list[i];
+        const long long ub = U_off[u], ue = U_off[u + 1], rb = ub + U_split[u];
+        const int k0 = (int)(ue - rb);
+        const uint32_t t = lane < k0 ? tall[rb + lane] : 0u;
+        const unsigned keep = __ballot_sync(FULL, t > 0);
+        const int k = __popc(keep);
+        if (k < 2) continue;
+        if (t > 0) {
+            const int q = __popc(keep & lanemask_lt());
+            S.x[q] = vid(U_col[rb + lane]);
+            S.t[q] = t;
+            S.at[q] = lane;
+        }
+        __syncwarp();
+        const uint32_t xmax = S.x[k - 1];
+        int cq = 0;
+        if (lane < k) {
+            const uint32_t v = S.x[lane];
+            const long long vb = U_off[v], ve = U_off[v + 1], nb = vb + U_split[v];
+            S.nb[lane] = nb;
+            if (EDGE) S.dg[lane] = (int)(ve - vb);
+            cq = (int)lower_bound_id(U_col + nb, ve - nb, xmax + 1);
+        }
+        int inc = cq;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(FULL, inc, o);
+            if (lane >= o) inc += y;
+        }
+        const int total = __shfl_sync(FULL, inc, 31);
+        S.pre[lane + 1] = inc;
+        if (lane == 0) S.pre[0] = 0;
+        W.row[lane] = 0;
+        S.c0[lane] = 0;
+        if (EDGE) S.c1[lane] = 0;
+        __syncwarp();
+        unsigned long long mine = 0;
+        const long long du = ue - ub;
+        auto walk = [&](auto hit) {
+            int q = 0;
+            for (int j = lane; j < total; j += 32) {
+                while (q + 1 < k && S.pre[q + 1] <= j) q++;
+                const long long slot = S.nb[q] + (j - S.pre[q]);
+                const int p = find_id(S.x, k, vid(U_col[slot]));
+                if (p >= 0) hit(q, p, slot);
+            }
+        };
+        walk([&](int q, int p, long long slot) {
+            atomicOr(&W.row[q], 1u << p);
+            atomicOr(&W.row[p], 1u << q);
+            credit_triangle<EDGE, 32>(S, q, p, slot, tall[slot], du, cr, mine);
+        });
+        __syncwarp();
+        unsigned n3 = 0;  // 4-cliques through u and X[lane]
+        if (lane < k) {
+            const uint32_t s = W.row[lane];
+            for (uint32_t m = s; m; m &= m - 1) n3 += __popc(s & W.row[__ffs(m) - 1]);
+            n3 /= 2;
+        }
+        const unsigned any = __ballot_sync(FULL, n3 > 0);
+        if (EDGE) {
+            if (lane < k) {
+                const long long e = rb + S.at[lane];
+                add_u64(&cr.to[2 * e], S.c0[lane]);
+                add_u64(&cr.to[2 * e + 1], S.c1[lane]);
+                add_u64(&cr.k4e[e], n3);
+            }
+            if (any)
+                walk([&](int q, int p, long long slot) {
+                    add_u64(&cr.k4e[slot], (unsigned long long)__popc(W.row[q] & W.row[p]));
+                });
+        } else {
+            if (lane < k) {
+                add_u64(&cr.d2[S.x[lane]], S.c0[lane]);
+                add_u64(&cr.k4v[S.x[lane]], n3);
+            }
+            mine = warp_sum_u64(mine);
+            const unsigned all = any ? __reduce_add_sync(FULL, n3) : 0u;
+            if (lane == 0) {
+                add_u64(&cr.d2[u], mine);
+                add_u64(&cr.k4v[u], all / 3);
+            }
+        }
+        __syncwarp();
+    }
+}
+
+// Roots with longer out-lists: a block per root.
+template <bool EDGE, int KM>
+struct BlockRoot {
+    RootState<EDGE, KM> r;
+    uint32_t row[KM * (KM / 32)];
+};
+template <bool EDGE, int KM, int BIN, int WORK>
+__global__ void __launch_bounds__(256) k_l_tri_block(Ctl* c, const int32_t* __restrict__ list,
+                                                     const long long* __restrict__ U_off,
+                                                     const uint32_t* __restrict__ U_col,
+                                                     const int32_t* __restrict__ U_split,
+                                                     const uint32_t* __restrict__ tall, TriCredits cr) {
+    pdl_enter();
+    extern __shared__ __align__(16) unsigned char lt_smem[];
+    BlockRoot<EDGE, KM>& B = *(BlockRoot<EDGE, KM>*)lt_smem;
+    RootState<EDGE, KM>& S = B.r;
+    __shared__ int s_idx, s_k, s_any;
+    __shared__ unsigned long long s_mine, s_all;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, NW = blockDim.x >> 5;
+    const int cnt = c->nbin[BIN];
+    for (;;) {
+        if (tid == 0) {
+            s_idx = (int)atomicAdd(&c->work[WORK], 1u);
+            s_any = 0;
+            s_mine = s_all = 0;
+        }
+        __syncthreads();
+        const int idx = s_idx;
+        if (idx >= cnt) break;
+        const uint32_t u = (uint32_t)list[idx];
+        const long long ub = U_off[u], ue = U_off[u + 1], rb = ub + U_split[u], du = ue - ub;
+        if (warp == 0) {
+            const int k0 = (int)(ue - rb);
+            int k = 0;
+            for (int b = 0; b < k0; b += 32) {
+                const uint32_t t = b + lane < k0 ? tall[rb + b + lane] : 0u;
+                const unsigned keep = __ballot_sync(FULL, t > 0);
+                if (t > 0) {
+                    const int q = k + __popc(keep & lanemask_lt());
+                    S.x[q] = vid(U_col[rb + b + lane]);
+                    S.t[q] = t;
+                    S.at[q] = b + lane;
+                }
+                k += __popc(keep);
+            }
+            if (lane == 0) s_k = k;
+        }
+        __syncthreads();
+        const int k = s_k, W = (k + 31) >> 5;
+        if (k < 2) {
+            __syncthreads();
+            continue;
+        }
+        const uint32_t xmax = S.x[k - 1];
+        for (int q = tid; q < k; q += blockDim.x) {
+            const uint32_t v = S.x[q];
+            const long long vb = U_off[v], ve = U_off[v + 1], nb = vb + U_split[v];
+            S.nb[q] = nb;
+            if (EDGE) S.dg[q] = (int)(ve - vb);
+            S.pre[q + 1] = (int)lower_bound_id(U_col + nb, ve - nb, xmax + 1);
+            S.c0[q] = 0;
+            if (EDGE) S.c1[q] = 0;
+        }
+        for (int j = tid; j < k * W; j += blockDim.x) B.row[j] = 0;
+        __syncthreads();
+        if (warp == 0) {  // inclusive scan of pre[1..k]
+            int carry = 0;
+            for (int b = 0; b < k; b += 32) {
+                int x = b + lane < k ? S.pre[b + lane + 1] : 0;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const int y = __shfl_up_sync(FULL, x, o);
+                    if (lane >= o) x += y;
+                }
+                if (b + lane < k) S.pre[b + lane + 1] = x + carry;
+                carry += __shfl_sync(FULL, x, 31);
+            }
+            if (lane == 0) S.pre[0] = 0;
+        }
+        __syncthreads();
+        const int total = S.pre[k];
+        unsigned long long mine = 0;
+        auto walk = [&](auto hit) {
+            for (int base = warp * 32; base < total; base += NW * 32) {
+                int q = 0, hi = k;  // row of candidate `base`
+                while (hi - q > 1) {
+                    const int mid = (q + hi) >> 1;
+                    if (S.pre[mid] <= base) q = mid;
+                    else hi = mid;
+                }
+                const int j = base + lane;
+                if (j >= total) continue;
+                while (q + 1 < k && S.pre[q + 1] <= j) q++;
+                const long long slot = S.nb[q] + (j - S.pre[q]);
+                const int p = find_id(S.x, k, vid(U_col[slot]));
+                if (p >= 0) hit(q, p, slot);
+            }
+        };
+        walk([&](int q, int p, long long slot) {
+            atomicOr(&B.row[q * W + (p >> 5)], 1u << (p & 31));
+            atomicOr(&B.row[p * W + (q >> 5)], 1u << (q & 31));
+            credit_triangle<EDGE, KM>(S, q, p, slot, tall[slot], du, cr, mine);
+        });
+        __syncthreads();
+        unsigned long long all = 0;
+        for (int q = tid; q < k; q += blockDim.x) {
+            const uint32_t* s = B.row + q * W;
+            unsigned long long n3 = 0;  // 4-cliques through u and X[q], twice
+            for (int i = 0; i < W; i++)
+                for (uint32_t m = s[i]; m; m &= m - 1) {
+                    const uint32_t* r = B.row + (i * 32 + __ffs(m) - 1) * W;
+                    for (int j = 0; j < W; j++) n3 += __popc(s[j] & r[j]);
+                }
+            n3 /= 2;
+            all += n3;
+            if (EDGE) {
+                const long long e = rb + S.at[q];
+                add_u64(&cr.to[2 * e], S.c0[q]);
+                add_u64(&cr.to[2 * e + 1], S.c1[q]);
+                add_u64(&cr.k4e[e], n3);
+            } else {
+                add_u64(&cr.d2[S.x[q]], S.c0[q]);
+                add_u64(&cr.k4v[S.x[q]], n3);
+            }
+        }
+        if (EDGE) {
+            if (all) s_any = 1;
+            __syncthreads();
+            if (s_any)
+                walk([&](int q, int p, long long slot) {
+                    unsigned x = 0;
+                    for (int j = 0; j < W; j++) x += __popc(B.row[q * W + j] & B.row[p * W + j]);
+                    add_u64(&cr.k4e[slot], x);
+                });
+        } else {
+            mine = warp_sum_u64(mine);
+            all = warp_sum_u64(all);
+            if (lane == 0 && (mine | all)) {
+                atomicAdd(&s_mine, mine);
+                atomicAdd(&s_all, all);
+            }
+            __syncthreads();
+            if (tid == 0) {
+                add_u64(&cr.d2[u], s_mine);
+                add_u64(&cr.k4v[u], s_all / 3);
+            }
+        }
+        __syncthreads();
+    }
+}
+
+// Roots with out-lists beyond the block tier: a warp per root, a lane per
+// out-edge e = (u, v) merging N+(u) after v with N+(v).
+template <bool EDGE>
+__global__ void k_l_tri_merge(const Ctl* c, const int32_t* __restrict__ list, const long long* __restrict__ U_off,
+                              const uint32_t* __restrict__ U_col, const int32_t* __restrict__ U_split,
+                              const uint32_t* __restrict__ tall, TriCredits cr) {
+    pdl_enter();
+    const int cnt = c->nbin[BIN_TRI_MERGE];
+    const int lane = threadIdx.x & 31;
+    const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int nwarps = (gridDim.x * blockDim.x) >> 5;
+    for (int wi = warp; wi < cnt; wi += nwarps) {
+        const uint32_t u = (uint32_t)list[wi];
+        const long long ob = U_off[u] + U_split[u], oe = U_off[u + 1], du = oe - U_off[u];
+        for (long long e = ob + lane; e < oe; e += 32) {
+            const unsigned long long te = tall[e];
+            if (!te) continue;
+            const uint32_t v = vid(U_col[e]);
+            const long long vb = U_off[v] + U_split[v], ve = U_off[v + 1], dv = ve - U_off[v];
+            long long i = e + 1, j = vb;
+            unsigned long long k4 = 0;
+            while (i < oe && j < ve) {
+                const uint32_t x = vid(U_col[i]), y = vid(U_col[j]);
+                if (x < y) {
+                    i++;
+                } else if (x > y) {
+                    j++;
+                } else {
+                    // triangle (u, v, y): t of uv, uy, vy at e, i, j
+                    const unsigned long long ti = tall[i], tj = tall[j];
+                    const long long yb = U_off[y] + U_split[y], ye = U_off[y + 1], dy = ye - U_off[y];
+                    if (EDGE) {
+                        add_u64(&cr.to[2 * e], (unsigned long long)(dy - 2));
+                        add_u64(&cr.to[2 * e + 1], ti + tj - 2);
+                        add_u64(&cr.to[2 * i], (unsigned long long)(dv - 2));
+                        add_u64(&cr.to[2 * i + 1], te + tj - 2);
+                        add_u64(&cr.to[2 * j], (unsigned long long)(du - 2));
+                        add_u64(&cr.to[2 * j + 1], te + ti - 2);
+                    } else {
+                        add_u64(&cr.d2[u], tj - 1);
+                        add_u64(&cr.d2[v], ti - 1);
+                        add_u64(&cr.d2[y], te - 1);
+                    }
+                    // 4-cliques (u, v, y, z), z > y in N+(u), N+(v), N+(y)
+                    long long p = i + 1, q = j + 1, r = yb;
+                    unsigned long long kk = 0;
+                    while (p < oe && q < ve && r < ye) {
+                        const uint32_t a = vid(U_col[p]), b = vid(U_col[q]), z = vid(U_col[r]);
+                        const uint32_t mx = max(a, max(b, z));
+                        if (a == mx && b == mx && z == mx) {
+                            if (EDGE) {
+                                atomicAdd(&cr.k4e[p], 1ull);
+                                atomicAdd(&cr.k4e[q], 1ull);
+                                atomicAdd(&cr.k4e[r], 1ull);
+                            } else {
+                                atomicAdd(&cr.k4v[a], 1ull);
+                            }
+                            kk++;
+                            p++;
+                            q++;
+                            r++;
+                        } else {
+                            if (a < mx) p++;
+                            if (b < mx) q++;
+                            if (z < mx) r++;
+                        }
+                    }
+                    if (EDGE) {
+                        add_u64(&cr.k4e[i], kk);
+                        add_u64(&cr.k4e[j], kk);
+                    } else {
+                        add_u64(&cr.k4v[v], kk);
+                        add_u64(&cr.k4v[y], kk);
+                    }
+                    k4 += kk;
+                    i++;
+                    j++;
+                }
+            }
+            add_u64(EDGE ? &cr.k4e[e] : &cr.k4v[u], k4);
+        }
+    }
+}
+
+template <bool EDGE>
+static int enqueue_tri_credits(Ctl* ctl, const int32_t* bins, int n, const long long* U_off, const uint32_t* U_col,
+                               const int32_t* U_split, const uint32_t* tall, const TriCredits& cr, int sms,
+                               cudaStream_t s) {
+    const auto small = k_l_tri_block<EDGE, TRI_KS, BIN_TRI_SMALL, WORK_LT_SMALL>;
+    const auto block = k_l_tri_block<EDGE, TRI_KM, BIN_TRI_BLOCK, WORK_LT_BLOCK>;
+    constexpr size_t sm_small = sizeof(BlockRoot<EDGE, TRI_KS>), sm_block = sizeof(BlockRoot<EDGE, TRI_KM>);
+    cudaFuncSetAttribute(block, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm_block);
+    auto list = [&](int b) { return bins + (size_t)b * n; };
+    pdl_launch(k_l_tri_warp<EDGE>, dim3(6 * sms), dim3(LT_WARPS * 32), 0, s, ctl, list(BIN_TRI_WARP), U_off, U_col,
+               U_split, tall, cr);
+    pdl_launch(small, dim3(8 * sms), dim3(256), sm_small, s, ctl, list(BIN_TRI_SMALL), U_off, U_col, U_split, tall, cr);
+    pdl_launch(block, dim3(2 * sms), dim3(256), sm_block, s, ctl, list(BIN_TRI_BLOCK), U_off, U_col, U_split, tall, cr);
+    pdl_launch(k_l_tri_merge<EDGE>, dim3(sms), dim3(256), 0, s, ctl, list(BIN_TRI_MERGE), U_off, U_col, U_split, tall,
+               cr);
+    return 4;
+}
+
+// ---- per vertex -----------------------------------------------------------------
+
+// The row terms of each vertex, the credits, and the inversion: orbit counts
+// by the triangular role containment; out[k v + j] by external id: the eleven
+// orbits (k = 11) or their sums per graphlet (k = 6).  A warp per vertex.
+__global__ void k_v_finalize(const Ctl* c, const int32_t* __restrict__ wlist, const long long* __restrict__ U_off,
+                             const uint32_t* __restrict__ U_col, const uint32_t* __restrict__ tall,
+                             const long long* __restrict__ sdeg, const unsigned long long* __restrict__ T2,
+                             const unsigned long long* __restrict__ d2, const unsigned long long* __restrict__ k4,
+                             const unsigned long long* __restrict__ c4, const int32_t* __restrict__ iperm, int k,
+                             unsigned long long* __restrict__ out) {
     pdl_enter();
     const int nW = c->nW;
     const int lane = threadIdx.x & 31;
@@ -114,302 +549,29 @@ __global__ void k_v_terms(const Ctl* c, const int32_t* __restrict__ wlist, const
         to = (long long)warp_sum_u64((unsigned long long)to);
         d3 = (long long)warp_sum_u64((unsigned long long)d3);
         if (lane == 0) {
-            long long* o = NV + NROLE * (size_t)v;
-            o[R_PEND] += pe - 2 * trv;
-            o[R_PMID] += pm;
-            o[R_SLEAF] += sl;
-            o[R_SCTR] += d * (d - 1) * (d - 2) / 6;
-            o[R_TTAIL] += tl;
-            o[R_TOTH] += to;
-            o[R_TATT] += trv * (d - 2);
-            o[R_D3] += d3;
-        }
-    }
-}
-
-// Triangles u < v < y (each once): the degree-2 corner part of the
-// diamonds (t of the opposite edge - 1 to each corner); 4-cliques
-// u < v < y < z (each once) credited to their four vertices.  A warp per
-// root u, a lane per out-edge (out-lists are short in the degree order).
-__global__ void k_v_tri_k4(const Ctl* c, const int32_t* __restrict__ wlist, const long long* __restrict__ U_off,
-                           const uint32_t* __restrict__ U_col, const int32_t* __restrict__ U_split,
-                           const uint32_t* __restrict__ tall, long long* __restrict__ NV) {
-    pdl_enter();
-    const int nW = c->nW;
-    const int lane = threadIdx.x & 31;
-    const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int nwarps = (gridDim.x * blockDim.x) >> 5;
-    for (int wi = warp; wi < nW; wi += nwarps) {
-        const uint32_t u = (uint32_t)wlist[wi];
-        const long long ob = U_off[u] + U_split[u], oe = U_off[u + 1];
-        for (long long e = ob + lane; e < oe; e += 32) {
-            const uint32_t v = vid(U_col[e]);
-            const long long vb = U_off[v] + U_split[v], ve = U_off[v + 1];
-            long long i = e + 1, j = vb;
-            long long k4u = 0;
-            while (i < oe && j < ve) {
-                const uint32_t x = vid(U_col[i]), y = vid(U_col[j]);
-                if (x < y) {
-                    i++;
-                } else if (x > y) {
-                    j++;
-                } else {
-                    // triangle (u, v, y): t of uv, uy, vy at e, i, j
-                    atomicAdd((unsigned long long*)&NV[NROLE * (size_t)u + R_D2],
-                              (unsigned long long)((long long)tall[j] - 1));
-                    atomicAdd((unsigned long long*)&NV[NROLE * (size_t)v + R_D2],
-                              (unsigned long long)((long long)tall[i] - 1));
-                    atomicAdd((unsigned long long*)&NV[NROLE * (size_t)y + R_D2],
-                              (unsigned long long)((long long)tall[e] - 1));
-                    // 4-cliques (u, v, y, z), z > y in N+(u), N+(v), N+(y)
-                    const long long yb = U_off[y] + U_split[y], ye = U_off[y + 1];
-                    long long p = i + 1, q = j + 1, r = yb, kk = 0;
-                    while (p < oe && q < ve && r < ye) {
-                        const uint32_t a = vid(U_col[p]), b = vid(U_col[q]), cc = vid(U_col[r]);
-                        const uint32_t mx = max(a, max(b, cc));
-                        if (a == mx && b == mx && cc == mx) {
-                            atomicAdd((unsigned long long*)&NV[NROLE * (size_t)a + R_K4], 1ull);
-                            kk++;
-                            p++;
-                            q++;
-                            r++;
-                        } else {
-                            if (a < mx) p++;
-                            if (b < mx) q++;
-                            if (cc < mx) r++;
-                        }
-                    }
-                    if (kk) {
-                        atomicAdd((unsigned long long*)&NV[NROLE * (size_t)v + R_K4], (unsigned long long)kk);
-                        atomicAdd((unsigned long long*)&NV[NROLE * (size_t)y + R_K4], (unsigned long long)kk);
-                        k4u += kk;
-                    }
-                    i++;
-                    j++;
-                }
-            }
-            if (k4u) atomicAdd((unsigned long long*)&NV[NROLE * (size_t)u + R_K4], (unsigned long long)k4u);
-        }
-    }
-}
-
-// 4-cycles, a block per pivot u (its highest vertex) with one dense counter
-// array of n words per block: walk 1 counts c_w over the wedges u-a-w
-// (a, w below u), walk 2 credits each middle a with c_w - 1, walk 3 takes
-// and clears c_w, crediting w and u with C(c_w, 2).
-__global__ void __launch_bounds__(1024) k_v_c4(const Ctl* c, const int32_t* __restrict__ wlist,
-                                               const long long* __restrict__ U_off,
-                                               const uint32_t* __restrict__ U_col,
-                                               const int32_t* __restrict__ U_split, uint32_t* __restrict__ cnt_all,
-                                               int n, const uint8_t* __restrict__ heavy,
-                                               long long* __restrict__ NV) {
-    pdl_enter();
-    const int nW = c->nW;
-    uint32_t* cnt = cnt_all + (size_t)blockIdx.x * (size_t)n;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, NWp = blockDim.x >> 5;
-    __shared__ unsigned long long s_u[32];
-    for (int pi = blockIdx.x; pi < nW; pi += gridDim.x) {
-        const uint32_t u = (uint32_t)wlist[pi];
-        if (heavy && heavy[u]) continue;  // taken by k_c4_group (same for the whole block)
-        const long long rb = U_off[u];
-        const int nlow = U_split[u];
-        unsigned long long usum = 0;
-        for (int pass = 0; pass < 3; pass++) {
-            for (int j = warp; j < nlow; j += NWp) {
-                const uint32_t a = vid(U_col[rb + j]);
-                const long long ab = U_off[a], ae = U_off[a + 1];
-                long long asum = 0;
-                for (long long q = ab + lane; q < ae; q += 32) {
-                    const uint32_t w = vid(U_col[q]);
-                    if (w >= u) break;  // rows are sorted: the rest is above u
-                    if (pass == 0) {
-                        atomicAdd(&cnt[w], 1u);
-                    } else if (pass == 1) {
-                        asum += (long long)__ldcg(&cnt[w]) - 1;
-                    } else {
-                        const uint32_t old = atomicExch(&cnt[w], 0u);
-                        if (old >= 2) {
-                            const unsigned long long cy = (unsigned long long)old * (old - 1) / 2;
-                            atomicAdd((unsigned long long*)&NV[NROLE * (size_t)w + R_C4], cy);
-                            usum += cy;
-                        }
-                    }
-                }
-                if (pass == 1) {
-                    asum = (long long)warp_sum_u64((unsigned long long)asum);
-                    if (lane == 0 && asum) atomicAdd((unsigned long long*)&NV[NROLE * (size_t)a + R_C4],
-                        (unsigned long long)asum);
-                }
-            }
-            __threadfence();
-            __syncthreads();
-        }
-        usum = warp_sum_u64(usum);
-        if (lane == 0) s_u[warp] = usum;
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            unsigned long long t = 0;
-            for (int w = 0; w < NWp; w++) t += s_u[w];
-            if (t) atomicAdd((unsigned long long*)&NV[NROLE * (size_t)u + R_C4], t);  // other blocks credit u too
-        }
-        __syncthreads();
-    }
-}
-
-// Heavy 4-cycle pivots of the local counts: w~(u) (the sum of the degrees
-// of u's lower neighbours, from the static pass) at least heavy_min.  They
-// are listed for k_c4_group and flagged so that the per-block walk skips
-// them.
-__global__ void k_c4_heavy_mark(const Ctl* c, const int32_t* __restrict__ wlist, const long long* __restrict__ U_wt,
-                                long long heavy_min, uint8_t* __restrict__ heavy, int32_t* __restrict__ hlist,
-                                int* __restrict__ hcount) {
-    pdl_enter();
-    const int nW = c->nW;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < nW; i += gridDim.x * blockDim.x) {
-        const int32_t u = wlist[i];
-        const bool h = U_wt[u] >= heavy_min;
-        heavy[u] = h ? 1 : 0;
-        if (h) hlist[atomicAdd(hcount, 1)] = u;
-    }
-}
-
-// One walk of the 4-cycle counting for up to C4G heavy pivots at once
-// (hlist[first .. first + count)), each with its own dense counter array of
-// n words (C4G arrays of 4 n bytes stay resident in L2 on graphs of a few
-// million vertices).  The whole grid shares the work: the (pivot, lower
-// neighbour a) pairs of the group are numbered and dealt to warps, the
-// lanes of a warp walk a's row below the pivot.  The three walks are three
-// launches (pass 0 count c_w, 1 credit c_w - 1, 2 clear), so the kernel
-// boundary is the only barrier between them.  EDGE: credits go to the two
-// entries of each wedge (per-edge 4-cycle role), else to the middle vertex
-// a in pass 1 and to the corners w and u with C(c_w, 2) in pass 2.
-template <bool EDGE>
-__global__ void k_c4_group(const int32_t* __restrict__ hlist, int first, int count,
-                           const long long* __restrict__ U_off, const uint32_t* __restrict__ U_col,
-                           const int32_t* __restrict__ U_split, uint32_t* __restrict__ cnt_g, int n, int pass,
-                           long long* __restrict__ acc) {
-    pdl_enter();
-    const int lane = threadIdx.x & 31;
-    const int gwarp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int nwarps = (gridDim.x * blockDim.x) >> 5;
-    // lane p < count holds slot p: its pivot and the inclusive prefix of the
-    // lower-neighbour counts
-    uint32_t up = 0;
-    long long nl = 0;
-    if (lane < count) {
-        up = (uint32_t)hlist[first + lane];
-        nl = U_split[up];
-    }
-    long long incl = nl;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const long long y = __shfl_up_sync(FULL, incl, o);
-        if (lane >= o) incl += y;
-    }
-    const long long total = __shfl_sync(FULL, incl, 31);
-    const long long excl = incl - nl;
-    for (long long k = gwarp; k < total; k += nwarps) {
-        const int p = __popc(__ballot_sync(FULL, incl <= k));  // the slot holding pair k
-        const uint32_t u = __shfl_sync(FULL, up, p);
-        const long long j = k - __shfl_sync(FULL, excl, p);
-        uint32_t* cnt = cnt_g + (size_t)p * (size_t)n;
-        const long long ea = U_off[u] + j;  // entry (u, a)
-        const uint32_t a = vid(U_col[ea]);
-        const long long ab = U_off[a], ae = U_off[a + 1];
-        long long asum = 0;
-        unsigned long long usum = 0;
-        for (long long q = ab + lane; q < ae; q += 32) {
-            const uint32_t w = vid(U_col[q]);
-            if (w >= u) break;  // rows are sorted: the rest is above u
-            if (pass == 0) {
-                atomicAdd(&cnt[w], 1u);
-            } else if (pass == 1) {
-                const long long x = (long long)__ldcg(&cnt[w]) - 1;
-                if (x > 0) {
-                    if (EDGE) atomicAdd((unsigned long long*)&acc[NEROLE * (size_t)q + E_C4], (unsigned long long)x);
-                    asum += x;
-                }
-            } else if (EDGE) {
-                cnt[w] = 0u;
+            const long long o14 = (long long)k4[v];
+            const long long o13 = d3 - 3 * o14;
+            const long long o12 = (long long)d2[v] - 3 * o14;
+            const long long o11 = trv * (d - 2) - 2 * o13 - 3 * o14;
+            const long long o10 = to - 2 * o12 - 2 * o13 - 6 * o14;
+            const long long o9 = tl - 2 * o12 - 3 * o14;
+            const long long o8 = (long long)c4[v] - o12 - o13 - 3 * o14;
+            const long long o7 = d * (d - 1) * (d - 2) / 6 - o11 - o13 - o14;
+            const long long o6 = sl - o9 - o10 - 2 * o12 - o13 - 3 * o14;
+            const long long o5 = pm - 2 * o8 - o10 - 2 * o11 - 2 * o12 - 4 * o13 - 6 * o14;
+            const long long o4 = pe - 2 * trv - 2 * o8 - 2 * o9 - o10 - 4 * o12 - 2 * o13 - 6 * o14;
+            unsigned long long* o = out + (size_t)k * iperm[v];
+            if (k == 11) {
+                const long long orb[11] = {o4, o5, o6, o7, o8, o9, o10, o11, o12, o13, o14};
+                for (int j = 0; j < 11; j++) o[j] = (unsigned long long)orb[j];
             } else {
-                const uint32_t old = atomicExch(&cnt[w], 0u);
-                if (old >= 2) {
-                    const unsigned long long cy = (unsigned long long)old * (old - 1) / 2;
-                    atomicAdd((unsigned long long*)&acc[NROLE * (size_t)w + R_C4], cy);
-                    usum += cy;
-                }
+                o[0] = (unsigned long long)(o4 + o5);
+                o[1] = (unsigned long long)(o6 + o7);
+                o[2] = (unsigned long long)o8;
+                o[3] = (unsigned long long)(o9 + o10 + o11);
+                o[4] = (unsigned long long)(o12 + o13);
+                o[5] = (unsigned long long)o14;
             }
-        }
-        if (pass == 1) {
-            asum = (long long)warp_sum_u64((unsigned long long)asum);
-            if (lane == 0 && asum) {
-                if (EDGE) atomicAdd((unsigned long long*)&acc[NEROLE * (size_t)ea + E_C4], (unsigned long long)asum);
-                else atomicAdd((unsigned long long*)&acc[NROLE * (size_t)a + R_C4], (unsigned long long)asum);
-            }
-        } else if (pass == 2 && !EDGE) {
-            usum = warp_sum_u64(usum);
-            if (lane == 0 && usum) atomicAdd((unsigned long long*)&acc[NROLE * (size_t)u + R_C4], usum);
-        }
-    }
-}
-
-// The heavy pivots: mark them, read their number back, then three launches
-// per group of C4G.  Returns the launches made, or -1 on a CUDA error.
-template <bool EDGE>
-static int enqueue_heavy_c4(const HeavyC4& h, Ctl* ctl, const int32_t* wlist, const long long* U_off,
-                            const uint32_t* U_col, const int32_t* U_split, int n, int sms, long long* acc,
-                            cudaStream_t s) {
-    if (h.heavy_min <= 0) return 0;
-    int nl = 0;
-    if (cudaMemsetAsync(h.hcount, 0, sizeof(int), s) != cudaSuccess) return -1;
-    pdl_launch(k_c4_heavy_mark, dim3(std::max(1, std::min(8 * sms, (n + 255) / 256))), dim3(256), 0, s, ctl, wlist,
-               h.U_wt, h.heavy_min, h.heavy, h.hlist, h.hcount);
-    nl++;
-    int H = 0;
-    if (cudaMemcpyAsync(&H, h.hcount, sizeof(int), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
-        cudaStreamSynchronize(s) != cudaSuccess)
-        return -1;
-    for (int first = 0; first < H; first += C4G) {
-        const int cnt = std::min(C4G, H - first);
-        for (int pass = 0; pass < 3; pass++) {
-            pdl_launch(k_c4_group<EDGE>, dim3(8 * sms), dim3(256), 0, s, (const int32_t*)h.hlist, first, cnt, U_off,
-                       U_col, U_split, h.cnt_g, n, pass, acc);
-            nl++;
-        }
-    }
-    return nl;
-}
-
-// Orbit counts per vertex by the triangular role containment; out[k v + j]
-// by external id: the eleven orbits (k = 11) or their sums per graphlet
-// (k = 6).
-__global__ void k_v_finalize(const long long* __restrict__ NV, int n, const int32_t* __restrict__ iperm, int k,
-                             unsigned long long* __restrict__ out) {
-    pdl_enter();
-    for (int v = blockIdx.x * blockDim.x + threadIdx.x; v < n; v += gridDim.x * blockDim.x) {
-        const long long* r = NV + NROLE * (size_t)v;
-        const long long o14 = r[R_K4];
-        const long long o13 = r[R_D3] - 3 * o14;
-        const long long o12 = r[R_D2] - 3 * o14;
-        const long long o11 = r[R_TATT] - 2 * o13 - 3 * o14;
-        const long long o10 = r[R_TOTH] - 2 * o12 - 2 * o13 - 6 * o14;
-        const long long o9 = r[R_TTAIL] - 2 * o12 - 3 * o14;
-        const long long o8 = r[R_C4] - o12 - o13 - 3 * o14;
-        const long long o7 = r[R_SCTR] - o11 - o13 - o14;
-        const long long o6 = r[R_SLEAF] - o9 - o10 - 2 * o12 - o13 - 3 * o14;
-        const long long o5 = r[R_PMID] - 2 * o8 - o10 - 2 * o11 - 2 * o12 - 4 * o13 - 6 * o14;
-        const long long o4 = r[R_PEND] - 2 * o8 - 2 * o9 - o10 - 4 * o12 - 2 * o13 - 6 * o14;
-        unsigned long long* o = out + (size_t)k * iperm[v];
-        if (k == 11) {
-            const long long orb[11] = {o4, o5, o6, o7, o8, o9, o10, o11, o12, o13, o14};
-            for (int j = 0; j < 11; j++) o[j] = (unsigned long long)orb[j];
-        } else {
-            o[0] = (unsigned long long)(o4 + o5);
-            o[1] = (unsigned long long)(o6 + o7);
-            o[2] = (unsigned long long)o8;
-            o[3] = (unsigned long long)(o9 + o10 + o11);
-            o[4] = (unsigned long long)(o12 + o13);
-            o[5] = (unsigned long long)o14;
         }
     }
 }
@@ -423,175 +585,52 @@ __global__ void k_v_finalize(const long long* __restrict__ NV, int n, const int3
 // (tri(x) = T2[x] / 2, s(x) = sum_{w in N(x)} (d_w - 1)):
 //   3-path end   (s(v) - (d_u - 1) - t) + (s(u) - (d_v - 1) - t)
 //   3-path middle (d_u - 1)(d_v - 1) - t;  3-star C(d_u - 1, 2) + C(d_v - 1, 2)
-//   4-cycle      credited by the pivot walk below
+//   4-cycle      credited by the counting pass (gc_cycles.cu)
 //   tail         (tri(u) - t) + (tri(v) - t);  attachment t (d_u + d_v - 4)
 //   opposite     sum over triangles {u, v, w} of d_w - 2
 //   diamond outer  sum over triangles {u, v, w} of t_uw + t_vw - 2
 //   chord C(t, 2);  4-clique credited by the clique listing
-// Credits land on either entry of the edge; the finalize adds both.
+// 4-cycle credits land on either entry of the edge (the finalize adds both),
+// triangle and 4-clique credits on the out-entry.
 
-// One sort key per entry: the out-entry (x < y) of an edge gets its
-// external pair (lo << nb) | hi, every in-entry the largest nb-bit pair,
-// so after the sort the first m keys are the edges in external order.
+// One sort key per edge, its external pair (lo << nb) | hi, from the
+// out-entries: vertex u's keys start at out_off[u].
+__global__ void k_e_outdeg(int n, const long long* __restrict__ U_off, const int32_t* __restrict__ U_split,
+                           int32_t* __restrict__ outdeg) {
+    pdl_enter();
+    for (int u = blockIdx.x * blockDim.x + threadIdx.x; u < n; u += gridDim.x * blockDim.x)
+        outdeg[u] = (int32_t)(U_off[u + 1] - U_off[u]) - U_split[u];
+}
 __global__ void k_e_keys(const Ctl* c, const int32_t* __restrict__ wlist, const long long* __restrict__ U_off,
                          const uint32_t* __restrict__ U_col, const int32_t* __restrict__ U_split,
-                         const int32_t* __restrict__ iperm, int nb, unsigned long long* __restrict__ keys) {
+                         const int32_t* __restrict__ iperm, int nb, const long long* __restrict__ out_off,
+                         unsigned long long* __restrict__ keys) {
     pdl_enter();
     const int nW = c->nW;
     const int lane = threadIdx.x & 31;
     const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int nwarps = (gridDim.x * blockDim.x) >> 5;
-    const unsigned long long none = (1ull << (2 * nb)) - 1;
     for (int i = warp; i < nW; i += nwarps) {
         const uint32_t u = (uint32_t)wlist[i];
-        const long long ob = U_off[u] + U_split[u];
+        const long long ob = U_off[u] + U_split[u], to = out_off[u] - ob;
         const unsigned long long a = (unsigned long long)iperm[u];
-        for (long long e = U_off[u] + lane; e < U_off[u + 1]; e += 32) {
-            if (e < ob) {
-                keys[e] = none;
-            } else {
-                const unsigned long long b = (unsigned long long)iperm[vid(U_col[e])];
-                keys[e] = a < b ? (a << nb) | b : (b << nb) | a;
-            }
-        }
-    }
-}
-
-// Triangles u < v < y (each once) credit the opposite and diamond-outer
-// terms of their three edges; 4-cliques u < v < y < z (each once) credit
-// their six edges.  A warp per root u, a lane per out-edge e = (u, v).
-__global__ void k_e_tri_k4(const Ctl* c, const int32_t* __restrict__ wlist, const long long* __restrict__ U_off,
-                           const uint32_t* __restrict__ U_col, const int32_t* __restrict__ U_split,
-                           const uint32_t* __restrict__ tall, long long* __restrict__ NE) {
-    pdl_enter();
-    const int nW = c->nW;
-    const int lane = threadIdx.x & 31;
-    const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int nwarps = (gridDim.x * blockDim.x) >> 5;
-    for (int wi = warp; wi < nW; wi += nwarps) {
-        const uint32_t u = (uint32_t)wlist[wi];
-        const long long ob = U_off[u] + U_split[u], oe = U_off[u + 1];
-        const long long du = U_off[u + 1] - U_off[u];
-        for (long long e = ob + lane; e < oe; e += 32) {
-            const uint32_t v = vid(U_col[e]);
-            const long long vb = U_off[v] + U_split[v], ve = U_off[v + 1];
-            const long long dv = U_off[v + 1] - U_off[v], te = tall[e];
-            long long i = e + 1, j = vb;
-            long long opp = 0, outer = 0, k4 = 0;
-            while (i < oe && j < ve) {
-                const uint32_t x = vid(U_col[i]), y = vid(U_col[j]);
-                if (x < y) {
-                    i++;
-                } else if (x > y) {
-                    j++;
-                } else {
-                    // triangle (u, v, y): edges uv, uy, vy at e, i, j
-                    const long long dy = U_off[y + 1] - U_off[y], ti = tall[i], tj = tall[j];
-                    opp += dy - 2;
-                    outer += ti + tj - 2;
-                    atomicAdd((unsigned long long*)&NE[NEROLE * (size_t)i + E_OPP], (unsigned long long)(dv - 2));
-                    atomicAdd((unsigned long long*)&NE[NEROLE * (size_t)i + E_OUTER],
-                              (unsigned long long)(te + tj - 2));
-                    atomicAdd((unsigned long long*)&NE[NEROLE * (size_t)j + E_OPP], (unsigned long long)(du - 2));
-                    atomicAdd((unsigned long long*)&NE[NEROLE * (size_t)j + E_OUTER],
-                              (unsigned long long)(te + ti - 2));
-                    // 4-cliques (u, v, y, z), z > y: edges uz, vz, yz at p, q, r
-                    const long long yb = U_off[y] + U_split[y], ye = U_off[y + 1];
-                    long long p = i + 1, q = j + 1, r = yb, kk = 0;
-                    while (p < oe && q < ve && r < ye) {
-                        const uint32_t a = vid(U_col[p]), b = vid(U_col[q]), cc = vid(U_col[r]);
-                        const uint32_t mx = max(a, max(b, cc));
-                        if (a == mx && b == mx && cc == mx) {
-                            atomicAdd((unsigned long long*)&NE[NEROLE * (size_t)p + E_K4], 1ull);
-                            atomicAdd((unsigned long long*)&NE[NEROLE * (size_t)q + E_K4], 1ull);
-                            atomicAdd((unsigned long long*)&NE[NEROLE * (size_t)r + E_K4], 1ull);
-                            kk++;
-                            p++;
-                            q++;
-                            r++;
-                        } else {
-                            if (a < mx) p++;
-                            if (b < mx) q++;
-                            if (cc < mx) r++;
-                        }
-                    }
-                    if (kk) {
-                        atomicAdd((unsigned long long*)&NE[NEROLE * (size_t)i + E_K4], (unsigned long long)kk);
-                        atomicAdd((unsigned long long*)&NE[NEROLE * (size_t)j + E_K4], (unsigned long long)kk);
-                        k4 += kk;
-                    }
-                    i++;
-                    j++;
-                }
-            }
-            if (opp) atomicAdd((unsigned long long*)&NE[NEROLE * (size_t)e + E_OPP], (unsigned long long)opp);
-            if (outer) atomicAdd((unsigned long long*)&NE[NEROLE * (size_t)e + E_OUTER], (unsigned long long)outer);
-            if (k4) atomicAdd((unsigned long long*)&NE[NEROLE * (size_t)e + E_K4], (unsigned long long)k4);
-        }
-    }
-}
-
-// 4-cycles per edge, a block per pivot u (the highest vertex of the cycle)
-// with one dense counter array of n words per block: walk 1 counts c_w over
-// the wedges u-a-w (a, w below u); walk 2 credits each wedge's two edges
-// u-a and a-w with c_w - 1 (the cycles u-a-w-b, b another middle); walk 3
-// clears the counters.
-__global__ void __launch_bounds__(1024) k_e_c4(const Ctl* c, const int32_t* __restrict__ wlist,
-                                               const long long* __restrict__ U_off,
-                                               const uint32_t* __restrict__ U_col,
-                                               const int32_t* __restrict__ U_split, uint32_t* __restrict__ cnt_all,
-                                               int n, const uint8_t* __restrict__ heavy,
-                                               long long* __restrict__ NE) {
-    pdl_enter();
-    const int nW = c->nW;
-    uint32_t* cnt = cnt_all + (size_t)blockIdx.x * (size_t)n;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, NWp = blockDim.x >> 5;
-    for (int pi = blockIdx.x; pi < nW; pi += gridDim.x) {
-        const uint32_t u = (uint32_t)wlist[pi];
-        if (heavy && heavy[u]) continue;  // taken by k_c4_group (same for the whole block)
-        const long long rb = U_off[u];
-        const int nlow = U_split[u];
-        for (int pass = 0; pass < 3; pass++) {
-            for (int j = warp; j < nlow; j += NWp) {
-                const uint32_t a = vid(U_col[rb + j]);
-                const long long ab = U_off[a], ae = U_off[a + 1];
-                long long asum = 0;
-                for (long long q = ab + lane; q < ae; q += 32) {
-                    const uint32_t w = vid(U_col[q]);
-                    if (w >= u) break;  // rows are sorted: the rest is above u
-                    if (pass == 0) {
-                        atomicAdd(&cnt[w], 1u);
-                    } else if (pass == 1) {
-                        const long long x = (long long)__ldcg(&cnt[w]) - 1;
-                        if (x > 0) {
-                            atomicAdd((unsigned long long*)&NE[NEROLE * (size_t)q + E_C4], (unsigned long long)x);
-                            asum += x;
-                        }
-                    } else {
-                        cnt[w] = 0u;
-                    }
-                }
-                if (pass == 1) {
-                    asum = (long long)warp_sum_u64((unsigned long long)asum);
-                    if (lane == 0 && asum)
-                        atomicAdd((unsigned long long*)&NE[NEROLE * (size_t)(rb + j) + E_C4], (unsigned long long)asum);
-                }
-            }
-            __threadfence();
-            __syncthreads();
+        for (long long e = ob + lane; e < U_off[u + 1]; e += 32) {
+            const unsigned long long b = (unsigned long long)iperm[vid(U_col[e])];
+            keys[to + e] = a < b ? (a << nb) | b : (b << nb) | a;
         }
     }
 }
 
 // Orbit counts per edge by the triangular edge-role containment.  A warp
-// per vertex x, a lane per out-entry e = (x, y); the credits of the twin
-// entry (x in y's row) are added, the edge's row in the output is the rank
+// per vertex x, a lane per out-entry e = (x, y); the 4-cycle credits of the
+// twin entry (x in y's row) are added, the edge's row in the output is the rank
 // of its key among the sorted keys.  out[k row + j]: the ten edge orbits
 // (k = 10) or their sums per graphlet (k = 6); edges[2 row] = (lo, hi).
 __global__ void k_e_finalize(const Ctl* c, const int32_t* __restrict__ wlist, const long long* __restrict__ U_off,
                              const uint32_t* __restrict__ U_col, const int32_t* __restrict__ U_split,
                              const uint32_t* __restrict__ tall, const long long* __restrict__ sdeg,
-                             const unsigned long long* __restrict__ T2, const long long* __restrict__ NE,
+                             const unsigned long long* __restrict__ T2, const unsigned long long* __restrict__ to,
+                             const unsigned long long* __restrict__ k4, const unsigned long long* __restrict__ c4,
                              const int32_t* __restrict__ iperm, const unsigned long long* __restrict__ skeys,
                              int nb, long long m, int k, unsigned long long* __restrict__ out,
                              int32_t* __restrict__ edges) {
@@ -609,10 +648,8 @@ __global__ void k_e_finalize(const Ctl* c, const int32_t* __restrict__ wlist, co
             const long long yb = U_off[y];
             const long long tw = yb + lower_bound_id(U_col + yb, U_split[y], x);
             const long long dy = U_off[y + 1] - yb, t = tall[e];
-            const long long* ra = NE + NEROLE * (size_t)e;
-            const long long* rt = NE + NEROLE * (size_t)tw;
-            const long long n_opp = ra[E_OPP] + rt[E_OPP], n_outer = ra[E_OUTER] + rt[E_OUTER];
-            const long long n_c4 = ra[E_C4] + rt[E_C4], n_k4 = ra[E_K4] + rt[E_K4];
+            const long long n_opp = (long long)to[2 * e], n_outer = (long long)to[2 * e + 1];
+            const long long n_c4 = (long long)(c4[e] + c4[tw]), n_k4 = (long long)k4[e];
             const long long n_pend = (sdeg[y] - (dx - 1) - t) + (sx - (dy - 1) - t);
             const long long n_pmid = (dx - 1) * (dy - 1) - t;
             const long long n_star = (dx - 1) * (dx - 2) / 2 + (dy - 1) * (dy - 2) / 2;
@@ -666,19 +703,20 @@ int enqueue_edge_counts(const EdgeArgs& a, cudaStream_t s) {
     int nl = 0;
     pdl_launch(k_v_tsym, dim3(gw), dim3(tpb), 0, s, a.ctl, a.wlist, a.U_off, a.U_col, a.U_split, a.tpack, a.tall);
     pdl_launch(k_v_s, dim3(gw), dim3(tpb), 0, s, a.ctl, a.wlist, a.U_off, a.U_col, a.sdeg);
+    pdl_launch(k_e_outdeg, dim3(std::max(1, std::min(gw, (a.n + 255) / 256))), dim3(256), 0, s, a.n, a.U_off, a.U_split,
+               a.outdeg);
+    nl += 3;
+    nl += scan_i32_to_i64(a.outdeg, a.out_off, nullptr, a.n, a.bsum, scan_grid(a.n, a.sms), nullptr, s);
     pdl_launch(k_e_keys, dim3(gw), dim3(tpb), 0, s, a.ctl, a.wlist, a.U_off, a.U_col, a.U_split, a.iperm, a.nb,
-               a.keys);
-    nl += 3;
-    nl += radix_sort_u64((uint64_t*)a.keys, (uint64_t*)a.keys_tmp, a.d_count, a.nU, 2 * a.nb, a.hist, a.sort_grid, s);
-    pdl_launch(k_e_tri_k4, dim3(gw), dim3(tpb), 0, s, a.ctl, a.wlist, a.U_off, a.U_col, a.U_split, a.tall, a.NE);
-    const int nh = enqueue_heavy_c4<true>(a.hv, a.ctl, a.wlist, a.U_off, a.U_col, a.U_split, a.n, a.sms, a.NE, s);
-    if (nh < 0) return -1;
-    nl += nh;
-    pdl_launch(k_e_c4, dim3(a.c4_blocks), dim3(1024), 0, s, a.ctl, a.wlist, a.U_off, a.U_col, a.U_split, a.cnt, a.n,
-               nh > 0 ? (const uint8_t*)a.hv.heavy : nullptr, a.NE);
+               a.out_off, a.keys);
+    nl++;
+    nl += radix_sort_u64((uint64_t*)a.keys, (uint64_t*)a.keys_tmp, a.out_off + a.n, a.m, 2 * a.nb, a.hist, a.sort_grid,
+                         s);
+    const TriCredits cr{nullptr, nullptr, a.to, a.k4};
+    nl += enqueue_tri_credits<true>(a.ctl, a.bins, a.n, a.U_off, a.U_col, a.U_split, a.tall, cr, a.sms, s);
     pdl_launch(k_e_finalize, dim3(gw), dim3(tpb), 0, s, a.ctl, a.wlist, a.U_off, a.U_col, a.U_split, a.tall, a.sdeg,
-               a.T2, a.NE, a.iperm, a.keys, a.nb, a.m, a.orbits ? 10 : 6, a.out, a.edges);
-    nl += 3;
+               a.T2, a.to, a.k4, a.c4, a.iperm, a.keys, a.nb, a.m, a.orbits ? 10 : 6, a.out, a.edges);
+    nl++;
     return nl;
 }
 
@@ -687,15 +725,11 @@ int enqueue_vertex_counts(const VertexArgs& a, cudaStream_t s) {
     int nl = 0;
     pdl_launch(k_v_tsym, dim3(gw), dim3(tpb), 0, s, a.ctl, a.wlist, a.U_off, a.U_col, a.U_split, a.tpack, a.tall);
     pdl_launch(k_v_s, dim3(gw), dim3(tpb), 0, s, a.ctl, a.wlist, a.U_off, a.U_col, a.sdeg);
-    pdl_launch(k_v_terms, dim3(gw), dim3(tpb), 0, s, a.ctl, a.wlist, a.U_off, a.U_col, a.tall, a.sdeg, a.T2, a.NV);
-    pdl_launch(k_v_tri_k4, dim3(gw), dim3(tpb), 0, s, a.ctl, a.wlist, a.U_off, a.U_col, a.U_split, a.tall, a.NV);
-    const int nh = enqueue_heavy_c4<false>(a.hv, a.ctl, a.wlist, a.U_off, a.U_col, a.U_split, a.n, a.sms, a.NV, s);
-    if (nh < 0) return -1;
-    nl += nh;
-    pdl_launch(k_v_c4, dim3(a.c4_blocks), dim3(1024), 0, s, a.ctl, a.wlist, a.U_off, a.U_col, a.U_split, a.cnt, a.n,
-               nh > 0 ? (const uint8_t*)a.hv.heavy : nullptr, a.NV);
-    pdl_launch(k_v_finalize, dim3((a.n + 255) / 256), dim3(256), 0, s, a.NV, a.n, a.iperm, a.orbits ? 11 : 6, a.out);
-    nl += 6;
+    const TriCredits cr{a.d2, a.k4, nullptr, nullptr};
+    nl += enqueue_tri_credits<false>(a.ctl, a.bins, a.n, a.U_off, a.U_col, a.U_split, a.tall, cr, a.sms, s);
+    pdl_launch(k_v_finalize, dim3(gw), dim3(tpb), 0, s, a.ctl, a.wlist, a.U_off, a.U_col, a.tall, a.sdeg, a.T2, a.d2,
+               a.k4, a.c4, a.iperm, a.orbits ? 11 : 6, a.out);
+    nl += 3;
     return nl;
 }
 
