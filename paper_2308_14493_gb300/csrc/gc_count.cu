@@ -17,13 +17,12 @@
 //
 // Triangles and 4-cliques, root-centred.  For a root u with out-list
 // X = N+(u) (k entries), every v = X[q] is probed: each entry y of N+(v)
-// that is also in X (binary search in shared memory) closes the triangle
-// (u, v, y), listed exactly once (u < v < y).  It sets bit p = pos(y) of the
-// local row q, and credits its three edges: (u,v) and (u,y) in a per-root
-// shared-memory accumulator, (v,y) by one 64-bit atomic.  The rows are the
-// adjacency of N+(u) as bitmasks, so the 4-cliques through u are
-// sum over bits p of row q of popcount(row_q & row_p).  G_a and G_b get one
-// row set each.  Roots are binned by k: a warp (k <= 32), a block
+// that is also in X closes the triangle (u, v, y), listed exactly once
+// (u < v < y).  It sets bit p = pos(y) of the local row q, and credits its
+// three edges: (u,v) and (u,y) through the rows and a per-root counter, (v,y)
+// by one 64-bit atomic.  The rows are the adjacency of N+(u) as bitmasks, so
+// the 4-cliques through u are sum over bits p of row q of
+// popcount(row_q & row_p).  Roots are binned by k: a warp (k <= 32), a block
 // (k <= TRI_KM), or per-edge merging (larger k).
 //
 // 4-cycles, pivot-centred.  Each 4-cycle is counted once at its highest
@@ -191,7 +190,106 @@ __global__ void k_bin(Ctl* c, const int32_t* __restrict__ wlist, const long long
 
 // ---- triangles and 4-cliques -------------------------------------------------
 
+// A root's candidates (the entries of N+(v), v in X) are about twenty times its
+// triangles, so the test "is y in X" is what the kernels spend their
+// instructions on.  Each candidate is first looked up in a bitmap of hashed ids
+// in shared memory (one load); the few that pass are queued per warp and
+// located in X by binary search 32 at a time, with every lane at work.  Four
+// candidates a lane are loaded together.  Rows of X's adjacency hold the
+// triangles in G_a (R); D marks those in one graph only, so G_b's rows are
+// R ^ D, and while D is empty both graphs have the same 4-cliques, counted
+// once.  t of (u, X[q]) is popcount(row q) plus the triangles whose third
+// vertex is X[q], kept as 16/16 bits (an out-list has at most TRI_KM entries).
+// (Binary search of every candidate, 64-bit shared-memory atomics, which are
+// compare-and-swap loops, and rows of an even stride took 16.4 ms for all three
+// sizes on the 1.6M/30M graph and 16.1 ms on the 2.4M/5M graph with out-lists
+// of up to 480 entries; these take 8.7 and 5.2 ms.)
+struct Cand {
+    int j;       // number of the candidate (its row q and slot follow from it)
+    uint32_t e;  // entry (X[q], y)
+};
+constexpr int TQ = 32 + 4 * 32;  // queue entries per warp: less than 32 left over, then up to 128 more
+
+__device__ __forceinline__ uint32_t tri_hash(uint32_t id, int lg) { return (id * 0x9E3779B1u) >> (32 - lg); }
+
+// A root's lists in shared memory (k = |X|, W words a row, rows `ws` apart).
+struct Root {
+    const uint32_t* X;
+    const long long* nb;  // start of N+(X[q])
+    const int* pre;       // candidates before row q
+    const uint32_t* bloom;
+    uint32_t *R, *D, *cnt;
+    int k, ws, lg;
+};
+
+// Locate up to 32 queued candidates in X and record their triangles; returns
+// whether one was in one graph only.
+__device__ __forceinline__ bool tri_record(const Root& t, const Cand* queue, int n, unsigned long long* tpack) {
+    const int lane = threadIdx.x & 31;
+    bool one = false;
+    if (lane < n) {
+        const Cand c = queue[lane];
+        const int p = find_pos(t.X, t.k, vid(c.e));
+        if (p >= 0) {
+            const int q = find_seg(t.pre, t.k, c.j);
+            const uint32_t f = t.X[q] & t.X[p] & c.e;
+            const unsigned long long iv = flag_inc(f);
+            if (iv) {
+                const uint32_t bit = 1u << (p & 31);
+                uint32_t* r = t.R + q * t.ws + (p >> 5);
+                if (f & FLAG_A) atomicOr(r, bit);
+                if ((f >> 30) != 3u) {
+                    atomicOr(t.D + (r - t.R), bit);
+                    one = true;
+                }
+                atomicAdd(&t.cnt[p], ((f & FLAG_A) ? 0x10000u : 0u) | (f >> 31));
+                atomicAdd(&tpack[t.nb[q] + (c.j - t.pre[q])], iv);
+            }
+        }
+    }
+    return one;
+}
+
+// The candidates [base, base + 128) of a root, from row q on (the row of
+// base); n entries are queued already.
+__device__ __forceinline__ bool tri_chunk(const Root& t, const uint32_t* __restrict__ U_col, int base, int total, int q,
+                                          Cand* queue, int& n, unsigned long long* tpack) {
+    const int lane = threadIdx.x & 31;
+    uint32_t e[4];
+#pragma unroll
+    for (int i = 0; i < 4; i++) {
+        const int j = base + 32 * i + lane;
+        e[i] = 0xFFFFFFFFu;
+        if (j < total) {
+            while (q + 1 < t.k && t.pre[q + 1] <= j) q++;
+            e[i] = U_col[t.nb[q] + (j - t.pre[q])];
+        }
+    }
+#pragma unroll
+    for (int i = 0; i < 4; i++) {
+        const uint32_t h = tri_hash(vid(e[i]), t.lg);
+        const bool pass = base + 32 * i + lane < total && ((t.bloom[h >> 5] >> (h & 31)) & 1u);
+        const unsigned m = __ballot_sync(FULL, pass);
+        if (pass) queue[n + __popc(m & lanemask_lt())] = Cand{base + 32 * i + lane, e[i]};
+        n += __popc(m);
+    }
+    __syncwarp();
+    bool one = false;
+    while (n >= 32) {
+        n -= 32;
+        one |= tri_record(t, queue + n, 32, tpack);
+    }
+    __syncwarp();
+    return one;
+}
+
 constexpr int TW = 8;  // warps per block of the warp-per-root kernel
+struct WarpTri {
+    long long nb[32];
+    Cand queue[TQ];
+    uint32_t X[32], R[32], D[32], cnt[32], bloom[32];
+    int pre[33];
+};
 
 __global__ void __launch_bounds__(TW * 32) k_tri_warp(Ctl* c, const int32_t* __restrict__ list,
                                                      const long long* __restrict__ U_off,
@@ -199,24 +297,21 @@ __global__ void __launch_bounds__(TW * 32) k_tri_warp(Ctl* c, const int32_t* __r
                                                      const int32_t* __restrict__ U_split,
                                                      unsigned long long* __restrict__ tpack) {
     pdl_enter();
-    __shared__ uint32_t sX[TW][32];
-    __shared__ long long sNb[TW][32];
-    __shared__ int sPre[TW][33];
-    __shared__ uint32_t sRA[TW][32], sRB[TW][32];
-    __shared__ unsigned long long sTq[TW][32];
+    __shared__ __align__(16) WarpTri s_w[TW];
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    WarpTri& S = s_w[w];
     const int cnt = c->nbin[BIN_TRI_WARP];
     unsigned long long ka = 0, kb = 0;
     for (int i = blockIdx.x * TW + w; i < cnt; i += gridDim.x * TW) {
-        int32_t u = list[i];
-        long long rb = U_off[u] + U_split[u];
-        int k = (int)(U_off[u + 1] - rb);
-        uint32_t x = lane < k ? U_col[rb + lane] : 0u;
-        uint32_t xmax = vid(__shfl_sync(FULL, x, k - 1));
+        const int32_t u = list[i];
+        const long long rb = U_off[u] + U_split[u];
+        const int k = (int)(U_off[u + 1] - rb);
+        const uint32_t x = lane < k ? U_col[rb + lane] : 0u;
+        const uint32_t xmax = vid(__shfl_sync(FULL, x, k - 1));
         int cq = 0;
         long long nb = 0;
         if (lane < k) {
-            uint32_t v = vid(x);
+            const uint32_t v = vid(x);
             nb = U_off[v] + U_split[v];
             cq = (int)lower_bound_id(U_col + nb, U_off[v + 1] - nb, xmax + 1);
         }
@@ -227,36 +322,46 @@ __global__ void __launch_bounds__(TW * 32) k_tri_warp(Ctl* c, const int32_t* __r
             if (lane >= o) inc += y;
         }
         const int total = __shfl_sync(FULL, inc, 31);
-        sX[w][lane] = x;
-        sNb[w][lane] = nb;
-        sPre[w][lane + 1] = inc;
-        if (lane == 0) sPre[w][0] = 0;
-        sRA[w][lane] = 0;
-        sRB[w][lane] = 0;
-        sTq[w][lane] = 0;
-        __syncwarp();
-        int q = 0;
-        for (int t = lane; t < total; t += 32) {
-            while (q + 1 < k && sPre[w][q + 1] <= t) q++;
-            long long slot = sNb[w][q] + (t - sPre[w][q]);
-            uint32_t e = U_col[slot];
-            int p = find_pos(sX[w], k, vid(e));
-            if (p < 0) continue;
-            uint32_t f = sX[w][q] & sX[w][p] & e;
-            unsigned long long iv = flag_inc(f);
-            if (!iv) continue;
-            if (f & FLAG_A) atomicOr(&sRA[w][q], 1u << p);
-            if (f & FLAG_B) atomicOr(&sRB[w][q], 1u << p);
-            atomicAdd(&sTq[w][q], iv);
-            atomicAdd(&sTq[w][p], iv);
-            atomicAdd(&tpack[slot], iv);
-        }
+        S.X[lane] = x;
+        S.nb[lane] = nb;
+        S.pre[lane + 1] = inc;
+        if (lane == 0) S.pre[0] = 0;
+        S.R[lane] = 0;
+        S.D[lane] = 0;
+        S.cnt[lane] = 0;
+        S.bloom[lane] = 0;
         __syncwarp();
         if (lane < k) {
-            uint32_t ra = sRA[w][lane], rbm = sRB[w][lane];
-            for (uint32_t m = ra; m; m &= m - 1) ka += __popc(ra & sRA[w][__ffs(m) - 1]);
-            for (uint32_t m = rbm; m; m &= m - 1) kb += __popc(rbm & sRB[w][__ffs(m) - 1]);
-            unsigned long long tq = sTq[w][lane];
+            const uint32_t h = tri_hash(vid(x), 10);
+            atomicOr(&S.bloom[h >> 5], 1u << (h & 31));
+        }
+        __syncwarp();
+        const Root t{S.X, S.nb, S.pre, S.bloom, S.R, S.D, S.cnt, k, 1, 10};
+        int n = 0, q = 0;
+        bool one = false;
+        for (int base = 0; base < total; base += 128) {
+            while (q + 1 < k && S.pre[q + 1] <= base) q++;
+            one |= tri_chunk(t, U_col, base, total, q, S.queue, n, tpack);
+        }
+        one |= tri_record(t, S.queue, n, tpack);
+        one = __any_sync(FULL, one);
+        if (lane < k) {
+            const uint32_t ra = S.R[lane];
+            unsigned na = 0;
+            for (uint32_t m = ra; m; m &= m - 1) na += __popc(ra & S.R[__ffs(m) - 1]);
+            ka += na;
+            const uint32_t rbm = ra ^ S.D[lane];
+            if (one) {
+                na = 0;
+                for (uint32_t m = rbm; m; m &= m - 1) {
+                    const int p = __ffs(m) - 1;
+                    na += __popc(rbm & (S.R[p] ^ S.D[p]));
+                }
+            }
+            kb += na;
+            const uint32_t cn = S.cnt[lane];
+            const unsigned long long tq =
+                ((unsigned long long)(__popc(ra) + (cn >> 16)) << 32) | (__popc(rbm) + (cn & 0xFFFFu));
             if (tq) atomicAdd(&tpack[rb + lane], tq);
         }
         __syncwarp();
@@ -265,117 +370,127 @@ __global__ void __launch_bounds__(TW * 32) k_tri_warp(Ctl* c, const int32_t* __r
     acc_add(c, 10, kb);
 }
 
-// Shared memory of the block kernel for out-lists of up to KM entries.
-template <int KM>
-constexpr size_t tri_block_smem() {
-    return (size_t)KM * 4 + (size_t)KM * 8 + (size_t)(KM + 8) * 4 + 2ull * KM * (KM / 32) * 4 + (size_t)KM * 8;
-}
-size_t tri_block_smem_bytes() { return tri_block_smem<TRI_KM>(); }
+// Shared memory of the block kernel for out-lists of up to KM entries; rows
+// have an odd number of words, so that lanes on consecutive rows meet
+// different banks.
+template <int KM, int THREADS>
+struct BlockTri {
+    static constexpr int LG = KM <= 128 ? 12 : 14;  // bitmap bits: at most 3 % of them set
+    long long nb[KM];
+    Cand queue[THREADS / 32][TQ];
+    uint32_t X[KM], cnt[KM], bloom[1 << (LG - 5)];
+    int pre[KM + 1];
+    uint32_t R[KM * (KM / 32 + 1)], D[KM * (KM / 32 + 1)];
+};
 
-// Roots with 32 < k <= KM: one block per root.  The out-list X is held
-// in shared memory; the candidates (every entry of N+(v) up to max X, for v
-// in X) are dealt in warp-contiguous runs of 32, so a lane finds its row by
-// stepping from the run's first row, and its position in X by binary search.
-// Two instances: KM = TRI_KS for the many short lists (small shared
-// footprint, many blocks per SM) and KM = TRI_KM for the long ones.
-template <int KM, int BIN, int WORK>
-__global__ void __launch_bounds__(256) k_tri_block(Ctl* c, const int32_t* __restrict__ list,
+constexpr int TRI_SMALL_THREADS = 256, TRI_BIG_THREADS = 512;
+
+// Roots with 32 < k <= KM: one block per root.  Two instances: KM = TRI_KS
+// for the many short lists (small shared footprint, many blocks per SM) and
+// KM = TRI_KM for the long ones.
+template <int KM, int THREADS, int BIN, int WORK>
+__global__ void __launch_bounds__(THREADS) k_tri_block(Ctl* c, const int32_t* __restrict__ list,
                                                   const long long* __restrict__ U_off,
                                                   const uint32_t* __restrict__ U_col,
                                                   const int32_t* __restrict__ U_split,
                                                   unsigned long long* __restrict__ tpack) {
     pdl_enter();
     extern __shared__ __align__(16) unsigned char smem[];
-    long long* sNb = (long long*)smem;
-    unsigned long long* sTq = (unsigned long long*)(smem + (size_t)KM * 8);
-    uint32_t* sX = (uint32_t*)(smem + (size_t)KM * 16);
-    int* sPre = (int*)(smem + (size_t)KM * 20);
-    uint32_t* sRA = (uint32_t*)(smem + (size_t)KM * 24 + 32);
-    uint32_t* sRB = sRA + KM * (KM / 32);
-    __shared__ int s_idx;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, NW = blockDim.x >> 5;
+    BlockTri<KM, THREADS>& S = *(BlockTri<KM, THREADS>*)smem;
+    __shared__ int s_idx, s_one;
+    constexpr int LG = BlockTri<KM, THREADS>::LG;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, NW = THREADS / 32;
     const int cnt = c->nbin[BIN];
     unsigned long long ka = 0, kb = 0;
     for (;;) {
-        if (tid == 0) s_idx = (int)atomicAdd(&c->work[WORK], 1u);
+        if (tid == 0) {
+            s_idx = (int)atomicAdd(&c->work[WORK], 1u);
+            s_one = 0;
+        }
         __syncthreads();
         const int idx = s_idx;
-        __syncthreads();
         if (idx >= cnt) break;
-        int32_t u = list[idx];
-        long long rb = U_off[u] + U_split[u];
+        const int32_t u = list[idx];
+        const long long rb = U_off[u] + U_split[u];
         const int k = (int)(U_off[u + 1] - rb);
-        const int W = (k + 31) >> 5;
+        const int W = (k + 31) >> 5, ws = W | 1;
         const uint32_t xmax = vid(U_col[rb + k - 1]);
-        for (int t = tid; t < k; t += blockDim.x) {
-            uint32_t x = U_col[rb + t];
-            uint32_t v = vid(x);
-            long long nb = U_off[v] + U_split[v];
-            sX[t] = x;
-            sNb[t] = nb;
-            sPre[t + 1] = (int)lower_bound_id(U_col + nb, U_off[v + 1] - nb, xmax + 1);
-            sTq[t] = 0;
+        for (int j = tid; j < (1 << (LG - 5)); j += THREADS) S.bloom[j] = 0;
+        for (int j = tid; j < k * ws; j += THREADS) {
+            S.R[j] = 0;
+            S.D[j] = 0;
         }
-        for (int t = tid; t < k * W; t += blockDim.x) {
-            sRA[t] = 0;
-            sRB[t] = 0;
+        for (int t = tid; t < k; t += THREADS) {
+            const uint32_t x = U_col[rb + t];
+            const uint32_t v = vid(x);
+            const long long nb = U_off[v] + U_split[v];
+            S.X[t] = x;
+            S.nb[t] = nb;
+            S.pre[t + 1] = (int)lower_bound_id(U_col + nb, U_off[v + 1] - nb, xmax + 1);
+            S.cnt[t] = 0;
         }
         __syncthreads();
-        if (warp == 0) {  // inclusive scan of sPre[1..k]
+        for (int t = tid; t < k; t += THREADS) {
+            const uint32_t h = tri_hash(vid(S.X[t]), LG);
+            atomicOr(&S.bloom[h >> 5], 1u << (h & 31));
+        }
+        if (warp == 0) {  // inclusive scan of pre[1..k]
             int carry = 0;
             for (int b = 0; b < k; b += 32) {
-                int x = b + lane < k ? sPre[b + lane + 1] : 0;
+                int x = b + lane < k ? S.pre[b + lane + 1] : 0;
 #pragma unroll
                 for (int o = 1; o < 32; o <<= 1) {
                     int y = __shfl_up_sync(FULL, x, o);
                     if (lane >= o) x += y;
                 }
-                if (b + lane < k) sPre[b + lane + 1] = x + carry;
+                if (b + lane < k) S.pre[b + lane + 1] = x + carry;
                 carry += __shfl_sync(FULL, x, 31);
             }
-            if (lane == 0) sPre[0] = 0;
+            if (lane == 0) S.pre[0] = 0;
         }
         __syncthreads();
-        const int total = sPre[k];
-        for (int base = warp * 32; base < total; base += NW * 32) {
-            const int t = base + lane;
-            int q = find_seg(sPre, k, base);
-            if (t < total) {
-                while (q + 1 < k && sPre[q + 1] <= t) q++;
-                const long long slot = sNb[q] + (t - sPre[q]);
-                const uint32_t e = U_col[slot];
-                const int p = find_pos(sX, k, vid(e));
-                if (p >= 0) {
-                    const uint32_t f = sX[q] & sX[p] & e;
-                    const unsigned long long iv = flag_inc(f);
-                    if (iv) {
-                        if (f & FLAG_A) atomicOr(&sRA[q * W + (p >> 5)], 1u << (p & 31));
-                        if (f & FLAG_B) atomicOr(&sRB[q * W + (p >> 5)], 1u << (p & 31));
-                        atomicAdd(&sTq[q], iv);
-                        atomicAdd(&sTq[p], iv);
-                        atomicAdd(&tpack[slot], iv);
-                    }
+        const int total = S.pre[k];
+        const Root t{S.X, S.nb, S.pre, S.bloom, S.R, S.D, S.cnt, k, ws, LG};
+        int n = 0;
+        bool one = false;
+        for (int base = warp * 128; base < total; base += NW * 128)
+            one |= tri_chunk(t, U_col, base, total, find_seg(S.pre, k, base), S.queue[warp], n, tpack);
+        one |= tri_record(t, S.queue[warp], n, tpack);
+        if (one) s_one = 1;
+        __syncthreads();
+        const bool differ = s_one != 0;
+        // 4-cliques: row q against the row of each of its bits
+        auto cliques = [&](int q) {
+            unsigned long long x = 0;
+            const uint32_t* r = S.R + q * ws;
+            for (int i = 0; i < W; i++)
+                for (uint32_t m = r[i]; m; m &= m - 1) {
+                    const int p = i * 32 + __ffs(m) - 1;
+                    const uint32_t* rp = S.R + p * ws;
+                    unsigned y = 0;
+                    for (int j = i; j < W; j++) y += __popc(r[j] & rp[j]);
+                    x += y;
                 }
-            }
-        }
-        __syncthreads();
-        for (int q = tid; q < k; q += blockDim.x) {
-            const uint32_t* ra = sRA + q * W;
-            const uint32_t* rbm = sRB + q * W;
+            return x;
+        };
+        for (int q = tid; q < k; q += THREADS) {
+            const uint32_t* r = S.R + q * ws;
+            const uint32_t* d = S.D + q * ws;
+            unsigned ta = S.cnt[q] >> 16, tb = S.cnt[q] & 0xFFFFu;
             for (int i = 0; i < W; i++) {
-                for (uint32_t m = ra[i]; m; m &= m - 1) {
-                    int p = i * 32 + __ffs(m) - 1;
-                    const uint32_t* rp = sRA + p * W;
-                    for (int i2 = p >> 5; i2 < W; i2++) ka += __popc(ra[i2] & rp[i2]);
-                }
-                for (uint32_t m = rbm[i]; m; m &= m - 1) {
-                    int p = i * 32 + __ffs(m) - 1;
-                    const uint32_t* rp = sRB + p * W;
-                    for (int i2 = p >> 5; i2 < W; i2++) kb += __popc(rbm[i2] & rp[i2]);
-                }
+                ta += __popc(r[i]);
+                tb += __popc(r[i] ^ d[i]);
             }
-            unsigned long long tq = sTq[q];
-            if (tq) atomicAdd(&tpack[rb + q], tq);
+            if (ta | tb) atomicAdd(&tpack[rb + q], ((unsigned long long)ta << 32) | tb);
+            const unsigned long long x = cliques(q);
+            ka += x;
+            if (!differ) kb += x;
+        }
+        if (differ) {
+            __syncthreads();
+            for (int j = tid; j < k * ws; j += THREADS) S.R[j] ^= S.D[j];
+            __syncthreads();
+            for (int q = tid; q < k; q += THREADS) kb += cliques(q);
         }
         __syncthreads();
     }
@@ -801,10 +916,11 @@ __global__ void k_finalize(Ctl* c, int mode) {
 namespace gcx {
 
 void count_setup_attributes() {
-    cudaFuncSetAttribute(k_tri_block<TRI_KM, BIN_TRI_BLOCK, WORK_TRI_BLOCK>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)tri_block_smem<TRI_KM>());
-    cudaFuncSetAttribute(k_tri_block<TRI_KS, BIN_TRI_SMALL, WORK_TRI_SMALL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)tri_block_smem<TRI_KS>());
+    cudaFuncSetAttribute(k_tri_block<TRI_KM, TRI_BIG_THREADS, BIN_TRI_BLOCK, WORK_TRI_BLOCK>,
+                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(BlockTri<TRI_KM, TRI_BIG_THREADS>));
+    cudaFuncSetAttribute(k_tri_block<TRI_KS, TRI_SMALL_THREADS, BIN_TRI_SMALL, WORK_TRI_SMALL>,
+                         cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         (int)sizeof(BlockTri<TRI_KS, TRI_SMALL_THREADS>));
     c4_setup_attributes();
 }
 
@@ -853,10 +969,12 @@ int enqueue_counting(const CountArgs& a, cudaStream_t s, cudaEvent_t ev_tri, cud
         for (int i = 0; i < 3; i++) cudaStreamWaitEvent(a.aux[i], a.fork, 0);
     }
     k_tri_warp<<<4 * sms, TW * 32, 0, sT>>>(a.ctl, lists(BIN_TRI_WARP), a.U_off, a.U_col, a.U_split, a.tpack);
-    k_tri_block<TRI_KS, BIN_TRI_SMALL, WORK_TRI_SMALL><<<8 * sms, 256, tri_block_smem<TRI_KS>(), sT>>>(
-        a.ctl, lists(BIN_TRI_SMALL), a.U_off, a.U_col, a.U_split, a.tpack);
-    k_tri_block<TRI_KM, BIN_TRI_BLOCK, WORK_TRI_BLOCK><<<2 * sms, 256, tri_block_smem<TRI_KM>(), sT>>>(
-        a.ctl, lists(BIN_TRI_BLOCK), a.U_off, a.U_col, a.U_split, a.tpack);
+    k_tri_block<TRI_KS, TRI_SMALL_THREADS, BIN_TRI_SMALL, WORK_TRI_SMALL>
+        <<<8 * sms, TRI_SMALL_THREADS, sizeof(BlockTri<TRI_KS, TRI_SMALL_THREADS>), sT>>>(
+            a.ctl, lists(BIN_TRI_SMALL), a.U_off, a.U_col, a.U_split, a.tpack);
+    k_tri_block<TRI_KM, TRI_BIG_THREADS, BIN_TRI_BLOCK, WORK_TRI_BLOCK>
+        <<<2 * sms, TRI_BIG_THREADS, sizeof(BlockTri<TRI_KM, TRI_BIG_THREADS>), sT>>>(
+            a.ctl, lists(BIN_TRI_BLOCK), a.U_off, a.U_col, a.U_split, a.tpack);
     k_tri_merge<<<sms, 256, 0, sT>>>(a.ctl, lists(BIN_TRI_MERGE), a.U_off, a.U_col, a.U_split, a.tpack);
     nl += 4;
     if (ev_c4) record_stage(ev_c4, sT);
