@@ -145,8 +145,8 @@ struct gc_graph {
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     cudaEvent_t ev[10] = {};  // stage boundaries, see gc_stats.ms_stage; [8], [9] around the
                               // heavy-pivot 4-cycle kernels (ms_stage[7])
-    cudaStream_t aux[3] = {};   // side streams of the counting pass
-    cudaEvent_t fork = nullptr, join[3] = {};
+    cudaStream_t aux[NAUX] = {};   // side streams of the counting pass
+    cudaEvent_t fork = nullptr, join[NAUX] = {};
     int launches = 0;        // kernels launched by the current call
     // device bytes held, for admission control
     std::unordered_map<void*, size_t> held;
@@ -659,7 +659,7 @@ static int count_region(gc_graph* g, int fin, bool set_F, bool timed, bool twin 
     ca.c4_credit = c4_credit;
     ca.local_heavy_min = g->loc_heavy_min;
     ca.sms = g->sms;
-    for (int i = 0; i < 3; i++) {
+    for (int i = 0; i < NAUX; i++) {
         ca.aux[i] = g->opt.serial_count ? nullptr : g->aux[i];
         ca.join[i] = g->join[i];
     }
@@ -1455,7 +1455,7 @@ static void destroy(gc_graph* g) {
     for (auto e : g->ev)
         if (e) cudaEventDestroy(e);
     if (g->e1) cudaEventDestroy(g->e1);
-    for (int i = 0; i < 3; i++) {
+    for (int i = 0; i < NAUX; i++) {
         if (g->aux[i]) cudaStreamDestroy(g->aux[i]);
         if (g->join[i]) cudaEventDestroy(g->join[i]);
     }
@@ -1728,7 +1728,7 @@ int gc_open(int32_t n, const int32_t* row_ptr, const int32_t* col, const gc_opti
         // side streams of the counting pass (they inherit nothing from the
         // caller's stream: every use is fenced by events on it)
         bool aux_ok = cudaEventCreateWithFlags(&g->fork, cudaEventDisableTiming) == cudaSuccess;
-        for (int i = 0; i < 3 && aux_ok; i++)
+        for (int i = 0; i < NAUX && aux_ok; i++)
             aux_ok = cudaStreamCreateWithFlags(&g->aux[i], cudaStreamNonBlocking) == cudaSuccess &&
                      cudaEventCreateWithFlags(&g->join[i], cudaEventDisableTiming) == cudaSuccess;
         if (!aux_ok) {

@@ -78,9 +78,10 @@ struct PivotArgs {
     unsigned long long* credit;  // C4_VERTEX: per vertex, C4_EDGE: per entry (added to)
 };
 
-// The hash-table tiers, then plan, run bounds and pivot kernels, on stream s
-// (bins: the work lists, NBINS * n); both return the launches made.
-int enqueue_c4_tables(const PivotArgs& a, int mode, const int32_t* bins, int sms, cudaStream_t s);
+// The hash-table tiers (the small one on stream s, the others on s2), then
+// plan, run bounds and pivot kernels (bins: the work lists, NBINS * n); all
+// return the launches made.
+int enqueue_c4_tables(const PivotArgs& a, int mode, const int32_t* bins, int sms, cudaStream_t s, cudaStream_t s2);
 // (the credits of the pivots below the tables: C4_VERTEX and C4_EDGE only)
 int enqueue_c4_warp_credit(const PivotArgs& a, int mode, const int32_t* bins, int sms, cudaStream_t s);
 int enqueue_c4_pivots(const PivotArgs& a, int mode, const C4Geom& g, cudaStream_t s);

@@ -814,10 +814,10 @@ struct C4Kernels {
         if constexpr (MODE != C4_COUNT)
             k_c4_warp_credit<MODE><<<4 * sms, CW_WARPS * 32, CW_WARPS * sizeof(CreditWarp), s>>>(a, bins);
     }
-    static int tables(const PivotArgs& a, const int32_t* bins, int sms, cudaStream_t s) {
+    static int tables(const PivotArgs& a, const int32_t* bins, int sms, cudaStream_t s, cudaStream_t s2) {
         tab_s<<<8 * sms, 128, table_smem<C4_TAB_S, 128>(), s>>>(a, bins + (size_t)BIN_C4_BSMALL * a.n);
-        tab_m<<<2 * sms, 512, table_smem<C4_TAB_M, 512>(), s>>>(a, bins + (size_t)BIN_C4_BLOCK * a.n);
-        tab_l<<<sms, 1024, table_smem<C4_TAB_L, 1024>(), s>>>(a, bins + (size_t)BIN_C4_BIG * a.n);
+        tab_m<<<2 * sms, 512, table_smem<C4_TAB_M, 512>(), s2>>>(a, bins + (size_t)BIN_C4_BLOCK * a.n);
+        tab_l<<<sms, 1024, table_smem<C4_TAB_L, 1024>(), s2>>>(a, bins + (size_t)BIN_C4_BIG * a.n);
         return 3;
     }
     static void pivots(const PivotArgs& a, const C4Geom& g, int c0, cudaStream_t s) {
@@ -851,10 +851,10 @@ void c4_setup_attributes() {
     C4Kernels<C4_EDGE>::attributes();
 }
 
-int enqueue_c4_tables(const PivotArgs& a, int mode, const int32_t* bins, int sms, cudaStream_t s) {
-    return mode == C4_VERTEX ? C4Kernels<C4_VERTEX>::tables(a, bins, sms, s)
-           : mode == C4_EDGE ? C4Kernels<C4_EDGE>::tables(a, bins, sms, s)
-                             : C4Kernels<C4_COUNT>::tables(a, bins, sms, s);
+int enqueue_c4_tables(const PivotArgs& a, int mode, const int32_t* bins, int sms, cudaStream_t s, cudaStream_t s2) {
+    return mode == C4_VERTEX ? C4Kernels<C4_VERTEX>::tables(a, bins, sms, s, s2)
+           : mode == C4_EDGE ? C4Kernels<C4_EDGE>::tables(a, bins, sms, s, s2)
+                             : C4Kernels<C4_COUNT>::tables(a, bins, sms, s, s2);
 }
 
 int enqueue_c4_warp_credit(const PivotArgs& a, int mode, const int32_t* bins, int sms, cudaStream_t s) {

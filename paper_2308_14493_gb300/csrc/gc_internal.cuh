@@ -146,6 +146,8 @@ struct Tuning {
 constexpr long long NEVER = 1ll << 62;
 inline Tuning default_tuning() { return Tuning{32, TRI_KS, TRI_KM, 32, C4_T1, C4_T2, 32768, NEVER, NEVER}; }
 
+constexpr int NAUX = 4;  // side streams of a counting pass
+
 // Handle-independent launch geometry.
 struct Dims {
     int sms;

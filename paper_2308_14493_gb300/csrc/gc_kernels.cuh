@@ -100,9 +100,9 @@ struct CountArgs {
     unsigned long long* c4_credit = nullptr;  // ... added here, per vertex or per entry
     long long local_heavy_min = 0;  // with credits: pivots of at least this bound (> 0) skip the tables
     int sms;
-    cudaStream_t aux[3] = {nullptr, nullptr, nullptr};  // side streams of the counting pass (or none)
+    cudaStream_t aux[NAUX] = {};    // side streams of the counting pass (or none)
     cudaEvent_t fork = nullptr;     // fork / join events for them (timing disabled)
-    cudaEvent_t join[3] = {nullptr, nullptr, nullptr};
+    cudaEvent_t join[NAUX] = {};
     cudaEvent_t ev_heavy[2] = {nullptr, nullptr};  // around the heavy-pivot 4-cycle kernels, on their stream
 };
 Tuning effective_tuning(const CountArgs& a);
