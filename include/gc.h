@@ -95,7 +95,7 @@ typedef struct {
     int64_t sums_a[6], sums_b[6];   /* [P, S, TT, D, K, Q]: non-induced 3-paths, 3-stars,
                                        tailed triangles, diamonds, 4-cliques, 4-cycles */
     int64_t num_edges;              /* edges of the graph after the batch */
-    float ms_device;                /* device time of the batch (CUDA events) */
+    float ms_device;                /* device time of the batch */
     float ms_wall;                  /* host wall time of the call */
     int32_t relayouts;              /* adjacency re-layouts the batch needed */
     int32_t path;                   /* 0: region recount (Algorithm 2); 2: a batched run whose
@@ -106,7 +106,7 @@ typedef struct {
                                        six induced / non-induced deltas and Cb / sums_b zero,
                                        C3a the 3-vertex deltas, work_triangles the probes */
     int32_t reserved[4];
-    /* device time per stage (CUDA events):
+    /* device time per stage (taken on the device, 32 ns steps):
        [0] normalise  [1] region walk  [2] union graph  [3] triangles + 4-cliques
        [4] 4-cycles   [5] edge terms + closed forms     [6] commit
        [7] the heavy-pivot 4-cycle kernels alone (plan, runs and k_c4_pivot),

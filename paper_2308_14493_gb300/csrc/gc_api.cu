@@ -143,8 +143,6 @@ struct gc_graph {
     gc_stats st{};
     std::string err;
     cudaEvent_t e0 = nullptr, e1 = nullptr;
-    cudaEvent_t ev[10] = {};  // stage boundaries, see gc_stats.ms_stage; [8], [9] around the
-                              // heavy-pivot 4-cycle kernels (ms_stage[7])
     cudaStream_t aux[NAUX] = {};   // side streams of the counting pass
     cudaEvent_t fork = nullptr, join[NAUX] = {};
     int launches = 0;        // kernels launched by the current call
@@ -244,6 +242,7 @@ namespace gcx {
 __global__ void k_begin_batch(Ctl* c, const long long* desc) {
     pdl_enter();
     if (threadIdx.x != 0) return;
+    c->ts[0] = global_ns();
     const bool run = c->halt == 0;
     c->active = run ? 1 : 0;
     // the descriptor is rewritten by host copies between calls: read it
@@ -277,6 +276,7 @@ __global__ void k_begin_batch(Ctl* c, const long long* desc) {
 __global__ void k_begin_twin(Ctl* c, const long long* desc) {
     pdl_enter();
     if (threadIdx.x != 0) return;
+    c->ts[0] = global_ns();
     c->active = 1;
     c->pairs_ins = (const int32_t*)__ldcg(desc);
     c->pairs_del = (const int32_t*)__ldcg(desc + 1);
@@ -309,7 +309,9 @@ __global__ void k_begin_twin(Ctl* c, const long long* desc) {
 // form 2: a twin pass writes the results of batches cur and cur + 1
 __global__ void k_end_batch(Ctl* c, unsigned long long* out, int commit, int form) {
     pdl_enter();
-    if (threadIdx.x != 0 || !c->active) return;
+    if (threadIdx.x != 0) return;
+    c->ts[7] = global_ns();
+    if (!c->active) return;
     if (form == 1 && c->cur > 0 && !c->err)
         for (int k = 0; k < 6; k++) out[6 * (long long)(c->cur - 1) + k] = c->prev_out[k];
     if (form == 2) {
@@ -613,11 +615,11 @@ static int ensure_desc(gc_graph* g, long long words) {
 
 // U build + counting + closed forms.
 //   fin: k_finalize mode (0 committed batch, 1 static, 2 independent batch)
-//   set_F: a static count that initialises F; timed: record stage events
+//   set_F: a static count that initialises F
 // all: the region is every vertex (no per-entry region test in the union
 // graph); twin: the twin pass's union graph of two batches
 // c4_mode, c4_credit: the 4-cycle credits of the local counts (static counts)
-static int count_region(gc_graph* g, int fin, bool set_F, bool timed, bool twin = false, bool all = false,
+static int count_region(gc_graph* g, int fin, bool set_F, bool twin = false, bool all = false,
                         int c4_mode = C4_COUNT, unsigned long long* c4_credit = nullptr) {
     cudaStream_t s = g->s;
     int gw = grid_warps(g);
@@ -664,22 +666,18 @@ static int count_region(gc_graph* g, int fin, bool set_F, bool timed, bool twin 
         ca.join[i] = g->join[i];
     }
     ca.fork = g->fork;
-    ca.ev_heavy[0] = timed ? g->ev[8] : nullptr;
-    ca.ev_heavy[1] = timed ? g->ev[9] : nullptr;
-    g->launches += enqueue_counting(ca, s, timed ? g->ev[3] : nullptr, timed ? g->ev[4] : nullptr,
-                                    timed ? g->ev[5] : nullptr, fin);
+    g->launches += enqueue_counting(ca, s, fin);
     if (set_F) {
         pdl_launch(k_set_F, dim3(1), dim3(32), 0, s, g->ctl);
         g->launches++;
     }
-    if (timed) CK(record_stage(g->ev[6], s));
     CKL();
     return GC_OK;
 }
 
 // Edge-local delta: union rows of the batch endpoints V_X (full rows), then
 // the local terms, 4-cliques and 4-cycles and their closed forms.
-static int count_local(gc_graph* g, int commit, bool timed, bool t2) {
+static int count_local(gc_graph* g, int commit, bool t2) {
     cudaStream_t s = g->s;
     int gw = grid_warps(g);
     pdl_launch(k_reset_count, dim3(1), dim3(32), 0, s, g->ctl);
@@ -732,9 +730,7 @@ static int count_local(gc_graph* g, int commit, bool timed, bool t2) {
     la.cap = g->l_cap;
     la.n = std::max(g->n, 1);
     la.sms = g->sms;
-    g->launches += enqueue_local(la, s, timed ? g->ev[3] : nullptr, timed ? g->ev[4] : nullptr,
-                                 timed ? g->ev[5] : nullptr, commit);
-    if (timed) CK(record_stage(g->ev[6], s));
+    g->launches += enqueue_local(la, s, commit);
     CKL();
     return GC_OK;
 }
@@ -776,7 +772,6 @@ static int enqueue_segments(gc_graph* g, bool clear) {
 // batch).  Grids are sized for batches of up to max_nk directed keys; the
 // actual sizes are read on the device.
 //   commit:     apply G <- G \ D u A (else an independent what-if batch)
-//   timed:      record the stage events (event-record nodes in the graph)
 //   local:      the edge-local delta instead of the region recount
 // role 0: the batch as Algorithm 2 (region, recount of G_a and G_b, commit);
 // the two-batch form (sequential runs whose regions cover the graph): role 1
@@ -786,10 +781,9 @@ static int enqueue_segments(gc_graph* g, bool clear) {
 // the twin pass, batches cur and cur + 1 keyed together with a batch tag and
 // counted over every vertex, G_a = G with the first, G_b = G with the second
 // (no commit).
-static int enqueue_batch(gc_graph* g, long long max_nk, bool commit, bool timed, bool local = false,
-                         bool t2 = false, int role = 0) {
+static int enqueue_batch(gc_graph* g, long long max_nk, bool commit, bool local = false, bool t2 = false,
+                         int role = 0) {
     cudaStream_t s = g->s;
-    if (timed) CK(record_stage(g->ev[0], s));
     const bool twin = role == 3;
     if (twin) pdl_launch(k_begin_twin, dim3(1), dim3(32), 0, s, g->ctl, g->desc);
     else pdl_launch(k_begin_batch, dim3(1), dim3(32), 0, s, g->ctl, g->desc);
@@ -826,7 +820,6 @@ static int enqueue_batch(gc_graph* g, long long max_nk, bool commit, bool timed,
         int rc = enqueue_segments(g, false);
         if (rc) return rc;
     }
-    if (timed) CK(record_stage(g->ev[1], s));
     CK(cudaMemsetAsync(g->visited, 0, sizeof(uint32_t) * (size_t)((g->n + 31) / 32 + 1), s));
     pdl_launch(k_bfs_sources, dim3(ge), dim3(TPB), 0, s, g->ctl, g->srcA.p, g->srcD.p, g->visited, g->wlist);
     pdl_launch(k_level_mark, dim3(1), dim3(1), 0, s, g->ctl, 0);
@@ -845,11 +838,10 @@ static int enqueue_batch(gc_graph* g, long long max_nk, bool commit, bool timed,
         g->launches++;
     }
     CKL();
-    if (timed) CK(record_stage(g->ev[2], s));
     int rc = GC_OK;
     if (role != 1) {
-        rc = local ? count_local(g, commit ? 1 : 0, timed, t2)
-                   : count_region(g, role == 2 ? 3 : role == 3 ? 4 : (commit ? 0 : 2), false, timed, twin,
+        rc = local ? count_local(g, commit ? 1 : 0, t2)
+                   : count_region(g, role == 2 ? 3 : role == 3 ? 4 : (commit ? 0 : 2), false, twin,
                                   role == 2);
         if (rc) return rc;
     }
@@ -867,7 +859,6 @@ static int enqueue_batch(gc_graph* g, long long max_nk, bool commit, bool timed,
         rc = enqueue_commit(g);
         if (rc) return rc;
     }
-    if (timed) CK(record_stage(g->ev[7], s));
     if (max_nk > 0) {
         rc = enqueue_segments(g, true);
         if (rc) return rc;
@@ -948,27 +939,23 @@ static int finish_pending_commit(gc_graph* g, int* relayouts) {
     return read_ctl(g);
 }
 
-static float elapsed(cudaEvent_t a, cudaEvent_t b) {
-    float x = 0.f;
-    if (cudaEventElapsedTime(&x, a, b) != cudaSuccess) {
-        cudaGetLastError();  // a stage the call did not run; not an error of the call
-        x = 0.f;
-    }
-    return x;
+// Milliseconds between two stage boundaries (0 when the call did not reach
+// both).
+static float elapsed(const Ctl& c, int a, int b) {
+    return c.ts[a] && c.ts[b] > c.ts[a] ? (float)(c.ts[b] - c.ts[a]) * 1e-6f : 0.f;
 }
 
-// Stage times of gc_stats.ms_stage from the boundary events ev[lo .. hi].
-// The triangle stage (ev3 -> ev4) and the 4-cycle stage (ev3 -> ev5) run
-// side by side from the same fork; the edge terms start after both.
-static void stage_times(gc_graph* g, int lo, int hi) {
+// gc_stats.ms_stage from the boundaries lo .. hi.  The triangle stage (3 -> 4)
+// and the 4-cycle stage (3 -> 5) run side by side from the same fork; the
+// edge terms start after both.
+static void stage_times(gc_graph* g, const Ctl& c, int lo, int hi) {
     for (int i = 0; i < 8; i++) g->st.ms_stage[i] = 0.f;
     for (int i = lo; i < hi; i++) {
-        if (i == 4) g->st.ms_stage[4] = elapsed(g->ev[3], g->ev[5]);
-        else if (i == 5) g->st.ms_stage[5] = std::min(elapsed(g->ev[4], g->ev[6]), elapsed(g->ev[5], g->ev[6]));
-        else g->st.ms_stage[i] = elapsed(g->ev[i], g->ev[i + 1]);
+        if (i == 4) g->st.ms_stage[4] = elapsed(c, 3, 5);
+        else if (i == 5) g->st.ms_stage[5] = elapsed(c, c.ts[4] > c.ts[5] ? 4 : 5, 6);
+        else g->st.ms_stage[i] = elapsed(c, i, i + 1);
     }
-    // the heavy-pivot 4-cycle kernels alone, on their own stream
-    if (lo <= 4 && hi > 4) g->st.ms_stage[7] = elapsed(g->ev[8], g->ev[9]);
+    if (lo <= 4 && hi > 4) g->st.ms_stage[7] = elapsed(c, 8, 9);
 }
 
 static void fill_stats(gc_graph* g, const Ctl& c) {
@@ -1035,11 +1022,11 @@ static int capture(gc_graph* g, cudaGraphExec_t* exec, int* launches, Enqueue en
 }
 
 // Capture the per-batch launch sequence (batch from the run cursor) into
-// *exec; timed: with the stage events as event-record nodes.
-static int capture_batch(gc_graph* g, long long shape_nk, bool commit, bool timed, cudaGraphExec_t* exec,
-                         int* launches, bool local = false, bool t2 = false, int role = 0) {
+// *exec.
+static int capture_batch(gc_graph* g, long long shape_nk, bool commit, cudaGraphExec_t* exec, int* launches,
+                         bool local = false, bool t2 = false, int role = 0) {
     return capture(g, exec, launches,
-                   [&] { return enqueue_batch(g, shape_nk, commit, timed, local, t2, role); });
+                   [&] { return enqueue_batch(g, shape_nk, commit, local, t2, role); });
 }
 
 // One batch whose pairs are already in device memory (plain form): the
@@ -1078,7 +1065,7 @@ static int apply_device(gc_graph* g, const int32_t* d_ins, long long n_ins, cons
         const bool t2 = g->t2_valid && (local || g->opt.local_max_pairs > 0);
         int* ex_t2 = local ? &g->l_t2 : &g->p_t2;
         if (!*ex || *ex_nk != shape_nk || *ex_commit != commit || *ex_gen != g->buf_gen || *ex_t2 != (int)t2) {
-            rc = capture_batch(g, shape_nk, commit != 0, true, ex, ex_launches, local, t2);
+            rc = capture_batch(g, shape_nk, commit != 0, ex, ex_launches, local, t2);
             if (rc) return rc;
             *ex_nk = shape_nk;
             *ex_commit = commit;
@@ -1095,9 +1082,7 @@ static int apply_device(gc_graph* g, const int32_t* d_ins, long long n_ins, cons
         pdl_launch(k_run_reset, dim3(1), dim3(32), 0, s, g->ctl);
         CKL();
         g->launches = *ex_launches + 1;
-        CK(cudaEventRecord(g->e0, s));
         CK(cudaGraphLaunch(*ex, s));
-        CK(cudaEventRecord(g->e1, s));
         rc = read_ctl(g);
         if (rc) return rc;
         if (g->h_ctl->err) {
@@ -1119,23 +1104,20 @@ static int apply_device(gc_graph* g, const int32_t* d_ins, long long n_ins, cons
         rc = finish_pending_commit(g, &relayouts);
         if (rc) return rc;
     }
-    Ctl c = *g->h_ctl;
-    float ms = 0.f;
-    cudaEventElapsedTime(&ms, g->e0, g->e1);
+    const Ctl& c = *g->h_ctl;
     fill_stats(g, c);
     g->st.n_ins_raw = n_ins;
     g->st.n_del_raw = n_del;
-    g->st.ms_device = ms;
+    g->st.ms_device = elapsed(c, 0, 7);
     g->st.relayouts = relayouts;
     g->st.launches = g->launches;
-    // [0] normalise: ev0->ev1, [1] region: ev1->ev2, [2] union graph: ev2->ev3,
-    // [3] triangles: ev3->ev4, [4] 4-cycles: ev4->ev5, [5] terms: ev5->ev6, [6] commit: ev6->ev7
     // (the edge-local path runs its stages one after the other)
     if (local) {
-        for (int i = 0; i < 8; i++) g->st.ms_stage[i] = i < 7 ? elapsed(g->ev[i], g->ev[i + 1]) : 0.f;
+        for (int i = 0; i < 8; i++) g->st.ms_stage[i] = i < 7 ? elapsed(c, i, i + 1) : 0.f;
     } else {
-        stage_times(g, 0, 7);
+        stage_times(g, c, 0, 7);
     }
+    if (!commit) g->st.ms_stage[6] = 0.f;
     g->st.path = local ? 1 : 0;
     if (commit && !local && g->opt.local_max_pairs <= 0) g->t2_valid = false;  // not kept without the local form
     if (commit) {
@@ -1208,7 +1190,7 @@ static int apply_batches_region(gc_graph* g, const int32_t* d_ins, const int32_t
     // (re)capture the per-batch graph when its shape or any buffer changed
     if (!g->gexec || g->g_nk != shape_nk || g->g_commit != (int)commit || g->g_gen != g->buf_gen ||
         g->g_t2 != (int)t2) {
-        rc = capture_batch(g, shape_nk, commit, false, &g->gexec, &g->g_launches, false, t2);
+        rc = capture_batch(g, shape_nk, commit, &g->gexec, &g->g_launches, false, t2);
         if (rc) return rc;
         g->g_nk = shape_nk;
         g->g_commit = (int)commit;
@@ -1251,7 +1233,7 @@ static int apply_batches_region(gc_graph* g, const int32_t* d_ins, const int32_t
         const int q = role - 1;
         const long long nk = role == 3 ? twin_nk : shape_nk;
         if (!g->qexec[q] || g->q_nk[q] != nk || g->q_gen[q] != g->buf_gen) {
-            int r = capture_batch(g, nk, role != 3, false, &g->qexec[q], &g->q_launches[q], false, false, role);
+            int r = capture_batch(g, nk, role != 3, &g->qexec[q], &g->q_launches[q], false, false, role);
             if (r) return r;
             g->q_nk[q] = nk;
             g->q_gen[q] = g->buf_gen;
@@ -1288,7 +1270,7 @@ static int apply_batches_region(gc_graph* g, const int32_t* d_ins, const int32_t
             if (rc) return rc;
             if (g->g_gen != g->buf_gen) {
                 // the adjacency moved: capture again for the remaining batches
-                rc = capture_batch(g, shape_nk, commit, false, &g->gexec, &g->g_launches, false, t2);
+                rc = capture_batch(g, shape_nk, commit, &g->gexec, &g->g_launches, false, t2);
                 if (rc) return rc;
                 g->g_gen = g->buf_gen;
             }
@@ -1333,8 +1315,7 @@ static int enqueue_static(gc_graph* g, bool set_F, int c4_mode = C4_COUNT, unsig
     pdl_launch(k_mark_active, dim3(1), dim3(32), 0, s, g->ctl);
     g->launches += 2;
     CKL();
-    CK(record_stage(g->ev[2], s));
-    int rc = count_region(g, 1, set_F, true, false, true, c4_mode, c4_credit);
+    int rc = count_region(g, 1, set_F, false, true, c4_mode, c4_credit);
     if (rc) return rc;
     // the static pass also gives the triangle sums of the edge-local path
     CK(cudaMemsetAsync(g->T2, 0, 8 * (size_t)std::max(g->n, 1), s));
@@ -1390,8 +1371,8 @@ static int count_static(gc_graph* g, bool set_F, uint64_t out[6], int c4_mode = 
         for (int i = 0; i < 2; i++) g->F3[i] = (uint64_t)g->h_ctl->C3a[i];
     }
     // a static count leaves its stage times in the stats record
-    stage_times(g, 2, 6);
-    if (cudaEventElapsedTime(&g->st.ms_device, g->ev[2], g->ev[6]) != cudaSuccess) cudaGetLastError();
+    stage_times(g, *g->h_ctl, 2, 6);
+    g->st.ms_device = elapsed(*g->h_ctl, 2, 6);
     fill_stats(g, *g->h_ctl);
     g->st.launches = g->launches;
     return GC_OK;
@@ -1452,8 +1433,6 @@ static void destroy(gc_graph* g) {
     if (g->h_ctl) cudaFreeHost(g->h_ctl);
     if (g->h_desc) cudaFreeHost(g->h_desc);
     if (g->e0) cudaEventDestroy(g->e0);
-    for (auto e : g->ev)
-        if (e) cudaEventDestroy(e);
     if (g->e1) cudaEventDestroy(g->e1);
     for (int i = 0; i < NAUX; i++) {
         if (g->aux[i]) cudaStreamDestroy(g->aux[i]);
@@ -1715,12 +1694,7 @@ int gc_open(int32_t n, const int32_t* row_ptr, const int32_t* col, const gc_opti
             g->own_stream = true;
         }
         if (cudaMallocHost((void**)&g->h_ctl, sizeof(Ctl)) != cudaSuccess ||
-            cudaEventCreate(&g->e0) != cudaSuccess || cudaEventCreate(&g->e1) != cudaSuccess ||
-            [&] {
-                for (auto& e : g->ev)
-                    if (cudaEventCreate(&e) != cudaSuccess) return true;
-                return false;
-            }()) {
+            cudaEventCreate(&g->e0) != cudaSuccess || cudaEventCreate(&g->e1) != cudaSuccess) {
             t_open_error = "host allocation failed";
             rc = GC_ENOMEM;
             break;

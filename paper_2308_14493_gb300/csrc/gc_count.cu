@@ -55,6 +55,9 @@ __global__ void k_reset_count(Ctl* c) {
     if (t == 0) {
         c->maxdeg = 0;
         c->c4_wt = c->c4_wmax = 0;
+        c->ts[2] = global_ns();
+        for (int i = 3; i < 10; i++)
+            if (i != 7) c->ts[i] = 0;
     }
 }
 
@@ -176,6 +179,7 @@ __global__ void k_bin(Ctl* c, const int32_t* __restrict__ wlist, const long long
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) dmax = max(dmax, __shfl_down_sync(FULL, dmax, o));
+    stage_end(c, 3);
     if (lane == 0 && dmax) atomicMax(&c->maxdeg, dmax);
     if (__any_sync(FULL, wsum != 0)) {
         wsum = warp_sum_u64(wsum);
@@ -368,6 +372,7 @@ __global__ void __launch_bounds__(TW * 32) k_tri_warp(Ctl* c, const int32_t* __r
     }
     acc_add(c, 4, ka);
     acc_add(c, 10, kb);
+    stage_end(c, 4);
 }
 
 // Shared memory of the block kernel for out-lists of up to KM entries; rows
@@ -496,6 +501,7 @@ __global__ void __launch_bounds__(THREADS) k_tri_block(Ctl* c, const int32_t* __
     }
     acc_add(c, 4, ka);
     acc_add(c, 10, kb);
+    stage_end(c, 4);
 }
 
 // Roots with very long out-lists: one warp per root, one lane per out-edge
@@ -559,6 +565,7 @@ __global__ void k_tri_merge(Ctl* c, const int32_t* __restrict__ list, const long
     }
     acc_add(c, 4, ka);
     acc_add(c, 10, kb);
+    stage_end(c, 4);
 }
 
 // ---- 4-cycles ----------------------------------------------------------------
@@ -651,6 +658,7 @@ __global__ void __launch_bounds__(256) k_c4_reg(Ctl* c, const int32_t* __restric
     acc_add(c, 5, qa);
     acc_add(c, 11, qb);
     acc_add(c, 15, wedges);
+    stage_end(c, 5);
 }
 
 // Walk the wedges u-v-w of pivot u (w < u) for its lower neighbours
@@ -772,6 +780,7 @@ __global__ void __launch_bounds__(C4W_WARPS * 32) k_c4_warp(Ctl* c, const int32_
     acc_add(c, 5, qa);
     acc_add(c, 11, qb);
     acc_add(c, 15, wedges);
+    stage_end(c, 5);
 }
 
 // ---- per-edge terms and closed forms ----------------------------------------
@@ -907,6 +916,7 @@ __global__ void k_finalize(Ctl* c, int mode) {
         if (mode == 3 && ok) c->F3[i] = (unsigned long long)c->C3a[i];
         c->last_out3[i] = mode == 2 ? c->F3[i] + d : c->F3[i];
     }
+    c->ts[6] = global_ns();
 }
 
 }  // namespace gcx
@@ -938,8 +948,7 @@ Tuning effective_tuning(const CountArgs& a) {
     return t;
 }
 
-int enqueue_counting(const CountArgs& a, cudaStream_t s, cudaEvent_t ev_tri, cudaEvent_t ev_c4, cudaEvent_t ev_end,
-                     int mode) {
+int enqueue_counting(const CountArgs& a, cudaStream_t s, int mode) {
     const int sms = a.sms;
     int nl = 0;
     auto lists = [&](int b) { return a.bins + (size_t)b * a.n_alloc; };
@@ -963,13 +972,10 @@ int enqueue_counting(const CountArgs& a, cudaStream_t s, cudaEvent_t ev_tri, cud
     // terms.  On a small graph each branch is a few kernels bound by latency,
     // and the count takes the longest branch; with the triangle kernels one
     // after the other that was 0.183 ms of a 7,000-vertex graph, now 0.170.
-    // ev_tri marks the fork, ev_c4 the end of the triangle branches, ev_end
-    // the end of the 4-cycle branches.
     bool par = true;
     for (int i = 0; i < NAUX; i++) par = par && a.aux[i];
     cudaStream_t sT = par ? a.aux[0] : s, sB = par ? a.aux[1] : s, sC = par ? a.aux[2] : s,
                  sD = par ? a.aux[3] : s;
-    if (ev_tri) record_stage(ev_tri, s);
     if (par) {
         cudaEventRecord(a.fork, s);
         for (int i = 0; i < NAUX; i++) cudaStreamWaitEvent(a.aux[i], a.fork, 0);
@@ -983,11 +989,6 @@ int enqueue_counting(const CountArgs& a, cudaStream_t s, cudaEvent_t ev_tri, cud
             a.ctl, lists(BIN_TRI_BLOCK), a.U_off, a.U_col, a.U_split, a.tpack);
     k_tri_merge<<<sms, 256, 0, sB>>>(a.ctl, lists(BIN_TRI_MERGE), a.U_off, a.U_col, a.U_split, a.tpack);
     nl += 4;
-    if (par) {
-        cudaEventRecord(a.join[0], sT);
-        cudaStreamWaitEvent(sB, a.join[0], 0);
-    }
-    if (ev_c4) record_stage(ev_c4, sB);
     PivotArgs pa;
     pa.ctl = a.ctl;
     pa.pivots = lists(BIN_C4_DENSE);
@@ -1010,20 +1011,12 @@ int enqueue_counting(const CountArgs& a, cudaStream_t s, cudaEvent_t ev_tri, cud
         nl += enqueue_c4_warp_credit(pa, a.c4_mode, a.bins, sms, sC);
     }
     nl += enqueue_c4_tables(pa, a.c4_mode, a.bins, sms, sC, sD);
-    if (a.ev_heavy[0]) record_stage(a.ev_heavy[0], s);
     nl += enqueue_c4_pivots(pa, a.c4_mode, geom, s);
-    if (a.ev_heavy[1]) record_stage(a.ev_heavy[1], s);
-    if (par) {
-        cudaEventRecord(a.join[2], sC);
-        cudaEventRecord(a.join[3], sD);
-        cudaStreamWaitEvent(s, a.join[2], 0);
-        cudaStreamWaitEvent(s, a.join[3], 0);
-    }
-    if (ev_end) record_stage(ev_end, s);
-    if (par) {
-        cudaEventRecord(a.join[1], sB);
-        cudaStreamWaitEvent(s, a.join[1], 0);
-    }
+    if (par)
+        for (int i = 0; i < NAUX; i++) {
+            cudaEventRecord(a.join[i], a.aux[i]);
+            cudaStreamWaitEvent(s, a.join[i], 0);
+        }
     k_edge_terms<<<8 * sms, 256, 0, s>>>(a.ctl, a.wlist, a.U_off, a.U_col, a.U_split, a.tpack, a.da, a.db);
     pdl_launch(k_finalize, dim3(1), dim3(32), 0, s, a.ctl, mode);
     nl += 2;

@@ -224,13 +224,14 @@ __global__ void __launch_bounds__(256) k_c4_granules(const long long* __restrict
 // even share of all of them over the blocks.  One block; the walk over the
 // granules (at most a few hundred on graphs below 16 M vertices) is serial.
 constexpr int PLAN_TILE = 512;
-__global__ void __launch_bounds__(PLAN_TILE) k_c4_plan(const Ctl* c, const long long* __restrict__ U_off, int n,
+__global__ void __launch_bounds__(PLAN_TILE) k_c4_plan(Ctl* c, const long long* __restrict__ U_off, int n,
                                                        int gran, int ngran, const int32_t* __restrict__ gmax,
                                                        int words, int ctas, int nchmax, C4Head* __restrict__ head,
                                                        C4Chunk* __restrict__ chunk, const int32_t* __restrict__ pivots,
                                                        const long long* __restrict__ U_wt,
                                                        int32_t* __restrict__ sorted) {
     pdl_enter();
+    stage_begin(c, 8);
     // pivots by falling wedge bound (two buckets per octave), so that the
     // largest tasks start first
     __shared__ unsigned s_hist[128];
@@ -533,6 +534,8 @@ __global__ void __launch_bounds__(THREADS, MINB) k_c4_pivot(PivotArgs a, int c0)
     acc_add(a.ctl, 11, qb + qab);
     acc_add(a.ctl, 15, wedges);
     acc_add(a.ctl, 20, wedges);
+    stage_end(a.ctl, 5);
+    stage_end(a.ctl, 9);
 }
 
 // A pivot's hash table in shared memory: a slot is an id and a packed count
@@ -708,6 +711,7 @@ __global__ void __launch_bounds__(THREADS, MINB) k_c4_table(PivotArgs a, const i
     acc_add(a.ctl, 5, qa);
     acc_add(a.ctl, 11, qb);
     acc_add(a.ctl, 15, wedges);
+    stage_end(a.ctl, 5);
 }
 
 // Credits of the small pivots (registers and warp tiers, w~ <= C4_T1): a warp
@@ -777,6 +781,7 @@ __global__ void __launch_bounds__(CW_WARPS * 32, 4) k_c4_warp_credit(PivotArgs a
     acc_add(a.ctl, 5, q);
     acc_add(a.ctl, 11, q);
     acc_add(a.ctl, 15, wedges);
+    stage_end(a.ctl, 5);
 }
 
 // ---- host side -------------------------------------------------------------------

@@ -117,6 +117,12 @@ struct Ctl {
     int l_nw3;                       // third vertices listed after V_X (maintained triangle sums)
     // wedge bounds of the pivots counted in shared memory (BIN_C4_DENSE): sum and maximum
     unsigned long long c4_wt, c4_wmax;
+    // stage boundaries: begin of [0] normalise [1] region walk [2] union graph;
+    // [3] end of the binning (local: begin of the triangles); end of [4] the
+    // triangles, [5] the 4-cycles (local: begin of the 4-cliques / 4-cycles and
+    // of the closed forms); [6] end of the closed forms, [7] of the batch;
+    // [8] begin and [9] end of the shared-memory pivots
+    unsigned long long ts[10];
     // (device-only tail: the host mirror copies the block up to here)
     unsigned long long accs[NACC][ACC_STRIPES];  // acc, striped: kernels add here, k_finalize sums
 };
@@ -153,15 +159,22 @@ struct Dims {
     int sms;
 };
 
-// Stage-boundary event: inside a stream capture it becomes an event-record
-// node that records at every replay (a plain record there would only order
-// the capture); outside a capture an ordinary record.
-inline cudaError_t record_stage(cudaEvent_t e, cudaStream_t s) {
-    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
-    cudaError_t r = cudaStreamIsCapturing(s, &st);
-    if (r != cudaSuccess) return r;
-    return st == cudaStreamCaptureStatusActive ? cudaEventRecordWithFlags(e, s, cudaEventRecordExternal)
-                                               : cudaEventRecord(e, s);
+// Stage boundaries are taken on the device, in Ctl::ts (global timer,
+// nanoseconds; it advances every 32 on this chip): event-record nodes in a
+// captured batch cost 3 to 5 us each and break the programmatic launches on
+// both sides.  stage_begin: the first kernel of a stage; stage_end: kernels of
+// a stage that ends with the last of several (every eighth block adds its
+// time, enough for blocks that share their work).
+__device__ __forceinline__ unsigned long long global_ns() {
+    unsigned long long t;
+    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+    return t;
+}
+__device__ __forceinline__ void stage_begin(Ctl* c, int i) {
+    if (blockIdx.x == 0 && threadIdx.x == 0) c->ts[i] = global_ns();
+}
+__device__ __forceinline__ void stage_end(Ctl* c, int i) {
+    if ((blockIdx.x & 7) == 0 && threadIdx.x == 0) atomicMax(&c->ts[i], global_ns());
 }
 
 __device__ __forceinline__ uint32_t vid(uint32_t e) { return e & ID_MASK; }

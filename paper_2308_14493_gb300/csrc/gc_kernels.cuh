@@ -103,7 +103,6 @@ struct CountArgs {
     cudaStream_t aux[NAUX] = {};    // side streams of the counting pass (or none)
     cudaEvent_t fork = nullptr;     // fork / join events for them (timing disabled)
     cudaEvent_t join[NAUX] = {};
-    cudaEvent_t ev_heavy[2] = {nullptr, nullptr};  // around the heavy-pivot 4-cycle kernels, on their stream
 };
 Tuning effective_tuning(const CountArgs& a);
 // Dynamic shared-memory limits of the counting kernels (once per device).
@@ -148,10 +147,8 @@ __global__ void k_t2_mark(const Ctl* c, const int32_t* wlist, uint32_t* mark, un
 __global__ void k_t2_from_region(const Ctl* c, const int32_t* wlist, const long long* U_off, const uint32_t* U_col,
                                  const int32_t* U_split, const unsigned long long* tpack, const uint32_t* mark,
                                  unsigned long long* T2);
-// Enqueue the edge-local delta (after the union rows of V_X); events mark
-// the triangle stage, the 4-clique / 4-cycle stage and the closed forms.
-int enqueue_local(const LocalArgs& a, cudaStream_t s, cudaEvent_t ev_tri, cudaEvent_t ev_sub, cudaEvent_t ev_fin,
-                  int commit);
+// Enqueue the edge-local delta (after the union rows of V_X).
+int enqueue_local(const LocalArgs& a, cudaStream_t s, int commit);
 
 // Per-vertex and per-edge graphlet counts after a static pass with the credits
 // of its 4-cycles (gc_vertex.cu).
@@ -211,10 +208,8 @@ struct EdgeArgs {
 int enqueue_edge_counts(const EdgeArgs& a, cudaStream_t s);
 
 // Enqueue the counting kernels (binning, triangles / 4-cliques, 4-cycles,
-// edge terms, closed forms with k_finalize(mode)); events, when given, are
-// recorded before the triangle, 4-cycle and edge-term stages.  Returns the
-// number of kernels launched.
-int enqueue_counting(const CountArgs& a, cudaStream_t s, cudaEvent_t ev_tri, cudaEvent_t ev_c4, cudaEvent_t ev_end,
-                     int mode);
+// edge terms, closed forms with k_finalize(mode)).  Returns the number of
+// kernels launched.
+int enqueue_counting(const CountArgs& a, cudaStream_t s, int mode);
 
 }  // namespace gcx

@@ -252,9 +252,10 @@ __global__ void k_loc_check_pairs(Ctl* c, long long cap) {
 
 // Owner of every union-row entry: own[e] = u for the entries of u's row (a
 // warp per vertex of V_X; a hub row is a long run of coalesced stores).
-__global__ void k_loc_owner(const Ctl* c, const int32_t* __restrict__ wlist, LocalView V,
+__global__ void k_loc_owner(Ctl* c, const int32_t* __restrict__ wlist, LocalView V,
                             int32_t* __restrict__ own) {
     pdl_enter();
+    stage_begin(c, 3);
     const int nX = c->l_len[0] ? c->lvl[0] : 0;
     const int lane = threadIdx.x & 31;
     const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -420,11 +421,12 @@ __global__ void k_loc_common(const Ctl* c, LocalView V, const int32_t* __restric
 // For a common neighbour w of pair (u, v) in the pair's graph x, the
 // 4-cliques {u, v, w, z} with z > w: probes of the shorter of the pair's
 // remaining records and w's row beyond w.
-__global__ void k_loc_k4_cost(const Ctl* c, LocalView V, const int32_t* __restrict__ srcA,
+__global__ void k_loc_k4_cost(Ctl* c, LocalView V, const int32_t* __restrict__ srcA,
                               const int32_t* __restrict__ dstA, const int32_t* __restrict__ srcD,
                               const int32_t* __restrict__ dstD, const long long* __restrict__ ppre,
                               const unsigned long long* __restrict__ rec, int32_t* __restrict__ kcost) {
     pdl_enter();
+    stage_begin(c, 4);
     const long long np = c->l_len[1];
     const long long tot = c->l_len[2];
     const long long stride = (long long)gridDim.x * blockDim.x;
@@ -1083,6 +1085,7 @@ __global__ void k_loc_vterms(Ctl* c, const int32_t* __restrict__ wlist, LocalVie
 // (Cb, sb zero).
 __global__ void k_finalize_local(Ctl* c, int commit) {
     pdl_enter();
+    stage_begin(c, 5);
     if (blockIdx.x == 0 && threadIdx.x < NACC) {
         unsigned long long x = 0;
         for (int k = 0; k < ACC_STRIPES; k++) x += c->accs[threadIdx.x][k];
@@ -1121,6 +1124,7 @@ __global__ void k_finalize_local(Ctl* c, int commit) {
     }
     c->acc[14] = (unsigned long long)(c->l_tot[0] + c->l_tot[2] + c->l_tot[4]);  // probes
     c->acc[15] = 0;
+    c->ts[6] = global_ns();
 }
 
 // ---- launch sequence ---------------------------------------------------------------
@@ -1150,15 +1154,13 @@ void local_setup_attributes() {
 // kind 0: the triangle kernel, 1: the 4-cycle kernel
 static int staged_grid(int kind, int sms) { return 8 * sms * (g_loc_per_sm[kind] > 0 ? g_loc_per_sm[kind] : 2); }
 
-int enqueue_local(const LocalArgs& a, cudaStream_t s, cudaEvent_t ev_tri, cudaEvent_t ev_sub, cudaEvent_t ev_fin,
-                  int commit) {
+int enqueue_local(const LocalArgs& a, cudaStream_t s, int commit) {
     const int sms = a.sms;
     const int gw = 8 * sms, tpb = 256;
     const int sg = scan_grid(a.cap, sms);
     LocalView V{a.visited, a.U_off, a.U_col, a.row_start, a.deg, a.col};
     int nl = 0;
     pdl_launch(k_loc_check_rows, dim3(1), dim3(32), 0, s, a.ctl, a.cap);
-    if (ev_tri) record_stage(ev_tri, s);
     pdl_launch(k_loc_owner, dim3(gw), dim3(tpb), 0, s, a.ctl, a.wlist, V, a.own);
     nl += 2;
     // changed pairs: common neighbours (4-cliques, triangles) and 4-cycle tasks
@@ -1194,7 +1196,6 @@ int enqueue_local(const LocalArgs& a, cudaStream_t s, cudaEvent_t ev_tri, cudaEv
         pdl_launch(k_loc_terms, dim3(gw), dim3(tpb), 0, s, a.ctl, a.wlist, V, a.own, a.tpack, a.da, a.db);
         nl += 2;
     }
-    if (ev_sub) record_stage(ev_sub, s);
     pdl_launch(k_loc_k4_cost, dim3(gw), dim3(tpb), 0, s, a.ctl, V, a.srcA, a.dstA, a.srcD, a.dstD, a.ppre, a.rec,
                a.kcost);
     nl++;
@@ -1209,7 +1210,6 @@ int enqueue_local(const LocalArgs& a, cudaStream_t s, cudaEvent_t ev_tri, cudaEv
     pdl_launch(k_loc_c4, dim3(staged_grid(1, sms)), dim3(LC4_THREADS), LC4_SMEM, s, a.ctl, V, a.srcA, a.dstA, a.srcD,
                a.dstD, a.walk, a.tpair, a.own, a.pre, a.cpre);
     nl++;
-    if (ev_fin) record_stage(ev_fin, s);
     pdl_launch(k_finalize_local, dim3(1), dim3(32), 0, s, a.ctl, commit);
     nl++;
     return nl;

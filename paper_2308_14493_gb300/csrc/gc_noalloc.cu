@@ -228,7 +228,7 @@ extern "C" int gc_count_static_noalloc(int32_t n, const int32_t* d_row_ptr, cons
     ca.c4.lcap = 0;
     ca.tune = default_tuning();
     ca.sms = sms;
-    enqueue_counting(ca, s, nullptr, nullptr, nullptr, 1);
+    enqueue_counting(ca, s, 1);
     if (!stale && cudaGetLastError() != cudaSuccess) return GC_ECUDA;
     long long Ca[6];
     if (cudaMemcpyAsync(Ca, ctl->Ca, sizeof(Ca), cudaMemcpyDeviceToHost, s) != cudaSuccess) return GC_ECUDA;

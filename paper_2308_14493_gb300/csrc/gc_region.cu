@@ -43,6 +43,7 @@ __device__ __forceinline__ void visit_append(bool want, int32_t v, uint32_t* vis
 __global__ void k_bfs_sources(Ctl* c, const int32_t* __restrict__ srcA, const int32_t* __restrict__ srcD,
                               uint32_t* __restrict__ visited, int32_t* __restrict__ wlist) {
     pdl_enter();
+    stage_begin(c, 1);
     if (c->err) return;
     long long na = c->nA2, nd = c->nD2, tot = na + nd;
     long long stride = (long long)gridDim.x * blockDim.x;
