@@ -258,7 +258,7 @@ __global__ void k_begin_batch(Ctl* c, const long long* desc) {
     c->nA2 = c->nD2 = 0;
     for (int k = 0; k < 8; k++) c->st[k] = 0;
     c->nW = 0;
-    for (int k = 0; k < MAX_HOPS + 2; k++) c->lvl[k] = 0;
+    for (int k = 0; k < MAX_HOPS + 2; k++) c->lvl[k] = c->lcnt[k] = 0;
     c->nU = 0;
     c->scratch_tail = 0;
     c->overflow = 0;
@@ -296,7 +296,7 @@ __global__ void k_begin_twin(Ctl* c, const long long* desc) {
     c->nA2 = c->nD2 = 0;
     for (int k = 0; k < 8; k++) c->st[k] = 0;
     c->nW = 0;
-    for (int k = 0; k < MAX_HOPS + 2; k++) c->lvl[k] = 0;
+    for (int k = 0; k < MAX_HOPS + 2; k++) c->lvl[k] = c->lcnt[k] = 0;
     c->nU = 0;
     c->scratch_tail = 0;
     c->overflow = 0;
@@ -677,17 +677,21 @@ static int count_region(gc_graph* g, int fin, bool set_F, bool twin = false, boo
 
 // Edge-local delta: union rows of the batch endpoints V_X (full rows), then
 // the local terms, 4-cliques and 4-cycles and their closed forms.
-static int count_local(gc_graph* g, int commit, bool t2) {
+// (laid_out: the normalisation has written the offsets of the union rows)
+static int count_local(gc_graph* g, int commit, bool t2, bool laid_out) {
     cudaStream_t s = g->s;
     int gw = grid_warps(g);
     pdl_launch(k_reset_count, dim3(1), dim3(32), 0, s, g->ctl);
     if (t2) CK(cudaMemsetAsync(g->visited2, 0, sizeof(uint32_t) * (size_t)((g->n + 31) / 32 + 1), s));
-    CK(cudaMemsetAsync(g->U_deg, 0, sizeof(int32_t) * (size_t)std::max(g->n, 1), s));
-    pdl_launch(k_u_count, dim3(gw), dim3(TPB), 0, s, g->ctl, g->wlist, g->visited, g->row_start, g->deg, g->col,
-               g->segA, g->U_deg, 1);
-    g->launches += 2;
-    g->launches += scan_i32_to_i64(g->U_deg, g->U_off, nullptr, g->n, g->bsum.p, scan_grid(g->n, g->sms), &g->ctl->nU,
-                                   s);
+    g->launches++;
+    if (!laid_out) {
+        CK(cudaMemsetAsync(g->U_deg, 0, sizeof(int32_t) * (size_t)std::max(g->n, 1), s));
+        pdl_launch(k_u_count, dim3(gw), dim3(TPB), 0, s, g->ctl, g->wlist, g->visited, g->row_start, g->deg, g->col,
+                   g->segA, g->U_deg, 1);
+        g->launches++;
+        g->launches += scan_i32_to_i64(g->U_deg, g->U_off, nullptr, g->n, g->bsum.p, scan_grid(g->n, g->sms), &g->ctl->nU,
+                                       s);
+    }
     pdl_launch(k_u_fill_all, dim3(gw), dim3(TPB), 0, s, g->ctl, g->wlist, g->row_start, g->deg, g->col, g->segA,
                g->segD, g->dstA.p,
                                     g->dstD.p, g->U_off, g->U_col.p, g->U_split, g->da, g->db);
@@ -785,12 +789,34 @@ static int enqueue_batch(gc_graph* g, long long max_nk, bool commit, bool local 
                          int role = 0) {
     cudaStream_t s = g->s;
     const bool twin = role == 3;
+    CK(cudaMemsetAsync(g->visited, 0, sizeof(uint32_t) * (size_t)((g->n + 31) / 32 + 1), s));
     if (twin) pdl_launch(k_begin_twin, dim3(1), dim3(32), 0, s, g->ctl, g->desc);
     else pdl_launch(k_begin_batch, dim3(1), dim3(32), 0, s, g->ctl, g->desc);
     g->launches++;
     const long long nkb = std::max<long long>(max_nk, 1);
     const int ge = grid_elems(g, nkb);
-    if (max_nk > 0) {
+    const bool small = !twin && max_nk <= SMALL_KEYS;
+    if (small) {
+        SmallBatch b;
+        b.ctl = g->ctl;
+        b.perm = g->perm;
+        b.n = g->n;
+        b.S = g->S;
+        b.row_start = g->row_start;
+        b.deg = g->deg;
+        b.col = g->col;
+        b.srcA = g->srcA.p;
+        b.dstA = g->dstA.p;
+        b.srcD = g->srcD.p;
+        b.dstD = g->dstD.p;
+        b.segA = g->segA;
+        b.segD = g->segD;
+        b.visited = g->visited;
+        b.wlist = g->wlist;
+        b.U_off = local ? g->U_off : nullptr;
+        pdl_launch(k_batch_small, dim3(1), dim3(1024), BATCH_SMALL_SMEM, s, b);
+        g->launches++;
+    } else {
         if (twin)
             pdl_launch(k_batch_keys_twin, dim3(grid_elems(g, nkb / 2)), dim3(TPB), 0, s, g->ctl, g->perm, g->n, g->S,
                        g->keys.p);
@@ -819,28 +845,26 @@ static int enqueue_batch(gc_graph* g, long long max_nk, bool commit, bool local 
         g->launches++;
         int rc = enqueue_segments(g, false);
         if (rc) return rc;
+        pdl_launch(k_bfs_sources, dim3(ge), dim3(TPB), 0, s, g->ctl, g->srcA.p, g->srcD.p, g->visited, g->wlist);
+        g->launches++;
     }
-    CK(cudaMemsetAsync(g->visited, 0, sizeof(uint32_t) * (size_t)((g->n + 31) / 32 + 1), s));
-    pdl_launch(k_bfs_sources, dim3(ge), dim3(TPB), 0, s, g->ctl, g->srcA.p, g->srcD.p, g->visited, g->wlist);
-    pdl_launch(k_level_mark, dim3(1), dim3(1), 0, s, g->ctl, 0);
-    g->launches += 2;
     if (role == 2 || role == 3) {
         pdl_launch(k_region_rest, dim3(grid_elems(g, g->n)), dim3(TPB), 0, s, g->ctl, g->n, g->visited, g->wlist);
         g->launches++;
-    }
-    for (int L = 1; L <= (local || role == 1 ? 0 : g->hops); L++) {
-        if (role == 0) {
+    } else if (role == 1) {
+        pdl_launch(k_level_ends, dim3(1), dim3(32), 0, s, g->ctl);
+        g->launches++;
+    } else if (!local) {
+        for (int L = 1; L <= g->hops; L++) {
             pdl_launch(k_bfs_expand, dim3(grid_warps(g)), dim3(TPB), 0, s, g->ctl, L, g->row_start, g->deg, g->col,
                        g->visited, g->wlist);
             g->launches++;
         }
-        pdl_launch(k_level_mark, dim3(1), dim3(1), 0, s, g->ctl, L);
-        g->launches++;
     }
     CKL();
     int rc = GC_OK;
     if (role != 1) {
-        rc = local ? count_local(g, commit ? 1 : 0, t2)
+        rc = local ? count_local(g, commit ? 1 : 0, t2, small)
                    : count_region(g, role == 2 ? 3 : role == 3 ? 4 : (commit ? 0 : 2), false, twin,
                                   role == 2);
         if (rc) return rc;
@@ -1572,6 +1596,7 @@ static int open_device(gc_graph* g, const int32_t* row_ptr, const int32_t* colh)
     // counting pass: work lists and the buffers of the shared-memory 4-cycle pivots
     count_setup_attributes();
     local_setup_attributes();
+    batch_setup_attributes();
     g->bins = (int32_t*)dalloc(g, sizeof(int32_t) * (size_t)NBINS * nn);
     if (!g->bins || !ensure_c4(g)) return nomem(g, "counting work lists");
     return count_static(g, true, nullptr);

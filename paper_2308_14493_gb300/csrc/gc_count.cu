@@ -56,6 +56,7 @@ __global__ void k_reset_count(Ctl* c) {
         c->maxdeg = 0;
         c->c4_wt = c->c4_wmax = 0;
         c->ts[2] = global_ns();
+        close_levels(c);
         for (int i = 3; i < 10; i++)
             if (i != 7) c->ts[i] = 0;
     }

@@ -70,6 +70,7 @@ struct Ctl {
     unsigned long long st[8];        // [0] repeats [1] cancelled [2] no-op ins [3] no-op del (directed)
     int nW;                          // region size
     int lvl[MAX_HOPS + 2];           // lvl[L]: end of BFS level L in the region list
+    int lcnt[MAX_HOPS + 2];          // vertices appended at each level (k_reset_count sums them up)
     long long nU;                    // entries of the region union graph
     unsigned long long acc[NACC];    // [0..5] sums of G_a, [6..11] sums of G_b: P, S, 2TT, D, K, Q
                                      // [12] |E(G_a)|, [13] |E(G_b)|, [14] triangle work, [15] wedges
@@ -318,6 +319,19 @@ __device__ __forceinline__ bool sorted_contains(const int32_t* a, long long len,
     long long p = lower_bound_i32(a, len, key);
     return p < len && a[p] == key;
 }
+
+// Ends of the BFS levels and the region size from the levels' counts.
+__device__ __forceinline__ void close_levels(Ctl* c) {
+    int e = 0;
+    for (int L = 0; L < MAX_HOPS + 2; L++) {
+        e += c->lcnt[L];
+        c->lvl[L] = e;
+    }
+    c->nW = e;
+}
+
+// Batches of up to this many keys are normalised by one block (k_batch_small).
+constexpr int SMALL_KEYS = 4096;
 
 // ---- host-side launchers implemented in the .cu files -------------------
 

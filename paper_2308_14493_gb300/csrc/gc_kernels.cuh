@@ -13,6 +13,22 @@ __global__ void k_batch_decide(const uint64_t* keys, Ctl* c, int S, const long l
 __global__ void k_batch_compact(const uint64_t* keys, const Ctl* c, int S, const int32_t* keepA,
                                 const int32_t* keepD, const long long* posA, const long long* posD, int32_t* srcA,
                                 int32_t* dstA, int32_t* srcD, int32_t* dstD);
+// Buffers of a small batch (at most SMALL_KEYS keys).
+struct SmallBatch {
+    Ctl* ctl;
+    const int32_t* perm;
+    int n, S;
+    const long long* row_start;
+    const int32_t *deg, *col;
+    int32_t *srcA, *dstA, *srcD, *dstD;
+    int2 *segA, *segD;
+    uint32_t* visited;
+    int32_t* wlist;
+    long long* U_off;   // edge-local form: union row offsets of the endpoints (else null)
+};
+__global__ void k_batch_small(SmallBatch b);
+void batch_setup_attributes();
+constexpr size_t BATCH_SMALL_SMEM = (size_t)SMALL_KEYS * 8;
 __global__ void k_batch_segments(const int32_t* src, const long long* d_len, int2* seg);
 __global__ void k_batch_clear_segments(const int32_t* src, const long long* d_len, int2* seg);
 __global__ void k_commit_plan(Ctl* c, const int32_t* wlist, const int2* segA, const int2* segD, const int32_t* deg,
@@ -43,7 +59,7 @@ __global__ void k_ext_degrees(const int32_t* deg, const int32_t* iperm, int n, i
 
 // gc_region.cu
 __global__ void k_bfs_sources(Ctl* c, const int32_t* srcA, const int32_t* srcD, uint32_t* visited, int32_t* wlist);
-__global__ void k_level_mark(Ctl* c, int L);
+__global__ void k_level_ends(Ctl* c);
 __global__ void k_region_rest(Ctl* c, int n, uint32_t* visited, int32_t* wlist);
 __global__ void k_u_count_twin(const Ctl* c, const int32_t* wlist, const int32_t* deg, const int2* segA,
                                int32_t* U_deg);

@@ -24,7 +24,9 @@ __device__ __forceinline__ bool in_region(const uint32_t* visited, int32_t v) {
 }
 
 // mark v; if it was unmarked, append it to the region list (warp-aggregated)
-__device__ __forceinline__ void visit_append(bool want, int32_t v, uint32_t* visited, int32_t* wlist, Ctl* c) {
+// (level L, which starts at wlist[first])
+__device__ __forceinline__ void visit_append(bool want, int32_t v, uint32_t* visited, int32_t* wlist, int first,
+                                             int* count) {
     bool fresh = false;
     if (want) {
         uint32_t bit = 1u << (v & 31);
@@ -34,7 +36,7 @@ __device__ __forceinline__ void visit_append(bool want, int32_t v, uint32_t* vis
     if (m) {
         int lane = threadIdx.x & 31, leader = __ffs(m) - 1;
         int base = 0;
-        if (lane == leader) base = atomicAdd(&c->nW, __popc(m));
+        if (lane == leader) base = first + atomicAdd(count, __popc(m));
         base = __shfl_sync(FULL, base, leader);
         if (fresh) wlist[base + __popc(m & lanemask_lt())] = v;
     }
@@ -53,11 +55,15 @@ __global__ void k_bfs_sources(Ctl* c, const int32_t* __restrict__ srcA, const in
     for (long long i = start; i < tot_r; i += stride) {
         bool ok = i < tot;
         int32_t v = ok ? (i < na ? srcA[i] : srcD[i - na]) : 0;
-        visit_append(ok, v, visited, wlist, c);
+        visit_append(ok, v, visited, wlist, 0, &c->lcnt[0]);
     }
 }
 
-__global__ void k_level_mark(Ctl* c, int L) { pdl_enter(); c->lvl[L] = c->nW; }
+// ends of the levels, for a batch that is committed without a count
+__global__ void k_level_ends(Ctl* c) {
+    pdl_enter();
+    if (threadIdx.x == 0) close_levels(c);
+}
 
 // The two-batch form's whole-graph pass: after the batch endpoints (level
 // 0), every other vertex joins the region, so W = V and the counts of G_a and
@@ -66,10 +72,11 @@ __global__ void k_level_mark(Ctl* c, int L) { pdl_enter(); c->lvl[L] = c->nW; }
 __global__ void k_region_rest(Ctl* c, int n, uint32_t* __restrict__ visited, int32_t* __restrict__ wlist) {
     pdl_enter();
     if (c->err || !c->active) return;
+    const int first = c->lcnt[0];
     const long long n_r = ((long long)n + 31) & ~31ll;  // warp-uniform bound for the ballot
     for (long long v = blockIdx.x * (long long)blockDim.x + threadIdx.x; v < n_r;
          v += (long long)gridDim.x * blockDim.x)
-        visit_append(v < n, (int32_t)(v < n ? v : 0), visited, wlist, c);
+        visit_append(v < n, (int32_t)(v < n ? v : 0), visited, wlist, first, &c->lcnt[1]);
 }
 
 __global__ void k_bfs_expand(Ctl* c, int L, const long long* __restrict__ row_start, const int32_t* __restrict__ deg,
@@ -77,8 +84,11 @@ __global__ void k_bfs_expand(Ctl* c, int L, const long long* __restrict__ row_st
                              int32_t* __restrict__ wlist) {
     pdl_enter();
     if (c->err) return;
-    int fb = L >= 2 ? c->lvl[L - 2] : 0;
-    int fe = c->lvl[L - 1];
+    int fb = 0, fe = c->lcnt[0];  // the level before
+    for (int i = 1; i < L; i++) {
+        fb = fe;
+        fe += c->lcnt[i];
+    }
     int lane = threadIdx.x & 31;
     int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     int nwarps = (gridDim.x * blockDim.x) >> 5;
@@ -89,7 +99,7 @@ __global__ void k_bfs_expand(Ctl* c, int L, const long long* __restrict__ row_st
         for (int b = 0; b < d; b += 32) {
             bool ok = b + lane < d;
             int32_t y = ok ? row[b + lane] : 0;
-            visit_append(ok, y, visited, wlist, c);
+            visit_append(ok, y, visited, wlist, fe, &c->lcnt[L]);
         }
     }
 }
@@ -100,7 +110,10 @@ __global__ void k_region_all(Ctl* c, int n, int32_t* __restrict__ wlist) {
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) wlist[i] = i;
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         c->nW = n;
-        for (int L = 0; L < MAX_HOPS + 2; L++) c->lvl[L] = n;
+        for (int L = 0; L < MAX_HOPS + 2; L++) {
+            c->lvl[L] = n;
+            c->lcnt[L] = L == 0 ? n : 0;
+        }
     }
 }
 
