@@ -510,7 +510,7 @@ __global__ void k_commit_plan(Ctl* c, const int32_t* __restrict__ wlist, const i
 // row \ D_u u A_u of every touched vertex into the scratch: a warp per
 // short row, a block per long one (every entry placed by binary searches,
 // so a hub row spreads over the block).
-constexpr long long LONG_ROW = 4096;
+constexpr long long LONG_ROW = 512;
 
 __global__ void k_commit_merge(const Ctl* c, const int32_t* __restrict__ wlist, const int2* __restrict__ segA,
                                const int2* __restrict__ segD, const int32_t* __restrict__ dstA,

@@ -40,163 +40,14 @@
 
 #include "gc_c4.cuh"
 #include "gc_kernels.cuh"
+#include "gc_walk.cuh"
 
 namespace gcx {
 
 namespace {
 
 constexpr unsigned long long RUN_LEN = (1ull << 28) - 1;
-constexpr int PV_UNROLL = 4;
 constexpr int C4_SPLITS = 18;  // chunks that the share limit may add
-
-constexpr int PV_LONG = 128;   // a run of at least this many entries is walked by the whole warp
-
-// Per-warp scratch: the short runs of up to 32 lower neighbours.
-struct __align__(16) ShortRun {
-    const uint32_t* p;
-    int len;
-    uint32_t fv;
-};
-struct WarpRuns {
-    ShortRun r[32];
-    int j[32];
-};
-
-// How a task's lower neighbours are dealt to warps.  Rows are sorted by id, so
-// the last lower neighbours have the longest rows, and those hold most of the
-// wedges: groups run from the end of the list, `lev` groups of 2^lm rows, then
-// as many of twice the size, and so on up to 32 times the size, so that the
-// groups are of similar work and the larger ones come first.  More groups
-// balance better, fewer start fewer chains of loads: lev is half a group per
-// warp for small tasks and two for large ones.  lm > 0 where runs are shorter
-// than 16 entries on average.
-struct Deal {
-    int lm, lev;
-};
-__device__ __forceinline__ Deal deal_groups(int nlow, float wedges, int warps) {
-    Deal d;
-    const int mul = (int)fminf(32.f, 16.f * (float)nlow / fmaxf(wedges, 1.f));
-    d.lm = mul >= 1 ? min(5, 32 - __clz(mul)) : 0;
-    d.lev = wedges < 512.f * (float)warps ? warps / 2 : wedges < 8192.f * (float)warps ? warps : 2 * warps;
-    return d;
-}
-
-// Walk the wedges of a pivot with lower neighbours row[0 .. nlow).  run(v, &p,
-// &len) gives the entries to walk of neighbour v.  The warps of the block
-// take groups of neighbours from *ctr; each lane loads one neighbour's run,
-// long runs are walked by all lanes and short ones by eight lanes a run, four
-// loads in flight per lane.  fn(q, e, f, x) takes four wedges at a time:
-// q[i] the address of the second edge's entry (null: no wedge), e[i] the
-// entry, f[i] the first edge's entry; with ACC it returns credits in x[i],
-// which are summed over each neighbour's run and given to rowfn(sum, v's
-// entry, its index in the row) by one lane.
-template <bool ACC, class RunFn, class Fn, class RowFn>
-__device__ __forceinline__ void walk_lower(const uint32_t* __restrict__ row, int nlow, Deal d, int* ctr, WarpRuns& W,
-                                           RunFn run, Fn fn, RowFn rowfn) {
-    const int lane = threadIdx.x & 31, sl = lane & 7;
-    const unsigned sub = 0xFFu << (lane & 24);
-    for (;;) {
-        int g = 0;
-        if (lane == 0) g = atomicAdd(ctr, 1);
-        g = __shfl_sync(FULL, g, 0);
-        const int q = min(g / d.lev, 5);
-        const int gs = (1 << q) << d.lm;
-        int j0 = (d.lev * ((1 << q) - 1) << d.lm) + (g - q * d.lev) * gs;
-        if (j0 >= nlow) break;
-        for (const int je = min(j0 + gs, nlow); j0 < je; j0 += 32) {
-            int len = 0, jr = 0;
-            const uint32_t* p = nullptr;
-            uint32_t fv = 0;
-            if (j0 + lane < je) {
-                jr = nlow - 1 - j0 - lane;
-                fv = row[jr];
-                run(vid(fv), &p, &len);
-            }
-            const bool brief = len > 0 && len < PV_LONG;
-            const unsigned ms = __ballot_sync(FULL, brief);
-            if (brief) {
-                const int slot = __popc(ms & lanemask_lt());
-                W.r[slot] = ShortRun{p, len, fv};
-                if (ACC) W.j[slot] = jr;
-            }
-            for (unsigned ml = __ballot_sync(FULL, len >= PV_LONG); ml; ml &= ml - 1) {
-                const int src = __ffs(ml) - 1;
-                const int n = __shfl_sync(FULL, len, src);
-                const uint32_t f0 = __shfl_sync(FULL, fv, src);
-                const uint32_t* q0 = (const uint32_t*)__shfl_sync(FULL, (unsigned long long)p, src) + lane;
-                unsigned long long acc = 0;
-                for (int rem = n - lane; rem + lane > 0; rem -= 32 * PV_UNROLL, q0 += 32 * PV_UNROLL) {
-                    const uint32_t* q[PV_UNROLL];
-                    uint32_t e[PV_UNROLL], f[PV_UNROLL], x[PV_UNROLL];
-#pragma unroll
-                    for (int i = 0; i < PV_UNROLL; i++) {
-                        q[i] = rem > 32 * i ? q0 + 32 * i : nullptr;
-                        f[i] = f0;
-                        e[i] = q[i] ? *q[i] : 0u;
-                    }
-                    fn(q, e, f, x);
-                    if (ACC) {
-#pragma unroll
-                        for (int i = 0; i < PV_UNROLL; i++) acc += q[i] ? x[i] : 0u;
-                    }
-                }
-                if (ACC) {
-                    acc = warp_sum_u64(acc);
-                    if (lane == 0 && acc) rowfn(acc, f0, nlow - 1 - j0 - src);
-                }
-            }
-            __syncwarp();
-            const int nr = __popc(ms);
-            // eight lanes a run: runs r = lane / 8, + 4, + 8, ...
-            int r = (lane >> 3) - 4, rem = 0, rc = -1;
-            uint32_t f0 = 0;
-            unsigned long long acc = 0;
-            auto flush = [&]() {  // the eight lanes' credits of run rc
-#pragma unroll
-                for (int o = 4; o > 0; o >>= 1) acc += __shfl_xor_sync(sub, acc, o);
-                if (sl == 0 && acc) rowfn(acc, W.r[rc].fv, W.j[rc]);
-                acc = 0;
-            };
-            while (__any_sync(FULL, r < nr)) {  // the warp stays together
-                const uint32_t* q[PV_UNROLL];
-                uint32_t e[PV_UNROLL], f[PV_UNROLL], x[PV_UNROLL];
-                int ri[PV_UNROLL];
-#pragma unroll
-                for (int i = 0; i < PV_UNROLL; i++) {
-                    r += rem <= 0 ? 4 : 0;
-                    if (rem <= 0 && r < nr) {
-                        const ShortRun t = W.r[r];
-                        p = t.p + sl;
-                        rem = t.len;
-                        f0 = t.fv;
-                    }
-                    q[i] = rem > sl ? p : nullptr;
-                    f[i] = f0;
-                    if (ACC) ri[i] = r;
-                    p += 8;
-                    rem -= 8;
-                }
-                __syncwarp();
-#pragma unroll
-                for (int i = 0; i < PV_UNROLL; i++) e[i] = q[i] ? *q[i] : 0u;
-                fn(q, e, f, x);
-                if (ACC) {
-#pragma unroll
-                    for (int i = 0; i < PV_UNROLL; i++) {
-                        if (ri[i] >= nr) break;  // same for the eight lanes
-                        if (ri[i] != rc) {
-                            if (rc >= 0) flush();
-                            rc = ri[i];
-                        }
-                        acc += q[i] ? x[i] : 0u;
-                    }
-                }
-            }
-            if (ACC && rc >= 0) flush();
-            __syncwarp();
-        }
-    }
-}
 
 __device__ __forceinline__ void red_u64(unsigned long long* p, unsigned long long x) { atomicAdd(p, x); }
 
@@ -403,8 +254,8 @@ __global__ void __launch_bounds__(THREADS, MINB) k_c4_pivot(PivotArgs a, int c0)
         const unsigned long long* const runs = a.b.run + (size_t)t.k * a.n;
         const float est = t.wt * ck.share;  // wedges of this task, about
         const Deal deal = deal_groups(nlow, est, NW);
-        auto run = [&](uint32_t v, const uint32_t** p, int* len) {
-            const unsigned long long r = runs[v];
+        auto run = [&](uint32_t fv, const uint32_t** p, int* len) {
+            const unsigned long long r = runs[vid(fv)];
             *len = (int)(r & RUN_LEN);
             *p = a.U_col + (r >> 28);
         };
@@ -672,7 +523,8 @@ __global__ void __launch_bounds__(THREADS, MINB) k_c4_table(PivotArgs a, const i
         const uint32_t* const row = a.U_col + t.rb;
         const Table T{keys, cnts, min((uint32_t)SLOTS, Table::size_for(t.k))};
         const Deal deal = deal_groups(t.nlow, (float)t.k, NW);
-        auto run = [&](uint32_t v, const uint32_t** p, int* len) {
+        auto run = [&](uint32_t fv, const uint32_t** p, int* len) {
+            const uint32_t v = vid(fv);
             const long long b = a.U_off[v];
             *p = a.U_col + b;
             *len = (int)(a.U_off[v + 1] - b);
@@ -744,7 +596,8 @@ __global__ void __launch_bounds__(CW_WARPS * 32, 4) k_c4_warp_credit(PivotArgs a
         const Table T{S.keys, S.cnts, min((uint32_t)CW_SLOTS, Table::size_for((int)a.U_wt[u]))};
         const uint32_t* const row = a.U_col + rb;
         const Deal deal{5, 1};  // 32 rows at a time
-        auto run = [&](uint32_t v, const uint32_t** p, int* len) {
+        auto run = [&](uint32_t fv, const uint32_t** p, int* len) {
+            const uint32_t v = vid(fv);
             const long long b = a.U_off[v];
             *p = a.U_col + b;
             *len = (int)(a.U_off[v + 1] - b);

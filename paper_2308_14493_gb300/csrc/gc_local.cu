@@ -44,6 +44,7 @@
 // directly (in both graphs: both flags implied).
 #include "gc_internal.cuh"
 #include "gc_kernels.cuh"
+#include "gc_walk.cuh"
 
 namespace gcx {
 
@@ -113,16 +114,28 @@ __device__ __forceinline__ long long locate(const long long* __restrict__ pre, l
     return lo;
 }
 
+// The same by a whole warp (every lane calls it with the same arguments): 32
+// boundaries a step, so a million tasks take four dependent loads instead of
+// twenty.
+__device__ __forceinline__ long long locate_all(const long long* __restrict__ pre, long long n, long long t,
+                                                long long lo = 0) {
+    long long hi = n;
+    while (hi - lo > 1) {
+        const long long step = (hi - lo + 31) >> 5;
+        const long long k = lo + step * ((threadIdx.x & 31) + 1);
+        lo += step * __popc(__ballot_sync(FULL, k < hi && pre[k] <= t));
+        hi = min(hi, lo + step);
+    }
+    return lo;
+}
+
 // The same for the 32 consecutive t of a warp (t non-decreasing over the
 // lanes; every lane calls it): one search for lane 0, then each lane steps
 // forward over a few task boundaries, or searches the rest when there are
 // more (runs of empty tasks).
 __device__ __forceinline__ long long locate_warp(const long long* __restrict__ pre, long long n, long long t,
                                                  bool valid) {
-    const long long t0 = __shfl_sync(FULL, t, 0);
-    long long e = 0;
-    if ((threadIdx.x & 31) == 0) e = locate(pre, n, t0);
-    e = __shfl_sync(FULL, e, 0);
+    long long e = locate_all(pre, n, __shfl_sync(FULL, t, 0));
     if (valid) {
         for (int k = 0; e + 1 < n && pre[e + 1] <= t; k++) {
             if (k == 4) {
@@ -173,11 +186,26 @@ __device__ __forceinline__ Pair pair_at(const Ctl* c, const int32_t* __restrict_
 
 // For the 4-cycles through a pair, the neighbours w of one endpoint v are
 // walked and each N(w) is intersected with the other endpoint's row; the
-// endpoint with the cheaper walk was chosen by k_loc_pair_cost (walk[i] = 1:
-// v = a).
-__device__ __forceinline__ void c4_orient(const Pair& p, int walk_a, uint32_t* v, uint32_t* u) {
-    *v = walk_a ? p.a : p.b;
-    *u = walk_a ? p.b : p.a;
+// endpoint with the cheaper walk was chosen by k_loc_pair_cost (bit 0 of
+// walk[i]: v = a).  A pair with enough work for it has u's row staged as a
+// bitmap of hashed ids in shared memory (WALK_STAGED), and N(w) is then walked
+// against it up to C4_WALK_MAX times the length of u's row; beyond, u's row is
+// walked and each entry searched in N(w).  Other pairs walk the shorter row.
+constexpr int WALK_STAGED = 2;
+constexpr int C4_WALK_MAX = 32;   // a bitmap test costs about 1 / 32 of a search in global memory
+constexpr int C4_SEARCH = 8;      // probes that a search counts for when work is dealt out
+constexpr int LC4_ROW_MIN = 64;   // rows shorter than this are searched, not staged
+__device__ __forceinline__ void c4_orient(const Pair& p, int walk, uint32_t* v, uint32_t* u) {
+    *v = (walk & 1) ? p.a : p.b;
+    *u = (walk & 1) ? p.b : p.a;
+}
+__device__ __forceinline__ unsigned long long c4_work(int rw, int ru) {
+    return (unsigned long long)min((long long)rw, (long long)C4_WALK_MAX * ru);
+}
+// probes of one task
+__device__ __forceinline__ int c4_cost(int rw, int ru, bool staged) {
+    if (!staged) return min(rw, ru);
+    return (long long)rw <= (long long)C4_WALK_MAX * ru ? rw : C4_SEARCH * ru;
 }
 
 __device__ __forceinline__ void acc_warp(Ctl* c, int slot, unsigned long long x) {
@@ -351,31 +379,61 @@ __global__ void k_loc_pair_cost(const Ctl* c, LocalView V, const int32_t* __rest
                                 const int32_t* __restrict__ dstD, int32_t* __restrict__ pcost,
                                 int32_t* __restrict__ ccnt, int32_t* __restrict__ walk) {
     pdl_enter();
-    // a warp per pair slot: the 4-cycle probes of walking either endpoint,
-    // sum over its neighbours w of min(|N(w)|, |other row|)
+    // the 4-cycle work of walking either endpoint, sum over its neighbours w
+    // of c4_work: a warp per pair slot, or a block when the rows are long (one
+    // hub of 10,000 neighbours took its warp 85 us)
+    __shared__ unsigned long long s_ca, s_cb;
     const long long np = c->l_len[1];
     const int lane = threadIdx.x & 31;
     const long long warp = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5;
     const long long nwarps = ((long long)gridDim.x * blockDim.x) >> 5;
+    auto put = [&](long long i, const Row& ra, const Row& rb, unsigned long long ca, unsigned long long cb) {
+        const int wa = ca < cb || (ca == cb && ra.len >= rb.len);
+        const int lu = wa ? rb.len : ra.len;
+        const bool staged = lu >= LC4_ROW_MIN && min(ca, cb) >= 4ull * (unsigned long long)lu;
+        pcost[i] = min(ra.len, rb.len);
+        ccnt[i] = wa ? ra.len : rb.len;
+        walk[i] = wa | (staged ? WALK_STAGED : 0);
+    };
+    auto sums = [&](const Row& ra, const Row& rb, int first, int step, unsigned long long& ca,
+                    unsigned long long& cb) {
+        ca = cb = 0;
+#pragma unroll 4
+        for (int j = first; j < ra.len; j += step) ca += c4_work(V.row(vid(ra.p[j])).len, rb.len);
+#pragma unroll 4
+        for (int j = first; j < rb.len; j += step) cb += c4_work(V.row(vid(rb.p[j])).len, ra.len);
+        ca = warp_sum_u64(ca);
+        cb = warp_sum_u64(cb);
+    };
+    constexpr int LONG_PAIR = 512;
     for (long long i = warp; i < np; i += nwarps) {
         const Pair p = pair_at(c, srcA, dstA, srcD, dstD, i);
-        int k = 0, m = 0, wa = 0;
-        if (p.a < p.b) {
-            const Row ra = V.urow(p.a), rb = V.urow(p.b);
-            unsigned long long ca = 0, cb = 0;
-            for (int j = lane; j < ra.len; j += 32) ca += (unsigned long long)min(V.row(vid(ra.p[j])).len, rb.len);
-            for (int j = lane; j < rb.len; j += 32) cb += (unsigned long long)min(V.row(vid(rb.p[j])).len, ra.len);
-            ca = warp_sum_u64(ca);
-            cb = warp_sum_u64(cb);
-            wa = ca < cb || (ca == cb && ra.len >= rb.len);
-            k = min(ra.len, rb.len);
-            m = wa ? ra.len : rb.len;
+        if (p.a > p.b) {
+            if (lane == 0) pcost[i] = ccnt[i] = walk[i] = 0;
+            continue;
         }
+        const Row ra = V.urow(p.a), rb = V.urow(p.b);
+        if (ra.len + rb.len > LONG_PAIR) continue;
+        unsigned long long ca, cb;
+        sums(ra, rb, lane, 32, ca, cb);
+        if (lane == 0) put(i, ra, rb, ca, cb);
+    }
+    for (long long i = blockIdx.x; i < np; i += gridDim.x) {
+        const Pair p = pair_at(c, srcA, dstA, srcD, dstD, i);
+        if (p.a > p.b) continue;
+        const Row ra = V.urow(p.a), rb = V.urow(p.b);
+        if (ra.len + rb.len <= LONG_PAIR) continue;
+        if (threadIdx.x == 0) s_ca = s_cb = 0;
+        __syncthreads();
+        unsigned long long ca, cb;
+        sums(ra, rb, threadIdx.x, blockDim.x, ca, cb);
         if (lane == 0) {
-            pcost[i] = k;
-            ccnt[i] = m;
-            walk[i] = wa;
+            atomicAdd(&s_ca, ca);
+            atomicAdd(&s_cb, cb);
         }
+        __syncthreads();
+        if (threadIdx.x == 0) put(i, ra, rb, s_ca, s_cb);
+        __syncthreads();
     }
 }
 
@@ -550,26 +608,20 @@ __global__ void k_loc_c4_tasks(const Ctl* c, LocalView V, const int32_t* __restr
         const uint32_t e = V.urow(v).p[j];
         const uint32_t w = vid(e);
         int k = 0;
-        if (w != u && (e & p.x)) k = min(V.row(w).len, (int)(V.U_off[u + 1] - V.U_off[u]));
+        if (w != u && (e & p.x))
+            k = c4_cost(V.row(w).len, (int)(V.U_off[u + 1] - V.U_off[u]), (walk[i] & WALK_STAGED) != 0);
         tpair[tau] = (int32_t)i;
         tent[tau] = j;
         tcost[tau] = k;
     }
 }
 
-// Each block takes one contiguous range of the probes (numbered pair by
-// pair, then task by task).  Before walking it the block picks the pair with
-// the most probes in the range and puts the other endpoint u's union row
-// (entries with their flags) into a bucketed hash table in shared memory,
-// when that row has between LC4_ROW_MIN and LC4_ROW_MAX entries and the
-// range holds at least two probes of the pair per entry; the probes of that
-// pair that walk N(w) then look z up there instead of binary-searching u's
-// row in global memory.  Probes that walk u's row (N(w) the longer) search
-// N(w) as before.  4 slots to a bucket, linear probing over buckets, at most
-// 3/4 of the slots filled, so every lookup ends at an empty slot.
+// The table of k_loc_tri: an owner's union row (entries with their flags) in a
+// bucketed hash in shared memory, for rows of LC4_ROW_MIN to LC4_ROW_MAX
+// entries.  4 slots to a bucket, linear probing over buckets, at most 3/4 of
+// the slots filled, so every lookup ends at an empty slot.
 constexpr int LC4_BUCKETS = 4096;
 constexpr int LC4_ROW_MAX = 3 * LC4_BUCKETS;
-constexpr int LC4_ROW_MIN = 64;
 constexpr uint32_t LC4_EMPTY = 0xFFFFFFFFu;  // ids stay below 2^30 - 1
 constexpr size_t LC4_SMEM = (size_t)LC4_BUCKETS * sizeof(uint4);
 constexpr int LC4_THREADS = 512;
@@ -581,14 +633,15 @@ __device__ __forceinline__ long long lc4_chunk(long long range) {
     return c < 128 ? 128 : c > LC4_CHUNK ? LC4_CHUNK : c;
 }
 // Blocks that take part for tot probes: about one per LC4_BLOCK_PROBES, at
-// least half and at most all of the launched grid (eight waves).  More and
-// smaller ranges put more of the probes under a staged row, fewer and larger
-// ones pay fewer table builds: 8 waves won at 10,000 updates on c3 (6.7
-// against 7.2 ms), 4 at 1,000 (1.60 against 1.78 ms).
-constexpr long long LC4_BLOCK_PROBES = 65536;
-__device__ __forceinline__ long long lc4_blocks(long long tot) {
+// most all of the launched grid (eight waves), at least an eighth (a quarter
+// for the 4-cycles) of it.  Fewer blocks set up less, more even out better: a
+// 100-update batch of the 1.6M/30M graph took 108 / 140 us for its triangles /
+// 4-cycles at one and two waves, 126 / 149 at four; 10,000 updates 2.09 ms for
+// the triangles at 32,768 probes, 2.45 at 131,072.
+constexpr long long LC4_BLOCK_PROBES = 32768;
+__device__ __forceinline__ long long lc4_blocks(long long tot, int least) {
     const long long g = (long long)gridDim.x, want = tot / LC4_BLOCK_PROBES;
-    return want < g / 2 ? g / 2 : want > g ? g : want;
+    return want < g / least ? g / least : want > g ? g : want;
 }
 
 __device__ __forceinline__ uint32_t lc4_bucket(uint32_t z, int lgb) { return (z * 0x9E3779B1u) >> (32 - lgb); }
@@ -628,7 +681,38 @@ __device__ __forceinline__ int lc4_stage(uint4* tab, const Row& r) {
     return lgb;
 }
 
-__global__ void __launch_bounds__(LC4_THREADS, 3) k_loc_c4(Ctl* c, LocalView V, const int32_t* __restrict__ srcA,
+// 4-cycles through the changed pairs.  A block takes one contiguous range of
+// the probes (numbered pair by pair, then task by task) and goes through it
+// pair by pair; the warps take chunks of a pair's part of the range in turn.
+// For a staged pair, u's row is entered into a bitmap of hashed ids; a warp
+// looks up 32 tasks of its chunk at a time (a lane each) and walks their rows
+// N(w) as the wedges of a pivot are walked (walk_group).  The few entries that
+// pass the bitmap (about one in twenty, hits included) are queued per warp and
+// searched in u's row 32 at a time.  Tasks whose N(w) is far longer than u's
+// row search that row's entries in N(w).  Runs of pairs too small to stage are
+// walked together, a search per probe.  Which pairs are staged, and how their
+// tasks are numbered, does not depend on the block, so a task that a chunk or
+// block boundary cuts is split exactly.
+// (With an exact table of u's row, four slots to a 16-byte bucket, for the one
+// pair with most probes of a range and a warp per task, the 4-clique and
+// 4-cycle stage took 4.35 ms for a 10,000-update batch of the 1.6M/30M graph;
+// hubs above 12,288 entries were not staged, and 439 pairs of the 2.4M/5M graph
+// took 7.3 ms.  Now 3.2 and 1.8.  Listing long rows for the whole block to
+// walk together, or leaving each row to the warp that starts it, was slower
+// than cutting the probes exactly: 4.4 and 3.8 ms.)
+constexpr int LB_LG_MAX = 18;  // 32 KB: one bit in six set by a row of 50,000
+struct C4Hit {
+    uint32_t e;  // entry (w, z)
+    uint32_t w;
+};
+constexpr int LQ = 32 + 4 * 32;
+struct C4Warp {
+    WarpRuns runs;
+    C4Hit queue[LQ];
+};
+constexpr size_t LC4_C4_SMEM = ((size_t)1 << (LB_LG_MAX - 3)) + (size_t)(LC4_THREADS / 32) * sizeof(C4Warp);
+
+__global__ void __launch_bounds__(LC4_THREADS, 2) k_loc_c4(Ctl* c, LocalView V, const int32_t* __restrict__ srcA,
                                                 const int32_t* __restrict__ dstA, const int32_t* __restrict__ srcD,
                                                 const int32_t* __restrict__ dstD, const int32_t* __restrict__ walk,
                                                 const int32_t* __restrict__ tpair, const int32_t* __restrict__ tent,
@@ -636,115 +720,194 @@ __global__ void __launch_bounds__(LC4_THREADS, 3) k_loc_c4(Ctl* c, LocalView V, 
                                                 const long long* __restrict__ cpre) {
     pdl_enter();
     extern __shared__ uint4 tab[];
-    __shared__ unsigned long long s_best, s_chunk;
-    __shared__ long long s_pair[2];
+    uint32_t* const bloom = (uint32_t*)tab;
+    __shared__ unsigned long long s_chunk;
+    __shared__ long long s_task[2];
+    __shared__ int s_next;
     const long long n = c->l_len[3];
     const long long tot = n ? tpre[n] : 0;
-    const long long nb = lc4_blocks(tot);
+    const long long nb = lc4_blocks(tot, 4);
     if (blockIdx.x >= nb) return;
     const long long lo = tot * blockIdx.x / nb, hi = tot * (blockIdx.x + 1) / nb;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    C4Warp& S = ((C4Warp*)(bloom + (1 << (LB_LG_MAX - 5))))[warp];
     unsigned long long qa = 0, qb = 0;
     if (lo < hi) {
-        // the pair with the most probes in [lo, hi) whose u row can be staged
-        if (threadIdx.x == 0) {
-            s_best = 0;
-            s_chunk = (unsigned long long)lo;
-            s_pair[0] = tpair[locate(tpre, n, lo)];
-            s_pair[1] = tpair[locate(tpre, n, hi - 1)];
+        // the tasks of the first and of the last probe
+        if (threadIdx.x < 64) {
+            const long long e = locate_all(tpre, n, warp ? hi - 1 : lo);
+            if (lane == 0) s_task[warp] = e;
         }
         __syncthreads();
-        for (long long i = s_pair[0] + threadIdx.x; i <= s_pair[1]; i += blockDim.x) {
-            const long long ta = cpre[i], tb = cpre[i + 1];
-            if (ta >= tb) continue;
-            const long long cnt = min(hi, tpre[tb]) - max(lo, tpre[ta]);
-            const Pair p = pair_at(c, srcA, dstA, srcD, dstD, i);
-            const uint32_t u = walk[i] ? p.b : p.a;
-            const long long len = V.U_off[u + 1] - V.U_off[u];
-            if (len < LC4_ROW_MIN || len > LC4_ROW_MAX || cnt < 2 * len) continue;
-            atomicMax(&s_best, ((unsigned long long)min(cnt, 0xFFFFFFFFll) << 32) | (unsigned long long)i);
-        }
-        __syncthreads();
-        const unsigned long long best = s_best;
-        const long long sp = best ? (long long)(uint32_t)best : -1;
-        int lgb = 0;
-        if (sp >= 0) {
-            const Pair p = pair_at(c, srcA, dstA, srcD, dstD, sp);
-            lgb = lc4_stage(tab, V.urow(walk[sp] ? p.b : p.a));
-        }
-        // the warps take chunks of the block's range in turn (probe costs
-        // differ tenfold, so equal shares would leave warps idle) and walk
-        // each chunk task by task: the task's pair, rows and walked entry
-        // once, then its probes 32 at a time
-        const int lane = threadIdx.x & 31;
-        const long long chunk = lc4_chunk(hi - lo);
-        long long tau = 0;
-        if (lane == 0) tau = locate(tpre, n, lo);
-        tau = __shfl_sync(FULL, tau, 0);
-        for (long long s = 0, whi = 0;;) {
-            if (s >= whi) {
-                long long c0 = 0;
-                if (lane == 0) c0 = (long long)atomicAdd(&s_chunk, (unsigned long long)chunk);
-                c0 = __shfl_sync(FULL, c0, 0);
-                if (c0 >= hi) break;
-                s = c0;
-                whi = min(hi, c0 + chunk);
+        const long long tf = s_task[0];
+        const int last = tpair[s_task[1]];
+        for (int i = tpair[tf]; i <= last;) {
+            // a staged pair, or the run of others up to the next one
+            if (threadIdx.x == 0) s_next = min(last + 1, i + LC4_THREADS);
+            __syncthreads();
+            {
+                const int k = i + threadIdx.x;
+                if (k <= last && (walk[k] & WALK_STAGED)) atomicMin(&s_next, k);
             }
-            tau = next_task(tpre, n, s, tau);
-            const long long pe = tpre[tau + 1], pb = tpre[tau];
-            const int k0 = (int)(s - pb), k1 = (int)(min(whi, pe) - pb);
-            s = min(whi, pe);
-            const int pi = tpair[tau];
-            const Pair p = pair_at(c, srcA, dstA, srcD, dstD, pi);
-            uint32_t v, u;
-            c4_orient(p, walk[pi], &v, &u);
-            const uint32_t ev = V.urow(v).p[tent[tau]];
-            const uint32_t w = vid(ev), fvw = ev & AB, x = p.x;
-            // the cycle u-v-w-z-u is counted at its smallest changed pair of graph x
-            const unsigned long long kp = pkey(p.a, p.b);
-            if (!(fvw & x) || (fvw == x && pkey(v, w) < kp)) continue;
-            const Row ru = V.urow(u), rw = V.row(w);
-            unsigned q4 = 0;
-            const bool staged = pi == sp;
-            // with u's row staged, a task whose N(w) is longer (at most four
-            // times) still walks N(w) when the task lies wholly in this
-            // block's range: its probe range [k0, k1) of u's row maps to the
-            // proportional range of N(w), so the chunks that split the task
-            // split N(w) exactly.  A task that a block boundary cuts keeps
-            // walking u's row in both blocks, whichever pairs they stage.
-            const bool walk_w =
-                rw.len <= ru.len || (staged && pb >= lo && pe <= hi && rw.len <= 4 * ru.len);
-            if (walk_w) {
-                const int j0 = rw.len <= ru.len ? k0 : (int)((long long)k0 * rw.len / ru.len);
-                const int j1 = rw.len <= ru.len ? k1 : (int)((long long)k1 * rw.len / ru.len);
-                for (int k = j0 + lane; k < j1; k += 32) {
-                    const uint32_t z = vid(rw.p[k]), fwz = flags_at(rw, k);
-                    if (z == v || !(fwz & x)) continue;
-                    uint32_t fuz;
-                    if (staged) {
-                        const uint32_t e = lc4_find(tab, lgb, z);
-                        if (e == LC4_EMPTY) continue;
-                        fuz = e & AB;
-                    } else {
-                        const int q = row_find(ru, 0, z);
-                        if (q < 0) continue;
-                        fuz = flags_at(ru, q);
+            __syncthreads();
+            const bool staged = s_next == i;
+            const int i1 = staged ? i + 1 : s_next;
+            const long long c0 = cpre[i], c1 = cpre[i1], a = max(lo, tpre[c0]), b = min(hi, tpre[c1]);
+            if (threadIdx.x == 0) s_chunk = (unsigned long long)a;
+            const long long chunk = lc4_chunk(b - a);
+            long long tau = max(tf, c0), s = 0, whi = 0;
+            // the next chunk of the part, in s .. whi (false: none is left)
+            auto next_chunk = [&]() {
+                long long at = 0;
+                if (lane == 0) at = (long long)atomicAdd(&s_chunk, (unsigned long long)chunk);
+                at = __shfl_sync(FULL, at, 0);
+                s = at;
+                whi = min(b, at + chunk);
+                return at < b;
+            };
+            if (a < b && staged) {
+                const Pair p = pair_at(c, srcA, dstA, srcD, dstD, i);
+                uint32_t v, u;
+                c4_orient(p, walk[i], &v, &u);
+                const Row ru = V.urow(u);
+                const uint32_t x = p.x;
+                const unsigned long long kp = pkey(p.a, p.b);
+                int lg = 12;
+                while (lg < LB_LG_MAX && (1ll << lg) < 16ll * ru.len) lg++;
+                for (int k = threadIdx.x; k < (1 << (lg - 7)); k += LC4_THREADS) tab[k] = make_uint4(0, 0, 0, 0);
+                __syncthreads();
+                for (int k = threadIdx.x; k < ru.len; k += LC4_THREADS) {
+                    const uint32_t h = (vid(ru.p[k]) * 0x9E3779B1u) >> (32 - lg);
+                    atomicOr(&bloom[h >> 5], 1u << (h & 31));
+                }
+                __syncthreads();
+                unsigned q4 = 0;
+                int nq = 0;
+                // search cnt queued entries, from queue[nq] on, in u's row
+                auto drain = [&](int cnt) {
+                    if (lane < cnt) {
+                        const C4Hit h = S.queue[nq + lane];
+                        const uint32_t z = vid(h.e), fwz = in_x(V.visited, h.w) ? h.e & AB : AB;
+                        if ((fwz & x) && !(fwz == x && pkey(h.w, z) < kp)) {
+                            const int q = row_find(ru, 0, z);
+                            if (q >= 0) {
+                                const uint32_t fuz = flags_at(ru, q);
+                                if ((fuz & x) && !(fuz == x && pkey(u, z) < kp)) q4++;
+                            }
+                        }
                     }
-                    if (!(fuz & x) || (fwz == x && pkey(w, z) < kp) || (fuz == x && pkey(u, z) < kp)) continue;
-                    q4++;
+                };
+                // a task's edge (v, w) is in graph x and holds no smaller pair
+                // (the cycle u-v-w-z-u is counted at its smallest changed pair)
+                auto open = [&](uint32_t ev) {
+                    const uint32_t w = vid(ev), fvw = ev & AB;
+                    return w != u && (fvw & x) && !(fvw == x && pkey(v, w) < kp);
+                };
+                const uint32_t* const row = V.urow(v).p;
+                while (next_chunk()) {
+                    tau = next_task(tpre, n, s, tau);
+                    for (bool more = true; more; tau += 32) {
+                        const long long t = tau + lane;
+                        int k0 = 0, k1 = 0;
+                        uint32_t ev = 0;
+                        Row rw{};
+                        if (t < c1) {
+                            const long long pb = tpre[t], pe = tpre[t + 1];
+                            if (pb < whi && pe > s) {
+                                ev = row[t - c0];
+                                if (open(ev)) {
+                                    k0 = (int)(max(s, pb) - pb);
+                                    k1 = (int)(min(whi, pe) - pb);
+                                    rw = V.row(vid(ev));
+                                }
+                            }
+                            more = pe < whi;
+                        } else {
+                            more = false;
+                        }
+                        more = __all_sync(FULL, more);
+                        const bool far = k1 > k0 && (long long)rw.len > (long long)C4_WALK_MAX * ru.len;
+                        walk_group<false>(
+                            rw.p + k0, far ? 0 : k1 - k0, ev, 0, S.runs,
+                            [&](const auto& q, const auto& e, const auto& f, auto&) {
+#pragma unroll
+                                for (int r = 0; r < PV_UNROLL; r++) {
+                                    const uint32_t z = vid(e[r]), h = (z * 0x9E3779B1u) >> (32 - lg);
+                                    const bool pass = q[r] && ((bloom[h >> 5] >> (h & 31)) & 1u) && z != v;
+                                    const unsigned m = __ballot_sync(FULL, pass);
+                                    if (pass) S.queue[nq + __popc(m & lanemask_lt())] = C4Hit{e[r], vid(f[r])};
+                                    nq += __popc(m);
+                                }
+                                __syncwarp();
+                                while (nq >= 32) {
+                                    nq -= 32;
+                                    drain(32);
+                                }
+                                __syncwarp();
+                            },
+                            [](unsigned long long, uint32_t, int) {});
+                        // far longer rows: u's row searched in N(w)
+                        for (unsigned m = __ballot_sync(FULL, far); m; m &= m - 1) {
+                            const int src = __ffs(m) - 1;
+                            const uint32_t w = vid(__shfl_sync(FULL, ev, src));
+                            const int j0 = __shfl_sync(FULL, k0, src) / C4_SEARCH;
+                            const int j1 = __shfl_sync(FULL, k1, src) / C4_SEARCH;
+                            const Row rf = V.row(w);
+                            for (int k = j0 + lane; k < j1; k += 32) {
+                                const uint32_t z = vid(ru.p[k]), fuz = flags_at(ru, k);
+                                if (z == v || !(fuz & x)) continue;
+                                const int q = row_find(rf, 0, z);
+                                if (q < 0) continue;
+                                const uint32_t fwz = flags_at(rf, q);
+                                if (!(fwz & x) || (fwz == x && pkey(w, z) < kp) || (fuz == x && pkey(u, z) < kp))
+                                    continue;
+                                q4++;
+                            }
+                        }
+                    }
+                    tau -= 32;  // (the last group may hold the next chunk's first task)
                 }
-            } else {
-                for (int k = k0 + lane; k < k1; k += 32) {
-                    const uint32_t z = vid(ru.p[k]), fuz = flags_at(ru, k);
-                    if (z == v || !(fuz & x)) continue;
-                    const int q = row_find(rw, 0, z);
-                    if (q < 0) continue;
-                    const uint32_t fwz = flags_at(rw, q);
-                    if (!(fwz & x) || (fwz == x && pkey(w, z) < kp) || (fuz == x && pkey(u, z) < kp)) continue;
-                    q4++;
+                const int left = nq;
+                nq = 0;
+                drain(left);
+                if (x == FLAG_A) qa += q4;
+                else qb += q4;
+            } else if (a < b) {
+                __syncthreads();
+                for (;;) {
+                    if (s >= whi && !next_chunk()) break;
+                    tau = next_task(tpre, n, s, tau);
+                    const long long pe = tpre[tau + 1], pb = tpre[tau];
+                    const int k0 = (int)(s - pb), k1 = (int)(min(whi, pe) - pb);
+                    s = min(whi, pe);
+                    const int pi = tpair[tau];
+                    const Pair p = pair_at(c, srcA, dstA, srcD, dstD, pi);
+                    uint32_t v, u;
+                    c4_orient(p, walk[pi], &v, &u);
+                    const uint32_t ev = V.urow(v).p[tent[tau]];
+                    const uint32_t w = vid(ev), fvw = ev & AB, x = p.x;
+                    const unsigned long long kp = pkey(p.a, p.b);
+                    if (!(fvw & x) || (fvw == x && pkey(v, w) < kp)) continue;
+                    const Row ru = V.urow(u), rw = V.row(w);
+                    const bool walk_w = rw.len <= ru.len;  // the shorter row, searched in the other
+                    const Row rs = walk_w ? rw : ru, rl = walk_w ? ru : rw;
+                    unsigned q4 = 0;
+                    for (int k = k0 + lane; k < k1; k += 32) {
+                        const uint32_t z = vid(rs.p[k]), fs = flags_at(rs, k);
+                        if (z == v || !(fs & x)) continue;
+                        const int q = row_find(rl, 0, z);
+                        if (q < 0) continue;
+                        const uint32_t fl = flags_at(rl, q);
+                        const uint32_t fwz = walk_w ? fs : fl, fuz = walk_w ? fl : fs;
+                        if (!(fl & x) || (fwz == x && pkey(w, z) < kp) || (fuz == x && pkey(u, z) < kp)) continue;
+                        q4++;
+                    }
+                    if (x == FLAG_A) qa += q4;
+                    else qb += q4;
                 }
             }
-            if (x == FLAG_A) qa += q4;
-            else qb += q4;
+            i = i1;
+            __syncthreads();  // the bitmap and the counters serve the next pair
         }
     }
     acc_warp(c, 5, qa);
@@ -768,19 +931,27 @@ __global__ void __launch_bounds__(LC4_THREADS, 3) k_loc_tri(const Ctl* c, LocalV
     pdl_enter();
     extern __shared__ uint4 tab[];
     __shared__ int32_t s_cand[3];
+    __shared__ long long s_task;
     __shared__ unsigned long long s_chunk;
     const long long n = c->l_len[0];
     if (n == 0) return;
     const long long tot = pre[n];
-    const long long nb = lc4_blocks(tot);
+    const long long nb = lc4_blocks(tot, 8);
     if (blockIdx.x >= nb) return;
     const long long lo = tot * blockIdx.x / nb, hi = tot * (blockIdx.x + 1) / nb;
     if (lo >= hi) return;
-    if (threadIdx.x < 3) {
-        const long long t = threadIdx.x == 0 ? lo : threadIdx.x == 1 ? lo + (hi - lo) / 2 : hi - 1;
-        s_cand[threadIdx.x] = own[locate(pre, n, t)];
+    const int lane = threadIdx.x & 31;
+    if (threadIdx.x < 96) {
+        const int k = threadIdx.x >> 5;
+        const long long e0 = locate_all(pre, n, k == 0 ? lo : k == 1 ? lo + (hi - lo) / 2 : hi - 1);
+        if (lane == 0) {
+            s_cand[k] = own[e0];
+            if (k == 0) {
+                s_task = e0;
+                s_chunk = (unsigned long long)lo;
+            }
+        }
     }
-    if (threadIdx.x == 0) s_chunk = (unsigned long long)lo;
     __syncthreads();
     long long su = -1, best = 0;
     for (int j = 0; j < 3; j++) {
@@ -793,11 +964,8 @@ __global__ void __launch_bounds__(LC4_THREADS, 3) k_loc_tri(const Ctl* c, LocalV
     }
     int lgb = 0;
     if (su >= 0) lgb = lc4_stage(tab, V.urow((uint32_t)su));
-    const int lane = threadIdx.x & 31;
     const long long chunk = lc4_chunk(hi - lo);
-    long long e = 0;
-    if (lane == 0) e = locate(pre, n, lo);
-    e = __shfl_sync(FULL, e, 0);
+    long long e = s_task;
     for (long long s = 0, whi = 0;;) {
         if (s >= whi) {
             long long c0 = 0;
@@ -1136,10 +1304,10 @@ __global__ void k_finalize_local(Ctl* c, int commit) {
 static int g_loc_per_sm[2] = {0, 0};
 
 template <typename K>
-static int staged_per_sm(K kernel) {
-    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)LC4_SMEM);
+static int staged_per_sm(K kernel, size_t smem) {
+    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     int per_sm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, LC4_THREADS, LC4_SMEM) != cudaSuccess) {
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, LC4_THREADS, smem) != cudaSuccess) {
         cudaGetLastError();
         per_sm = 0;
     }
@@ -1147,8 +1315,8 @@ static int staged_per_sm(K kernel) {
 }
 
 void local_setup_attributes() {
-    g_loc_per_sm[0] = staged_per_sm(k_loc_tri);
-    g_loc_per_sm[1] = staged_per_sm(k_loc_c4);
+    g_loc_per_sm[0] = staged_per_sm(k_loc_tri, LC4_SMEM);
+    g_loc_per_sm[1] = staged_per_sm(k_loc_c4, LC4_C4_SMEM);
 }
 
 // kind 0: the triangle kernel, 1: the 4-cycle kernel
@@ -1207,7 +1375,7 @@ int enqueue_local(const LocalArgs& a, cudaStream_t s, int commit) {
                                       a.cost);
     nl += 2;
     nl += scan_i32_to_i64(a.cost, a.pre, &a.ctl->l_len[3], 0, a.bsum, sg, &a.ctl->l_tot[4], s);
-    pdl_launch(k_loc_c4, dim3(staged_grid(1, sms)), dim3(LC4_THREADS), LC4_SMEM, s, a.ctl, V, a.srcA, a.dstA, a.srcD,
+    pdl_launch(k_loc_c4, dim3(staged_grid(1, sms)), dim3(LC4_THREADS), LC4_C4_SMEM, s, a.ctl, V, a.srcA, a.dstA, a.srcD,
                a.dstD, a.walk, a.tpair, a.own, a.pre, a.cpre);
     nl++;
     pdl_launch(k_finalize_local, dim3(1), dim3(32), 0, s, a.ctl, commit);

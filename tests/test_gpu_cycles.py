@@ -117,3 +117,33 @@ def test_repeated_static_counts(gcb):
             for _ in range(5):
                 assert g.count_static() == og.F
             assert g.counts() == og.F
+
+
+@pytest.mark.parametrize("mid_degree,hub_degree", [(63, 5000), (64, 2048), (70, 3000), (150, 5000)])
+def test_local_pairs_between_mid_vertices_under_hubs(gcb, mid_degree, hub_degree):
+    """Edge-local 4-cycles where the staged rows have about 64 entries (the
+    shortest staged) and the walked rows are hubs on both sides of 32 times
+    their length (walked, or searched)."""
+    n, mids = 8000, 60
+    rng = np.random.default_rng(mid_degree + hub_degree)
+    keys = set(int(k) for k in gen.er_graph(n, 4000, 5))
+    for h in (0, 1):
+        for v in rng.choice(np.arange(2, n), hub_degree, replace=False):
+            keys.add((h << 32) | int(v))
+    for u in range(2, 2 + mids):
+        keys.add(u)  # (0, u): every mid vertex hangs on the first hub
+        for v in rng.choice(np.arange(100, n), mid_degree, replace=False):
+            keys.add((u << 32) | int(v))
+    keys = np.array(sorted(keys), dtype=np.uint64)
+    rp, col = gen.csr_from_keys(n, keys)
+    F0 = oracle.static_counts(rp, col)
+    have = set(int(k) for k in keys)
+    pairs = [(a, b) for a in range(2, 2 + mids) for b in range(a + 1, 2 + mids)]
+    rng.shuffle(pairs)
+    ins = np.array([p for p in pairs if ((p[0] << 32) | p[1]) not in have][:200], np.int32)
+    dels = gen.random_batch(n, keys, 0, 150, 9)[1]
+    r = oracle.fdgc_step(rp, col, ins, dels, F0)
+    with gcb.Graph(n, rp, col, local_max_pairs=100000) as g:
+        assert g.apply(ins, dels) == r["F"]
+        assert g.stats()["path"] == 1
+        assert g.apply(dels, ins) == F0
