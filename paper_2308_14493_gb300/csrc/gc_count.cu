@@ -853,71 +853,78 @@ __global__ void k_edge_terms(Ctl* c, const int32_t* __restrict__ wlist, const lo
     acc_add(c, 14, work);
 }
 
-// mode 0: batch (F += C_a - C_b unless the batch was rejected); 1: static
+// The closed forms and the results, by one warp (lane i < 6 holds graphlet i,
+// so the loads of one result are in flight together).
+// mode 0: committed batch, F += C_a - C_b (unless the batch was rejected);
+// mode 2: independent batch, the result is F + C_a - C_b and F stays; mode 1:
+// static count; mode 3: a committed batch whose pass covered every vertex, so
+// C_a and C_b are the whole graph's counts after and before it: F = C_a, and
+// C_b is the result of the batch before it (committed without a count of its
+// own); mode 4: two independent batches counted over every vertex (the twin
+// pass): C_a and C_b are the whole graph's counts with the first and with the
+// second batch applied; F stays
 __global__ void k_finalize(Ctl* c, int mode) {
     pdl_enter();
-    // fold the striped accumulators (one warp: lane i sums slot i's copies
-    // and slot i + 16's if any)
-    if (blockIdx.x == 0 && threadIdx.x < NACC) {
-        unsigned long long x = 0;
-        for (int k = 0; k < ACC_STRIPES; k++) x += c->accs[threadIdx.x][k];
-        c->acc[threadIdx.x] += x;
-    }
-    __syncwarp();
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
-    for (int g = 0; g < 2; g++) {
-        const unsigned long long* s = c->acc + 6 * g;
-        long long P = (long long)s[0], S = (long long)s[1], TT = (long long)(s[2] / 2), D = (long long)s[3],
-                  K = (long long)s[4], Q = (long long)s[5];
-        long long g6 = K;
-        long long g5 = D - 6 * K;
-        long long g3 = Q - g5 - 3 * K;
-        long long g4 = TT - 4 * g5 - 12 * K;
-        long long g2 = S - g4 - 2 * g5 - 4 * K;
-        long long g1 = P - 2 * g4 - 4 * g3 - 6 * g5 - 12 * K;
-        long long* C = g == 0 ? c->Ca : c->Cb;
-        long long* sm = g == 0 ? c->sa : c->sb;
-        C[0] = g1; C[1] = g2; C[2] = g3; C[3] = g4; C[4] = g5; C[5] = g6;
-        sm[0] = P; sm[1] = S; sm[2] = TT; sm[3] = D; sm[4] = K; sm[5] = Q;
-    }
-    // mode 0: committed batch, F += C_a - C_b; mode 2: independent batch,
-    // the result is F + C_a - C_b and F stays; mode 1: static count; mode 3:
-    // a committed batch whose pass covered every vertex, so C_a and C_b are
-    // the whole graph's counts after and before it: F = C_a, and C_b is the
-    // result of the batch before it (committed without a count of its own);
-    // mode 4: see below
+    __shared__ unsigned long long s_acc[32];
+    const int t = threadIdx.x;
+    if (blockIdx.x != 0 || t >= 32) return;
     const bool ok = c->err == 0 && c->active;
-    for (int i = 0; i < 6; i++) {
-        unsigned long long d = (unsigned long long)(c->Ca[i] - c->Cb[i]);
-        if (mode == 0 && ok) c->F[i] += d;
+    unsigned long long x = 0;  // fold the striped accumulators
+    if (t < NACC) {
+        x = c->acc[t];
+#pragma unroll
+        for (int k = 0; k < ACC_STRIPES; k++) x += c->accs[t][k];
+        c->acc[t] = x;
+    }
+    s_acc[t] = x;
+    const unsigned long long F = t < 6 ? c->F[t] : 0ull, F3 = t < 2 ? c->F3[t] : 0ull;
+    __syncwarp();
+    long long C[2] = {0, 0};
+    for (int g = 0; g < 2; g++) {
+        const unsigned long long* s = s_acc + 6 * g;
+        const long long P = (long long)s[0], S = (long long)s[1], TT = (long long)(s[2] / 2), D = (long long)s[3],
+                        K = (long long)s[4], Q = (long long)s[5];
+        const long long g6 = K;
+        const long long g5 = D - 6 * K;
+        const long long g3 = Q - g5 - 3 * K;
+        const long long g4 = TT - 4 * g5 - 12 * K;
+        const long long g2 = S - g4 - 2 * g5 - 4 * K;
+        const long long g1 = P - 2 * g4 - 4 * g3 - 6 * g5 - 12 * K;
+        C[g] = t == 0 ? g1 : t == 1 ? g2 : t == 2 ? g3 : t == 3 ? g4 : t == 4 ? g5 : g6;
+        if (t < 6) {
+            (g == 0 ? c->Ca : c->Cb)[t] = C[g];
+            (g == 0 ? c->sa : c->sb)[t] = t == 0 ? P : t == 1 ? S : t == 2 ? TT : t == 3 ? D : t == 4 ? K : Q;
+        }
+    }
+    if (t < 6) {
+        const unsigned long long d = (unsigned long long)(C[0] - C[1]);
+        unsigned long long f = F;
+        if (mode == 0 && ok) f = F + d;
         if (mode == 3 && ok) {
-            c->prev_out[i] = (unsigned long long)c->Cb[i];
-            c->F[i] = (unsigned long long)c->Ca[i];
+            c->prev_out[t] = (unsigned long long)C[1];
+            f = (unsigned long long)C[0];
         }
-        c->last_out[i] = mode == 2 ? c->F[i] + d : c->F[i];
-        // mode 4: two independent batches counted over every vertex (the
-        // twin pass): C_a and C_b are the whole graph's counts with the
-        // first and with the second batch applied; F stays
-        if (mode == 4) {
-            c->last_out[i] = (unsigned long long)c->Ca[i];
-            c->prev_out[i] = (unsigned long long)c->Cb[i];
-        }
+        if (f != F) c->F[t] = f;
+        c->last_out[t] = mode == 2 ? F + d : mode == 4 ? (unsigned long long)C[0] : f;
+        if (mode == 4) c->prev_out[t] = (unsigned long long)C[1];
     }
     // 3-vertex graphlets from the same sums: triangles = (sum t_e) / 3,
     // induced 2-paths = sum C(d, 2) - 3 triangles
-    for (int g = 0; g < 2; g++) {
-        long long* C3 = g == 0 ? c->C3a : c->C3b;
-        const unsigned long long t3 = c->acc[16 + g], w2 = c->acc[18 + g];
-        C3[0] = (long long)(w2 - t3);
-        C3[1] = (long long)(t3 / 3);
+    if (t < 2) {
+        long long C3[2];
+        for (int g = 0; g < 2; g++) {
+            const unsigned long long t3 = s_acc[16 + g], w2 = s_acc[18 + g];
+            C3[g] = t == 0 ? (long long)(w2 - t3) : (long long)(t3 / 3);
+            (g == 0 ? c->C3a : c->C3b)[t] = C3[g];
+        }
+        const unsigned long long d = (unsigned long long)(C3[0] - C3[1]);
+        unsigned long long f = F3;
+        if (mode == 0 && ok) f = F3 + d;
+        if (mode == 3 && ok) f = (unsigned long long)C3[0];
+        if (f != F3) c->F3[t] = f;
+        c->last_out3[t] = mode == 2 ? F3 + d : f;
     }
-    for (int i = 0; i < 2; i++) {
-        unsigned long long d = (unsigned long long)(c->C3a[i] - c->C3b[i]);
-        if (mode == 0 && ok) c->F3[i] += d;
-        if (mode == 3 && ok) c->F3[i] = (unsigned long long)c->C3a[i];
-        c->last_out3[i] = mode == 2 ? c->F3[i] + d : c->F3[i];
-    }
-    c->ts[6] = global_ns();
+    if (t == 0) c->ts[6] = global_ns();
 }
 
 }  // namespace gcx

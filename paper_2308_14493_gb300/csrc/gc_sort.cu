@@ -33,44 +33,35 @@ __global__ void __launch_bounds__(RS_BLOCK) k_rs_hist(const uint64_t* __restrict
     chunk_of(*d_count, beg, end);
     for (long long i = beg + threadIdx.x; i < end; i += RS_BLOCK) atomicAdd(&h[(keys[i] >> shift) & 255], 1u);
     __syncthreads();
-    hist[(size_t)threadIdx.x * gridDim.x + blockIdx.x] = h[threadIdx.x];
+    hist[(size_t)blockIdx.x * 256 + threadIdx.x] = h[threadIdx.x];
 }
 
-// In-place exclusive scan of a[0..len) by one block of 1024 threads: each
-// thread sums a contiguous slice, the 1024 slice sums are scanned with warp
-// shuffles (two levels), then each thread rewrites its slice.
-__global__ void __launch_bounds__(1024) k_scan_u32_one_block(uint32_t* a, int len) {
-    pdl_enter();
-    __shared__ uint32_t wsum[32];
-    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-    const int per = (len + 1023) / 1024;
-    const int beg = t * per, end = min(beg + per, len);
-    uint32_t s = 0;
-    for (int i = beg; i < end; i++) s += a[i];
-    uint32_t x = s;  // inclusive scan within the warp
+// Where this block's keys of each digit go: the keys of smaller digits in all
+// blocks, then those of the digit in earlier blocks.  hist holds a row of 256
+// counts per block; thread d sums column d (coalesced across the block), so no
+// scan kernel stands between the histogram and the scatter (one block scanning
+// 256 x 304 counts took 107 us a pass; reading them costs each block a few us).
+__device__ __forceinline__ uint32_t digit_base(const uint32_t* __restrict__ hist) {
+    __shared__ uint32_t wsum[RS_WARPS];
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5, me = blockIdx.x, G = gridDim.x;
+    uint32_t before = 0, all = 0;
+#pragma unroll 8
+    for (int b = 0; b < G; b++) {
+        const uint32_t x = hist[(size_t)b * 256 + t];
+        all += x;
+        before += b < me ? x : 0u;
+    }
+    uint32_t y = all;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t y = __shfl_up_sync(FULL, x, o);
-        if (lane >= o) x += y;
+        const uint32_t z = __shfl_up_sync(FULL, y, o);
+        if (lane >= o) y += z;
     }
-    if (lane == 31) wsum[warp] = x;
+    if (lane == 31) wsum[warp] = y;
     __syncthreads();
-    if (warp == 0) {
-        uint32_t w = wsum[lane];
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const uint32_t y = __shfl_up_sync(FULL, w, o);
-            if (lane >= o) w += y;
-        }
-        wsum[lane] = w;
-    }
-    __syncthreads();
-    uint32_t run = x - s + (warp > 0 ? wsum[warp - 1] : 0u);
-    for (int i = beg; i < end; i++) {
-        const uint32_t v = a[i];
-        a[i] = run;
-        run += v;
-    }
+    uint32_t w = 0;
+    for (int k = 0; k < warp; k++) w += wsum[k];
+    return w + y - all + before;
 }
 
 // Stable scatter: each tile of RS_BLOCK keys is ranked within warps with
@@ -78,12 +69,12 @@ __global__ void __launch_bounds__(1024) k_scan_u32_one_block(uint32_t* a, int le
 // per-digit base carries the order across tiles.
 __global__ void __launch_bounds__(RS_BLOCK) k_rs_scatter(const uint64_t* __restrict__ in, uint64_t* __restrict__ out,
                                                         const long long* d_count, int shift,
-                                                        const uint32_t* __restrict__ offs) {
+                                                        const uint32_t* __restrict__ hist) {
     pdl_enter();
     __shared__ uint32_t base[256];
     __shared__ uint32_t wcnt[RS_WARPS][256];
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-    base[t] = offs[(size_t)t * gridDim.x + blockIdx.x];
+    base[t] = digit_base(hist);
     long long beg, end;
     chunk_of(*d_count, beg, end);
     for (long long tile = beg; tile < end; tile += RS_BLOCK) {
@@ -161,15 +152,6 @@ __global__ void __launch_bounds__(SC_BLOCK) k_scan_partials(const int32_t* __res
     if (threadIdx.x == SC_BLOCK - 1) bsum[blockIdx.x] = s;
 }
 
-__global__ void __launch_bounds__(1024) k_scan_top(long long* bsum, int G) {
-    pdl_enter();
-    __shared__ long long sh[32];
-    // G <= 1024
-    long long x = threadIdx.x < G ? bsum[threadIdx.x] : 0;
-    long long inc = block_incl_scan_i64(x, sh);
-    if (threadIdx.x < G) bsum[threadIdx.x] = inc - x;
-}
-
 __global__ void __launch_bounds__(SC_BLOCK) k_scan_apply(const int32_t* __restrict__ in, long long* __restrict__ out,
                                                         const long long* d_len, long long host_len,
                                                         const long long* __restrict__ bsum, long long* total_out) {
@@ -178,7 +160,15 @@ __global__ void __launch_bounds__(SC_BLOCK) k_scan_apply(const int32_t* __restri
     long long n = d_len ? *d_len : host_len;
     long long beg, end;
     chunk_of(n, beg, end);
-    long long run = bsum[blockIdx.x];
+    // the chunks before this one (at most 1,024 sums: two loads a thread, in
+    // place of a kernel that scans them)
+    __shared__ long long s_run;
+    long long before = 0;
+    for (int b = threadIdx.x; b < (int)blockIdx.x; b += SC_BLOCK) before += bsum[b];
+    before = block_incl_scan_i64(before, sh);
+    if (threadIdx.x == SC_BLOCK - 1) s_run = before;
+    __syncthreads();
+    long long run = s_run;
     for (long long tile = beg; tile < end; tile += SC_BLOCK) {
         long long i = tile + threadIdx.x;
         long long x = i < end ? in[i] : 0;
@@ -212,13 +202,12 @@ int radix_grid(long long max_count, int sms) {
 int radix_sort_u64(uint64_t* keys, uint64_t* tmp, const long long* d_count, long long max_count, int bits,
                    uint32_t* hist, int grid, cudaStream_t s) {
     int passes = (bits + 7) / 8;
-    int launches = 3 * passes;
+    int launches = 2 * passes;
     uint64_t* a = keys;
     uint64_t* b = tmp;
     for (int p = 0; p < passes; p++) {
         int shift = 8 * p;
         pdl_launch(k_rs_hist, dim3(grid), dim3(RS_BLOCK), 0, s, a, d_count, shift, hist);
-        pdl_launch(k_scan_u32_one_block, dim3(1), dim3(1024), 0, s, hist, 256 * grid);
         pdl_launch(k_rs_scatter, dim3(grid), dim3(RS_BLOCK), 0, s, a, b, d_count, shift, hist);
         uint64_t* t = a;
         a = b;
@@ -245,9 +234,8 @@ int scan_grid(long long max_len, int sms) {
 int scan_i32_to_i64(const int32_t* in, long long* out, const long long* d_len, long long host_len, long long* bsum,
                     int grid, long long* total_out, cudaStream_t s) {
     pdl_launch(k_scan_partials, dim3(grid), dim3(SC_BLOCK), 0, s, in, d_len, host_len, bsum);
-    pdl_launch(k_scan_top, dim3(1), dim3(1024), 0, s, bsum, grid);
     pdl_launch(k_scan_apply, dim3(grid), dim3(SC_BLOCK), 0, s, in, out, d_len, host_len, bsum, total_out);
-    return 3;
+    return 2;
 }
 
 }  // namespace gcx
