@@ -588,7 +588,6 @@ static size_t carve_c4(const gc_graph* g, C4Bufs* b) {
     o.head = (C4Head*)take(sizeof(C4Head));
     o.chunk = (C4Chunk*)take(sizeof(C4Chunk) * (size_t)m.nchmax);
     o.gmax = (int32_t*)take(4 * (size_t)m.ngran);
-    o.sorted = (int32_t*)take(4 * (size_t)n);
     o.list = (uint32_t*)take(4 * (size_t)m.ctas * C4_LIST);
     o.lcap = C4_LIST;
     o.run = (unsigned long long*)take(8 * (size_t)m.group * (size_t)n);

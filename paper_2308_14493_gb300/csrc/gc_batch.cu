@@ -231,7 +231,7 @@ __global__ void k_batch_clear_segments(const int32_t* __restrict__ src, const lo
 // by a block scan, segments written, and the endpoints put on the region list
 // (ascending).  The kernels above take about 27 launches for it, each a few
 // microseconds of dependent latency whatever its size: 55 us for 1,000 pairs
-// on a 7,000-vertex graph, SMALL_NOW here.  For the edge-local form the block
+// on a 7,000-vertex graph, 27 here.  For the edge-local form the block
 // also lays out the union rows: the offsets of the endpoints, in id order
 // (only U_off[u] and U_off[u + 1] of an endpoint u are read there), in place
 // of a scan over all vertices.

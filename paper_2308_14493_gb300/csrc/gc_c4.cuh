@@ -54,7 +54,6 @@ struct C4Bufs {
     C4Head* head;               // 1
     C4Chunk* chunk;             // nchmax
     int32_t* gmax;              // ngran
-    int32_t* sorted;            // n: the pivots by falling wedge bound
     unsigned long long* run;    // group * n packed runs (start << 28 | length)
     uint32_t* list;             // ctas * lcap
     long long lcap;
@@ -66,7 +65,7 @@ enum { C4_COUNT = 0, C4_VERTEX = 1, C4_EDGE = 2 };
 
 struct PivotArgs {
     Ctl* ctl;
-    const int32_t* pivots;      // BIN_C4_DENSE
+    const int32_t* pivots;      // BIN_C4_DENSE, by falling wedge bound
     const long long* U_off;
     const uint32_t* U_col;
     const int32_t* U_split;
@@ -78,9 +77,10 @@ struct PivotArgs {
     unsigned long long* credit;  // C4_VERTEX: per vertex, C4_EDGE: per entry (added to)
 };
 
-// The hash-table tiers (the small one on stream s, the others on s2), then
-// plan, run bounds and pivot kernels (bins: the work lists, NBINS * n); all
-// return the launches made.
+// Plan and run bounds of the pivots (needs k_wedge_bound's sums; not the bins);
+// the hash-table tiers (the small one on stream s, the others on s2) and the
+// pivot kernel (bins: the work lists, NBINS * n).  All return the launches made.
+int enqueue_c4_plan(const PivotArgs& a, const C4Geom& g, cudaStream_t s);
 int enqueue_c4_tables(const PivotArgs& a, int mode, const int32_t* bins, int sms, cudaStream_t s, cudaStream_t s2);
 // (the credits of the pivots below the tables: C4_VERTEX and C4_EDGE only)
 int enqueue_c4_warp_credit(const PivotArgs& a, int mode, const int32_t* bins, int sms, cudaStream_t s);

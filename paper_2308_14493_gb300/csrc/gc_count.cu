@@ -52,6 +52,7 @@ __global__ void k_reset_count(Ctl* c) {
     for (int i = t; i < NACC * ACC_STRIPES; i += blockDim.x) (&c->accs[0][0])[i] = 0;
     if (t < NWORK) c->work[t] = 0;
     if (t < NBINS) c->nbin[t] = 0;
+    for (int i = t; i < 128; i += blockDim.x) c->c4_hist[i] = c->c4_cur[i] = 0;
     if (t == 0) {
         c->maxdeg = 0;
         c->c4_wt = c->c4_wmax = 0;
@@ -98,17 +99,35 @@ __device__ __forceinline__ int find_seg(const int* pre, int k, int t) {
 
 // ---- binning ---------------------------------------------------------------
 
+// Tier of a 4-cycle pivot with wedge bound wt.
+__device__ __forceinline__ int c4_bin(const Tuning& t, long long wt) {
+    return wt <= t.c4_reg_max                         ? BIN_C4_REG
+           : wt <= t.c4_warp_max                      ? BIN_C4_WARP
+           : wt <= min(t.c4_block_max, C4B_SMALL_MAX) ? BIN_C4_BSMALL
+           : wt <= t.c4_block_max                     ? BIN_C4_BLOCK
+           : wt <= t.c4_cta_max                       ? BIN_C4_BIG
+                                                      : BIN_C4_DENSE;
+}
+// Bucket of a wedge bound, two per octave, the largest bounds first.
+__device__ __forceinline__ int wedge_bucket(long long w) {
+    const int lg = 63 - __clzll(w | 1);
+    return 127 - (2 * lg + (lg > 0 ? (int)((w >> (lg - 1)) & 1) : 0));
+}
+
 // Wedge bound of every 4-cycle pivot: w~(u) = sum of the union-graph degrees
 // of its lower neighbours.  A warp per vertex (hubs with tens of thousands
-// of lower neighbours spread over the grid like everyone else).
-__global__ void k_wedge_bound(const Ctl* c, const int32_t* __restrict__ wlist, const long long* __restrict__ U_off,
+// of lower neighbours spread over the grid like everyone else).  The sums over
+// the largest tier, which plan its chunks, are made here, so that the plan
+// need not wait for the bins.
+__global__ void k_wedge_bound(Ctl* c, const int32_t* __restrict__ wlist, const long long* __restrict__ U_off,
                               const uint32_t* __restrict__ U_col, const int32_t* __restrict__ U_split,
-                              long long* __restrict__ U_wt) {
+                              long long* __restrict__ U_wt, Tuning t) {
     pdl_enter();
     const int nW = c->nW;
     const int lane = threadIdx.x & 31;
     const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int nwarps = (gridDim.x * blockDim.x) >> 5;
+    unsigned long long wsum = 0, wmax = 0;  // of the pivots for shared memory
     for (int i = warp; i < nW; i += nwarps) {
         const int32_t u = wlist[i];
         const int sp = U_split[u];
@@ -123,7 +142,18 @@ __global__ void k_wedge_bound(const Ctl* c, const int32_t* __restrict__ wlist, c
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(FULL, part, o);
         }
-        if (lane == 0) U_wt[u] = part;
+        if (lane == 0) {
+            U_wt[u] = part;
+            if (sp >= 2 && c4_bin(t, part) == BIN_C4_DENSE) {
+                wsum += (unsigned long long)part;
+                wmax = max(wmax, (unsigned long long)part);
+                atomicAdd(&c->c4_hist[wedge_bucket(part)], 1u);
+            }
+        }
+    }
+    if (lane == 0 && wsum) {
+        atomicAdd(&c->c4_wt, wsum);
+        atomicMax(&c->c4_wmax, wmax);
     }
 }
 
@@ -137,10 +167,9 @@ __global__ void k_bin(Ctl* c, const int32_t* __restrict__ wlist, const long long
     const long long stride = (long long)gridDim.x * blockDim.x;
     const long long nW_r = ((long long)nW + 31) & ~31ll;
     int dmax = 0;
-    unsigned long long wsum = 0, wmax = 0;  // of the pivots for shared memory
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < nW_r; i += stride) {
         const bool valid = i < nW;
-        int tb = -1, cb = -1;
+        int tb = -1, cb = -1, bk = -1;
         const int32_t u = valid ? wlist[i] : 0;
         if (valid) {
             const long long rb = U_off[u], re = U_off[u + 1];
@@ -154,16 +183,8 @@ __global__ void k_bin(Ctl* c, const int32_t* __restrict__ wlist, const long long
                                             : BIN_TRI_MERGE;
             if (split >= 2) {
                 const long long wt = U_wt[u];
-                cb = wt <= t.c4_reg_max                         ? BIN_C4_REG
-                     : wt <= t.c4_warp_max                      ? BIN_C4_WARP
-                     : wt <= min(t.c4_block_max, C4B_SMALL_MAX) ? BIN_C4_BSMALL
-                     : wt <= t.c4_block_max                     ? BIN_C4_BLOCK
-                     : wt <= t.c4_cta_max                       ? BIN_C4_BIG
-                                                                : BIN_C4_DENSE;
-                if (cb == BIN_C4_DENSE) {
-                    wsum += (unsigned long long)wt;
-                    wmax = max(wmax, (unsigned long long)wt);
-                }
+                cb = c4_bin(t, wt);
+                if (cb == BIN_C4_DENSE) bk = wedge_bucket(wt);
             }
         }
 #pragma unroll 1
@@ -174,7 +195,30 @@ __global__ void k_bin(Ctl* c, const int32_t* __restrict__ wlist, const long long
                 int leader = __ffs(m) - 1, base = 0;
                 if (lane == leader) base = atomicAdd(&c->nbin[b], __popc(m));
                 base = __shfl_sync(FULL, base, leader);
-                if (mine) bins[(size_t)b * n + base + __popc(m & lanemask_lt())] = u;
+                if (b == BIN_C4_DENSE) {  // by falling wedge bound: behind the buckets before
+                    unsigned before[4], run = 0;
+#pragma unroll
+                    for (int q = 0; q < 4; q++) {
+                        const unsigned x = c->c4_hist[32 * q + lane];
+                        unsigned y = x;
+#pragma unroll
+                        for (int o = 1; o < 32; o <<= 1) {
+                            const unsigned z = __shfl_up_sync(FULL, y, o);
+                            if (lane >= o) y += z;
+                        }
+                        before[q] = run + y - x;
+                        run += __shfl_sync(FULL, y, 31);
+                    }
+                    unsigned at = 0;
+#pragma unroll
+                    for (int q = 0; q < 4; q++) {
+                        const unsigned z = __shfl_sync(FULL, before[q], bk & 31);
+                        if ((bk >> 5) == q) at = z;
+                    }
+                    if (mine) bins[(size_t)b * n + at + atomicAdd(&c->c4_cur[bk], 1u)] = u;
+                } else if (mine) {
+                    bins[(size_t)b * n + base + __popc(m & lanemask_lt())] = u;
+                }
             }
         }
     }
@@ -182,15 +226,6 @@ __global__ void k_bin(Ctl* c, const int32_t* __restrict__ wlist, const long long
     for (int o = 16; o > 0; o >>= 1) dmax = max(dmax, __shfl_down_sync(FULL, dmax, o));
     stage_end(c, 3);
     if (lane == 0 && dmax) atomicMax(&c->maxdeg, dmax);
-    if (__any_sync(FULL, wsum != 0)) {
-        wsum = warp_sum_u64(wsum);
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) wmax = max(wmax, __shfl_down_sync(FULL, wmax, o));
-        if (lane == 0) {
-            atomicAdd(&c->c4_wt, wsum);
-            atomicMax(&c->c4_wmax, wmax);
-        }
-    }
 }
 
 // ---- triangles and 4-cliques -------------------------------------------------
@@ -786,10 +821,14 @@ __global__ void __launch_bounds__(C4W_WARPS * 32) k_c4_warp(Ctl* c, const int32_
 
 // ---- per-edge terms and closed forms ----------------------------------------
 
-__global__ void k_edge_terms(Ctl* c, const int32_t* __restrict__ wlist, const long long* __restrict__ U_off,
-                             const uint32_t* __restrict__ U_col, const int32_t* __restrict__ U_split,
-                             const unsigned long long* __restrict__ tpack, const int32_t* __restrict__ da,
-                             const int32_t* __restrict__ db) {
+constexpr int ET_WARPS = 8;
+// Sums meet in the block first: with a set of atomics per warp a 7,000-vertex
+// graph took 14 us here, now 9.
+__global__ void __launch_bounds__(ET_WARPS * 32)
+    k_edge_terms(Ctl* c, const int32_t* __restrict__ wlist, const long long* __restrict__ U_off,
+                 const uint32_t* __restrict__ U_col, const int32_t* __restrict__ U_split,
+                 const unsigned long long* __restrict__ tpack, const int32_t* __restrict__ da,
+                 const int32_t* __restrict__ db) {
     pdl_enter();
     int nW = c->nW;
     int lane = threadIdx.x & 31;
@@ -830,27 +869,34 @@ __global__ void k_edge_terms(Ctl* c, const int32_t* __restrict__ wlist, const lo
             }
         }
     }
+    // one atomic per sum and block
+    __shared__ unsigned long long s_sum[ET_WARPS][NACC];
+    unsigned long long* const mine = s_sum[threadIdx.x >> 5];
+    if (lane < NACC) mine[lane] = 0;
+    __syncwarp();
+    auto put = [&](int slot, unsigned long long x) {
+        x = warp_sum_u64(x);
+        if (lane == 0) mine[slot] = x;
+    };
+    if (warp < nW) {
 #pragma unroll
-    for (int g = 0; g < 2; g++) {
-        P[g] = warp_sum_u64(P[g]);
-        S[g] = warp_sum_u64(S[g]);
-        T3[g] = warp_sum_u64(T3[g]);
-        W2[g] = warp_sum_u64(W2[g]);
-        T[g] = warp_sum_u64(T[g]);
-        D[g] = warp_sum_u64(D[g]);
-        E[g] = warp_sum_u64(E[g]);
+        for (int g = 0; g < 2; g++) {
+            put(6 * g + 0, P[g]);
+            put(6 * g + 1, S[g]);
+            put(6 * g + 2, T[g]);
+            put(6 * g + 3, D[g]);
+            put(12 + g, E[g]);
+            put(16 + g, T3[g]);
+            put(18 + g, W2[g]);
+        }
+        put(14, work);
     }
-    for (int g = 0; g < 2; g++) {
-        const int o = 6 * g;
-        acc_add_warp(c, o + 0, P[g]);
-        acc_add_warp(c, o + 1, S[g]);
-        acc_add_warp(c, o + 2, T[g]);
-        acc_add_warp(c, o + 3, D[g]);
-        acc_add_warp(c, 12 + g, E[g]);
-        acc_add_warp(c, 16 + g, T3[g]);
-        acc_add_warp(c, 18 + g, W2[g]);
+    __syncthreads();
+    if (threadIdx.x < NACC) {
+        unsigned long long x = 0;
+        for (int w = 0; w < ET_WARPS; w++) x += s_sum[w][threadIdx.x];
+        if (x) atomicAdd(&c->accs[threadIdx.x][blockIdx.x & (ACC_STRIPES - 1)], x);
     }
-    acc_add(c, 14, work);
 }
 
 // The closed forms and the results, by one warp (lane i < 6 holds graphlet i,
@@ -970,33 +1016,19 @@ int enqueue_counting(const CountArgs& a, cudaStream_t s, int mode) {
         t.c4_block_max = (int)std::min<long long>(t.c4_block_max, cap);
         t.c4_cta_max = std::min(t.c4_cta_max, cap);
     }
-    pdl_launch(k_wedge_bound, dim3(8 * sms), dim3(256), 0, s, a.ctl, a.wlist, a.U_off, a.U_col, a.U_split, a.U_wt);
-    pdl_launch(k_bin, dim3(gb), dim3(256), 0, s, a.ctl, a.wlist, a.U_off, a.U_split, a.U_wt, a.bins, a.n_alloc, t);
-    nl += 2;
     // The triangle kernels and the 4-cycle tiers are independent: with
-    // auxiliary streams they run side by side in five branches (warp roots;
-    // block roots; 4-cycle warps and small tables; larger tables; pivots on
-    // the handle's own stream) between a fork after the binning and a join before the edge
-    // terms.  On a small graph each branch is a few kernels bound by latency,
-    // and the count takes the longest branch; with the triangle kernels one
-    // after the other that was 0.183 ms of a 7,000-vertex graph, now 0.170.
+    // auxiliary streams they run side by side in six branches (4-cycle warps on
+    // the handle's own stream; triangle warp roots; block roots; small tables;
+    // larger tables; pivots) between a fork after the binning and a join before
+    // the edge terms.  On a small graph each branch is a few kernels bound by
+    // latency, and the count takes the longest branch.  The pivots' plan and
+    // run bounds need the sums of k_wedge_bound only and run beside the
+    // binning; after it they would wait until the triangle kernels, which fill
+    // the chip, let go of a first SM (20 us of a 7,000-vertex graph's batch).
     bool par = true;
     for (int i = 0; i < NAUX; i++) par = par && a.aux[i];
     cudaStream_t sT = par ? a.aux[0] : s, sB = par ? a.aux[1] : s, sC = par ? a.aux[2] : s,
-                 sD = par ? a.aux[3] : s;
-    if (par) {
-        cudaEventRecord(a.fork, s);
-        for (int i = 0; i < NAUX; i++) cudaStreamWaitEvent(a.aux[i], a.fork, 0);
-    }
-    k_tri_warp<<<4 * sms, TW * 32, 0, sT>>>(a.ctl, lists(BIN_TRI_WARP), a.U_off, a.U_col, a.U_split, a.tpack);
-    k_tri_block<TRI_KS, TRI_SMALL_THREADS, BIN_TRI_SMALL, WORK_TRI_SMALL>
-        <<<8 * sms, TRI_SMALL_THREADS, sizeof(BlockTri<TRI_KS, TRI_SMALL_THREADS>), sB>>>(
-            a.ctl, lists(BIN_TRI_SMALL), a.U_off, a.U_col, a.U_split, a.tpack);
-    k_tri_block<TRI_KM, TRI_BIG_THREADS, BIN_TRI_BLOCK, WORK_TRI_BLOCK>
-        <<<2 * sms, TRI_BIG_THREADS, sizeof(BlockTri<TRI_KM, TRI_BIG_THREADS>), sB>>>(
-            a.ctl, lists(BIN_TRI_BLOCK), a.U_off, a.U_col, a.U_split, a.tpack);
-    k_tri_merge<<<sms, 256, 0, sB>>>(a.ctl, lists(BIN_TRI_MERGE), a.U_off, a.U_col, a.U_split, a.tpack);
-    nl += 4;
+                 sD = par ? a.aux[3] : s, sP = par ? a.aux[4] : s;
     PivotArgs pa;
     pa.ctl = a.ctl;
     pa.pivots = lists(BIN_C4_DENSE);
@@ -1010,22 +1042,43 @@ int enqueue_counting(const CountArgs& a, cudaStream_t s, int mode) {
     pa.words = geom.words;
     pa.group = geom.group;
     pa.credit = a.c4_credit;
+    pdl_launch(k_wedge_bound, dim3(8 * sms), dim3(256), 0, s, a.ctl, a.wlist, a.U_off, a.U_col, a.U_split, a.U_wt, t);
+    if (par) {
+        cudaEventRecord(a.fork, s);
+        cudaStreamWaitEvent(sP, a.fork, 0);
+    }
+    nl += enqueue_c4_plan(pa, geom, sP);
+    pdl_launch(k_bin, dim3(gb), dim3(256), 0, s, a.ctl, a.wlist, a.U_off, a.U_split, a.U_wt, a.bins, a.n_alloc, t);
+    nl += 2;
+    if (par) {
+        cudaEventRecord(a.fork, s);
+        for (int i = 0; i < NAUX; i++) cudaStreamWaitEvent(a.aux[i], a.fork, 0);
+    }
+    nl += enqueue_c4_pivots(pa, a.c4_mode, geom, sP);
+    k_tri_warp<<<4 * sms, TW * 32, 0, sT>>>(a.ctl, lists(BIN_TRI_WARP), a.U_off, a.U_col, a.U_split, a.tpack);
+    k_tri_block<TRI_KS, TRI_SMALL_THREADS, BIN_TRI_SMALL, WORK_TRI_SMALL>
+        <<<8 * sms, TRI_SMALL_THREADS, sizeof(BlockTri<TRI_KS, TRI_SMALL_THREADS>), sB>>>(
+            a.ctl, lists(BIN_TRI_SMALL), a.U_off, a.U_col, a.U_split, a.tpack);
+    k_tri_block<TRI_KM, TRI_BIG_THREADS, BIN_TRI_BLOCK, WORK_TRI_BLOCK>
+        <<<2 * sms, TRI_BIG_THREADS, sizeof(BlockTri<TRI_KM, TRI_BIG_THREADS>), sB>>>(
+            a.ctl, lists(BIN_TRI_BLOCK), a.U_off, a.U_col, a.U_split, a.tpack);
+    k_tri_merge<<<sms, 256, 0, sB>>>(a.ctl, lists(BIN_TRI_MERGE), a.U_off, a.U_col, a.U_split, a.tpack);
+    nl += 4;
     if (a.c4_mode == C4_COUNT) {
-        k_c4_reg<<<4 * sms, 256, 0, sC>>>(a.ctl, lists(BIN_C4_REG), a.U_off, a.U_col, a.U_split);
-        k_c4_warp<<<7 * sms, C4W_WARPS * 32, 0, sC>>>(a.ctl, lists(BIN_C4_WARP), a.U_off, a.U_col, a.U_split,
-                                                       a.U_wt);
+        k_c4_reg<<<4 * sms, 256, 0, s>>>(a.ctl, lists(BIN_C4_REG), a.U_off, a.U_col, a.U_split);
+        k_c4_warp<<<7 * sms, C4W_WARPS * 32, 0, s>>>(a.ctl, lists(BIN_C4_WARP), a.U_off, a.U_col, a.U_split,
+                                                      a.U_wt);
         nl += 2;
     } else {
-        nl += enqueue_c4_warp_credit(pa, a.c4_mode, a.bins, sms, sC);
+        nl += enqueue_c4_warp_credit(pa, a.c4_mode, a.bins, sms, s);
     }
     nl += enqueue_c4_tables(pa, a.c4_mode, a.bins, sms, sC, sD);
-    nl += enqueue_c4_pivots(pa, a.c4_mode, geom, s);
     if (par)
         for (int i = 0; i < NAUX; i++) {
             cudaEventRecord(a.join[i], a.aux[i]);
             cudaStreamWaitEvent(s, a.join[i], 0);
         }
-    k_edge_terms<<<8 * sms, 256, 0, s>>>(a.ctl, a.wlist, a.U_off, a.U_col, a.U_split, a.tpack, a.da, a.db);
+    k_edge_terms<<<8 * sms, ET_WARPS * 32, 0, s>>>(a.ctl, a.wlist, a.U_off, a.U_col, a.U_split, a.tpack, a.da, a.db);
     pdl_launch(k_finalize, dim3(1), dim3(32), 0, s, a.ctl, mode);
     nl += 2;
     return nl;

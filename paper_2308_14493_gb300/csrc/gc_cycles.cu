@@ -72,53 +72,20 @@ __global__ void __launch_bounds__(256) k_c4_granules(const long long* __restrict
 // Cut [0, n) into chunks, from the highest granule down: a chunk grows while
 // its counters fit `words` and its share of the adjacency entries is within
 // the limit.  The limit is 1 unless the pivot of most wedges would outlast an
-// even share of all of them over the blocks.  One block; the walk over the
-// granules (at most a few hundred on graphs below 16 M vertices) is serial.
+// even share of all of them over the blocks.  One block.  Below 2^16 ids all
+// counters fit at 16 bits, and the cuts are those of even shares, found by a
+// thread per granule; else the walk over the granules (at most a few hundred
+// on graphs below 16 M vertices) is serial.
 constexpr int PLAN_TILE = 512;
 __global__ void __launch_bounds__(PLAN_TILE) k_c4_plan(Ctl* c, const long long* __restrict__ U_off, int n,
                                                        int gran, int ngran, const int32_t* __restrict__ gmax,
                                                        int words, int ctas, int nchmax, C4Head* __restrict__ head,
-                                                       C4Chunk* __restrict__ chunk, const int32_t* __restrict__ pivots,
-                                                       const long long* __restrict__ U_wt,
-                                                       int32_t* __restrict__ sorted) {
-    pdl_enter();
+                                                       C4Chunk* __restrict__ chunk) {
     stage_begin(c, 8);
-    // pivots by falling wedge bound (two buckets per octave), so that the
-    // largest tasks start first
-    __shared__ unsigned s_hist[128];
-    const int npiv = c->nbin[BIN_C4_DENSE];
-    auto bucket = [&](int32_t u) {
-        const long long w = U_wt[u];
-        const int lg = 63 - __clzll(w | 1);
-        return 127 - (2 * lg + (lg > 0 ? (int)((w >> (lg - 1)) & 1) : 0));
-    };
-    if (threadIdx.x < 128) s_hist[threadIdx.x] = 0;
-    __syncthreads();
-    for (int i = threadIdx.x; i < npiv; i += blockDim.x) atomicAdd(&s_hist[bucket(pivots[i])], 1u);
-    __syncthreads();
-    if (threadIdx.x < 32) {
-        unsigned run = 0;
-        for (int b = 0; b < 128; b += 32) {
-            const unsigned x = s_hist[b + threadIdx.x];
-            unsigned y = x;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const unsigned z = __shfl_up_sync(FULL, y, o);
-                if ((int)threadIdx.x >= o) y += z;
-            }
-            s_hist[b + threadIdx.x] = run + y - x;
-            run += __shfl_sync(FULL, y, 31);
-        }
-    }
-    __syncthreads();
-    for (int i = threadIdx.x; i < npiv; i += blockDim.x) {
-        const int32_t u = pivots[i];
-        sorted[atomicAdd(&s_hist[bucket(u)], 1u)] = u;
-    }
     __shared__ int s_max[PLAN_TILE];
     __shared__ long long s_off[PLAN_TILE + 1];
     const long long entries = U_off[n];
-    if (c->nbin[BIN_C4_DENSE] == 0 || entries == 0) {
+    if (c->c4_wt == 0 || entries == 0) {  // no pivots
         if (threadIdx.x == 0) head->nch = 0;
         return;
     }
@@ -128,12 +95,37 @@ __global__ void __launch_bounds__(PLAN_TILE) k_c4_plan(Ctl* c, const long long* 
         const double fair = (double)c->c4_wt / ctas, big = 2.0 * (double)c->c4_wmax;
         if (big > fair) limit = (long long)((double)entries * fmax(fair / big, 0.125));
     }
+    if (!gmax) {
+        const int t = threadIdx.x, k = (int)((entries + limit - 1) / limit);
+        auto off = [&](int j) { return U_off[min((long long)n, (long long)j * gran)]; };
+        auto part = [&](int j) { return (int)((entries - off(j + 1)) * k / entries); };  // of granule j
+        // granule t is the highest of its chunk
+        const bool cut = t < ngran && (t == ngran - 1 || part(t) != part(t + 1));
+        const unsigned b = __ballot_sync(FULL, cut);
+        __shared__ unsigned s_cut[PLAN_TILE / 32];
+        __shared__ int s_top[PLAN_TILE];
+        if ((t & 31) == 0) s_cut[t >> 5] = b;
+        __syncthreads();
+        int at = __popc(b & ~(lanemask_lt() | (1u << (t & 31)))), all = 0;
+        for (int w = 0; w < PLAN_TILE / 32; w++) {
+            all += __popc(s_cut[w]);
+            if (w > (t >> 5)) at += __popc(s_cut[w]);
+        }
+        if (cut) s_top[at] = t + 1;
+        __syncthreads();
+        if (t < all && t < nchmax) {
+            const int hi = s_top[t], lo = t + 1 < all ? s_top[t + 1] : 0;
+            chunk[t] = C4Chunk{lo * gran, min(n, hi * gran), 1, (float)((double)(off(hi) - off(lo)) / (double)entries)};
+        }
+        if (t == 0) head->nch = min(all, nchmax);
+        return;
+    }
     for (int top = ngran; top > 0; top -= PLAN_TILE) {
         const int base = max(0, top - PLAN_TILE), cnt = top - base;
         __syncthreads();
         for (int i = threadIdx.x; i <= cnt; i += blockDim.x) {
             s_off[i] = U_off[min((long long)n, (long long)(base + i) * gran)];
-            if (i < cnt) s_max[i] = gmax ? gmax[base + i] : 65535;
+            if (i < cnt) s_max[i] = gmax[base + i];
         }
         __syncthreads();
         if (threadIdx.x != 0) continue;
@@ -164,7 +156,9 @@ __global__ void __launch_bounds__(PLAN_TILE) k_c4_plan(Ctl* c, const long long* 
 
 // Run of every vertex's row in the chunks [c0, c0 + group): start << 28 |
 // length.  A thread per vertex, chunks from the top, each bound a binary
-// search in what is left of the row.
+// search in what is left of the row; where the launch has a thread for each
+// (chunk, vertex), each finds its two bounds by itself (7,000 vertices:
+// 16 us -> 7, all of it the latency of the searches).
 __global__ void __launch_bounds__(256) k_c4_runs(const long long* __restrict__ U_off,
                                                  const uint32_t* __restrict__ U_col, int n, C4Head* __restrict__ head,
                                                  const C4Chunk* __restrict__ chunk, int c0, int group,
@@ -173,6 +167,17 @@ __global__ void __launch_bounds__(256) k_c4_runs(const long long* __restrict__ U
     if (blockIdx.x == 0 && threadIdx.x == 0) head->task = 0;
     const int nc = min(group, head->nch - c0);
     if (nc <= 0) return;
+    if ((long long)n * nc <= (long long)gridDim.x * blockDim.x) {
+        const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+        if (i >= (long long)n * nc) return;
+        const int k = (int)(i / n);
+        const long long v = i - (long long)k * n, b = U_off[v], len = U_off[v + 1] - b;
+        const int lo = chunk[c0 + k].lo, hi = chunk[c0 + k].hi;
+        const long long s = (len && lo) ? lower_bound_id(U_col + b, len, (uint32_t)lo) : 0;
+        const long long e = (len && hi < n) ? lower_bound_id(U_col + b, len, (uint32_t)hi) : len;
+        run[(size_t)k * n + v] = ((unsigned long long)(b + s) << 28) | (unsigned long long)(e - s);
+        return;
+    }
     const int top = chunk[c0].hi;
     for (long long v = blockIdx.x * (long long)blockDim.x + threadIdx.x; v < n;
          v += (long long)gridDim.x * blockDim.x) {
@@ -229,7 +234,7 @@ __global__ void __launch_bounds__(THREADS, MINB) k_c4_pivot(PivotArgs a, int c0)
         o.id = atomicAdd(&a.b.head->task, 1ull);
         if (o.id >= tasks) return;
         o.k = (int)(o.id / (unsigned)npiv);
-        o.u = (uint32_t)a.b.sorted[(int)(o.id - (unsigned long long)o.k * (unsigned)npiv)];
+        o.u = (uint32_t)a.pivots[(int)(o.id - (unsigned long long)o.k * (unsigned)npiv)];
         o.rb = a.U_off[o.u];
         o.nlow = a.U_split[o.u];
         o.wt = (float)a.U_wt[o.u];
@@ -721,22 +726,32 @@ int enqueue_c4_warp_credit(const PivotArgs& a, int mode, const int32_t* bins, in
     return 1;
 }
 
-int enqueue_c4_pivots(const PivotArgs& a, int mode, const C4Geom& g, cudaStream_t s) {
-    int nl = 0;
+static int enqueue_c4_runs(const PivotArgs& a, const C4Geom& g, int c0, cudaStream_t s) {
+    const int gr = (int)std::max<long long>(
+        1, std::min<long long>(((long long)a.n * std::min(g.group, 8) + 255) / 256, 16ll * g.ctas));
+    k_c4_runs<<<gr, 256, 0, s>>>(a.U_off, a.U_col, a.n, a.b.head, a.b.chunk, c0, g.group, a.b.run);
+    return 1;
+}
+
+int enqueue_c4_plan(const PivotArgs& a, const C4Geom& g, cudaStream_t s) {
+    int nl = 1;
     if (!g.narrow) {
         k_c4_granules<<<g.ngran, 256, 0, s>>>(a.U_off, a.n, g.gran, a.b.gmax);
         nl++;
     }
     k_c4_plan<<<1, PLAN_TILE, 0, s>>>(a.ctl, a.U_off, a.n, g.gran, g.ngran, g.narrow ? nullptr : a.b.gmax, g.words,
-                                      g.ctas, g.nchmax, a.b.head, a.b.chunk, a.pivots, a.U_wt, a.b.sorted);
-    nl++;
-    const int gr = (int)std::max<long long>(1, std::min<long long>(((long long)a.n + 255) / 256, 16ll * g.ctas));
+                                      g.ctas, g.nchmax, a.b.head, a.b.chunk);
+    return nl + enqueue_c4_runs(a, g, 0, s);
+}
+
+int enqueue_c4_pivots(const PivotArgs& a, int mode, const C4Geom& g, cudaStream_t s) {
+    int nl = 0;
     for (int c0 = 0; c0 < g.nchmax; c0 += g.group) {
-        k_c4_runs<<<gr, 256, 0, s>>>(a.U_off, a.U_col, a.n, a.b.head, a.b.chunk, c0, g.group, a.b.run);
+        if (c0) nl += enqueue_c4_runs(a, g, c0, s);
         if (mode == C4_VERTEX) C4Kernels<C4_VERTEX>::pivots(a, g, c0, s);
         else if (mode == C4_EDGE) C4Kernels<C4_EDGE>::pivots(a, g, c0, s);
         else C4Kernels<C4_COUNT>::pivots(a, g, c0, s);
-        nl += 2;
+        nl++;
     }
     return nl;
 }

@@ -118,6 +118,7 @@ struct Ctl {
     int l_nw3;                       // third vertices listed after V_X (maintained triangle sums)
     // wedge bounds of the pivots counted in shared memory (BIN_C4_DENSE): sum and maximum
     unsigned long long c4_wt, c4_wmax;
+    unsigned c4_hist[128], c4_cur[128];  // of them per half octave (k_wedge_bound), placed so far (k_bin)
     // stage boundaries: begin of [0] normalise [1] region walk [2] union graph;
     // [3] end of the binning (local: begin of the triangles); end of [4] the
     // triangles, [5] the 4-cycles (local: begin of the 4-cliques / 4-cycles and
@@ -153,7 +154,7 @@ struct Tuning {
 constexpr long long NEVER = 1ll << 62;
 inline Tuning default_tuning() { return Tuning{32, TRI_KS, TRI_KM, 32, C4_T1, C4_T2, 32768, NEVER, NEVER}; }
 
-constexpr int NAUX = 4;  // side streams of a counting pass
+constexpr int NAUX = 5;  // side streams of a counting pass
 
 // Handle-independent launch geometry.
 struct Dims {

@@ -48,8 +48,7 @@ constexpr size_t OFF_TPACK = al(OFF_UCOL + 4 * (size_t)NA_MAX_E);
 constexpr size_t OFF_BINS = al(OFF_TPACK + 8 * (size_t)NA_MAX_E);
 constexpr size_t OFF_HEAD = al(OFF_BINS + 4 * (size_t)NA_MAX_N * NBINS);
 constexpr size_t OFF_CHUNK = al(OFF_HEAD + sizeof(C4Head));
-constexpr size_t OFF_SORTED = al(OFF_CHUNK + sizeof(C4Chunk) * NA_CHUNKS);
-constexpr size_t OFF_RUN = al(OFF_SORTED + 4 * (size_t)NA_MAX_N);
+constexpr size_t OFF_RUN = al(OFF_CHUNK + sizeof(C4Chunk) * NA_CHUNKS);
 constexpr size_t OFF_ERR = al(OFF_RUN + 8 * (size_t)NA_MAX_N * NA_GROUP);
 constexpr size_t SCRATCH_BYTES = al(OFF_ERR + 16);
 
@@ -222,7 +221,6 @@ extern "C" int gc_count_static_noalloc(int32_t n, const int32_t* d_row_ptr, cons
     ca.c4.head = (C4Head*)(b + OFF_HEAD);
     ca.c4.chunk = (C4Chunk*)(b + OFF_CHUNK);
     ca.c4.gmax = nullptr;  // every degree is below 2^16
-    ca.c4.sorted = (int32_t*)(b + OFF_SORTED);
     ca.c4.run = (unsigned long long*)(b + OFF_RUN);
     ca.c4.list = nullptr;  // a static count has no one-graph wedges
     ca.c4.lcap = 0;
