@@ -624,22 +624,22 @@ static int count_region(gc_graph* g, int fin, bool set_F, bool twin = false, boo
     int gw = grid_warps(g);
     pdl_launch(k_reset_count, dim3(1), dim3(32), 0, s, g->ctl);
     CK(cudaMemsetAsync(g->U_deg, 0, sizeof(int32_t) * (size_t)std::max(g->n, 1), s));
-    if (twin)
-        pdl_launch(k_u_count_twin, dim3(grid_elems(g, g->n)), dim3(TPB), 0, s, g->ctl, g->wlist, g->deg, g->segA,
+    if (all || twin)
+        pdl_launch(k_u_count_all, dim3(grid_elems(g, g->n)), dim3(TPB), 0, s, g->ctl, g->wlist, g->deg, g->segA,
                    g->U_deg);
     else
         pdl_launch(k_u_count, dim3(gw), dim3(TPB), 0, s, g->ctl, g->wlist, g->visited, g->row_start, g->deg, g->col,
-                   g->segA, g->U_deg, all ? 1 : 0);
+                   g->segA, g->U_deg);
     g->launches += 2;
     g->launches += scan_i32_to_i64(g->U_deg, g->U_off, nullptr, g->n, g->bsum.p, scan_grid(g->n, g->sms), &g->ctl->nU,
                                    s);
-    if (twin)
-        pdl_launch(k_u_fill_twin, dim3(gw), dim3(TPB), 0, s, g->ctl, g->wlist, g->row_start, g->deg, g->col, g->segA,
-                   g->segD, g->dstA.p, g->dstD.p, g->U_off, g->U_col.p, g->U_split, g->da, g->db);
+    if (all || twin)
+        pdl_launch(twin ? k_u_fill_twin : k_u_fill_rows, dim3(gw), dim3(TPB), 0, s, g->ctl, g->wlist,
+                   g->row_start, g->deg, g->col, g->segA, g->segD, g->dstA.p, g->dstD.p, g->U_off, g->U_col.p,
+                   g->U_split, g->da, g->db);
     else
         pdl_launch(k_u_fill, dim3(gw), dim3(TPB), 0, s, g->ctl, g->wlist, g->visited, g->row_start, g->deg, g->col,
-                   g->segA, g->segD, g->dstA.p, g->dstD.p, g->U_off, g->U_col.p, g->U_split, g->da, g->db,
-                   all ? 1 : 0);
+                   g->segA, g->segD, g->dstA.p, g->dstD.p, g->U_off, g->U_col.p, g->U_split, g->da, g->db);
     pdl_launch(k_zero_u64, dim3(grid_elems(g, (long long)g->U_col.cap)), dim3(TPB), 0, s, g->tpack.p, &g->ctl->nU);
     g->launches += 2;
     CountArgs ca;
@@ -685,8 +685,8 @@ static int count_local(gc_graph* g, int commit, bool t2, bool laid_out) {
     g->launches++;
     if (!laid_out) {
         CK(cudaMemsetAsync(g->U_deg, 0, sizeof(int32_t) * (size_t)std::max(g->n, 1), s));
-        pdl_launch(k_u_count, dim3(gw), dim3(TPB), 0, s, g->ctl, g->wlist, g->visited, g->row_start, g->deg, g->col,
-                   g->segA, g->U_deg, 1);
+        pdl_launch(k_u_count_all, dim3(grid_elems(g, g->n)), dim3(TPB), 0, s, g->ctl, g->wlist, g->deg, g->segA,
+                   g->U_deg);
         g->launches++;
         g->launches += scan_i32_to_i64(g->U_deg, g->U_off, nullptr, g->n, g->bsum.p, scan_grid(g->n, g->sms), &g->ctl->nU,
                                        s);

@@ -115,42 +115,109 @@ __device__ __forceinline__ int wedge_bucket(long long w) {
 }
 
 // Wedge bound of every 4-cycle pivot: w~(u) = sum of the union-graph degrees
-// of its lower neighbours.  A warp per vertex (hubs with tens of thousands
-// of lower neighbours spread over the grid like everyone else).  The sums over
-// the largest tier, which plan its chunks, are made here, so that the plan
-// need not wait for the bins.
-__global__ void k_wedge_bound(Ctl* c, const int32_t* __restrict__ wlist, const long long* __restrict__ U_off,
+// of its lower neighbours.  Bound by the latency of entry and degree loads.
+// Up to four vertices a warp, a warp takes one at a time.  Beyond, eight lanes
+// take a vertex and a warp 32, since a warp per vertex has one short row in
+// flight (1.53 ms on a graph of 4.8 M vertices and 69 M edges, 0.84 now), and
+// long lists wait for the whole block.  The sums over the largest tier, which
+// plan its chunks, are made here, so that the plan need not wait for the bins.
+constexpr int WB_LONG = 256;
+constexpr int WB_LONGS = 256;  // a block's list of them (a warp takes each further one)
+__global__ void __launch_bounds__(256) k_wedge_bound(Ctl* c, const int32_t* __restrict__ wlist, const long long* __restrict__ U_off,
                               const uint32_t* __restrict__ U_col, const int32_t* __restrict__ U_split,
                               long long* __restrict__ U_wt, Tuning t) {
     pdl_enter();
     const int nW = c->nW;
     const int lane = threadIdx.x & 31;
-    const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int nwarps = (gridDim.x * blockDim.x) >> 5;
+    const long long warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const long long nwarps = (gridDim.x * blockDim.x) >> 5;
     unsigned long long wsum = 0, wmax = 0;  // of the pivots for shared memory
-    for (int i = warp; i < nW; i += nwarps) {
-        const int32_t u = wlist[i];
-        const int sp = U_split[u];
-        long long part = 0;
-        if (sp >= 2) {
-            const long long rb = U_off[u];
-#pragma unroll 4
-            for (int j = lane; j < sp; j += 32) {
-                const uint32_t v = vid(U_col[rb + j]);
-                part += U_off[v + 1] - U_off[v];
-            }
-#pragma unroll
-            for (int o = 16; o > 0; o >>= 1) part += __shfl_xor_sync(FULL, part, o);
+    auto put = [&](int32_t u, int sp, long long w) {
+        U_wt[u] = w;
+        if (sp >= 2 && c4_bin(t, w) == BIN_C4_DENSE) {
+            wsum += (unsigned long long)w;
+            wmax = max(wmax, (unsigned long long)w);
+            atomicAdd(&c->c4_hist[wedge_bucket(w)], 1u);
         }
-        if (lane == 0) {
-            U_wt[u] = part;
-            if (sp >= 2 && c4_bin(t, part) == BIN_C4_DENSE) {
-                wsum += (unsigned long long)part;
-                wmax = max(wmax, (unsigned long long)part);
-                atomicAdd(&c->c4_hist[wedge_bucket(part)], 1u);
+    };
+    auto sum = [&](long long b, int len, int first, int step) {
+        long long part = 0;
+#pragma unroll 4
+        for (int j = first; j < len; j += step) {
+            const uint32_t v = vid(U_col[b + j]);
+            part += U_off[v + 1] - U_off[v];
+        }
+        return part;
+    };
+    auto by_warp = [&](int32_t u, int sp, long long rb) {
+        long long w = sp >= 2 ? sum(rb, sp, lane, 32) : 0;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) w += __shfl_xor_sync(FULL, w, o);
+        if (lane == 0) put(u, sp, w);
+    };
+    __shared__ int32_t s_long[WB_LONGS];
+    __shared__ int s_nlong;
+    __shared__ long long s_part[8];
+    if (threadIdx.x == 0) s_nlong = 0;
+    __syncthreads();
+    const bool few = nW <= 4 * nwarps;
+    if (few)
+        for (long long i = warp; i < nW; i += nwarps) {
+            const int32_t u = wlist[i];
+            by_warp(u, U_split[u], U_off[u]);
+        }
+    // eight quads of neighbouring vertices, spread over the ids
+    const int quads = few ? 0 : (nW + 3) / 4;
+    for (long long base = warp; base < quads; base += 8 * nwarps) {
+        const long long i = 4 * (base + (lane >> 2) * nwarps) + (lane & 3);
+        int32_t u = -1;
+        int sp = 0;
+        long long rb = 0;
+        bool over = false;  // long, and the block's list is full
+        if (i < nW) {
+            u = wlist[i];
+            sp = U_split[u];
+            rb = U_off[u];
+            if (sp > WB_LONG) {
+                const int at = atomicAdd(&s_nlong, 1);
+                over = at >= WB_LONGS;
+                if (!over) s_long[at] = u;
             }
+        }
+#pragma unroll 2
+        for (int r = 0; r < 8; r++) {
+            const int src = 4 * r + (lane >> 3);
+            const int32_t x = __shfl_sync(FULL, u, src);
+            const int len = __shfl_sync(FULL, sp, src);
+            const long long b = __shfl_sync(FULL, rb, src);
+            long long w = len >= 2 && len <= WB_LONG ? sum(b, len, lane & 7, 8) : 0;
+#pragma unroll
+            for (int o = 4; o > 0; o >>= 1) w += __shfl_xor_sync(FULL, w, o);
+            if ((lane & 7) == 0 && x >= 0 && len <= WB_LONG) put(x, len, w);
+        }
+        for (unsigned m = __ballot_sync(FULL, over); m; m &= m - 1) {
+            const int src = __ffs(m) - 1;
+            by_warp(__shfl_sync(FULL, u, src), __shfl_sync(FULL, sp, src), __shfl_sync(FULL, rb, src));
         }
     }
+    __syncthreads();
+    const int nlong = min(s_nlong, WB_LONGS);
+    for (int k = 0; k < nlong; k++) {
+        const int32_t u = s_long[k];
+        const int sp = U_split[u];
+        const long long w = (long long)warp_sum_u64((unsigned long long)sum(U_off[u], sp, threadIdx.x, blockDim.x));
+        if (lane == 0) s_part[threadIdx.x >> 5] = w;
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            long long all = 0;
+            for (int i = 0; i < (int)(blockDim.x >> 5); i++) all += s_part[i];
+            put(u, sp, all);
+        }
+        __syncthreads();
+    }
+    wsum = warp_sum_u64(wsum);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) wmax = max(wmax, __shfl_xor_sync(FULL, wmax, o));
     if (lane == 0 && wsum) {
         atomicAdd(&c->c4_wt, wsum);
         atomicMax(&c->c4_wmax, wmax);
@@ -822,52 +889,117 @@ __global__ void __launch_bounds__(C4W_WARPS * 32) k_c4_warp(Ctl* c, const int32_
 // ---- per-edge terms and closed forms ----------------------------------------
 
 constexpr int ET_WARPS = 8;
-// Sums meet in the block first: with a set of atomics per warp a 7,000-vertex
-// graph took 14 us here, now 9.
-__global__ void __launch_bounds__(ET_WARPS * 32)
+constexpr int ET_LONG = 256;  // longer out-lists are walked one at a time
+struct EdgeRow {
+    long long b;      // first entry of the out-list
+    int k;            // its length
+    uint32_t da, db;  // degrees in G_a, G_b
+};
+// Bound by latency: two random degree loads per edge behind a chain of three.
+// A warp takes 32 vertices and walks their out-lists as one run, four edges a
+// lane ahead, so rows of a few entries fill the lanes (a warp per row: 3.25 ms
+// for the 69 M edges of a 4.8 M-vertex graph, 0.60 now).  The sums meet in the
+// block before the atomics (a 7,000-vertex graph: 14 us with a set per warp,
+// now 9).
+__global__ void __launch_bounds__(ET_WARPS * 32, 4)
     k_edge_terms(Ctl* c, const int32_t* __restrict__ wlist, const long long* __restrict__ U_off,
                  const uint32_t* __restrict__ U_col, const int32_t* __restrict__ U_split,
                  const unsigned long long* __restrict__ tpack, const int32_t* __restrict__ da,
                  const int32_t* __restrict__ db) {
     pdl_enter();
-    int nW = c->nW;
-    int lane = threadIdx.x & 31;
-    int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    int nwarps = (gridDim.x * blockDim.x) >> 5;
-    unsigned long long P[2] = {0, 0}, S[2] = {0, 0}, T[2] = {0, 0}, D[2] = {0, 0}, E[2] = {0, 0}, work = 0;
+    __shared__ EdgeRow s_row[ET_WARPS * 32];
+    __shared__ int s_pre[ET_WARPS][33];
+    const int nW = c->nW;
+    const int lane = threadIdx.x & 31;
+    const long long warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const long long nwarps = (gridDim.x * blockDim.x) >> 5;
+    EdgeRow* const rows = s_row + (threadIdx.x & ~31);
+    int* const pre = s_pre[threadIdx.x >> 5];
+    unsigned long long P[2] = {0, 0}, S[2] = {0, 0}, T[2] = {0, 0}, D[2] = {0, 0}, work = 0;
     unsigned long long T3[2] = {0, 0}, W2[2] = {0, 0};  // sum of t_e; sum of C(d, 2)
-    for (int wi = warp; wi < nW; wi += nwarps) {
-        int32_t u = wlist[wi];
-        long long dau = da[u], dbu = db[u];
-        if (lane == 0) {
-            S[0] += choose3((unsigned long long)dau);
-            S[1] += choose3((unsigned long long)dbu);
-            W2[0] += choose2((unsigned long long)dau);
-            W2[1] += choose2((unsigned long long)dbu);
+    unsigned E[2] = {0, 0};
+    auto edge = [&](const EdgeRow& r, uint32_t fe, unsigned long long t, uint32_t dva, uint32_t dvb) {
+        auto add = [&](int g, uint32_t du, uint32_t dv, uint32_t tt) {
+            P[g] += (unsigned long long)(du - 1) * (dv - 1);
+            T[g] += (unsigned long long)tt * (du + dv - 4);  // (an edge in a triangle has du, dv >= 2)
+            D[g] += (unsigned long long)tt * tt;
+            T3[g] += tt;
+            E[g]++;
+        };
+        if (fe & FLAG_A) add(0, r.da, dva, (uint32_t)(t >> 32));
+        if (fe & FLAG_B) add(1, r.db, dvb, (uint32_t)t);
+    };
+    const int quads = (nW + 3) / 4;
+    // eight quads of neighbouring vertices, spread over the ids (hubs have
+    // neighbouring ids)
+    for (long long base = warp; base < quads; base += 8 * nwarps) {
+        const long long i = 4 * (base + (lane >> 2) * nwarps) + (lane & 3);
+        EdgeRow r{};
+        if (i < nW) {
+            const int32_t u = wlist[i];
+            r.da = (uint32_t)da[u];
+            r.db = (uint32_t)db[u];
+            S[0] += choose3(r.da);
+            S[1] += choose3(r.db);
+            W2[0] += choose2(r.da);
+            W2[1] += choose2(r.db);
+            const long long b = U_off[u], e = U_off[u + 1];
+            r.b = b + U_split[u];
+            r.k = (int)(e - r.b);
+            // rows walked for the triangles: both out-lists of every edge, so
+            // a vertex's own once for each of its edges
+            work += (unsigned long long)r.k * (unsigned long long)(e - b);
         }
-        long long ob = U_off[u] + U_split[u], oe = U_off[u + 1];
-        for (long long e = ob + lane; e < oe; e += 32) {
-            uint32_t fe = U_col[e];
-            uint32_t v = vid(fe);
-            unsigned long long t = tpack[e];
-            work += (unsigned long long)((oe - ob) + (U_off[v + 1] - U_off[v] - U_split[v]));
-            if (fe & FLAG_A) {
-                long long dv = da[v], tt = (long long)(t >> 32);
-                P[0] += (unsigned long long)((dau - 1) * (dv - 1) - tt);
-                T[0] += (unsigned long long)(tt * (dau + dv - 4));
-                D[0] += choose2((unsigned long long)tt);
-                T3[0] += (unsigned long long)tt;
-                E[0] += 1;
+        const bool is_long = r.k > ET_LONG;
+        rows[lane] = r;
+        int x = is_long ? 0 : r.k;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int y = __shfl_up_sync(FULL, x, o);
+            if (lane >= o) x += y;
+        }
+        pre[lane + 1] = x;
+        if (lane == 0) pre[0] = 0;
+        const int total = __shfl_sync(FULL, x, 31);
+        __syncwarp();
+        int q = 0;
+        for (int j0 = lane; j0 < total; j0 += 128) {
+            int at[4];
+            uint32_t fe[4], va[4], vb[4];
+            unsigned long long t[4];
+#pragma unroll
+            for (int k = 0; k < 4; k++) {
+                const int j = j0 + 32 * k;
+                if (j < total)
+                    while (pre[q + 1] <= j) q++;
+                at[k] = q;
+                const long long e = rows[q].b + (j - pre[q]);
+                fe[k] = j < total ? U_col[e] : 0u;
+                t[k] = j < total ? tpack[e] : 0ull;
             }
-            if (fe & FLAG_B) {
-                long long dv = db[v], tt = (long long)(t & 0xFFFFFFFFull);
-                P[1] += (unsigned long long)((dbu - 1) * (dv - 1) - tt);
-                T[1] += (unsigned long long)(tt * (dbu + dv - 4));
-                D[1] += choose2((unsigned long long)tt);
-                T3[1] += (unsigned long long)tt;
-                E[1] += 1;
+#pragma unroll
+            for (int k = 0; k < 4; k++) {
+                va[k] = (fe[k] & FLAG_A) ? (uint32_t)da[vid(fe[k])] : 0u;
+                vb[k] = (fe[k] & FLAG_B) ? (uint32_t)db[vid(fe[k])] : 0u;
+            }
+#pragma unroll
+            for (int k = 0; k < 4; k++) edge(rows[at[k]], fe[k], t[k], va[k], vb[k]);
+        }
+        for (unsigned m = __ballot_sync(FULL, is_long); m; m &= m - 1) {
+            const EdgeRow l = rows[__ffs(m) - 1];
+#pragma unroll 4
+            for (int j = lane; j < l.k; j += 32) {
+                const uint32_t fe = U_col[l.b + j];
+                edge(l, fe, tpack[l.b + j], (fe & FLAG_A) ? (uint32_t)da[vid(fe)] : 0u,
+                     (fe & FLAG_B) ? (uint32_t)db[vid(fe)] : 0u);
             }
         }
+        __syncwarp();
+    }
+#pragma unroll
+    for (int g = 0; g < 2; g++) {
+        P[g] -= T3[g];             // sum of (du - 1)(dv - 1) - t
+        D[g] = (D[g] - T3[g]) / 2;  // sum of C(t, 2), exact: every term is even
     }
     // one atomic per sum and block
     __shared__ unsigned long long s_sum[ET_WARPS][NACC];
@@ -878,7 +1010,7 @@ __global__ void __launch_bounds__(ET_WARPS * 32)
         x = warp_sum_u64(x);
         if (lane == 0) mine[slot] = x;
     };
-    if (warp < nW) {
+    if (warp < quads) {
 #pragma unroll
         for (int g = 0; g < 2; g++) {
             put(6 * g + 0, P[g]);

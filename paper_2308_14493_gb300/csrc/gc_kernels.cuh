@@ -61,8 +61,12 @@ __global__ void k_ext_degrees(const int32_t* deg, const int32_t* iperm, int n, i
 __global__ void k_bfs_sources(Ctl* c, const int32_t* srcA, const int32_t* srcD, uint32_t* visited, int32_t* wlist);
 __global__ void k_level_ends(Ctl* c);
 __global__ void k_region_rest(Ctl* c, int n, uint32_t* visited, int32_t* wlist);
-__global__ void k_u_count_twin(const Ctl* c, const int32_t* wlist, const int32_t* deg, const int2* segA,
-                               int32_t* U_deg);
+__global__ void k_u_count_all(const Ctl* c, const int32_t* wlist, const int32_t* deg, const int2* segA,
+                              int32_t* U_deg);
+__global__ void k_u_fill_rows(const Ctl* c, const int32_t* wlist, const long long* row_start, const int32_t* deg,
+                              const int32_t* col, const int2* segA, const int2* segD, const int32_t* dstA,
+                              const int32_t* dstD, const long long* U_off, uint32_t* U_col, int32_t* U_split,
+                              int32_t* da, int32_t* db);
 __global__ void k_u_fill_twin(const Ctl* c, const int32_t* wlist, const long long* row_start, const int32_t* deg,
                               const int32_t* col, const int2* segA, const int2* segD, const int32_t* dstA,
                               const int32_t* dstD, const long long* U_off, uint32_t* U_col, int32_t* U_split,
@@ -76,13 +80,13 @@ __global__ void k_batch_compact_twin(const uint64_t* keys, const Ctl* c, int S, 
 __global__ void k_bfs_expand(Ctl* c, int L, const long long* row_start, const int32_t* deg, const int32_t* col,
                              uint32_t* visited, int32_t* wlist);
 __global__ void k_region_all(Ctl* c, int n, int32_t* wlist);
-// all = 1: every entry of each row (the edge-local path), else N(u) n W
+// N(u) n W and the insertions
 __global__ void k_u_count(const Ctl* c, const int32_t* wlist, const uint32_t* visited, const long long* row_start,
-                          const int32_t* deg, const int32_t* col, const int2* segA, int32_t* U_deg, int all);
+                          const int32_t* deg, const int32_t* col, const int2* segA, int32_t* U_deg);
 __global__ void k_u_fill(const Ctl* c, const int32_t* wlist, const uint32_t* visited, const long long* row_start,
                          const int32_t* deg, const int32_t* col, const int2* segA, const int2* segD,
                          const int32_t* dstA, const int32_t* dstD, const long long* U_off, uint32_t* U_col,
-                         int32_t* U_split, int32_t* da, int32_t* db, int all);
+                         int32_t* U_split, int32_t* da, int32_t* db);
 
 __global__ void k_u_fill_all(const Ctl* c, const int32_t* wlist, const long long* row_start, const int32_t* deg,
                              const int32_t* col, const int2* segA, const int2* segD, const int32_t* dstA,

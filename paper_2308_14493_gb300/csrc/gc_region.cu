@@ -120,7 +120,7 @@ __global__ void k_region_all(Ctl* c, int n, int32_t* __restrict__ wlist) {
 __global__ void k_u_count(const Ctl* c, const int32_t* __restrict__ wlist, const uint32_t* __restrict__ visited,
                           const long long* __restrict__ row_start, const int32_t* __restrict__ deg,
                           const int32_t* __restrict__ col, const int2* __restrict__ segA,
-                          int32_t* __restrict__ U_deg, int all) {
+                          int32_t* __restrict__ U_deg) {
     pdl_enter();
     int nW = c->nW;
     int lane = threadIdx.x & 31;
@@ -128,14 +128,10 @@ __global__ void k_u_count(const Ctl* c, const int32_t* __restrict__ wlist, const
     int nwarps = (gridDim.x * blockDim.x) >> 5;
     for (int i = warp; i < nW; i += nwarps) {
         int32_t u = wlist[i];
-        if (all) {  // the full row and the insertions
-            if (lane == 0) U_deg[u] = deg[u] + (segA[u].y - segA[u].x);
-            continue;
-        }
         const int32_t* row = col + row_start[u];
         int d = deg[u], cnt = 0;
         for (int b = 0; b < d; b += 32) {
-            bool ok = b + lane < d && (all || in_region(visited, row[b + lane]));
+            bool ok = b + lane < d && in_region(visited, row[b + lane]);
             cnt += __popc(__ballot_sync(FULL, ok));
         }
         if (lane == 0) {
@@ -151,7 +147,7 @@ __global__ void k_u_fill(const Ctl* c, const int32_t* __restrict__ wlist, const 
                          const int2* __restrict__ segD, const int32_t* __restrict__ dstA,
                          const int32_t* __restrict__ dstD, const long long* __restrict__ U_off,
                          uint32_t* __restrict__ U_col, int32_t* __restrict__ U_split, int32_t* __restrict__ da,
-                         int32_t* __restrict__ db, int all) {
+                         int32_t* __restrict__ db) {
     pdl_enter();
     int nW = c->nW;
     int lane = threadIdx.x & 31;
@@ -165,7 +161,7 @@ __global__ void k_u_fill(const Ctl* c, const int32_t* __restrict__ wlist, const 
         uint32_t* out = U_col + U_off[u];
         long long len = warp_merge_row(
             col + row_start[u], deg[u], dstA + a.x, na, out, FLAG_A,
-            [&](int32_t v) { return all || in_region(visited, v); },
+            [&](int32_t v) { return in_region(visited, v); },
             [&](int32_t v) { return FLAG_B | ((nd == 0 || !sorted_contains(dl, nd, v)) ? FLAG_A : 0u); });
         __syncwarp();
         if (lane == 0) {
@@ -176,15 +172,9 @@ __global__ void k_u_fill(const Ctl* c, const int32_t* __restrict__ wlist, const 
     }
 }
 
-// Twin pass (two independent batches, W = V): row u of U is N(u) plus the
-// insertions of either batch; the kept entries carry the batches' mask in
-// their two low bits (dst << 2 | mask, one entry per vertex pair, sorted).
-// A G entry loses FLAG_A (FLAG_B) if the first (second) batch deletes it; an
-// insertion has FLAG_A (FLAG_B) if the first (second) batch makes it.  Every
-// entry is placed by binary searches: a row element after the insertions
-// below it, an insertion after the row elements below it.
-__global__ void k_u_count_twin(const Ctl* c, const int32_t* __restrict__ wlist, const int32_t* __restrict__ deg,
-                               const int2* __restrict__ segA, int32_t* __restrict__ U_deg) {
+// W = V: row u of U is all of N(u) plus the insertions.
+__global__ void k_u_count_all(const Ctl* c, const int32_t* __restrict__ wlist, const int32_t* __restrict__ deg,
+                              const int2* __restrict__ segA, int32_t* __restrict__ U_deg) {
     pdl_enter();
     const int nW = c->nW;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < nW; i += gridDim.x * blockDim.x) {
@@ -193,61 +183,196 @@ __global__ void k_u_count_twin(const Ctl* c, const int32_t* __restrict__ wlist, 
     }
 }
 
-__global__ void k_u_fill_twin(const Ctl* c, const int32_t* __restrict__ wlist, const long long* __restrict__ row_start,
-                              const int32_t* __restrict__ deg, const int32_t* __restrict__ col,
-                              const int2* __restrict__ segA, const int2* __restrict__ segD,
-                              const int32_t* __restrict__ dstA, const int32_t* __restrict__ dstD,
-                              const long long* __restrict__ U_off, uint32_t* __restrict__ U_col,
-                              int32_t* __restrict__ U_split, int32_t* __restrict__ da, int32_t* __restrict__ db) {
-    pdl_enter();
-    const int nW = c->nW;
-    const int lane = threadIdx.x & 31;
-    const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int nwarps = (gridDim.x * blockDim.x) >> 5;
-    for (int i = warp; i < nW; i += nwarps) {
-        const int32_t u = wlist[i];
-        const int2 a = segA[u], d = segD[u];
-        const int32_t* A = dstA + a.x;
-        const int32_t* D = dstD + d.x;
-        const long long na = a.y - a.x, nd = d.y - d.x;
-        const int32_t* row = col + row_start[u];
-        const int du = deg[u];
-        uint32_t* out = U_col + U_off[u];
-        for (int p = lane; p < du; p += 32) {
-            const int32_t v = row[p];
-            uint32_t fl = FLAG_A | FLAG_B;
-            if (nd) {
-                const long long q = lower_bound_i32(D, nd, v << 2);
-                if (q < nd && (D[q] >> 2) == v) {
-                    if (D[q] & 1) fl &= ~FLAG_A;
-                    if (D[q] & 2) fl &= ~FLAG_B;
-                }
-            }
-            out[p + (na ? lower_bound_i32(A, na, v << 2) : 0)] = (uint32_t)v | fl;
-        }
-        int cA = 0, cB = 0;  // insertions into G_a / G_b minus deletions from them
-        for (long long q = lane; q < na; q += 32) {
-            const int32_t x = A[q] >> 2, m = A[q] & 3;
-            out[q + lower_bound_i32(row, du, x)] = (uint32_t)x | ((m & 1) ? FLAG_A : 0u) | ((m & 2) ? FLAG_B : 0u);
-            cA += (m & 1) ? 1 : 0;
-            cB += (m & 2) ? 1 : 0;
-        }
-        for (long long q = lane; q < nd; q += 32) {
-            cA -= (D[q] & 1) ? 1 : 0;
-            cB -= (D[q] & 2) ? 1 : 0;
-        }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            cA += __shfl_xor_sync(FULL, cA, o);
-            cB += __shfl_xor_sync(FULL, cB, o);
-        }
-        __syncwarp();
-        if (lane == 0) {
-            U_split[u] = (int32_t)(lower_bound_i32(row, du, u + 1) + (na ? lower_bound_i32(A, na, (u + 1) << 2) : 0));
-            da[u] = du + cA;
-            db[u] = du + cB;
+// Rows of U for W = V.  Every entry is placed by binary searches: a row element
+// after the insertions below it, an insertion after the row elements below it.
+// TWIN (two independent batches): the kept entries carry the batches' mask in
+// their two low bits (dst << 2 | mask, one entry per vertex pair, sorted); a G
+// entry loses FLAG_A (FLAG_B) if the first (second) batch deletes it, an
+// insertion has FLAG_A (FLAG_B) if the first (second) batch makes it.
+//
+// Mostly a copy, bound by memory if enough loads are in flight.  A warp per row
+// had one row's chain of a dozen dependent loads in flight for 30 entries: 2.66
+// ms for the 138 M entries of a 4.8 M-vertex graph, 0.67 now.  So a warp
+// takes 32 rows: a lane reads each row's header, and the lanes copy the rows'
+// entries as one run, four loads ahead.  Long rows go to the whole block.  The
+// rows of a block are spread over the ids in quads, since hubs have
+// neighbouring ids.
+constexpr int UF_T = 256;
+constexpr int U_LONG_ROW = 512;
+constexpr int U_LONG_ROWS = 128;  // a block's list of them (a warp copies each further one)
+struct UfRow {
+    const int32_t* row;
+    const int32_t *A, *D;
+    uint32_t* out;
+    int du, na, nd;
+};
+template <bool TWIN>
+__device__ __forceinline__ void uf_entry(const UfRow& r, int p, int32_t v) {
+    uint32_t fl = FLAG_A | FLAG_B;
+    const int32_t key = TWIN ? v << 2 : v;
+    if (r.nd) {
+        const long long q = lower_bound_i32(r.D, r.nd, key);
+        if (q < r.nd) {
+            const int32_t d = r.D[q];
+            if (TWIN ? (d >> 2) == v : d == v)
+                fl = TWIN ? fl & ~(((d & 1) ? FLAG_A : 0u) | ((d & 2) ? FLAG_B : 0u)) : FLAG_B;
         }
     }
+    r.out[p + (r.na ? lower_bound_i32(r.A, r.na, key) : 0)] = (uint32_t)v | fl;
+}
+template <bool TWIN>
+__device__ __forceinline__ void uf_insertion(const UfRow& r, int q) {
+    const int32_t a = r.A[q], x = TWIN ? a >> 2 : a;
+    const uint32_t fl = TWIN ? ((a & 1) ? FLAG_A : 0u) | ((a & 2) ? FLAG_B : 0u) : FLAG_A;
+    r.out[q + lower_bound_i32(r.row, r.du, x)] = (uint32_t)x | fl;
+}
+// inclusive prefix sums over the lanes to pre[1 ..], pre[0] = 0; the total
+__device__ __forceinline__ int uf_prefix(int x, int* pre) {
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(FULL, x, o);
+        if (lane >= o) x += y;
+    }
+    pre[lane + 1] = x;
+    if (lane == 0) pre[0] = 0;
+    __syncwarp();
+    return __shfl_sync(FULL, x, 31);
+}
+template <bool TWIN>
+__device__ __forceinline__ void u_fill_rows(const Ctl* c, const int32_t* __restrict__ wlist,
+                                            const long long* __restrict__ row_start, const int32_t* __restrict__ deg,
+                                            const int32_t* __restrict__ col, const int2* __restrict__ segA,
+                                            const int2* __restrict__ segD, const int32_t* __restrict__ dstA,
+                                            const int32_t* __restrict__ dstD, const long long* __restrict__ U_off,
+                                            uint32_t* __restrict__ U_col, int32_t* __restrict__ U_split,
+                                            int32_t* __restrict__ da, int32_t* __restrict__ db) {
+    __shared__ UfRow s_row[UF_T], s_long[U_LONG_ROWS];
+    __shared__ int s_pre[UF_T / 32][2][33];
+    __shared__ int32_t s_longu[U_LONG_ROWS];
+    __shared__ int s_nlong, s_cnt[2];
+    const int nW = c->nW, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    UfRow* const rows = s_row + 32 * warp;
+    int(*const pre)[33] = s_pre[warp];
+    if (tid == 0) s_nlong = 0;
+    __syncthreads();
+    // quad (it, tid / 4) of this block: vertices 4 ((64 it + tid / 4) grid + block) ..
+    for (long long it = 0; it * UF_T * gridDim.x + 4ll * blockIdx.x < nW; it++) {
+        const long long i = ((it * (UF_T / 4) + (tid >> 2)) * gridDim.x + blockIdx.x) * 4 + (tid & 3);
+        UfRow r{};
+        int32_t u = 0;
+        bool over = false;  // long, and the list is full
+        if (i < nW) {
+            u = wlist[i];
+            const int2 a = segA[u], d = segD[u];
+            r.row = col + row_start[u];
+            r.A = dstA + a.x;
+            r.D = dstD + d.x;
+            r.out = U_col + U_off[u];
+            r.du = deg[u];
+            r.na = a.y - a.x;
+            r.nd = d.y - d.x;
+            U_split[u] = (int32_t)(lower_bound_i32(r.row, r.du, u + 1) +
+                                   (r.na ? lower_bound_i32(r.A, r.na, TWIN ? (u + 1) << 2 : u + 1) : 0));
+            if ((long long)r.du + r.na > U_LONG_ROW) {
+                const int at = atomicAdd(&s_nlong, 1);
+                over = at >= U_LONG_ROWS;
+                if (!over) {
+                    s_long[at] = r;
+                    s_longu[at] = u;
+                    r.du = r.na = r.nd = 0;
+                    u = -1;
+                }
+            }
+        }
+        rows[lane] = r;
+        const int total = uf_prefix(over ? 0 : r.du, pre[0]);
+        int q = 0;
+        for (int b = lane; b < total; b += 128) {
+            int at[4], p[4];
+            int32_t v[4];
+#pragma unroll
+            for (int k = 0; k < 4; k++) {
+                const int j = b + 32 * k;
+                if (j < total)
+                    while (pre[0][q + 1] <= j) q++;
+                at[k] = q;
+                p[k] = j - pre[0][q];
+                v[k] = j < total ? rows[q].row[p[k]] : 0;
+            }
+#pragma unroll
+            for (int k = 0; k < 4; k++)
+                if (b + 32 * k < total) uf_entry<TWIN>(rows[at[k]], p[k], v[k]);
+        }
+        if (__any_sync(FULL, r.na != 0 && !over)) {
+            const int ins = uf_prefix(over ? 0 : r.na, pre[1]);
+            q = 0;
+            for (int j = lane; j < ins; j += 32) {
+                while (pre[1][q + 1] <= j) q++;
+                uf_insertion<TWIN>(rows[q], j - pre[1][q]);
+            }
+        }
+        for (unsigned m = __ballot_sync(FULL, over); m; m &= m - 1) {
+            const UfRow l = rows[__ffs(m) - 1];
+            for (int p = lane; p < l.du; p += 32) uf_entry<TWIN>(l, p, l.row[p]);
+            for (int p = lane; p < l.na; p += 32) uf_insertion<TWIN>(l, p);
+        }
+        if (i < nW && u >= 0) {
+            int cA = r.na - r.nd, cB = 0;  // insertions into G_a / G_b minus deletions from them
+            if (TWIN) {
+                cA = 0;
+                for (int k = 0; k < r.na; k++) cA += r.A[k] & 1, cB += (r.A[k] >> 1) & 1;
+                for (int k = 0; k < r.nd; k++) cA -= r.D[k] & 1, cB -= (r.D[k] >> 1) & 1;
+            }
+            da[u] = r.du + cA;
+            db[u] = r.du + cB;
+        }
+        __syncwarp();
+    }
+    __syncthreads();
+    for (int k = 0; k < min(s_nlong, U_LONG_ROWS); k++) {
+        const UfRow l = s_long[k];
+#pragma unroll 4
+        for (int p = tid; p < l.du; p += UF_T) uf_entry<TWIN>(l, p, l.row[p]);
+        for (int q = tid; q < l.na; q += UF_T) uf_insertion<TWIN>(l, q);
+        if (tid < 2) s_cnt[tid] = 0;
+        __syncthreads();
+        if (TWIN && l.na + l.nd) {
+            int cA = 0, cB = 0;
+            for (int j = tid; j < l.na; j += UF_T) cA += l.A[j] & 1, cB += (l.A[j] >> 1) & 1;
+            for (int j = tid; j < l.nd; j += UF_T) cA -= l.D[j] & 1, cB -= (l.D[j] >> 1) & 1;
+            cA = __reduce_add_sync(FULL, cA);
+            cB = __reduce_add_sync(FULL, cB);
+            if (lane == 0) {
+                atomicAdd(&s_cnt[0], cA);
+                atomicAdd(&s_cnt[1], cB);
+            }
+        }
+        __syncthreads();
+        if (tid == 0) {
+            da[s_longu[k]] = l.du + (TWIN ? s_cnt[0] : l.na - l.nd);
+            db[s_longu[k]] = l.du + (TWIN ? s_cnt[1] : 0);
+        }
+        __syncthreads();
+    }
+}
+__global__ void __launch_bounds__(UF_T, 6) k_u_fill_rows(
+    const Ctl* c, const int32_t* __restrict__ wlist, const long long* __restrict__ row_start,
+    const int32_t* __restrict__ deg, const int32_t* __restrict__ col, const int2* __restrict__ segA,
+    const int2* __restrict__ segD, const int32_t* __restrict__ dstA, const int32_t* __restrict__ dstD,
+    const long long* __restrict__ U_off, uint32_t* __restrict__ U_col, int32_t* __restrict__ U_split,
+    int32_t* __restrict__ da, int32_t* __restrict__ db) {
+    pdl_enter();
+    u_fill_rows<false>(c, wlist, row_start, deg, col, segA, segD, dstA, dstD, U_off, U_col, U_split, da, db);
+}
+__global__ void __launch_bounds__(UF_T, 6) k_u_fill_twin(
+    const Ctl* c, const int32_t* __restrict__ wlist, const long long* __restrict__ row_start,
+    const int32_t* __restrict__ deg, const int32_t* __restrict__ col, const int2* __restrict__ segA,
+    const int2* __restrict__ segD, const int32_t* __restrict__ dstA, const int32_t* __restrict__ dstD,
+    const long long* __restrict__ U_off, uint32_t* __restrict__ U_col, int32_t* __restrict__ U_split,
+    int32_t* __restrict__ da, int32_t* __restrict__ db) {
+    pdl_enter();
+    u_fill_rows<true>(c, wlist, row_start, deg, col, segA, segD, dstA, dstD, U_off, U_col, U_split, da, db);
 }
 
 // Union rows over the full adjacency (the edge-local path): a block per
