@@ -202,6 +202,14 @@ struct C4Task {
     float wt;
 };
 
+// The lowest bit of each of the word's counters (32 >> s bits) that is 2 or more.
+__device__ __forceinline__ uint32_t counters_above_1(uint32_t w, int s) {
+    return s == 3   ? ((w >> 1) | (w >> 2) | (w >> 3)) & 0x11111111u
+           : s == 2 ? __vcmpgtu4(w, 0x01010101u) & 0x01010101u
+           : s == 1 ? __vcmpgtu2(w, 0x00010001u) & 0x00010001u
+                    : (w > 1 ? 1u : 0u);
+}
+
 // The pivots of BIN_C4_DENSE, a block per (chunk, pivot).  Bound by issue
 // slots (about 60 instructions per 32 wedges, a third of them the short
 // runs' bookkeeping) and by the chain of three loads that starts each group
@@ -320,14 +328,19 @@ __global__ void __launch_bounds__(THREADS, MINB) k_c4_pivot(PivotArgs a, int c0)
             if (MODE == C4_EDGE) {
                 for (int i = tid; i < (used + 3) / 4; i += THREADS) c4[i] = make_uint4(0, 0, 0, 0);
             } else {
-                for (int i = tid; i < used; i += THREADS) {
-                    uint32_t w = cnt[i];
-                    if (!w) continue;
-                    cnt[i] = 0;
-                    for (int b = 0; w; b++, w = s ? w >> (32 >> s) : 0u) {
-                        const unsigned long long c = w & cmask;
-                        if (c >= 2) red_u64(&a.credit[lo + ((uint32_t)i << s) + b], c * (c - 1) / 2);
-                    }
+                // C(c, 2) to every id counted twice or more
+                for (int i = tid; i < (used + 3) / 4; i += THREADS) {
+                    const uint4 v = c4[i];
+                    if (!(v.x | v.y | v.z | v.w)) continue;
+                    c4[i] = make_uint4(0, 0, 0, 0);
+                    const uint32_t w4[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+                    for (int k = 0; k < 4; k++)
+                        for (uint32_t m = counters_above_1(w4[k], s); m; m &= m - 1) {
+                            const int sh = __ffs(m) - 1;
+                            const unsigned long long c = (w4[k] >> sh) & cmask;
+                            red_u64(&a.credit[lo + ((uint32_t)(4 * i + k) << s) + (sh >> ls)], c * (c - 1) / 2);
+                        }
                 }
             }
             __syncthreads();

@@ -46,7 +46,8 @@ __device__ __forceinline__ Deal deal_groups(int nlow, float wedges, int warps) {
 // walked by all lanes, shorter ones by eight lanes a run, four loads in flight
 // per lane.  fn(q, e, f, x), which the whole warp calls together, takes four
 // entries at a time: q[i] the address (null: none), e[i] the entry, f[i] the
-// neighbour's entry; with ACC it returns credits in x[i], which are summed over
+// neighbour's entry; with ACC it returns credits in x[i] (0 where q[i] is null;
+// below 2^28, as the lower neighbours of a pivot are), which are summed over
 // each run and given to rowfn(sum, fv, jr) by one lane.
 template <bool ACC, class Fn, class RowFn>
 __device__ __forceinline__ void walk_group(const uint32_t* p, int len, uint32_t fv, int jr, WarpRuns& W, Fn fn,
@@ -76,10 +77,7 @@ __device__ __forceinline__ void walk_group(const uint32_t* p, int len, uint32_t 
                 e[i] = q[i] ? *q[i] : 0u;
             }
             fn(q, e, f, x);
-            if (ACC) {
-#pragma unroll
-                for (int i = 0; i < PV_UNROLL; i++) acc += q[i] ? x[i] : 0u;
-            }
+            if (ACC) acc += x[0] + x[1] + x[2] + x[3];
         }
         if (ACC) {
             acc = warp_sum_u64(acc);
@@ -130,7 +128,7 @@ __device__ __forceinline__ void walk_group(const uint32_t* p, int len, uint32_t 
                     if (rc >= 0) flush();
                     rc = ri[i];
                 }
-                acc += q[i] ? x[i] : 0u;
+                acc += x[i];
             }
         }
     }
