@@ -119,35 +119,118 @@ __device__ __forceinline__ int find_id(const uint32_t* s, int k, uint32_t y) {
     return (lo < k && s[lo] == y) ? lo : -1;
 }
 
+// 64-bit sum in two shared words (a 64-bit shared atomic is a loop).
+struct Sum64 {
+    uint32_t lo, hi;
+    __device__ __forceinline__ void add(uint32_t x) {
+        if (atomicAdd(&lo, x) > ~x) atomicAdd(&hi, 1u);
+    }
+    __device__ __forceinline__ unsigned long long get() const { return ((unsigned long long)hi << 32) | lo; }
+};
+
 // Shared state of one root with up to KM kept entries.
 template <bool EDGE, int KM>
 struct RootState {
     long long nb[KM];                 // start of N+(X[q])
-    unsigned long long c0[KM];        // per vertex: D2 of X[q]; per edge: E_OPP of (u, X[q])
-    unsigned long long c1[EDGE ? KM : 1];  // E_OUTER of (u, X[q])
+    Sum64 t3[EDGE ? KM : 1];          // sum of t of the edges (X[q], X[p]) over its triangles
     uint32_t x[KM];                   // ids
     uint32_t t[KM];                   // t of (u, X[q])
     int pre[KM + 1];                  // candidates before row q
     int at[KM];                       // position in u's out-list
     int dg[EDGE ? KM : 1];            // degrees
+    uint32_t bloom[KM];               // a bit per hashed id of X
 };
 
-// One triangle (u, X[q], X[p]) whose third edge is entry `slot`.
+// A candidate that passed the filter: id, its row q, its number.
+struct Candidate {
+    uint32_t y;
+    int q, j;
+};
+
+__device__ __forceinline__ uint32_t lt_hash(uint32_t y, int km) { return __umulhi(y * 0x9E3779B1u, 32u * km); }
+
+// The candidates lo .. hi - 1 of a root (rows of X one after the other) by one
+// warp: those that a bit filter of X lets pass are queued, and 32 at a time
+// searched in X; hit(q, p, slot) for each entry `slot` = (X[q], X[p]).
+template <bool EDGE, int KM, class Hit>
+__device__ __forceinline__ void walk_candidates(const RootState<EDGE, KM>& S, int k, int lo, int hi,
+                                                const uint32_t* __restrict__ U_col, Candidate* queue, Hit hit) {
+    const int lane = threadIdx.x & 31;
+    int q = 0, end = k, nq = 0;  // q: row of candidate lo
+    while (end - q > 1) {
+        const int mid = (q + end) >> 1;
+        if (S.pre[mid] <= lo) q = mid;
+        else end = mid;
+    }
+    auto drain = [&](int n) {
+        if (lane < n) {
+            const Candidate c = queue[nq + lane];
+            const int p = find_id(S.x, k, c.y);
+            if (p >= 0) hit(c.q, p, S.nb[c.q] + (c.j - S.pre[c.q]));
+        }
+        __syncwarp();
+    };
+    for (int base = lo; base < hi; base += 128) {
+        uint32_t y[4];
+        int row[4];
+#pragma unroll
+        for (int i = 0; i < 4; i++) {
+            const int j = base + 32 * i + lane;
+            if (j < hi)
+                while (q + 1 < k && S.pre[q + 1] <= j) q++;
+            row[i] = q;
+            y[i] = j < hi ? vid(U_col[S.nb[q] + (j - S.pre[q])]) : 0u;
+        }
+#pragma unroll
+        for (int i = 0; i < 4; i++) {
+            const int j = base + 32 * i + lane;
+            const uint32_t h = lt_hash(y[i], KM);
+            const bool pass = j < hi && ((S.bloom[h >> 5] >> (h & 31)) & 1u);
+            const unsigned m = __ballot_sync(FULL, pass);
+            if (pass) queue[nq + __popc(m & lanemask_lt())] = Candidate{y[i], row[i], j};
+            nq += __popc(m);
+            __syncwarp();
+            if (nq >= 32) {
+                nq -= 32;
+                drain(32);
+            }
+        }
+    }
+    const int left = nq;
+    nq = 0;
+    drain(left);
+}
+
+// Credits of one triangle (u, X[q], X[p]) that the bit rows do not give: its
+// third edge is entry `slot`.
 template <bool EDGE, int KM>
 __device__ __forceinline__ void credit_triangle(RootState<EDGE, KM>& S, int q, int p, long long slot, uint32_t t3,
                                                 long long du, const TriCredits& cr, unsigned long long& mine) {
-    const unsigned long long tq = S.t[q], tp = S.t[p];
     if (EDGE) {
-        atomicAdd(&S.c0[q], (unsigned long long)(S.dg[p] - 2));
-        atomicAdd(&S.c1[q], tp + t3 - 2);
-        atomicAdd(&S.c0[p], (unsigned long long)(S.dg[q] - 2));
-        atomicAdd(&S.c1[p], tq + t3 - 2);
+        S.t3[q].add(t3);
+        S.t3[p].add(t3);
         add_u64(&cr.to[2 * slot], (unsigned long long)(du - 2));
-        add_u64(&cr.to[2 * slot + 1], tq + tp - 2);
+        add_u64(&cr.to[2 * slot + 1], (unsigned long long)S.t[q] + S.t[p] - 2);
     } else {
         mine += t3 - 1;
-        if (tp > 1) atomicAdd(&S.c0[q], tp - 1);
-        if (tq > 1) atomicAdd(&S.c0[p], tq - 1);
+    }
+}
+
+// Credits of (u, X[q]) or X[q] from its bit row (n: partners p; each(fn) runs
+// fn(p) over them): 4-cliques n3, and per vertex t of the opposite edges - 1,
+// per edge the opposite corners' degrees - 2 and the outer edges' t - 2.
+template <bool EDGE, int KM>
+__device__ __forceinline__ void credit_member(const RootState<EDGE, KM>& S, int q, long long rb, uint64_t n,
+                                              unsigned long long sum, unsigned long long tsum, uint64_t n3,
+                                              const TriCredits& cr) {
+    if (EDGE) {
+        const long long e = rb + S.at[q];
+        add_u64(&cr.to[2 * e], sum - 2 * n);
+        add_u64(&cr.to[2 * e + 1], tsum + S.t3[q].get() - 2 * n);
+        add_u64(&cr.k4e[e], n3);
+    } else {
+        add_u64(&cr.d2[S.x[q]], tsum - n);
+        add_u64(&cr.k4v[S.x[q]], n3);
     }
 }
 
@@ -157,6 +240,7 @@ template <bool EDGE>
 struct WarpRoot {
     RootState<EDGE, 32> r;
     uint32_t row[32];
+    Candidate queue[64];
 };
 template <bool EDGE>
 __global__ void __launch_bounds__(LT_WARPS * 32) k_l_tri_warp(const Ctl* c, const int32_t* __restrict__ list,
@@ -204,21 +288,17 @@ __global__ void __launch_bounds__(LT_WARPS * 32) k_l_tri_warp(const Ctl* c, cons
         S.pre[lane + 1] = inc;
         if (lane == 0) S.pre[0] = 0;
         W.row[lane] = 0;
-        S.c0[lane] = 0;
-        if (EDGE) S.c1[lane] = 0;
+        S.bloom[lane] = 0;
+        if (EDGE) S.t3[lane] = Sum64{0, 0};
+        __syncwarp();
+        if (lane < k) {
+            const uint32_t h = lt_hash(S.x[lane], 32);
+            atomicOr(&S.bloom[h >> 5], 1u << (h & 31));
+        }
         __syncwarp();
         unsigned long long mine = 0;
         const long long du = ue - ub;
-        auto walk = [&](auto hit) {
-            int q = 0;
-            for (int j = lane; j < total; j += 32) {
-                while (q + 1 < k && S.pre[q + 1] <= j) q++;
-                const long long slot = S.nb[q] + (j - S.pre[q]);
-                const int p = find_id(S.x, k, vid(U_col[slot]));
-                if (p >= 0) hit(q, p, slot);
-            }
-        };
-        walk([&](int q, int p, long long slot) {
+        walk_candidates(S, k, 0, total, U_col, W.queue, [&](int q, int p, long long slot) {
             atomicOr(&W.row[q], 1u << p);
             atomicOr(&W.row[p], 1u << q);
             credit_triangle<EDGE, 32>(S, q, p, slot, tall[slot], du, cr, mine);
@@ -227,26 +307,23 @@ __global__ void __launch_bounds__(LT_WARPS * 32) k_l_tri_warp(const Ctl* c, cons
         unsigned n3 = 0;  // 4-cliques through u and X[lane]
         if (lane < k) {
             const uint32_t s = W.row[lane];
-            for (uint32_t m = s; m; m &= m - 1) n3 += __popc(s & W.row[__ffs(m) - 1]);
+            unsigned long long sum = 0, tsum = 0;
+            for (uint32_t m = s; m; m &= m - 1) {
+                const int p = __ffs(m) - 1;
+                n3 += __popc(s & W.row[p]);
+                tsum += S.t[p];
+                if (EDGE) sum += (unsigned)S.dg[p];
+            }
             n3 /= 2;
+            credit_member<EDGE, 32>(S, lane, rb, __popc(s), sum, tsum, n3, cr);
         }
         const unsigned any = __ballot_sync(FULL, n3 > 0);
         if (EDGE) {
-            if (lane < k) {
-                const long long e = rb + S.at[lane];
-                add_u64(&cr.to[2 * e], S.c0[lane]);
-                add_u64(&cr.to[2 * e + 1], S.c1[lane]);
-                add_u64(&cr.k4e[e], n3);
-            }
             if (any)
-                walk([&](int q, int p, long long slot) {
+                walk_candidates(S, k, 0, total, U_col, W.queue, [&](int q, int p, long long slot) {
                     add_u64(&cr.k4e[slot], (unsigned long long)__popc(W.row[q] & W.row[p]));
                 });
         } else {
-            if (lane < k) {
-                add_u64(&cr.d2[S.x[lane]], S.c0[lane]);
-                add_u64(&cr.k4v[S.x[lane]], n3);
-            }
             mine = warp_sum_u64(mine);
             const unsigned all = any ? __reduce_add_sync(FULL, n3) : 0u;
             if (lane == 0) {
@@ -262,7 +339,8 @@ __global__ void __launch_bounds__(LT_WARPS * 32) k_l_tri_warp(const Ctl* c, cons
 template <bool EDGE, int KM>
 struct BlockRoot {
     RootState<EDGE, KM> r;
-    uint32_t row[KM * (KM / 32)];
+    uint32_t row[KM * (KM / 32 | 1)];
+    Candidate queue[8][64];
 };
 template <bool EDGE, int KM, int BIN, int WORK>
 __global__ void __launch_bounds__(256) k_l_tri_block(Ctl* c, const int32_t* __restrict__ list,
@@ -306,7 +384,7 @@ __global__ void __launch_bounds__(256) k_l_tri_block(Ctl* c, const int32_t* __re
             if (lane == 0) s_k = k;
         }
         __syncthreads();
-        const int k = s_k, W = (k + 31) >> 5;
+        const int k = s_k, W = (k + 31) >> 5, ST = W | 1;  // (odd stride: no bank conflicts)
         if (k < 2) {
             __syncthreads();
             continue;
@@ -318,11 +396,15 @@ __global__ void __launch_bounds__(256) k_l_tri_block(Ctl* c, const int32_t* __re
             S.nb[q] = nb;
             if (EDGE) S.dg[q] = (int)(ve - vb);
             S.pre[q + 1] = (int)lower_bound_id(U_col + nb, ve - nb, xmax + 1);
-            S.c0[q] = 0;
-            if (EDGE) S.c1[q] = 0;
+            if (EDGE) S.t3[q] = Sum64{0, 0};
         }
-        for (int j = tid; j < k * W; j += blockDim.x) B.row[j] = 0;
+        for (int j = tid; j < k * ST; j += blockDim.x) B.row[j] = 0;
+        for (int j = tid; j < KM; j += blockDim.x) S.bloom[j] = 0;
         __syncthreads();
+        for (int q = tid; q < k; q += blockDim.x) {
+            const uint32_t h = lt_hash(S.x[q], KM);
+            atomicOr(&S.bloom[h >> 5], 1u << (h & 31));
+        }
         if (warp == 0) {  // inclusive scan of pre[1..k]
             int carry = 0;
             for (int b = 0; b < k; b += 32) {
@@ -340,56 +422,40 @@ __global__ void __launch_bounds__(256) k_l_tri_block(Ctl* c, const int32_t* __re
         __syncthreads();
         const int total = S.pre[k];
         unsigned long long mine = 0;
-        auto walk = [&](auto hit) {
-            for (int base = warp * 32; base < total; base += NW * 32) {
-                int q = 0, hi = k;  // row of candidate `base`
-                while (hi - q > 1) {
-                    const int mid = (q + hi) >> 1;
-                    if (S.pre[mid] <= base) q = mid;
-                    else hi = mid;
-                }
-                const int j = base + lane;
-                if (j >= total) continue;
-                while (q + 1 < k && S.pre[q + 1] <= j) q++;
-                const long long slot = S.nb[q] + (j - S.pre[q]);
-                const int p = find_id(S.x, k, vid(U_col[slot]));
-                if (p >= 0) hit(q, p, slot);
-            }
-        };
-        walk([&](int q, int p, long long slot) {
-            atomicOr(&B.row[q * W + (p >> 5)], 1u << (p & 31));
-            atomicOr(&B.row[p * W + (q >> 5)], 1u << (q & 31));
+        const int lo = (int)((long long)total * warp / NW), hi = (int)((long long)total * (warp + 1) / NW);
+        walk_candidates(S, k, lo, hi, U_col, B.queue[warp], [&](int q, int p, long long slot) {
+            atomicOr(&B.row[q * ST + (p >> 5)], 1u << (p & 31));
+            atomicOr(&B.row[p * ST + (q >> 5)], 1u << (q & 31));
             credit_triangle<EDGE, KM>(S, q, p, slot, tall[slot], du, cr, mine);
         });
         __syncthreads();
         unsigned long long all = 0;
         for (int q = tid; q < k; q += blockDim.x) {
-            const uint32_t* s = B.row + q * W;
-            unsigned long long n3 = 0;  // 4-cliques through u and X[q], twice
+            const uint32_t* s = B.row + q * ST;
+            unsigned long long n3 = 0, sum = 0, tsum = 0;  // n3: 4-cliques through u and X[q], twice
+            unsigned n = 0;
             for (int i = 0; i < W; i++)
                 for (uint32_t m = s[i]; m; m &= m - 1) {
-                    const uint32_t* r = B.row + (i * 32 + __ffs(m) - 1) * W;
-                    for (int j = 0; j < W; j++) n3 += __popc(s[j] & r[j]);
+                    const int p = i * 32 + __ffs(m) - 1;
+                    const uint32_t* r = B.row + p * ST;
+                    unsigned x = 0;
+                    for (int j = 0; j < W; j++) x += __popc(s[j] & r[j]);
+                    n3 += x;
+                    tsum += S.t[p];
+                    if (EDGE) sum += (unsigned)S.dg[p];
+                    n++;
                 }
             n3 /= 2;
             all += n3;
-            if (EDGE) {
-                const long long e = rb + S.at[q];
-                add_u64(&cr.to[2 * e], S.c0[q]);
-                add_u64(&cr.to[2 * e + 1], S.c1[q]);
-                add_u64(&cr.k4e[e], n3);
-            } else {
-                add_u64(&cr.d2[S.x[q]], S.c0[q]);
-                add_u64(&cr.k4v[S.x[q]], n3);
-            }
+            credit_member<EDGE, KM>(S, q, rb, n, sum, tsum, n3, cr);
         }
         if (EDGE) {
             if (all) s_any = 1;
             __syncthreads();
             if (s_any)
-                walk([&](int q, int p, long long slot) {
+                walk_candidates(S, k, lo, hi, U_col, B.queue[warp], [&](int q, int p, long long slot) {
                     unsigned x = 0;
-                    for (int j = 0; j < W; j++) x += __popc(B.row[q * W + j] & B.row[p * W + j]);
+                    for (int j = 0; j < W; j++) x += __popc(B.row[q * ST + j] & B.row[p * ST + j]);
                     add_u64(&cr.k4e[slot], x);
                 });
         } else {
