@@ -1790,6 +1790,16 @@ int gc_counts_all(const gc_graph* g, uint64_t out[22]) {
     return GC_OK;
 }
 
+static SideStreams side_streams(const gc_graph* g) {
+    SideStreams o;
+    for (int i = 0; i < 3 && !g->opt.serial_count; i++) {
+        o.aux[i] = g->aux[i];
+        o.join[i] = g->join[i];
+    }
+    o.fork = g->fork;
+    return o;
+}
+
 static int vertex_counts(gc_graph* g, uint64_t* out, int orbits) {
     if (!g || (!out && g->n > 0)) return GC_EINVAL;
     if (!on_device(g)) {
@@ -1843,6 +1853,7 @@ static int vertex_counts(gc_graph* g, uint64_t* out, int orbits) {
     va.out = dout;
     va.orbits = orbits;
     va.sms = g->sms;
+    va.side = side_streams(g);
     if (ce == cudaSuccess) {
         g->launches += enqueue_vertex_counts(va, s);
         ce = cudaEventRecord(g->e1, s);
@@ -1947,6 +1958,7 @@ static int edge_counts(gc_graph* g, int32_t* edges, uint64_t* out, int orbits) {
     ea.edges = dedges;
     ea.orbits = orbits;
     ea.sms = g->sms;
+    ea.side = side_streams(g);
     if (ce == cudaSuccess) {
         g->launches += enqueue_edge_counts(ea, s);
         ce = cudaEventRecord(g->e1, s);

@@ -170,6 +170,24 @@ __global__ void k_t2_from_region(const Ctl* c, const int32_t* wlist, const long 
 // Enqueue the edge-local delta (after the union rows of V_X).
 int enqueue_local(const LocalArgs& a, cudaStream_t s, int commit);
 
+// Streams for the independent kernels of the local counts, between a fork and a
+// join on the handle's stream (null: all on that stream).
+struct SideStreams {
+    cudaStream_t aux[3] = {};
+    cudaEvent_t fork = nullptr, join[3] = {};
+    cudaStream_t on(int i, cudaStream_t s) const { return aux[i] ? aux[i] : s; }
+    void begin(cudaStream_t s) const {
+        if (aux[0]) cudaEventRecord(fork, s);
+        for (int i = 0; i < 3 && aux[0]; i++) cudaStreamWaitEvent(aux[i], fork, 0);
+    }
+    void end(cudaStream_t s) const {
+        for (int i = 0; i < 3 && aux[0]; i++) {
+            cudaEventRecord(join[i], aux[i]);
+            cudaStreamWaitEvent(s, join[i], 0);
+        }
+    }
+};
+
 // Per-vertex and per-edge graphlet counts after a static pass with the credits
 // of its 4-cycles (gc_vertex.cu).
 struct VertexArgs {
@@ -190,6 +208,7 @@ struct VertexArgs {
     unsigned long long* out;       // 6 n (graphlets) or 11 n (orbits), by external id
     int orbits;
     int sms;
+    SideStreams side;
 };
 // Returns the kernels launched.
 int enqueue_vertex_counts(const VertexArgs& a, cudaStream_t s);
@@ -223,6 +242,7 @@ struct EdgeArgs {
     int32_t* edges;                // 2 m: (lo, hi) per output row
     int orbits;
     int sms;
+    SideStreams side;
 };
 // Returns the kernels launched.
 int enqueue_edge_counts(const EdgeArgs& a, cudaStream_t s);
