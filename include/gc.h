@@ -55,7 +55,9 @@ typedef struct {
        stream), or NULL, which makes the call that needed it return
        GC_ENOMEM with the graph and its counts unchanged; free releases a
        pointer alloc returned, in the order of `stream`.  NULL for both: the
-       library uses cudaMallocAsync / cudaFreeAsync on its stream.  The
+       library uses cudaMallocAsync / cudaFreeAsync on its stream (the scratch
+       of the local counts from a pool that keeps up to 2 GiB per device
+       mapped until the last such handle closes).  The
        Python binding's TorchAllocator passes PyTorch's caching allocator. */
     void *(*alloc)(size_t bytes, void *stream, void *ctx);
     void (*free)(void *ptr, void *stream, void *ctx);
