@@ -896,8 +896,8 @@ static int enqueue_batch(gc_graph* g, long long max_nk, bool commit, bool local 
                        g->col, g->keepA.p, g->keepD.p);
         g->launches++;
         int sg = scan_grid(nkb, g->sms);
-        g->launches += scan_i32_to_i64(g->keepA.p, g->posA.p, &g->ctl->nkeys, 0, g->bsum.p, sg, &g->ctl->nA2, s);
-        g->launches += scan_i32_to_i64(g->keepD.p, g->posD.p, &g->ctl->nkeys, 0, g->bsum.p, sg, &g->ctl->nD2, s);
+        g->launches += scan2_i32_to_i64(g->keepA.p, g->posA.p, &g->ctl->nA2, g->keepD.p, g->posD.p, &g->ctl->nD2,
+                                        &g->ctl->nkeys, g->bsum.p, sg, s);
         if (twin)
             pdl_launch(k_batch_compact_twin, dim3(ge), dim3(TPB), 0, s, g->keys.p, g->ctl, g->S, g->keepA.p,
                        g->keepD.p, g->posA.p, g->posD.p, g->srcA.p, g->dstA.p, g->srcD.p, g->dstD.p);
@@ -1561,7 +1561,7 @@ static int open_device(gc_graph* g, const int32_t* row_ptr, const int32_t* colh)
         !g->row_start || !g->U_off || !g->U_wt || !g->ctl || !g->segA || !g->segD || !g->visited)
         return nomem(g, "graph state");
     if (ensure_desc(g, 16)) return GC_ENOMEM;
-    if (!ensure(g, g->bsum, 1024)) return nomem(g, "scan scratch");
+    if (!ensure(g, g->bsum, 2048)) return nomem(g, "scan scratch");
     CK(cudaMemsetAsync(g->segA, 0, sizeof(int2) * nn, s));
     CK(cudaMemsetAsync(g->segD, 0, sizeof(int2) * nn, s));
     Ctl zero{};

@@ -345,10 +345,13 @@ int radix_sort_u64(uint64_t* keys, uint64_t* tmp, const long long* d_count, long
                    uint32_t* hist, int grid, cudaStream_t s);
 int radix_grid(long long max_count, int sms);
 // Exclusive prefix sum of int32 in[0..len) into int64 out[0..len], out[len] = total.
-// len = *d_len when d_len != null, else host_len.  `bsum` holds `grid` int64.
+// len = *d_len when d_len != null, else host_len.  `bsum` holds 2,048 int64.
 // If total_out != null the total is also stored there.
 int scan_i32_to_i64(const int32_t* in, long long* out, const long long* d_len, long long host_len,
                     long long* bsum, int grid, long long* total_out, cudaStream_t s);
+// Two of them of the same length *d_len in the same launches.
+int scan2_i32_to_i64(const int32_t* in0, long long* out0, long long* total0, const int32_t* in1, long long* out1,
+                     long long* total1, const long long* d_len, long long* bsum, int grid, cudaStream_t s);
 int scan_grid(long long max_len, int sms);
 
 }  // namespace gcx

@@ -154,7 +154,7 @@ struct LocalArgs {
     long long* dtri2;              // n zeroed words: its change in the batch (cleared after)
     uint32_t* visited2;            // n bits, zeroed: third vertices already listed
     int32_t* wlist_w;              // = wlist (third vertices are appended after V_X)
-    long long* bsum;               // 1024 words
+    long long* bsum;               // 2048 words
     long long cap;
     int n;                         // vertex id bound (U_off has n + 1 entries)
     int sms;
@@ -229,7 +229,7 @@ struct EdgeArgs {
     const unsigned long long* c4;  // nU: 4-cycle credits of each entry
     int32_t* outdeg;               // n
     long long* out_off;            // n + 1
-    long long* bsum;               // 1024
+    long long* bsum;               // 2048
     unsigned long long* keys;      // m sort keys
     unsigned long long* keys_tmp;  // m
     uint32_t* hist;                // 256 sort_grid

@@ -1335,8 +1335,8 @@ int enqueue_local(const LocalArgs& a, cudaStream_t s, int commit) {
     pdl_launch(k_loc_pair_cost, dim3(gw), dim3(tpb), 0, s, a.ctl, V, a.srcA, a.dstA, a.srcD, a.dstD, a.pcost, a.ccnt,
                a.walk);
     nl++;
-    nl += scan_i32_to_i64(a.pcost, a.ppre, &a.ctl->l_len[1], 0, a.bsum, sg, &a.ctl->l_tot[1], s);
-    nl += scan_i32_to_i64(a.ccnt, a.cpre, &a.ctl->l_len[1], 0, a.bsum, sg, &a.ctl->l_tot[3], s);
+    nl += scan2_i32_to_i64(a.pcost, a.ppre, &a.ctl->l_tot[1], a.ccnt, a.cpre, &a.ctl->l_tot[3], &a.ctl->l_len[1],
+                           a.bsum, sg, s);
     pdl_launch(k_loc_check_pairs, dim3(1), dim3(32), 0, s, a.ctl, a.cap);
     pdl_launch(k_loc_common, dim3(gw), dim3(tpb), 0, s, a.ctl, V, a.srcA, a.dstA, a.srcD, a.dstD, a.ppre, a.rec);
     nl += 2;

@@ -139,27 +139,50 @@ __device__ __forceinline__ long long block_incl_scan_i64(long long x, long long*
     return r;
 }
 
-__global__ void __launch_bounds__(SC_BLOCK) k_scan_partials(const int32_t* __restrict__ in, const long long* d_len,
+// One or two scans of the same length in a launch (blockIdx.y picks one).
+struct ScanJob {
+    const int32_t* in;
+    long long* out;
+    long long* total;
+};
+constexpr int SC_SUMS = 1024;  // bsum words per scan
+
+// a block's part of the entries, from a multiple of four
+__device__ __forceinline__ void scan_chunk(long long n, long long& beg, long long& end) {
+    const long long chunk = ((n + gridDim.x - 1) / gridDim.x + 3) & ~3ll;
+    beg = min(n, (long long)blockIdx.x * chunk);
+    end = min(n, beg + chunk);
+}
+
+__global__ void __launch_bounds__(SC_BLOCK) k_scan_partials(ScanJob j0, ScanJob j1, const long long* d_len,
                                                            long long host_len, long long* __restrict__ bsum) {
     pdl_enter();
     __shared__ long long sh[32];
+    const int32_t* __restrict__ in = (blockIdx.y ? j1 : j0).in;
     long long n = d_len ? *d_len : host_len;
     long long beg, end;
-    chunk_of(n, beg, end);
+    scan_chunk(n, beg, end);
     long long s = 0;
+#pragma unroll 4
     for (long long i = beg + threadIdx.x; i < end; i += SC_BLOCK) s += in[i];
     s = block_incl_scan_i64(s, sh);
-    if (threadIdx.x == SC_BLOCK - 1) bsum[blockIdx.x] = s;
+    if (threadIdx.x == SC_BLOCK - 1) bsum[SC_SUMS * blockIdx.y + blockIdx.x] = s;
 }
 
-__global__ void __launch_bounds__(SC_BLOCK) k_scan_apply(const int32_t* __restrict__ in, long long* __restrict__ out,
-                                                        const long long* d_len, long long host_len,
-                                                        const long long* __restrict__ bsum, long long* total_out) {
+// Four entries a thread and tile: the tiles of a block are a chain of five
+// barriers each (10,000 pairs on 7,000 vertices: normalisation 60 -> 50 us,
+// with two scans in one launch).
+__global__ void __launch_bounds__(SC_BLOCK) k_scan_apply(ScanJob j0, ScanJob j1, const long long* d_len,
+                                                        long long host_len, const long long* __restrict__ bsum) {
     pdl_enter();
     __shared__ long long sh[32];
+    const ScanJob j = blockIdx.y ? j1 : j0;
+    const int32_t* __restrict__ in = j.in;
+    long long* __restrict__ out = j.out;
+    bsum += SC_SUMS * blockIdx.y;
     long long n = d_len ? *d_len : host_len;
     long long beg, end;
-    chunk_of(n, beg, end);
+    scan_chunk(n, beg, end);
     // the chunks before this one (at most 1,024 sums: two loads a thread, in
     // place of a kernel that scans them)
     __shared__ long long s_run;
@@ -169,11 +192,30 @@ __global__ void __launch_bounds__(SC_BLOCK) k_scan_apply(const int32_t* __restri
     if (threadIdx.x == SC_BLOCK - 1) s_run = before;
     __syncthreads();
     long long run = s_run;
-    for (long long tile = beg; tile < end; tile += SC_BLOCK) {
-        long long i = tile + threadIdx.x;
-        long long x = i < end ? in[i] : 0;
-        long long inc = block_incl_scan_i64(x, sh);
-        if (i < end) out[i] = run + inc - x;
+    const bool wide = (((uintptr_t)in | (uintptr_t)out) & 15) == 0;
+    for (long long tile = beg; tile < end; tile += 4 * SC_BLOCK) {
+        const long long i = tile + 4 * threadIdx.x;
+        int4 x = make_int4(0, 0, 0, 0);
+        if (wide && i + 3 < end) {
+            x = *(const int4*)(in + i);
+        } else {
+            if (i < end) x.x = in[i];
+            if (i + 1 < end) x.y = in[i + 1];
+            if (i + 2 < end) x.z = in[i + 2];
+            if (i + 3 < end) x.w = in[i + 3];
+        }
+        const long long mine = (long long)x.x + x.y + x.z + x.w;
+        const long long inc = block_incl_scan_i64(mine, sh);
+        const long long o0 = run + inc - mine, o1 = o0 + x.x, o2 = o1 + x.y, o3 = o2 + x.z;
+        if (wide && i + 3 < end) {
+            *(longlong2*)(out + i) = make_longlong2(o0, o1);
+            *(longlong2*)(out + i + 2) = make_longlong2(o2, o3);
+        } else {
+            if (i < end) out[i] = o0;
+            if (i + 1 < end) out[i + 1] = o1;
+            if (i + 2 < end) out[i + 2] = o2;
+            if (i + 3 < end) out[i + 3] = o3;
+        }
         // total of this tile = inclusive value of the last thread
         __shared__ long long tile_total;
         if (threadIdx.x == SC_BLOCK - 1) tile_total = inc;
@@ -182,8 +224,10 @@ __global__ void __launch_bounds__(SC_BLOCK) k_scan_apply(const int32_t* __restri
         __syncthreads();
     }
     if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) {
+        // (with chunks of whole fours the last blocks may be empty; their run
+        // is the total all the same)
         out[n] = run;
-        if (total_out) *total_out = run;
+        if (j.total) *j.total = run;
     }
 }
 
@@ -231,11 +275,22 @@ int scan_grid(long long max_len, int sms) {
     return (int)g;
 }
 
+static int scan_jobs(const ScanJob& a, const ScanJob& b, int jobs, const long long* d_len, long long host_len,
+                     long long* bsum, int grid, cudaStream_t s) {
+    pdl_launch(k_scan_partials, dim3(grid, jobs), dim3(SC_BLOCK), 0, s, a, b, d_len, host_len, bsum);
+    pdl_launch(k_scan_apply, dim3(grid, jobs), dim3(SC_BLOCK), 0, s, a, b, d_len, host_len, bsum);
+    return 2;
+}
+
 int scan_i32_to_i64(const int32_t* in, long long* out, const long long* d_len, long long host_len, long long* bsum,
                     int grid, long long* total_out, cudaStream_t s) {
-    pdl_launch(k_scan_partials, dim3(grid), dim3(SC_BLOCK), 0, s, in, d_len, host_len, bsum);
-    pdl_launch(k_scan_apply, dim3(grid), dim3(SC_BLOCK), 0, s, in, out, d_len, host_len, bsum, total_out);
-    return 2;
+    const ScanJob j{in, out, total_out};
+    return scan_jobs(j, j, 1, d_len, host_len, bsum, grid, s);
+}
+
+int scan2_i32_to_i64(const int32_t* in0, long long* out0, long long* total0, const int32_t* in1, long long* out1,
+                     long long* total1, const long long* d_len, long long* bsum, int grid, cudaStream_t s) {
+    return scan_jobs(ScanJob{in0, out0, total0}, ScanJob{in1, out1, total1}, 2, d_len, 0, bsum, grid, s);
 }
 
 }  // namespace gcx
