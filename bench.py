@@ -57,20 +57,15 @@ BENCH = {
 }
 STAGES = ["normalise", "region", "union_graph", "triangles_k4", "four_cycles", "terms_closed_forms", "commit"]
 KERNEL_OF_STAGE = {3: "k_tri_warp + k_tri_block + k_tri_merge (triangles, 4-cliques)",
-                   4: "k_c4_reg + k_c4_warp + k_c4_block + k_c4_dense + k_c4_hash (4-cycles)"}
-HEAVY_KERNEL = "k_c4_dense_t (heavy 4-cycle pivots; with k_c4_chunk when the tuning enables it)"
-# L2 atomic throughput of this GPU, measured by a probe kernel: random 32-bit
-# updates from 1,024-thread CTAs on every SM into 19 per-cluster arrays of
-# 3.2 MB (61 MB in all, the footprint of the heavy-pivot kernel's counters
-# on the 1.6M-vertex graph): reductions that return nothing, and atomics
-# that return the old value
-PROBE_L2_RED_PER_S = 125e9
-PROBE_L2_ATOM_PER_S = 134.5e9
-# DRAM bytes (read + written) per wedge of the heavy-pivot kernel, from one
-# ncu capture of it on the half-size graph (n=800,000 m=15M, same generator):
-# 1.403 GB over 1.302e9 wedges;
-# None once the kernel changes
-HEAVY_DRAM_BYTES_PER_WEDGE = (1.399486e9 + 3.768832e6) / 1.301926991e9
+                   4: "k_c4_reg + k_c4_warp + k_c4_table + k_c4_pivot (4-cycles)"}
+HEAVY_KERNEL = "k_c4_pivot (4-cycle pivots counted in shared memory)"
+# shared-memory atomic throughput of this GPU, measured by a probe kernel:
+# random 32-bit updates from 1,024-thread blocks on every SM
+PROBE_SHARED_ATOM_PER_S = 1.8e12
+# DRAM bytes (read + written) per wedge of that kernel, from one ncu capture
+# of it on the half-size graph (n=800,000 m=15M, same generator): 0.830 GB
+# over 1.345e9 wedges; None once the kernel changes
+HEAVY_DRAM_BYTES_PER_WEDGE = (826.703360e6 + 3.603712e6) / 1.345478987e9
 WORKLOADS_DESC_C4 = ("Chung-Lu n=2.4M m=5M gamma=1.8 dmax=100,000; 64 independent batches, sizes log-uniform "
                      "10..50,000, 50% ins / 50% del")
 
@@ -283,7 +278,7 @@ def stage_means(recs):
 def roofline(recs, peak, peak_kind):
     """Dominant counting kernel: algorithmic bytes = 4 bytes per adjacency
     element the kernel's method reads (triangles: |N+(u)| + |N+(v)| per
-    out-edge; 4-cycles: one element per wedge), over its CUDA-event time."""
+    out-edge; 4-cycles: one element per wedge), over its time on the device's clock."""
     sm = stage_means(recs)
     k = 3 if sm[3] >= sm[4] else 4
     work = statistics.mean(r["stats"]["work_triangles"] if k == 3 else r["stats"]["work_wedges"] for r in recs)
@@ -297,17 +292,14 @@ def roofline(recs, peak, peak_kind):
 
 
 def heavy_roofline(recs, peak, peak_kind):
-    """Roofline of the dominant kernel: the heavy-pivot 4-cycle kernels,
-    timed by the library with CUDA events on the stream they run on
-    (gc_stats.ms_stage[7]; alone when the records come from a serial-count
-    handle).  Algorithmic bytes = 4 bytes per wedge they walk
-    (one adjacency element each).  Beside the HBM roofline, the L2-atomic
-    one: the counter updates they send to L2 over the time the probe rates
-    would need for them."""
+    """Roofline of the dominant kernel: the 4-cycle pivots counted in shared
+    memory, from the first of its launches to the end of the last on the
+    device's clock (gc_stats.ms_stage[7]; alone when the records come from a
+    serial-count handle).  Algorithmic bytes = 4 bytes per wedge they walk
+    (one adjacency element each).  Beside the HBM roofline, the one of the
+    shared-memory atomics: one counter update per wedge over the probe rate."""
     ms = statistics.mean(r["stats"]["ms_stage"][7] for r in recs)
     wedges = statistics.mean(r["stats"]["work_wedges_heavy"] for r in recs)
-    red = statistics.mean(r["stats"]["l2_red_heavy"] for r in recs)
-    atom = statistics.mean(r["stats"]["l2_atom_heavy"] for r in recs)
     bytes_ = 4.0 * wedges
     sec = ms / 1e3
     achieved = bytes_ / sec / 1e9 if sec > 0 else None
@@ -319,10 +311,9 @@ def heavy_roofline(recs, peak, peak_kind):
             "traffic": HEAVY_DRAM_BYTES_PER_WEDGE * wedges if HEAVY_DRAM_BYTES_PER_WEDGE else None,
             "traffic_source": "ncu dram__bytes_read.sum + dram__bytes_write.sum of one launch on the n=800,000 "
                               "m=15M graph, per wedge, times this launch's wedges",
-            "l2_atomics": {"reductions": red, "returning": atom,
-                           "ops_per_s": (red + atom) / sec if sec > 0 else None,
-                           "probe_red_per_s": PROBE_L2_RED_PER_S, "probe_atom_per_s": PROBE_L2_ATOM_PER_S,
-                           "frac": (red / PROBE_L2_RED_PER_S + atom / PROBE_L2_ATOM_PER_S) / sec if sec > 0 else None},
+            "shared_atomics": {"updates": wedges, "ops_per_s": wedges / sec if sec > 0 else None,
+                               "probe_ops_per_s": PROBE_SHARED_ATOM_PER_S,
+                               "frac": wedges / PROBE_SHARED_ATOM_PER_S / sec if sec > 0 else None},
             "stage_ms": dict(zip(STAGES, [round(x, 4) for x in sm]))}
 
 
@@ -544,8 +535,9 @@ def paper_regime(gcb, torch, n, keys, rp, col, stream, flush, static_ms):
 def local_counts_line(gcb, n, rp, col):
     """Per-vertex graphlet counts (gc_vertex_counts) and per-edge orbit
     counts (gc_edge_orbits) of the graph: device time of their kernels
-    (after the static pass they start from) and of that static pass; the
-    sums over vertices and over edges checked against the global counts."""
+    (the static pass that they start from, which credits the 4-cycles,
+    included) and of a plain static pass; the sums over vertices and over
+    edges checked against the global counts."""
     per_orbit = [(0, 2), (0, 1), (1, 3), (2, 4), (3, 1), (3, 1), (3, 2), (4, 4), (4, 1), (5, 6)]
     with gcb.Graph(n, rp, col) as g:
         g.vertex_counts()  # warm-up

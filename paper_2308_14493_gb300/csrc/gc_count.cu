@@ -123,9 +123,10 @@ __device__ __forceinline__ int wedge_bucket(long long w) {
 // plan its chunks, are made here, so that the plan need not wait for the bins.
 constexpr int WB_LONG = 256;
 constexpr int WB_LONGS = 256;  // a block's list of them (a warp takes each further one)
-__global__ void __launch_bounds__(256) k_wedge_bound(Ctl* c, const int32_t* __restrict__ wlist, const long long* __restrict__ U_off,
-                              const uint32_t* __restrict__ U_col, const int32_t* __restrict__ U_split,
-                              long long* __restrict__ U_wt, Tuning t) {
+__global__ void __launch_bounds__(256)
+    k_wedge_bound(Ctl* c, const int32_t* __restrict__ wlist, const long long* __restrict__ U_off,
+                  const uint32_t* __restrict__ U_col, const int32_t* __restrict__ U_split,
+                  long long* __restrict__ U_wt, Tuning t) {
     pdl_enter();
     const int nW = c->nW;
     const int lane = threadIdx.x & 31;

@@ -36,6 +36,9 @@
 // w and its two middle vertices (or its four edges).  Once a task's c_w are
 // known, a second walk adds c_w - 1 to each middle vertex (to both edges of
 // each wedge), and the sweep that clears the counters adds C(c_w, 2) to w.
+// On the 1.6M/30M graph the pivots take 24 ms with the credits per vertex, 11.7
+// without; 33.5 when the sweep looked at every counter of a word and runs were
+// summed by shuffles.
 #include <algorithm>
 
 #include "gc_c4.cuh"

@@ -44,9 +44,9 @@ def main():
     ap.add_argument("--heavy-min", default="",
                     help="with --vertex / --edge: comma-separated local_c4_heavy_min values, each timed in turn")
     ap.add_argument("--chunk-threshold", type=int, default=0,
-                    help="wedge bound above which 4-cycle pivots use the chunked shared-memory kernel")
+                    help="gc_options.chunk_threshold (accepted; no effect)")
     ap.add_argument("--tuning", default="", help="JSON object of bin boundaries to set after the open "
-                                                 "(e.g. '{\"c4_chunk_min\": 262144}'), applied after --autotune")
+                                                 "(e.g. '{\"c4_cta_max\": 8192}'), applied after --autotune")
     a = ap.parse_args()
     keys = gen.chung_lu_graph(a.n, a.m, a.gamma, a.dmax, a.seed)
     rp, col = gen.csr_from_keys(a.n, keys)
