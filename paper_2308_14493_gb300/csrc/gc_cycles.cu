@@ -96,7 +96,7 @@ __global__ void __launch_bounds__(PLAN_TILE) k_c4_plan(Ctl* c, const long long* 
     long long cmass = 0, limit = entries;
     {
         const double fair = (double)c->c4_wt / ctas, big = 2.0 * (double)c->c4_wmax;
-        if (big > fair) limit = (long long)((double)entries * fmax(fair / big, 0.125));
+        if (big > fair) limit = max(1ll, (long long)((double)entries * fmax(fair / big, 0.125)));
     }
     if (!gmax) {
         const int t = threadIdx.x, k = (int)((entries + limit - 1) / limit);
@@ -716,6 +716,7 @@ C4Geom c4_geom(long long n, int sms) {
     g.ctas = small ? 3 * sms : sms;
     g.gran = 64;
     while (g.gran < n / 512 && g.gran < 32768) g.gran <<= 1;
+    while (g.narrow && (long long)g.gran * PLAN_TILE < n) g.gran <<= 1;  // k_c4_plan: a thread per granule
     g.ngran = (int)((n + g.gran - 1) / g.gran);
     const long long least = (g.narrow ? 2ll * g.words : (long long)g.words) - g.gran + 1;
     g.nchmax = (int)(n / std::max<long long>(least, 1)) + 1 + C4_SPLITS;

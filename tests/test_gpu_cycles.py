@@ -147,3 +147,14 @@ def test_local_pairs_between_mid_vertices_under_hubs(gcb, mid_degree, hub_degree
         assert g.apply(ins, dels) == r["F"]
         assert g.stats()["path"] == 1
         assert g.apply(dels, ins) == F0
+
+
+# a plan with one thread per granule of ids: around the number of ids that
+# fills its threads (512 granules of 64)
+@pytest.mark.parametrize("n", [32767, 32768, 32769, 33279, 33280])
+def test_pivot_plans_cover_every_id(gcb, n):
+    keys = hub_graph(n, 2 * n, 4000, n)
+    rp, col = gen.csr_from_keys(n, keys)
+    with gcb.Graph(n, rp, col) as g:
+        g.set_tuning(**ALL_DENSE)
+        assert g.count_static() == oracle.static_counts(rp, col)
