@@ -214,11 +214,11 @@ __device__ __forceinline__ uint32_t counters_above_1(uint32_t w, int s) {
 }
 
 // The pivots of BIN_C4_DENSE, a block per (chunk, pivot).  Bound by issue
-// slots (about 60 instructions per 32 wedges, a third of them the short
-// runs' bookkeeping) and by the chain of three loads that starts each group
-// of lower neighbours.  The counters are cleared by a fill, or, when the task
-// has few wedges for its counters, by walking them again.  MODE: C4_COUNT,
-// C4_VERTEX or C4_EDGE (credits; every entry is then in both graphs).
+// slots (78 instructions per 32 wedges, 68 % of the cycles issue) and by the
+// chain of three loads that starts each group of lower neighbours.  The
+// counters are cleared by a fill, or, when the task has few wedges for its
+// counters, by walking them again.  MODE: C4_COUNT, C4_VERTEX or C4_EDGE
+// (credits; every entry is then in both graphs).
 // Measured (pivots above w~ = 19,456, kernel alone): 11.7 ms for 2.85e9 wedges
 // of the 1.6M/30M graph, where L2 reductions by clusters of eight blocks took
 // 30 ms; 2.8 ms against 11 for 1.09e9 wedges of the 2.4M/5M graph with hubs of
